@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <vector>
 
@@ -602,10 +603,18 @@ static void head_granules(const wnw_cache *c, int layer, int mode, const SeqHost
 // single piece of the same size).  So heads are cut as little as the balance allows: for a piece size T a head becomes
 // round(work / T) even pieces (at least one), the pieces go longest-first to the least loaded CTA, and T is the candidate
 // between 0.3 and three even shares of the launch that gives the shortest longest CTA under that cost model.
+struct CutMemo {   // piece sizes found for one work list, by the launch's head sizes
+  struct Entry { std::vector<int> sizes; double T; };
+  std::vector<Entry> entries;
+  const Entry *find(const std::vector<int> &sizes) const {
+    for (const Entry &e : entries) if (e.sizes == sizes) return &e;
+    return nullptr;
+  }
+};
 static void build_throughput_items(const wnw_cache *c, int layer, int mode, const std::vector<int> &seq_ids,
                                    const std::vector<int> &n_gran, const std::vector<int> &n_work, std::vector<WorkItem> &items,
                                    std::vector<HeadItems> &heads, LayerWork &lw, std::vector<int32_t> &order,
-                                   std::vector<int32_t> &ranges) {
+                                   std::vector<int32_t> &ranges, CutMemo *memo) {
   const Geometry &G = c->geo;
   const int nw = attn_warps(true), n_heads = (int)seq_ids.size() * G.Hkv;
   const double cost_whole = 5.0, cost_piece = 16.0;   // fixed cost of an item in granules' worth: finished in the CTA / left as a partial
@@ -616,20 +625,55 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   const int P = (int)std::min<double>(per_sm * c->n_sm, std::max(1.0, total / (2.0 * nw)));   // at least two granules per warp and CTA
   const bool may_finish = mode != ATTN_PREFILL;       // the prefill scoring pass leaves partials whatever the cut
   auto pieces_of = [&](int hd, double T) { return std::max(1, (int)std::lround(n_work[hd] / T)); };
+  // Longest-first onto the least loaded CTA (the lower index on equal loads).  The pieces of a head cost the same, so heads are
+  // sorted instead of pieces; as long as all loads are equal a run of equal pieces goes round robin (one division, which is
+  // the whole assignment where all heads are alike); after that a heap finds the least loaded CTA.
+  struct Run { double cost; int hd, np; };
+  std::vector<Run> runs(n_heads);
+  std::vector<double> load(P);
+  typedef std::pair<double, int> Slot;
+  std::vector<Slot> heap;
   auto makespan = [&](double T, std::vector<std::vector<std::pair<int, int>>> *assign) {
-    std::vector<std::pair<double, std::pair<int, int>>> its;   // cost, (head, piece)
     for (int hd = 0; hd < n_heads; ++hd) {
       const int np = pieces_of(hd, T);
-      for (int x = 0; x < np; ++x)
-        its.push_back({(double)n_work[hd] / np + ((np > 1 || !may_finish) ? cost_piece : cost_whole), {hd, x}});
+      runs[hd] = Run{(double)n_work[hd] / np + ((np > 1 || !may_finish) ? cost_piece : cost_whole), hd, np};
     }
-    std::stable_sort(its.begin(), its.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
-    std::vector<double> load(P, 0.0);
+    std::stable_sort(runs.begin(), runs.end(), [](const Run &x, const Run &y) { return x.cost > y.cost; });
     if (assign) assign->assign(P, {});
-    for (const auto &e : its) {
-      const int cta = (int)(std::min_element(load.begin(), load.end()) - load.begin());
-      load[cta] += e.first;
-      if (assign) (*assign)[cta].push_back(e.second);
+    size_t r = 0;
+    int next = 0;          // the CTA whose turn it is while all loads are equal but for one piece
+    double level = 0.0;    // load of the CTAs from `next` on
+    while (r < runs.size()) {
+      long long n = 0;
+      size_t e = r;
+      for (; e < runs.size() && runs[e].cost == runs[r].cost; ++e) n += runs[e].np;
+      if (assign) {
+        int cta = 0;
+        for (size_t x = r; x < e; ++x)
+          for (int y = 0; y < runs[x].np; ++y) { (*assign)[cta].push_back({runs[x].hd, y}); cta = cta + 1 == P ? 0 : cta + 1; }
+      }
+      level += (double)(n / P) * runs[r].cost;
+      next = (int)(n % P);
+      const double step = runs[r].cost;
+      r = e;
+      if (next == 0) continue;
+      for (int x = 0; x < P; ++x) load[x] = x < next ? level + step : level;
+      break;
+    }
+    if (next == 0) load.assign(P, level);
+    else if (r < runs.size()) {
+      heap.resize(P);
+      for (int x = 0; x < P; ++x) heap[x] = Slot(load[x], x);
+      std::make_heap(heap.begin(), heap.end(), std::greater<Slot>());
+      for (; r < runs.size(); ++r)
+        for (int y = 0; y < runs[r].np; ++y) {
+          std::pop_heap(heap.begin(), heap.end(), std::greater<Slot>());
+          Slot &s = heap.back();
+          s.first += runs[r].cost;
+          if (assign) (*assign)[s.second].push_back({runs[r].hd, y});
+          std::push_heap(heap.begin(), heap.end(), std::greater<Slot>());
+        }
+      for (const Slot &s : heap) load[s.second] = s.first;
     }
     // the longest CTA bounds the launch; the mean load counts too: while some CTAs sit in item overheads the others can
     // only use the bandwidth they leave if there is work left to overlap, so overhead is never free
@@ -638,10 +682,25 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
     return *std::max_element(load.begin(), load.end()) + mean_weight * sum / P;
   };
   const double share = std::max(total / P, (double)(4 * nw));
-  double best_T = share, best = 1e300;
-  for (int k = 6; k <= 60; ++k) {   // T from 0.3 to three shares in steps of 5 %; ties go to the larger T (fewer items)
-    const double T = share * k / 20.0, ms = makespan(T, nullptr);
-    if (ms <= best) { best = ms; best_T = T; }
+  // Layers of a stack differ in which heads play which role, hardly ever in how many play it: the search depends on the
+  // launch's head sizes alone and is made once for all layers of a list.
+  std::vector<int> sizes(n_work.begin(), n_work.begin() + n_heads);
+  std::sort(sizes.begin(), sizes.end());
+  double best_T = share;
+  const CutMemo::Entry *known = memo ? memo->find(sizes) : nullptr;
+  if (known) best_T = known->T;
+  else {
+    double best = 1e300;
+    std::vector<int> np_now(n_heads), np_last;
+    for (int k = 6; k <= 60; ++k) {   // T from 0.3 to three shares in steps of 5 %; ties go to the larger T (fewer items)
+      const double T = share * k / 20.0;
+      for (int hd = 0; hd < n_heads; ++hd) np_now[hd] = pieces_of(hd, T);
+      if (np_now == np_last) continue;   // cuts every head as the candidate before it
+      const double ms = makespan(T, nullptr);
+      if (ms <= best) { best = ms; best_T = T; }
+      np_last = np_now;
+    }
+    if (memo) memo->entries.push_back(CutMemo::Entry{sizes, best_T});
   }
   std::vector<std::vector<std::pair<int, int>>> assign;
   makespan(best_T, &assign);
@@ -680,7 +739,7 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
 // Appends the items of one layer for the given sequences.
 static void build_layer_items(const wnw_cache *c, int layer, int mode, const std::vector<int> &seq_ids,
                               std::vector<WorkItem> &items, std::vector<HeadItems> &heads, LayerWork &lw,
-                              std::vector<int32_t> &order, std::vector<int32_t> &ranges) {
+                              std::vector<int32_t> &order, std::vector<int32_t> &ranges, CutMemo *memo = nullptr) {
   const Geometry &G = c->geo;
   // n_gran: the head's whole virtual key space (what the items must cover); n_work: the granules expected to hold data
   // (what the items are sized by): the dynamic slots of a SEGMENT_LAG table are about half empty and cost nothing then
@@ -721,7 +780,7 @@ static void build_layer_items(const wnw_cache *c, int layer, int mode, const std
   lw.head_items_off = (int)heads.size();
   lw.max_count = 0;
   if (throughput) {
-    build_throughput_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw, order, ranges);
+    build_throughput_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw, order, ranges, memo);
     return;
   }
   for (size_t i = 0; i < seq_ids.size(); ++i)
@@ -760,7 +819,7 @@ static void build_layer_items(const wnw_cache *c, int layer, int mode, const std
     items.resize(lw.first_item);
     heads.resize(lw.head_items_off);
     lw.throughput = true;
-    build_throughput_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw, order, ranges);
+    build_throughput_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw, order, ranges, memo);
     return;
   }
   if (!throughput && overlapped && attn_xpref_fits(G.g, G.d) &&
@@ -853,8 +912,9 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
     }
   }
   size_t part_total = 0;
+  CutMemo memo;
   for (int l = 0; l < G.L; ++l) {
-    build_layer_items(c, l, mode, c->active, items, heads, c->wl_layers[l], order, ranges);
+    build_layer_items(c, l, mode, c->active, items, heads, c->wl_layers[l], order, ranges, &memo);
     c->wl_layers[l].part_off = part_total;
     part_total += (size_t)c->wl_layers[l].n_items;
   }
