@@ -220,8 +220,12 @@ __device__ __forceinline__ GranDesc decode_granule(const CacheView &cv, const At
 //   (chunk, head, K|V).  The bytes become fp16 fragments on their way from ldmatrix to mma.sync (one conversion per two
 //   elements, exact), and the products with such a granule run on the fp16 form of mma.sync with q and P taken as fp16 (q
 //   exactly while its elements lie in fp16's normal range; P in [0,1] with three more mantissa bits than bf16 gives it).  The
-//   K scale multiplies the logits; the V scale enters the exponent of the granule's weights (see the softmax step).  The
-//   default path (VAR 0) carries none of either variant's branches.
+//   K scale multiplies the logits; the V scale enters the exponent of the granule's weights (see the softmax step).
+// VAR 3 (UNI): all heads are alike and cut into the same number of even pieces: a CTA's item follows from its index, no list
+//   is built, uploaded or read, and the grid is not bound by the length of one;
+// VAR 4 (UNI, KO): the prefill scoring pass: scores need K alone, so V is neither fetched nor multiplied and a warp's ring
+//   holds twice the granules; grid row y scores text query y.
+//   The default path (VAR 0) carries none of any variant's branches.
 // bid: the CTA's index within its layer's launch (a launch may carry the CTAs of several layers back to back);
 // inl: the layer's work items when they travel in the kernel parameters, else null (read from a.items).
 template <int D, bool G16, int NW, int VAR>
@@ -237,8 +241,9 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   constexpr int PPR = D / 8;              // 16-byte pieces per row
   constexpr int KK = D / 16;              // k16 steps of QK^T; also pairs of n8 tiles of PV
   constexpr int NQ = G16 ? 4 : 2;
-  constexpr bool TB = VAR == 1, F8 = VAR == 2;
-  constexpr int NSTAGE = nstage_of(NW);
+  constexpr bool TB = VAR == 1, F8 = VAR == 2, UNI = VAR == 3 || VAR == 4, KO = VAR == 4;
+  constexpr int NSTAGE = KO ? 2 * nstage_of(NW) : nstage_of(NW);
+  constexpr int STAGEB = KO ? TILEB : 2 * TILEB;   // a stage holds a granule's K rows, then its V rows
   static_assert(!F8 || D == 128, "an e4m3 row must fill one 128-byte swizzle atom");
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -261,7 +266,8 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   __shared__ int2 ring[NW][NSTAGE];                              // per stage: visible rows | loaded << 8, score index
   __shared__ __align__(8) unsigned long long bars[NW][NSTAGE];   // one mbarrier per stage, producer = consumer = this warp
   __shared__ int s_flag;
-  const uint32_t my_base = smem_u32(smem + (size_t)warp * NSTAGE * 2 * TILEB);
+  if (VAR == 3) asm volatile("griddepcontrol.wait;\n" ::: "memory");   // the caller's buffer may be what the preceding work wrote
+  const uint32_t my_base = smem_u32(smem + (size_t)warp * NSTAGE * STAGEB);
   if (lane == 0) {
 #pragma unroll
     for (int st = 0; st < NSTAGE; ++st) mbar_init(smem_u32(&bars[warp][st]), 1);
@@ -281,7 +287,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   // One work item per CTA when the launch fits the machine; otherwise a persistent CTA per SM walks the items the
   // host assigned to it (balanced by size), so no SM idles through a partial last wave.
   int q_begin = bid, q_end = bid + 1;
-  if (a.cta_ranges) { q_begin = a.cta_ranges[bid]; q_end = a.cta_ranges[bid + 1]; }
+  if (!UNI && a.cta_ranges) { q_begin = a.cta_ranges[bid]; q_end = a.cta_ranges[bid + 1]; }
 
   // What a warp needs to address the granules of one work item.
   struct Ctx {
@@ -314,15 +320,24 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   };
   int parity_b = -1, parity_v = 0;   // slot-table copy of the sequence whose tidal items this CTA is serving
   auto load_ctx = [&](Ctx &c, int qi, bool for_loads) {
-    c.item_idx = a.cta_ranges ? a.order[qi] : qi;
-    // short item lists travel in the kernel parameters: no global load before the first K/V load is issued
-    c.it = (inl && a.n_items <= INLINE_ITEMS_MAX) ? inl->it[c.item_idx] : a.items[c.item_idx];
-    c.T_t = cv.text_len[c.it.b] + a.has_new;
+    if constexpr (UNI) {
+      const int np = a.uni.hd_count, h = qi / np, x = qi - h * np, n = a.uni.g1;
+      c.item_idx = qi;
+      c.it = a.uni;
+      c.it.h = c.it.ridx = h; c.it.hd_first = h * np;
+      c.it.g0 = (int)((long long)n * x / np); c.it.g1 = (int)((long long)n * (x + 1) / np);
+      c.T_t = a.uni.T_hint;   // exact: nothing is appended
+    } else {
+      c.item_idx = a.cta_ranges ? a.order[qi] : qi;
+      // short item lists travel in the kernel parameters: no global load before the first K/V load is issued
+      c.it = (inl && a.n_items <= INLINE_ITEMS_MAX) ? inl->it[c.item_idx] : a.items[c.item_idx];
+      c.T_t = cv.text_len[c.it.b] + a.has_new;
+    }
     if (c.it.role == ROLE_ANCHOR) { c.v_delta_audio = G.T_a_pad; c.map_audio = &maps.anchor; }       // rows between a
     else if (c.it.role == ROLE_TIDAL) { c.v_delta_audio = G.ncp; c.map_audio = &maps.pool; }          // granule's K and
     else { c.v_delta_audio = G.FB * G.ncp; c.map_audio = &maps.fixed; }                            // V rows
     c.m_full = c.m_tail = 0;
-    if (c.it.role == ROLE_TIDAL && cv.steps && c.it.b != parity_b) {   // once per sequence a CTA serves, not per item
+    if (!UNI && c.it.role == ROLE_TIDAL && c.it.b != parity_b) {   // once per sequence a CTA serves, not per item
       parity_b = c.it.b;
       parity_v = (int)(cv.steps[c.it.b] & 1);
     }
@@ -391,15 +406,15 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
     // The boxes of a granule (K and V, HALVES each) are issued by as many lanes at once, one box per lane: lane = 2 * half + (V).
     // The stage's barrier cannot complete before lane 0 has arrived with the byte count, whichever copy lands first.
     const bool f8g = F8 && !is_text && c.it.role == ROLE_TIDAL;   // an e4m3 granule: one box of 16 rows x 128 bytes each for K and V
-    if (load && lane < (f8g ? 2 : 2 * HALVES)) {
+    if (load && lane < (KO ? HALVES : f8g ? 2 : 2 * HALVES)) {
       const int stage = (int)(seq % NSTAGE);
       const uint32_t bar = smem_u32(&bars[warp][stage]);
       const CUtensorMap *map = is_text ? &maps.text : (base_blk ? &maps.fixed : c.map_audio);
       const int v_delta = is_text ? v_delta_text : (base_blk ? G.FB * G.ncp : c.v_delta_audio);
-      const int hf = lane >> 1, isv = lane & 1;
+      const int hf = KO ? lane : lane >> 1, isv = KO ? 0 : lane & 1;
       fence_proxy_async();  // the stage was last read through the generic proxy (ldmatrix)
-      if (lane == 0) mbar_expect_tx(bar, f8g ? 2 * HALFB : 2 * TILEB);
-      tma_load_2d(my_base + stage * 2 * TILEB + isv * TILEB + hf * HALFB, map, hf * 64, row + isv * v_delta, bar);
+      if (lane == 0) mbar_expect_tx(bar, f8g ? 2 * HALFB : STAGEB);
+      tma_load_2d(my_base + stage * STAGEB + isv * TILEB + hf * HALFB, map, hf * 64, row + isv * v_delta, bar);
     }
     return load;
   };
@@ -455,8 +470,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   }
   const WorkItem &it = cc.it;
   const int item_idx = cc.item_idx;
-  if (cv.step_snap && it.h == 0 && it.g0 == 0 && threadIdx.x == 0 && a.mode != ATTN_PREFILL)   // (no cache state behind the
-    cv.step_snap[(long long)it.b * G.L + a.layer] = cv.steps[it.b];                            //  allocation-free entry)
+  if (!UNI && it.h == 0 && it.g0 == 0 && threadIdx.x == 0) cv.step_snap[(long long)it.b * G.L + a.layer] = cv.steps[it.b];
   const int b = it.b, ridx = it.ridx, T_t = cc.T_t;
   const int first = cc.first, n_my = cc.n_my;
 #ifdef WNW_PHASE_STAMPS
@@ -493,7 +507,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
           else { phase_bits ^= 1u << stage; prewaited |= 1u << stage; }
         }
         if (valid > 0 && valid < GR && !timed_out) {
-          const uint32_t sVz = my_base + stage * 2 * TILEB + TILEB;
+          const uint32_t sVz = my_base + stage * STAGEB + TILEB;
           for (int r = valid + (lane >> 3); r < GR; r += 4)
 #pragma unroll
             for (int hf = 0; hf < HALVES; ++hf)
@@ -525,7 +539,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   const int r0 = lane >> 2, cq = (lane & 3) * 2;
   uint32_t qa[KK][NQ];
   {
-    const bf16 *qb = a.q + ((long long)it.i * G.Hq + (long long)it.h * g) * D;
+    const bf16 *qb = a.q + ((long long)(KO ? blockIdx.y : it.i) * G.Hq + (long long)it.h * g) * D;
 #pragma unroll
     for (int kk = 0; kk < KK; ++kk) {
       qa[kk][0] = r0 < g ? __ldcg(reinterpret_cast<const uint32_t *>(qb + r0 * D + kk * 16 + cq)) : 0u;
@@ -690,7 +704,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
           }
           if (r0 == 0) {
             const int hq = nt * 8 + cq;
-            float2 *ge = a.gran_em + ((long long)it.i * a.n_aq + (long long)ridx * g + hq) * a.n_ag_max + sidxs[u];
+            float2 *ge = a.gran_em + ((long long)(KO ? blockIdx.y : it.i) * a.n_aq + (long long)ridx * g + hq) * a.n_ag_max + sidxs[u];
             if (hq < g) ge[0] = make_float2(eA, mnA);
             if (hq + 1 < g) ge[a.n_ag_max] = make_float2(eB, mnB);
           }
@@ -710,7 +724,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       for (int t = 0; t < D / 16; ++t) { oT[nt][t][0] *= alA; oT[nt][t][1] *= alB; oT[nt][t][2] *= alA; oT[nt][t][3] *= alB; }
     }
     STAMP(26);
-    {
+    if constexpr (!KO) {
       const int mtx = lane >> 3;
       const uint32_t lane_v = (uint32_t)((((mtx & 1) << 3) + (lane & 7)) * 128 + (((mtx >> 1) ^ (lane & 7)) << 4));   // as lane_k above
       auto pv_bf16 = [&](int t2, int u) {
@@ -777,7 +791,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
         if (!timed_out) ++adv;
         if (n == 0 && u == 0) STAMP(24);
         if (valid > 0 && !timed_out) {
-          const uint32_t sK = my_base + stage * 2 * TILEB, sV = sK + TILEB;
+          const uint32_t sK = my_base + stage * STAGEB, sV = sK + TILEB;
           // the row of the token being generated: take it from k_new/v_new and store it into the text region
           const int j = first + (n + u) * NW;
           if (j == new_j) {
@@ -791,7 +805,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
               asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst), "r"(val.x), "r"(val.y), "r"(val.z), "r"(val.w) : "memory");
             }
           }
-          if (valid < GR && !pre) {
+          if (!KO && valid < GR && !pre) {
             // rows past the visible ones get probability 0, but 0 x NaN is NaN and a caller-owned buffer (the allocation-free
             // entry) may hold anything there: clear those V rows (a masked K row only spoils logits that are replaced anyway)
             for (int r = valid + (lane >> 3); r < GR; r += 4)
@@ -833,7 +847,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   // ---- merge the warps' partial states through shared memory ----
   // scratch: behind the stages when the pipeline runs across items (copies of the next item are landing in them),
   // otherwise the stages themselves, which are idle by now
-  unsigned char *scratch = xpref ? smem + (size_t)NW * NSTAGE * 2 * TILEB : smem;
+  unsigned char *scratch = xpref ? smem + (size_t)NW * NSTAGE * STAGEB : smem;
   constexpr int RS = D + 2;   // row stride of red_o in floats: spreads the transposed accumulators' stores over the banks (two-way
                               // conflicts left; four more bytes per row and a group of 8 heads no longer fits behind the stages)
   float2 *red_ml = reinterpret_cast<float2 *>(scratch);                           // [NW][16]
@@ -845,6 +859,19 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       red_ml[warp * 16 + nt * 8 + cq + 1] = make_float2(mrun[nt][1], lrun[nt][1]);
     }
     if (!G16) { red_ml[warp * 16 + 8 + cq] = make_float2(-INFINITY, 0.f); red_ml[warp * 16 + 9 + cq] = make_float2(-INFINITY, 0.f); }
+  }
+  if constexpr (KO) {   // a head's share of (max, denominator): all that the placement needs of a piece
+    __syncthreads();
+    if (threadIdx.x < g) {
+      float M = -INFINITY, L = 0.f;
+#pragma unroll
+      for (int w = 0; w < NW; ++w) M = fmaxf(M, red_ml[w * 16 + threadIdx.x].x);
+      if (M > -INFINITY)
+#pragma unroll
+        for (int w = 0; w < NW; ++w) L += red_ml[w * 16 + threadIdx.x].y * exp2f(red_ml[w * 16 + threadIdx.x].x - M);
+      a.part_ml[((long long)blockIdx.y * gridDim.x + item_idx) * g + threadIdx.x] = make_float2(M, L);
+    }
+    continue;
   }
 #pragma unroll
   for (int nt = 0; nt < NTN; ++nt) {
@@ -863,10 +890,10 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   }
   __syncthreads();
   // A head served by a single CTA is finished here (bf16 output, final max and denominator); otherwise the CTA
-  // leaves one partial in global memory.  The prefill scoring pass always leaves partials.
+  // leaves one partial in global memory.
   STAMP(20);
   const HeadItems hi{it.hd_first, it.hd_count};   // travels with the item: no load on the way to the merge
-  const bool direct = hi.count == 1 && a.mode != ATTN_PREFILL;
+  const bool direct = hi.count == 1;
   if (hi.count > 0) STAMP(21);
   for (int pr = threadIdx.x; pr < g * D / 2; pr += NW * 32) {
     const int idx = pr * 2, row = idx / D;
@@ -895,7 +922,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   }
   STAMP(3);
   KSTAMP_MAX(kslot, 2);
-  if (direct || a.mode == ATTN_PREFILL) continue;
+  if (direct) continue;
 
   // ---- the CTA that finishes this head last merges its split partials ----
   // Every thread's partial stores are ordered before the barrier; thread 0's fence after it makes them visible device-wide
@@ -990,6 +1017,14 @@ __global__ void __launch_bounds__(NW * 32, NW == NW_THR ? (G16 ? 2 : WNW_THR_CTA
   attn_body<D, G16, NW, VAR>(cv, a, &inl, maps, (int)blockIdx.x);
 }
 
+// All heads cut alike (VAR 3, 4): the item list is in the launch shape.
+template <int D, bool G16, int VAR>
+__global__ void __launch_bounds__(NW_LAT * 32, 1) wnw_attn_uniform_kernel(const __grid_constant__ CacheView cv,
+                                                                         const __grid_constant__ AttnArgs a,
+                                                                         const __grid_constant__ TmaMaps maps) {
+  attn_body<D, G16, NW_LAT, VAR>(cv, a, nullptr, maps, (int)blockIdx.x);
+}
+
 // The CTAs of several layers in one launch (layers whose inputs are all ready and whose outputs are read after the
 // step): CTA x belongs to the layer whose range of the prefix table holds x and does exactly what it would do in that
 // layer's own launch.
@@ -1044,6 +1079,34 @@ static cudaError_t launch_tb(const CacheView &cv, const AttnArgs &a, cudaStream_
   }
   return cudaLaunchKernelEx(&cfg, wnw_attn_kernel<D, G16, NW, VAR>, cv, a, inl, *a.maps);
 }
+static size_t uniform_smem(int d) { return (size_t)NW_LAT * nstage_of(NW_LAT) * 2 * GR * d * 2 + 1024; }
+template <int D, bool G16, int VAR>
+static cudaError_t launch_uniform_t(const CacheView &cv, const AttnArgs &a, int n_ctas, int n_rows, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)n_ctas, (unsigned)n_rows, 1);
+  cfg.blockDim = dim3(NW_LAT * 32, 1, 1);
+  cfg.dynamicSmemBytes = uniform_smem(D);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  if (a.pdl) {
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, wnw_attn_uniform_kernel<D, G16, VAR>, cv, a, *a.maps);
+}
+cudaError_t launch_attn_uniform(const CacheView &cv, const AttnArgs &a, int n_heads, int n_queries, cudaStream_t st) {
+  const int n = n_heads * a.uni.hd_count, d = cv.geo.d;
+  const bool g16 = cv.geo.g > 8;
+  if (!a.maps || n < 1 || n_queries < 1 || (d != 64 && d != 128)) return cudaErrorInvalidValue;
+  if (a.mode == ATTN_PREFILL) {
+    if (d == 128) return g16 ? launch_uniform_t<128, true, 4>(cv, a, n, n_queries, st) : launch_uniform_t<128, false, 4>(cv, a, n, n_queries, st);
+    return g16 ? launch_uniform_t<64, true, 4>(cv, a, n, n_queries, st) : launch_uniform_t<64, false, 4>(cv, a, n, n_queries, st);
+  }
+  if (d == 128) return g16 ? launch_uniform_t<128, true, 3>(cv, a, n, 1, st) : launch_uniform_t<128, false, 3>(cv, a, n, 1, st);
+  return g16 ? launch_uniform_t<64, true, 3>(cv, a, n, 1, st) : launch_uniform_t<64, false, 3>(cv, a, n, 1, st);
+}
+
 template <int D, bool G16, int NW>
 static cudaError_t launch_t(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
   if constexpr (D == 128)
@@ -1107,6 +1170,11 @@ static cudaError_t configure_t() {
   if (e != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(wnw_attn_multi_kernel<D, G16, NW, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(wnw_attn_multi_kernel<D, G16, NW, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e;
+  if constexpr (NW == NW_LAT) {
+    const int ub = (int)uniform_smem(D);
+    if ((e = cudaFuncSetAttribute(wnw_attn_uniform_kernel<D, G16, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, ub)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(wnw_attn_uniform_kernel<D, G16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, ub)) != cudaSuccess) return e;
+  }
   if constexpr (D == 128) {   // the e4m3 tidal tier
     if ((e = cudaFuncSetAttribute(wnw_attn_kernel<D, G16, NW, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(wnw_attn_multi_kernel<D, G16, NW, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e;

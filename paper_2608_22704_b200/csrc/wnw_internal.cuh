@@ -128,6 +128,11 @@ __host__ __device__ inline long long mirror_off(const Geometry &G, const LayerIn
   return (((long long)C_b * li.tid_prefix + (long long)c * li.n_tidal + t_idx) * 2 + kv) * G.ncp * G.d;
 }
 
+// the same inside one layer's part of the mirror (which is one contiguous run, chunk by chunk)
+__host__ __device__ inline long long mirror_block_off(const Geometry &G, const LayerInfo &li, int c, int t_idx, int kv) {
+  return (((long long)c * li.n_tidal + t_idx) * 2 + kv) * G.ncp * G.d;
+}
+
 // ---- e4m3 tidal tier ----
 // Offsets into the pool and the mirrors count ELEMENTS; an element is one byte there (two as bf16).
 __host__ __device__ inline int tidal_elem_bytes(const Geometry &G) { return G.kv8 ? 1 : 2; }
@@ -179,7 +184,7 @@ struct AttnArgs {
   int32_t pdl;                   // launch with programmatic stream serialization (previous stream op is a layer kernel)
   int xpref;        // the CTAs serve several work items each and keep their copy pipeline running across them
   int wait_inputs;  // q/k_new/v_new come from the preceding work on the stream: wait for it before reading them
-  const HeadItems *head_items;  // [n_active][Hkv] work items of each head (first is relative to `items`)
+  WorkItem uni;     // uniform launches: what all items share; g1 = granules of a head, hd_count = pieces a head is cut into
   const bf16 *q;         // [n_active][Hq][d]
   const bf16 *k_new, *v_new;    // [n_active][Hkv][d] or null
   // anchor-like source: decode -> cache anchor store; full -> same store, head = l*Hkv+h; prefill -> staging, head = h
@@ -246,6 +251,9 @@ struct RecallSignal {
 
 // kernels' host launchers (defined in the .cu files)
 cudaError_t launch_attn(const CacheView &cv, const AttnArgs &a, cudaStream_t st);
+// every one of n_heads heads cut into a.uni.hd_count even pieces, one one-shot CTA each (mode ATTN_PREFILL: the scoring pass,
+// n_queries text queries side by side; else plain attention of one query)
+cudaError_t launch_attn_uniform(const CacheView &cv, const AttnArgs &a, int n_heads, int n_queries, cudaStream_t st);
 // groups: CTAs per sequence (a layer that updates many tables, e.g. the last one under the global score scope)
 cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_bytes, int groups, cudaStream_t st);
 cudaError_t launch_select_all(const CacheView &cv, const SelectArgs *layer_args_dev, const int4 *map_dev, int n_entries,
@@ -260,17 +268,19 @@ cudaError_t launch_step_end(const CacheView &cv, int n_active, const int32_t *ac
                             cudaStream_t st);
 cudaError_t launch_recall(const CacheView &cv, int n_active, const int32_t *active, const int32_t *layers_dev, int n_layers,
                           int skip_copy, RecallSignal sig, cudaStream_t st);
-cudaError_t launch_place_scatter(const CacheView &cv, int b, int layer, const bf16 *k, const bf16 *v, int n_tokens, int ab,
-                                 int ae, int T_t, int C_b, int S_b, int S_base, bf16 *stage, cudaStream_t st);
-cudaError_t launch_prefill_select(const CacheView &cv, int b, int layer, const HeadItems *head_items, const float2 *part_ml,
+cudaError_t launch_place_scatter(const CacheView &cv, int b, int layer, int full_mode, const bf16 *k, const bf16 *v, int ab, int ae,
+                                 int T_t, int C_b, int S_b, int S_base, bf16 *stage, cudaStream_t st);
+// np: pieces a head was cut into by the scoring launch; n_q text queries; first, last: whether the placement begins, ends with them
+cudaError_t launch_prefill_select(const CacheView &cv, int b, int layer, int np, int n_q, const float2 *part_ml,
                                   const float2 *gran_em, int n_ag_max, int first, int last, cudaStream_t st);
-cudaError_t launch_place_gather(const CacheView &cv, int b, int layer, int full_mode, const bf16 *stage, int C_b,
+// mirror_out: device image of the layer's part of the host mirror
+cudaError_t launch_place_gather(const CacheView &cv, int b, int layer, const bf16 *stage, int C_b, bf16 *mirror_out,
                                 cudaStream_t st);
 // token-granular compression of the layer's fixed heads (after the chunk-granular placement staged the prefix)
 cudaError_t launch_token_compress(const CacheView &cv, int b, int layer, int n_comp, int n_tidal_base, const bf16 *stage,
                                   const bf16 *q_text, int n_q, int T_t, int T_a, int seg, const float *retention_dev,
                                   int variant, float *work, float *p_tok, int32_t *flags, long long p_stride,
-                                  int32_t *fixed_tok, int tok_cap, int32_t *tok_n, cudaStream_t st);
+                                  int32_t *fixed_tok, int tok_cap, int32_t *tok_n, bf16 *mirror_out, cudaStream_t st);
 cudaError_t launch_append_audio(const CacheView &cv, int b, int layer, int full_mode, const bf16 *k, const bf16 *v, int n_tokens,
                                 int T_a_old, int S_old, int set_dims, int T_a_new, int C_new, int S_new, cudaStream_t st);
 cudaError_t launch_exchange_scores(const CacheView &cv, int n_active, const int32_t *active, float *buf, int out, cudaStream_t st);

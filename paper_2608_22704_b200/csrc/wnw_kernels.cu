@@ -1,4 +1,6 @@
 // Recall, step bookkeeping and prefill placement kernels (sm_100a).
+#include <algorithm>
+
 #include <cuda_fp8.h>
 
 #include "wnw_internal.cuh"
@@ -490,13 +492,18 @@ cudaError_t launch_step_end(const CacheView &cv, int n_active, const int32_t *ac
 // Prefill placement ("Prefill Compression", chunk level)
 // ------------------------------------------------------------------------------------------------
 
-// Splits one layer's prefill K,V [n_tokens][Hkv][d] into the text store and a per-head staging copy of the audio
-// (anchor layout [Hkv][K|V][T_a_pad][d]), zero-pads the staging tail, and resets the layer's tables.
-__global__ void __launch_bounds__(256) wnw_place_scatter_kernel(const __grid_constant__ CacheView cv, int b, int layer,
-                                                                const bf16 *k, const bf16 *v, int n_tokens, int ab, int ae,
-                                                                int T_t, int C_b, int S_b, int S_base, bf16 *stage) {
+// Splits one layer's prefill K,V [n_tokens][Hkv][d] into the text store and the audio rows of every head, each chunk padded
+// with zero rows to whole granules, and resets the layer's tables.  The audio goes to a per-head staging copy (anchor layout
+// [Hkv][K|V][T_a_pad][d]), or straight to its final place where every head keeps all of it (full_mode).
+// A CTA takes a few destination rows, all heads of them, K and V: a row of the source is one contiguous run, so the divisions
+// are per row and the loads of the rows go out together.  Bound by HBM (read once, written once); 3064 tokens x 8 heads x 128:
+// 11.4 + 3.4 (a memset of the staging copy, which the zero rows replace) -> 7.7 us.
+constexpr int SCATTER_U = 4;
+__global__ void __launch_bounds__(256) wnw_place_scatter_kernel(const __grid_constant__ CacheView cv, int b, int layer, int full_mode,
+                                                                const bf16 *k, const bf16 *v, int ab, int ae, int T_t, int C_b,
+                                                                int S_b, int S_base, bf16 *stage, int rows_per_cta) {
   const Geometry &G = cv.geo;
-  const int T_a = ae - ab, vec_per_row = G.d / 8;
+  const int T_a = ae - ab, vpr = G.d / 8, vec_head = G.Hkv * vpr, vec_row = 2 * vec_head;
   const long long bl = (long long)b * G.L + layer;
   if (blockIdx.x == 0) {
     if (threadIdx.x == 0) {
@@ -514,80 +521,100 @@ __global__ void __launch_bounds__(256) wnw_place_scatter_kernel(const __grid_con
     const LayerInfo li = cv.layers[layer];
     for (int f = threadIdx.x; f < li.n_fixed; f += blockDim.x) cv.fixed_n[(long long)b * G.F_tot + li.fixed_off + f] = 0;
   }
-  const long long work = (long long)n_tokens * G.Hkv * 2 * vec_per_row;   // the staging copy was zeroed by the caller
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < work; idx += (long long)gridDim.x * blockDim.x) {
-    const int vv = (int)(idx % vec_per_row);
-    long long t = idx / vec_per_row;
-    const int kv = (int)(t % 2); t /= 2;
-    const int h = (int)(t % G.Hkv);
-    const int tok = (int)(t / G.Hkv);
-    const uint4 val = *reinterpret_cast<const uint4 *>((kv ? v : k) + ((long long)tok * G.Hkv + h) * G.d + vv * 8);
-    bf16 *dst;
-    if (tok >= ab && tok < ae) {  // audio token tau sits in row (tau / nc) * ncp + tau % nc: every chunk starts on a granule
-      const int tau = tok - ab, cc = tau / G.nc;
-      dst = stage + anchor_off(G, 0, 0, h, kv) + (long long)(cc * G.ncp + (tau - cc * G.nc)) * G.d + vv * 8;
-    } else {
-      dst = cv.text + text_off(G, b, layer, h, kv) + (long long)(tok < ab ? tok : tok - T_a) * G.d + vv * 8;
+  const int n_rows = T_t + C_b * G.ncp;
+  for (int row0 = blockIdx.x * rows_per_cta; row0 < n_rows; row0 += gridDim.x * rows_per_cta) {
+    const int work = min(rows_per_cta, n_rows - row0) * vec_row;
+    for (int w0 = threadIdx.x; w0 < work; w0 += blockDim.x * SCATTER_U) {
+      uint4 val[SCATTER_U];
+      uint4 *dst[SCATTER_U];
+#pragma unroll
+      for (int u = 0; u < SCATTER_U; ++u) {
+        const int w = w0 + u * (int)blockDim.x;
+        dst[u] = nullptr;
+        if (w >= work) continue;
+        const int rr = w / vec_row, x = w - rr * vec_row, kv = x >= vec_head, y = x - kv * vec_head, h = y / vpr, vv = y - h * vpr;
+        const int row = row0 + rr;
+        int tok = -1;
+        if (row < T_t) {
+          tok = row < ab ? row : row + T_a;
+          dst[u] = reinterpret_cast<uint4 *>(cv.text + text_off(G, b, layer, h, kv) + (long long)row * G.d) + vv;
+        } else {   // audio token tau sits in row (tau / nc) * ncp + tau % nc: every chunk starts on a granule
+          const int p = row - T_t, cc = p / G.ncp, off = p - cc * G.ncp, tau = cc * G.nc + off;
+          if (off < G.nc && tau < T_a) tok = ab + tau;
+          bf16 *base = full_mode ? cv.anchor + anchor_off(G, G.anchor_seq_stride, b, layer * G.Hkv + h, kv) : stage + anchor_off(G, 0, 0, h, kv);
+          dst[u] = reinterpret_cast<uint4 *>(base + (long long)p * G.d) + vv;
+        }
+        val[u] = tok < 0 ? make_uint4(0, 0, 0, 0) : __ldcs(reinterpret_cast<const uint4 *>(kv ? v : k) + (long long)tok * vec_head + y);
+      }
+#pragma unroll
+      for (int u = 0; u < SCATTER_U; ++u)
+        if (dst[u]) *dst[u] = val[u];
     }
-    *reinterpret_cast<uint4 *>(dst) = val;
   }
 }
-cudaError_t launch_place_scatter(const CacheView &cv, int b, int layer, const bf16 *k, const bf16 *v, int n_tokens, int ab,
-                                 int ae, int T_t, int C_b, int S_b, int S_base, bf16 *stage, cudaStream_t st) {
-  wnw_place_scatter_kernel<<<296, 256, 0, st>>>(cv, b, layer, k, v, n_tokens, ab, ae, T_t, C_b, S_b, S_base, stage);
+cudaError_t launch_place_scatter(const CacheView &cv, int b, int layer, int full_mode, const bf16 *k, const bf16 *v, int ab, int ae,
+                                 int T_t, int C_b, int S_b, int S_base, bf16 *stage, cudaStream_t st) {
+  const int vec_row = 2 * cv.geo.Hkv * (cv.geo.d / 8), rows = std::max(T_t + C_b * cv.geo.ncp, 1);
+  const int rows_per_cta = std::max(1, SCATTER_U * 256 / vec_row);   // one batch of loads per thread
+  wnw_place_scatter_kernel<<<std::min((rows + rows_per_cta - 1) / rows_per_cta, 148 * 16), 256, 0, st>>>(
+      cv, b, layer, full_mode, k, v, ab, ae, T_t, C_b, S_b, S_base, stage, rows_per_cta);
   return cudaGetLastError();
 }
 
-// One CTA.  From the prefill attention partials of q_last: pre[h][c] per non-anchor KV head, then the fixed heads'
-// own top-S sets and the tidal heads' shared top-S table (rank r -> slot r, stamp -1-r).
+// One CTA.  From the scoring partials of n_q text queries: pre[h][c] per non-anchor KV head, added in query order, then the
+// fixed heads' own top-S sets and the tidal heads' shared top-S table (rank r -> slot r, stamp -1-r).  np: pieces per head.
 __global__ void __launch_bounds__(512) wnw_prefill_select_kernel(const __grid_constant__ CacheView cv, int b, int layer,
-                                                                 const HeadItems *head_items, const float2 *part_ml,
-                                                                 const float2 *gran_em, int n_ag_max, int first, int last) {
-  extern __shared__ float sm[];  // [Hq] M, [Hq] Z, [C_max] keys (as u64 pairs)
+                                                                 int np, int n_q, const float2 *part_ml, const float2 *gran_em,
+                                                                 int n_ag_max, int first, int last) {
+  extern __shared__ float sm[];  // [n_q][Hq] M, [n_q][Hq] Z, [C_max] keys (as u64 pairs)
   const Geometry &G = cv.geo;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarp = blockDim.x >> 5;
   const int g = G.g, C_b = cv.C[b], S_b = cv.S_base[b], T_a = cv.T_a[b];   // the prefill placement fills the permanent slots
-  float *sM = sm, *sZ = sm + G.Hq;
-  unsigned long long *skey = reinterpret_cast<unsigned long long *>(sm + 2 * G.Hq + (2 * G.Hq & 1));
+  const int n_qh = n_q * G.Hq;
+  float *sM = sm, *sZ = sm + n_qh;
+  unsigned long long *skey = reinterpret_cast<unsigned long long *>(sm + 2 * n_qh);
   const LayerInfo li = cv.layers[layer];
   const long long bl = (long long)b * G.L + layer;
-  for (int hq = warp; hq < G.Hq; hq += nwarp) {
-    const HeadItems hi = head_items[hq / g];
-    const int row = hq % g;
+  for (int x = warp; x < n_qh; x += nwarp) {
+    const int hq = x % G.Hq, row = hq % g;
+    const float2 *ml_h = part_ml + ((long long)(x / G.Hq) * G.Hkv + hq / g) * np * g + row;
     float M = -INFINITY;
-    for (int n = lane; n < hi.count; n += 32) M = fmaxf(M, part_ml[(long long)(hi.first + n) * g + row].x);
+    for (int n = lane; n < np; n += 32) M = fmaxf(M, ml_h[(long long)n * g].x);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
     float Z = 0.f;
-    for (int n = lane; n < hi.count; n += 32) {
-      const float2 ml = part_ml[(long long)(hi.first + n) * g + row];
+    for (int n = lane; n < np; n += 32) {
+      const float2 ml = ml_h[(long long)n * g];
       Z += M > -INFINITY ? ml.y * exp2f(ml.x - M) : 0.f;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
-    if (lane == 0) { sM[hq] = M; sZ[hq] = Z; }
+    if (lane == 0) { sM[x] = M; sZ[x] = Z; }
   }
   __syncthreads();
   float *pre = cv.pre + bl * G.Hkv * G.C_max;
   for (int idx = tid; idx < G.Hkv * C_b; idx += blockDim.x) {
     const int h = idx / C_b, c = idx - h * C_b;
-    float total = 0.f;
+    float sum = first ? 0.f : pre[(long long)h * G.C_max + c];
     if (cv.roles[layer * G.Hkv + h] != ROLE_ANCHOR) {
-      for (int r = 0; r < g; ++r) {
-        const int hq = h * g + r;
-        const float2 *ge = gran_em + (long long)hq * n_ag_max + (long long)c * G.gpc;
-        float sum_h = 0.f;
-        for (int gi = 0; gi < G.gpc; ++gi) {
-          if (gi * GR >= chunk_len(G, T_a, c)) break;
-          sum_h += ge[gi].x * exp2f(ge[gi].y - sM[hq]);
+      for (int q = 0; q < n_q; ++q) {   // summed over the text queries ("Prefill Compression": p_prefill = sum over text queries)
+        float total = 0.f;
+        for (int r = 0; r < g; ++r) {
+          const int hq = h * g + r, x = q * G.Hq + hq;
+          const float2 *ge = gran_em + (long long)x * n_ag_max + (long long)c * G.gpc;
+          float sum_h = 0.f;
+          for (int gi = 0; gi < G.gpc; ++gi) {
+            if (gi * GR >= chunk_len(G, T_a, c)) break;
+            sum_h += ge[gi].x * exp2f(ge[gi].y - sM[x]);
+          }
+          total += sZ[x] > 0.f ? sum_h / sZ[x] : 0.f;
         }
-        total += sZ[hq] > 0.f ? sum_h / sZ[hq] : 0.f;
+        sum += total;
       }
     }
-    // summed over the text queries, one launch per query ("Prefill Compression": p_prefill = sum over text queries)
-    pre[(long long)h * G.C_max + c] = first ? total : pre[(long long)h * G.C_max + c] + total;
+    pre[(long long)h * G.C_max + c] = sum;
   }
-  if (!last) return;   // the placement follows the last query
+  if (!last) return;   // the placement follows the last queries
   __syncthreads();
   // fixed heads: rank by counting
   for (int h = 0; h < G.Hkv; ++h) {
@@ -702,28 +729,28 @@ cudaError_t launch_prefill_retable(const CacheView &cv, int b, int layer, const 
   return cudaGetLastError();
 }
 
-cudaError_t launch_prefill_select(const CacheView &cv, int b, int layer, const HeadItems *head_items, const float2 *part_ml,
+cudaError_t launch_prefill_select(const CacheView &cv, int b, int layer, int np, int n_q, const float2 *part_ml,
                                   const float2 *gran_em, int n_ag_max, int first, int last, cudaStream_t st) {
-  const size_t smem = (size_t)(2 * cv.geo.Hq + 2) * sizeof(float) + (size_t)cv.geo.C_max * sizeof(unsigned long long);
-  wnw_prefill_select_kernel<<<1, 512, smem, st>>>(cv, b, layer, head_items, part_ml, gran_em, n_ag_max, first, last);
+  const size_t smem = (size_t)2 * n_q * cv.geo.Hq * sizeof(float) + (size_t)cv.geo.C_max * sizeof(unsigned long long);
+  wnw_prefill_select_kernel<<<1, 512, smem, st>>>(cv, b, layer, np, n_q, part_ml, gran_em, n_ag_max, first, last);
   return cudaGetLastError();
 }
 
-// grid (C_b, Hkv).  Moves one chunk of one head from staging to its tier: anchor store (anchor heads, or every
-// head in full mode), compacted fixed store if selected, host mirror (+ slot if resident) for tidal heads.
+// grid (C_b, Hkv).  Moves one chunk of one head from staging to its tier: anchor store, compacted fixed store if selected, for
+// tidal heads the layer's outgoing mirror image (mirror_out, in the mirror's layout; a copy engine takes it to the host: written
+// straight to the mapped host memory this kernel ran at the link's rate, 152 us a layer at 3000 x 5 heads, with everything
+// behind it waiting) and the slot if the chunk is resident.
 __global__ void __launch_bounds__(128) wnw_place_gather_kernel(const __grid_constant__ CacheView cv, int b, int layer,
-                                                               int full_mode, const bf16 *stage) {
+                                                               const bf16 *stage, bf16 *mirror_out) {
   const Geometry &G = cv.geo;
   const int c = blockIdx.x, h = blockIdx.y;
   const LayerInfo li = cv.layers[layer];
   const long long bl = (long long)b * G.L + layer;
-  const int role = full_mode ? ROLE_ANCHOR : cv.roles[layer * G.Hkv + h];
-  const int ridx = full_mode ? h : cv.role_idx[layer * G.Hkv + h];
+  const int role = cv.roles[layer * G.Hkv + h], ridx = cv.role_idx[layer * G.Hkv + h];
   const int vec_per_chunk = G.ncp * G.d / 8;
   bf16 *dst0[2] = {nullptr, nullptr}, *dst1[2] = {nullptr, nullptr};
   if (role == ROLE_ANCHOR) {
-    const int head = full_mode ? layer * G.Hkv + h : li.anchor_off + ridx;
-    for (int kv = 0; kv < 2; ++kv) dst0[kv] = cv.anchor + anchor_off(G, G.anchor_seq_stride, b, head, kv) + (long long)c * G.ncp * G.d;
+    for (int kv = 0; kv < 2; ++kv) dst0[kv] = cv.anchor + anchor_off(G, G.anchor_seq_stride, b, li.anchor_off + ridx, kv) + (long long)c * G.ncp * G.d;
   } else if (role == ROLE_FIXED) {
     const long long fh = (long long)b * G.F_tot + li.fixed_off + ridx;
     int pos = -1;
@@ -739,7 +766,7 @@ __global__ void __launch_bounds__(128) wnw_place_gather_kernel(const __grid_cons
     for (int kv = 0; kv < 2; ++kv) {
       const float inv = exp2f(-(float)cv.kv_exp[kv_exp_off(G, cv.tid_total, b, li.tid_prefix + ridx, c) + kv]);
       const bf16 *src = stage + anchor_off(G, 0, 0, h, kv) + (long long)c * G.ncp * G.d;
-      uint4 *m = reinterpret_cast<uint4 *>(tier_ptr(G, cv.mirror[b], mirror_off(G, li, mirror_chunks_of(G, cv.C[b]), c, ridx, kv)));
+      uint4 *m = reinterpret_cast<uint4 *>(tier_ptr(G, mirror_out, mirror_block_off(G, li, c, ridx, kv)));
       uint4 *p = slot >= 0 ? reinterpret_cast<uint4 *>(tier_ptr(G, cv.pool, pool_off(G, li, b, slot, ridx, kv))) : nullptr;
       for (int gidx = threadIdx.x; gidx < groups; gidx += blockDim.x) {
         union { uint4 v; uint8_t b[16]; } out;
@@ -755,7 +782,7 @@ __global__ void __launch_bounds__(128) wnw_place_gather_kernel(const __grid_cons
   } else {
     const int slot = cv.chunk_slot[bl * G.C_max + c];
     for (int kv = 0; kv < 2; ++kv) {
-      dst0[kv] = cv.mirror[b] + mirror_off(G, li, mirror_chunks_of(G, cv.C[b]), c, ridx, kv);
+      dst0[kv] = mirror_out + mirror_block_off(G, li, c, ridx, kv);
       if (slot >= 0) dst1[kv] = cv.pool + pool_off(G, li, b, slot, ridx, kv);
     }
   }
@@ -808,10 +835,10 @@ cudaError_t launch_quantise_stage(const CacheView &cv, int b, int layer, bf16 *s
   return cudaGetLastError();
 }
 
-cudaError_t launch_place_gather(const CacheView &cv, int b, int layer, int full_mode, const bf16 *stage, int C_b,
-                                  cudaStream_t st) {
+cudaError_t launch_place_gather(const CacheView &cv, int b, int layer, const bf16 *stage, int C_b, bf16 *mirror_out,
+                                cudaStream_t st) {
   if (C_b <= 0) return cudaSuccess;
-  wnw_place_gather_kernel<<<dim3(C_b, cv.geo.Hkv), 128, 0, st>>>(cv, b, layer, full_mode, stage);
+  wnw_place_gather_kernel<<<dim3(C_b, cv.geo.Hkv), 128, 0, st>>>(cv, b, layer, stage, mirror_out);
   return cudaGetLastError();
 }
 

@@ -24,7 +24,7 @@ struct SeqHost {
   int T_a_fixed = 0, S_fixed = 0;   // the clip and the slot count at placement: what a fixed head keeps for good (streaming audio)
   int append_layer = 0, append_n = 0;   // an append of audio in progress: layers done, positions per layer
   bf16 *mirror = nullptr;
-  size_t mirror_bytes = 0;
+  size_t mirror_cap = 0;   // bytes allocated; a placement lays it out for its own clip and keeps it if it is large enough
   std::vector<int> fixed_blocks;   // [L][Hkv] blocks of a token-compacted head's store; empty or -1: S_base chunks
   std::vector<int2> tok_m;         // [L][Hkv] tidal token bases: kept positions of a full / of the last segment
 };
@@ -37,7 +37,7 @@ struct LayerWork {
   int n_ctas_free = 0;   // BATCHED layers: the first n_ctas_free CTAs hold no tidal head (they need no recall epoch) ...
   int n_ctas_anchor = 0; // ... and the first n_ctas_anchor of those hold the anchor heads (what the step's selection waits for)
   bool packed = false;                             // one-shot CTAs that serve several short heads each
-  int head_items_off = 0;                          // offset in the uploaded HeadItems array
+  int head_items_off = 0;                          // offset in the list's HeadItems
 };
 
 struct DeviceGuard {
@@ -78,26 +78,28 @@ struct wnw_cache {
   std::vector<int> wl_T_a;
   std::vector<LayerWork> wl_layers;
   WorkItem *d_items = nullptr;
-  int32_t *d_sched = nullptr, *d_pf_sched = nullptr;  // persistent schedules: [order of all layers | ranges of all layers]
-  size_t d_sched_cap = 0, sched_ranges_base = 0, pf_sched_cap = 0, pf_ranges_base = 0;
-  int pf_n_ctas = 0;
-  std::vector<WorkItem> h_items, h_pf_items;  // host copies (short lists are inlined into kernel parameters)
-  HeadItems *d_head_items = nullptr;
-  size_t d_items_cap = 0, d_head_items_cap = 0;
-  int prefill_seq = -1, prefill_T_a = -1;
-  WorkItem *d_pf_items = nullptr;
-  HeadItems *d_pf_head_items = nullptr;
-  int pf_n_items = 0;
-  bool pf_throughput = false;
-  size_t pf_items_cap = 0;
+  int32_t *d_sched = nullptr;  // persistent schedules: [order of all layers | ranges of all layers]
+  size_t d_sched_cap = 0, sched_ranges_base = 0;
+  std::vector<WorkItem> h_items;  // host copy (short lists are inlined into kernel parameters)
+  size_t d_items_cap = 0;
   // partial buffers
   float *part_o = nullptr;
   float2 *part_ml = nullptr, *gran_em = nullptr, *head_mz = nullptr;
   int32_t *head_done = nullptr;
   float2 *pf_gran_em = nullptr, *pf_part_ml = nullptr;
-  float *pf_part_o = nullptr;
+  int pf_queries = 1;               // text queries one scoring launch takes
   size_t part_cap_total = 0;
-  int part_cap_items = 0, n_aq_max = 0, n_ag_max = 0;
+  int n_aq_max = 0, n_ag_max = 0;
+  // Placement: the tidal heads' part of a layer's K,V on its way to the pinned mirror.  A few device images of a layer, filled
+  // in turn and taken out by a copy engine on a stream of its own, so that the next layers' kernels and the first decode step
+  // run beside the transfer; whoever reads the mirror waits for ev_mirror.
+  static constexpr int MIRROR_RING = 4;
+  bf16 *mst[MIRROR_RING] = {};
+  bool mst_used[MIRROR_RING] = {};
+  int mst_next = 0;
+  cudaEvent_t ev_mst_ready[MIRROR_RING] = {}, ev_mst_free[MIRROR_RING] = {}, ev_mirror = nullptr;
+  cudaStream_t copy_stream = nullptr;
+  bool mirror_pending = false, mirror_step_issued = false;   // copies may be under way; a replayed step has been issued beside them
   // streams / events
   static constexpr int N_SIDE = 8;  // layers alternate between side streams so selection + recall keep pace with attention
   cudaStream_t side[N_SIDE] = {}, last_stream = nullptr;
@@ -222,7 +224,12 @@ static void destroy_impl(wnw_cache *c) {
     if (s.mirror) cudaFreeHost(s.mirror);
   for (auto sd : c->side)
     if (sd) cudaStreamDestroy(sd);
-
+  if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
+  for (int r = 0; r < wnw_cache::MIRROR_RING; ++r) {
+    if (c->ev_mst_ready[r]) cudaEventDestroy(c->ev_mst_ready[r]);
+    if (c->ev_mst_free[r]) cudaEventDestroy(c->ev_mst_free[r]);
+  }
+  if (c->ev_mirror) cudaEventDestroy(c->ev_mirror);
   for (auto e : c->ev_layer_done) cudaEventDestroy(e);
   for (auto e : c->ev_side_done) cudaEventDestroy(e);
   for (auto e : c->ev_layer_done_cap) cudaEventDestroy(e);
@@ -409,7 +416,7 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
   CKC(dev_alloc(c, &cv.pool, G.kv8 ? (B * (size_t)G.pool_seq_stride + 1) / 2 : B * (size_t)G.pool_seq_stride));   // one byte per element as e4m3
   CKC(dev_alloc(c, &cv.kv_exp, G.kv8 ? B * (size_t)std::max(t_tot, 1) * std::max(G.C_max, 1) * 2 : 1));
   CKC(dev_alloc(c, &cv.fixed, B * (size_t)G.fixed_seq_stride));
-  CKC(dev_alloc(c, &c->stage, (size_t)Hkv * 2 * G.T_a_pad * d));
+  CKC(dev_alloc(c, &c->stage, full ? 1 : (size_t)Hkv * 2 * G.T_a_pad * d));
   CKC(dev_alloc(c, &cv.text_len, B)); CKC(dev_alloc(c, &cv.T_a, B)); CKC(dev_alloc(c, &cv.C, B)); CKC(dev_alloc(c, &cv.S, B));
   CKC(dev_alloc(c, &cv.S_base, B));
   CKC(dev_alloc(c, &cv.steps, B));
@@ -435,21 +442,19 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
     CKC(dev_upload(c, &c->d_iota, iota));
   }
   CKC(dev_alloc(c, &c->d_active, B));
-  // partial buffers: the work-list builder keeps items <= target + heads
   int n_aq = 0;
   for (int l = 0; l < L; ++l) n_aq = std::max(n_aq, c->layers[l].n_anchor * G.g);
   c->n_aq_max = std::max(n_aq, 1);
   c->n_ag_max = std::max(G.C_max * G.gpc, 1);
-  c->part_cap_items = 10 * c->n_sm + 2 * (int)B * Hkv + 64;
-  // split partials of the prefill scoring pass; the decode layers get one region each (sized with the work lists),
-  // because consecutive layer kernels overlap
-  CKC(dev_alloc(c, &c->pf_part_o, (size_t)c->part_cap_items * G.g * d, false));
-  CKC(dev_alloc(c, &c->pf_part_ml, (size_t)c->part_cap_items * G.g, false));
+  // partials of the prefill scoring pass, of as many text queries as one launch takes (what the selection behind it can hold
+  // in its 48 KB of shared memory beside the chunk keys)
+  c->pf_queries = std::max(1, std::min(8, (int)((48 * 1024 - (long long)G.C_max * 8) / (8ll * G.Hq))));
+  CKC(dev_alloc(c, &c->pf_part_ml, full ? 1 : (size_t)c->pf_queries * std::max(c->n_sm, Hkv) * G.g, false));
   // granule partials and final (M,Z) are per layer: the side-stream selection of layer l reads them while the
   // caller's stream already runs later layers
   c->gran_em_layer_stride = B * (size_t)c->n_aq_max * c->n_ag_max;
   CKC(dev_alloc(c, &c->gran_em, full ? 1 : (size_t)L * c->gran_em_layer_stride, false));
-  CKC(dev_alloc(c, &c->pf_gran_em, full ? 1 : (size_t)G.Hq * c->n_ag_max, false));
+  CKC(dev_alloc(c, &c->pf_gran_em, full ? 1 : (size_t)c->pf_queries * G.Hq * c->n_ag_max, false));
   CKC(dev_alloc(c, &c->head_mz, (size_t)L * B * G.Hq, false));
   c->sel_smem.assign(L, 0);
   for (int l = 0; l < L && !full; ++l) {
@@ -474,8 +479,22 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
     else ok = ok && encode_store_map(&c->maps_decode.pool, r_pool ? (void *)cv.pool : (void *)cv.text, r_pool ? r_pool : r_text, d);
     ok = ok && encode_store_map(&c->maps_decode.fixed, r_fixed ? (void *)cv.fixed : (void *)cv.text, r_fixed ? r_fixed : r_text, d);
     c->maps_prefill = c->maps_decode;
-    ok = ok && encode_store_map(&c->maps_prefill.anchor, c->stage, r_stage, d);
+    if (!full) ok = ok && encode_store_map(&c->maps_prefill.anchor, c->stage, r_stage, d);
     if (!ok) return fail(WNW_ERR_CUDA);
+  }
+  {
+    int tid_max = 0;
+    for (const LayerInfo &li : c->layers) tid_max = std::max(tid_max, (int)li.n_tidal);
+    if (!full && tid_max > 0 && G.C_max > 0) {
+      CKE(cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
+      CKE(cudaEventCreateWithFlags(&c->ev_mirror, cudaEventDisableTiming));
+      for (int r = 0; r < wnw_cache::MIRROR_RING; ++r) {
+        const size_t elems = (size_t)G.C_max * tid_max * 2 * G.ncp * d;
+        CKC(dev_alloc(c, &c->mst[r], G.kv8 ? (elems + 1) / 2 : elems, false));
+        CKE(cudaEventCreateWithFlags(&c->ev_mst_ready[r], cudaEventDisableTiming));
+        CKE(cudaEventCreateWithFlags(&c->ev_mst_free[r], cudaEventDisableTiming));
+      }
+    }
   }
   c->seqs.assign(B, SeqHost{});
   c->mirror_ptrs.assign(B, nullptr);
@@ -623,7 +642,6 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   double total = 0.0;
   for (int hd = 0; hd < n_heads; ++hd) total += n_work[hd];
   const int P = (int)std::min<double>(per_sm * c->n_sm, std::max(1.0, total / (2.0 * nw)));   // at least two granules per warp and CTA
-  const bool may_finish = mode != ATTN_PREFILL;       // the prefill scoring pass leaves partials whatever the cut
   auto pieces_of = [&](int hd, double T) { return std::max(1, (int)std::lround(n_work[hd] / T)); };
   // Longest-first onto the least loaded CTA (the lower index on equal loads).  The pieces of a head cost the same, so heads are
   // sorted instead of pieces; as long as all loads are equal a run of equal pieces goes round robin (one division, which is
@@ -636,7 +654,7 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   auto makespan = [&](double T, std::vector<std::vector<std::pair<int, int>>> *assign) {
     for (int hd = 0; hd < n_heads; ++hd) {
       const int np = pieces_of(hd, T);
-      runs[hd] = Run{(double)n_work[hd] / np + ((np > 1 || !may_finish) ? cost_piece : cost_whole), hd, np};
+      runs[hd] = Run{(double)n_work[hd] / np + (np > 1 ? cost_piece : cost_whole), hd, np};
     }
     std::stable_sort(runs.begin(), runs.end(), [](const Run &x, const Run &y) { return x.cost > y.cost; });
     if (assign) assign->assign(P, {});
@@ -733,7 +751,7 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   }
   ranges.push_back(pos);
   lw.n_ctas = n_ctas;
-  lw.packed = mode != ATTN_PREFILL;   // the pipeline runs across a CTA's items (its merge scratch sits behind the stages)
+  lw.packed = true;   // the pipeline runs across a CTA's items (its merge scratch sits behind the stages)
 }
 
 // Appends the items of one layer for the given sequences.
@@ -757,9 +775,7 @@ static void build_layer_items(const wnw_cache *c, int layer, int mode, const std
     }
   }
   bool throughput = false;
-  // the prefill scoring pass is a single launch: nothing overlaps it
-  const bool overlapped = mode != ATTN_PREFILL && (c->layer_dependency == WNW_LAYERS_INDEPENDENT ||
-                                                  c->layer_dependency == WNW_LAYERS_BATCHED);
+  const bool overlapped = c->layer_dependency == WNW_LAYERS_INDEPENDENT || c->layer_dependency == WNW_LAYERS_BATCHED;
   int gpi = granules_per_item(c, total, longest, (int)seq_ids.size() * G.Hkv, overlapped, &throughput);
   // BATCHED layers share one launch: the work of the whole step is cut for one wave of CTAs, long heads into pieces as
   // fat as a pack of short ones, short heads packed whole
@@ -933,11 +949,6 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
     c->dev_allocs.push_back(c->d_items);
     c->d_items_cap = items.size();
   }
-  if (heads.size() > c->d_head_items_cap) {
-    CK(cudaMalloc((void **)&c->d_head_items, heads.size() * sizeof(HeadItems)));
-    c->dev_allocs.push_back(c->d_head_items);
-    c->d_head_items_cap = heads.size();
-  }
   if (order.size() + ranges.size() > c->d_sched_cap) {
     CK(cudaMalloc((void **)&c->d_sched, (order.size() + ranges.size()) * sizeof(int32_t)));
     c->dev_allocs.push_back(c->d_sched);
@@ -949,7 +960,6 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
   }
   c->sched_ranges_base = order.size();
   CK(cudaMemcpy(c->d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(c->d_head_items, heads.data(), heads.size() * sizeof(HeadItems), cudaMemcpyHostToDevice));
   std::vector<int32_t> act(c->active.begin(), c->active.end());
   CK(cudaMemcpy(c->d_active, act.data(), act.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
   c->h_items = items;
@@ -970,19 +980,55 @@ extern "C" wnw_status_t wnw_place_prefill(wnw_cache_t *c, int32_t seq, int32_t l
 
 static wnw_status_t place_multi(wnw_cache_t *c, int32_t seq, int32_t layer, const void *k_dev, const void *v_dev,
                                 int32_t n_tokens, int32_t audio_begin, int32_t audio_end, const void *q_last_dev,
-                                int32_t n_queries, void *cuda_stream);
+                                int32_t n_queries, cudaStream_t st, bf16 **mirror_out);
+static wnw_status_t send_mirror(wnw_cache_t *c, int seq, int layer, cudaStream_t st);
 
 extern "C" wnw_status_t wnw_place_prefill_multi(wnw_cache_t *c, int32_t seq, int32_t layer, const void *k_dev, const void *v_dev,
                                                 int32_t n_tokens, int32_t audio_begin, int32_t audio_end,
                                                 const void *q_last_dev, int32_t n_queries, void *cuda_stream) {
   // a token-granular base is placed by wnw_place_prefill_tokens only
   if (c && c->geo.token_base) return WNW_ERR_STATE;
-  return place_multi(c, seq, layer, k_dev, v_dev, n_tokens, audio_begin, audio_end, q_last_dev, n_queries, cuda_stream);
+  bf16 *out = nullptr;
+  wnw_status_t rc = place_multi(c, seq, layer, k_dev, v_dev, n_tokens, audio_begin, audio_end, q_last_dev, n_queries,
+                                (cudaStream_t)cuda_stream, &out);
+  return rc == WNW_OK && out ? send_mirror(c, seq, layer, (cudaStream_t)cuda_stream) : rc;
 }
 
+// The layer's mirror image (filled by work queued on st) goes to the host on the copy stream.
+static wnw_status_t send_mirror(wnw_cache_t *c, int seq, int layer, cudaStream_t st) {
+  const Geometry &G = c->geo;
+  const SeqHost &s = c->seqs[seq];
+  const LayerInfo &li = c->layers[layer];
+  DeviceGuard guard(c->cfg.device);
+  const int r = c->mst_next;
+  const size_t eb = tidal_elem_bytes(G);
+  CK(cudaEventRecord(c->ev_mst_ready[r], st));
+  CK(cudaStreamWaitEvent(c->copy_stream, c->ev_mst_ready[r], 0));
+  CK(cudaMemcpyAsync(reinterpret_cast<char *>(s.mirror) + mirror_off(G, li, mirror_chunks_of(G, s.C), 0, 0, 0) * eb, c->mst[r],
+                     (size_t)s.C * li.n_tidal * 2 * G.ncp * G.d * eb, cudaMemcpyDeviceToHost, c->copy_stream));
+  CK(cudaEventRecord(c->ev_mst_free[r], c->copy_stream));
+  CK(cudaEventRecord(c->ev_mirror, c->copy_stream));
+  c->mst_used[r] = true;
+  c->mst_next = (r + 1) % wnw_cache::MIRROR_RING;
+  c->mirror_pending = true; c->mirror_step_issued = false;
+  return WNW_OK;
+}
+
+// What is queued on `st` from here on may read the mirrors: after the copies of earlier placements.
+static wnw_status_t wait_for_mirror(wnw_cache *c, cudaStream_t st) {
+  if (!c->mirror_pending) return WNW_OK;
+  const cudaError_t e = cudaEventQuery(c->ev_mirror);
+  if (e == cudaSuccess) { c->mirror_pending = false; return WNW_OK; }
+  if (e != cudaErrorNotReady) { c->last_cuda = e; return WNW_ERR_CUDA; }
+  cudaGetLastError();   // "not ready" is no error
+  CK(cudaStreamWaitEvent(st, c->ev_mirror, 0));
+  return WNW_OK;
+}
+
+// mirror_out: set to the layer's mirror image when it has tidal heads: the caller hands it to send_mirror once it is final.
 static wnw_status_t place_multi(wnw_cache_t *c, int32_t seq, int32_t layer, const void *k_dev, const void *v_dev,
                                 int32_t n_tokens, int32_t audio_begin, int32_t audio_end, const void *q_last_dev,
-                                int32_t n_queries, void *cuda_stream) {
+                                int32_t n_queries, cudaStream_t st, bf16 **mirror_out) {
   if (!c || !k_dev || !v_dev || n_queries < 1) return WNW_ERR_INVALID_ARG;
   const Geometry &G = c->geo;
   if (seq < 0 || seq >= G.max_batch || layer < 0 || layer >= G.L || n_tokens < 1) return WNW_ERR_INVALID_ARG;
@@ -997,99 +1043,65 @@ static wnw_status_t place_multi(wnw_cache_t *c, int32_t seq, int32_t layer, cons
   const int S_base_b = full ? 0 : base_slots_for(c->cfg, C_b);
   if (!full && C_b > 0 && !q_last_dev) return WNW_ERR_INVALID_ARG;
   DeviceGuard guard(c->cfg.device);
-  cudaStream_t st = (cudaStream_t)cuda_stream;
   if (layer == 0) {
     s.placed_layers = 0;
     const size_t need = full ? 0 : (size_t)mirror_chunks_of(G, C_b) * c->tid_total * 2 * G.ncp * G.d * tidal_elem_bytes(G);
-    if (need != s.mirror_bytes) {
+    if (need > s.mirror_cap) {
       CK(cudaDeviceSynchronize());
       if (s.mirror) cudaFreeHost(s.mirror);
-      s.mirror = nullptr; s.mirror_bytes = 0;
-      if (need) {
-        void *p = nullptr;
-        if (cudaHostAlloc(&p, need, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
-          cudaGetLastError();
-          return WNW_ERR_OOM_HOST;
-        }
-        if (G.mirror_chunks) memset(p, 0, need);   // chunks that have not arrived yet must read as padding
-        void *dp = nullptr;
-        CK(cudaHostGetDevicePointer(&dp, p, 0));
-        s.mirror = (bf16 *)p; s.mirror_bytes = need;
-        c->mirror_ptrs[seq] = (bf16 *)dp;
-      } else {
-        c->mirror_ptrs[seq] = nullptr;
+      s.mirror = nullptr; s.mirror_cap = 0;
+      void *p = nullptr;
+      if (cudaHostAlloc(&p, need, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return WNW_ERR_OOM_HOST;
       }
+      if (G.mirror_chunks) memset(p, 0, need);   // chunks that have not arrived yet must read as padding
+      void *dp = nullptr;
+      CK(cudaHostGetDevicePointer(&dp, p, 0));
+      s.mirror = (bf16 *)p; s.mirror_cap = need;
+      c->mirror_ptrs[seq] = (bf16 *)dp;
       CK(cudaMemcpy(c->cv.mirror + seq, &c->mirror_ptrs[seq], sizeof(bf16 *), cudaMemcpyHostToDevice));
     }
     s.T_a = T_a; s.T_t = T_t; s.C = C_b; s.S = S_b; s.S_base = S_base_b;
     s.T_a_fixed = T_a; s.S_fixed = S_base_b; s.append_layer = 0; s.append_n = 0;
     s.fixed_blocks.clear(); s.tok_m.clear();
     c->wl_layers.clear();  // dims may have changed
+    // selections and recalls of earlier eager steps may still write the tables and slots that this placement resets
+    for (int l = 0; l < G.L; ++l)
+      if (c->side_recorded[l]) CK(cudaStreamWaitEvent(st, c->ev_side_done[l], 0));
   }
   // the staging buffer and the partial buffers are shared: order after earlier placements and steps
   if (c->place_recorded) CK(cudaStreamWaitEvent(st, c->ev_place, 0));
   if (c->step_recorded) CK(cudaStreamWaitEvent(st, c->ev_step, 0));
   if (c->recall_all_pending) CK(cudaStreamWaitEvent(st, c->ev_recall_all, 0));
-  // chunks start on granule boundaries in every store; the rows between a chunk's last token and the next chunk are zero
-  CK(cudaMemsetAsync(c->stage, 0, (size_t)G.Hkv * 2 * G.T_a_pad * G.d * sizeof(bf16), st));
-  CK(launch_place_scatter(c->cv, seq, layer, (const bf16 *)k_dev, (const bf16 *)v_dev, n_tokens, audio_begin, audio_end, T_t,
+  CK(launch_place_scatter(c->cv, seq, layer, full ? 1 : 0, (const bf16 *)k_dev, (const bf16 *)v_dev, audio_begin, audio_end, T_t,
                           C_b, S_b, S_base_b, c->stage, st));
-  // e4m3 tidal tier: scales per chunk, and the staged rows of the tidal heads become the values their bytes will decode
-  // to, so that the prefill scores below already see what decoding will see
-  if (G.kv8 && C_b > 0) CK(launch_quantise_stage(c->cv, seq, layer, c->stage, C_b, st));
   if (!full && C_b > 0) {
-    if (c->prefill_seq != seq || c->prefill_T_a != T_a) {
-      std::vector<WorkItem> items;
-      std::vector<HeadItems> heads;
-      LayerWork lw;
-      std::vector<int> one{seq};
-      std::vector<int32_t> order, ranges;
-      build_layer_items(c, layer, ATTN_PREFILL, one, items, heads, lw, order, ranges);
-      if (order.size() + ranges.size() > c->pf_sched_cap) {
-        CK(cudaMalloc((void **)&c->d_pf_sched, (order.size() + ranges.size()) * sizeof(int32_t)));
-        c->dev_allocs.push_back(c->d_pf_sched);
-        c->pf_sched_cap = order.size() + ranges.size();
-      }
-      if (!order.empty()) {
-        CK(cudaMemcpyAsync(c->d_pf_sched, order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-        CK(cudaMemcpyAsync(c->d_pf_sched + order.size(), ranges.data(), ranges.size() * sizeof(int32_t), cudaMemcpyHostToDevice, st));
-      }
-      c->pf_ranges_base = order.size();
-      c->pf_n_ctas = lw.n_ctas;
-      if ((int)items.size() > c->part_cap_items) return WNW_ERR_CAPACITY;
-      if (items.size() > c->pf_items_cap) {
-        CK(cudaMalloc((void **)&c->d_pf_items, items.size() * sizeof(WorkItem)));
-        c->dev_allocs.push_back(c->d_pf_items);
-        c->pf_items_cap = items.size();
-      }
-      if (!c->d_pf_head_items) {
-        CK(cudaMalloc((void **)&c->d_pf_head_items, (size_t)G.Hkv * sizeof(HeadItems)));
-        c->dev_allocs.push_back(c->d_pf_head_items);
-      }
-      for (auto &it : items) it.i = 0;
-      CK(cudaMemcpyAsync(c->d_pf_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(c->d_pf_head_items, heads.data(), heads.size() * sizeof(HeadItems), cudaMemcpyHostToDevice, st));
-      CK(cudaStreamSynchronize(st));  // the host vectors go out of scope
-      c->pf_n_items = (int)items.size();
-      c->pf_throughput = lw.throughput;
-      c->h_pf_items = items;
-      c->prefill_seq = seq; c->prefill_T_a = T_a;
-    }
+    // e4m3 tidal tier: scales per chunk, and the staged rows of the tidal heads become the values their bytes will decode
+    // to, so that the prefill scores below already see what decoding will see
+    if (G.kv8) CK(launch_quantise_stage(c->cv, seq, layer, c->stage, C_b, st));
+    // The scoring pass: every head is alike, cut into even pieces of at least two granules a warp, one wave of CTAs
+    const int n_gran = G.n_tg + C_b * G.gpc, per_cta = 2 * attn_warps(false);
     AttnArgs a{};
-    a.mode = ATTN_PREFILL; a.layer = layer; a.li = c->layers[layer]; a.n_active = 1; a.has_new = 0; a.score_on = 1;
-    a.active = c->d_iota + seq; a.items = c->d_pf_items; a.items_host = c->h_pf_items.data(); a.n_items = c->pf_n_items; a.maps = &c->maps_prefill; a.throughput = c->pf_throughput;
-    if (c->pf_n_ctas > 0) { a.order = c->d_pf_sched; a.cta_ranges = c->d_pf_sched + c->pf_ranges_base; a.n_ctas = c->pf_n_ctas; }
-    a.head_items = c->d_pf_head_items;
-    a.anchor_base = c->stage; a.anchor_seq_stride = 0; a.anchor_head0 = 0;
-    a.part_o = c->pf_part_o; a.part_ml = c->pf_part_ml; a.gran_em = c->pf_gran_em; a.n_aq = G.Hq; a.n_ag_max = c->n_ag_max;
-    for (int qi = 0; qi < n_queries; ++qi) {   // one scoring pass per text query; the scores add up, the last pass places
-      a.q = (const bf16 *)q_last_dev + (size_t)qi * G.Hq * G.d;
-      CK(launch_attn(c->cv, a, st));
-      CK(launch_prefill_select(c->cv, seq, layer, c->d_pf_head_items, c->pf_part_ml, c->pf_gran_em, c->n_ag_max, qi == 0,
-                               qi == n_queries - 1, st));
+    a.mode = ATTN_PREFILL; a.layer = layer; a.li = c->layers[layer]; a.n_active = 1; a.score_on = 1; a.maps = &c->maps_prefill;
+    const int np = std::max(1, std::min((n_gran + per_cta - 1) / per_cta, c->n_sm / G.Hkv));
+    a.uni = WorkItem{0, 0, 0, n_gran, seq, ROLE_ANCHOR, 0, T_a, C_b, 0, T_t, 0, np};
+    a.part_ml = c->pf_part_ml; a.gran_em = c->pf_gran_em; a.n_aq = G.Hq; a.n_ag_max = c->n_ag_max;
+    for (int q0 = 0; q0 < n_queries; q0 += c->pf_queries) {   // the scores of the text queries add up, the last ones place
+      const int nq = std::min(c->pf_queries, n_queries - q0);
+      a.q = (const bf16 *)q_last_dev + (size_t)q0 * G.Hq * G.d;
+      CK(launch_attn_uniform(c->cv, a, G.Hkv, nq, st));
+      CK(launch_prefill_select(c->cv, seq, layer, np, nq, c->pf_part_ml, c->pf_gran_em, c->n_ag_max, q0 == 0, q0 + nq == n_queries, st));
     }
+    bf16 *out = nullptr;
+    if (c->layers[layer].n_tidal > 0) {
+      const int r = c->mst_next;
+      if (c->mst_used[r]) CK(cudaStreamWaitEvent(st, c->ev_mst_free[r], 0));
+      out = c->mst[r];
+    }
+    CK(launch_place_gather(c->cv, seq, layer, c->stage, C_b, out, st));
+    *mirror_out = out;
   }
-  CK(launch_place_gather(c->cv, seq, layer, full ? 1 : 0, c->stage, C_b, st));
   CK(cudaEventRecord(c->ev_place, st));
   c->place_recorded = true;
   c->last_stream = st;
@@ -1133,7 +1145,6 @@ extern "C" wnw_status_t wnw_append_audio(wnw_cache_t *c, int32_t seq, int32_t la
   if (last) {
     s.T_a = T_new; s.C = C_new; s.S = S_new; s.S_base = S_new;
     c->wl_layers.clear();   // the heads grew: the next step cuts its work anew
-    c->prefill_seq = -1;
   }
   return WNW_OK;
 }
@@ -1183,10 +1194,12 @@ extern "C" wnw_status_t wnw_place_prefill_tokens(wnw_cache_t *c, int32_t seq, in
       m_host[h] = variant != 0 ? make_int2(-1, -1)
                                : make_int2((int)std::floor((double)retention[h] * (double)G.nc), (int)std::floor((double)retention[h] * (double)tail_len));
   }
-  wnw_status_t rc = place_multi(c, seq, layer, k_dev, v_dev, n_tokens, audio_begin, audio_end, q_text_dev, n_queries, cuda_stream);
-  if (rc != WNW_OK || n_comp == 0 || T_a == 0) return rc;
-  DeviceGuard guard(c->cfg.device);
   cudaStream_t st = (cudaStream_t)cuda_stream;
+  bf16 *out = nullptr;
+  wnw_status_t rc = place_multi(c, seq, layer, k_dev, v_dev, n_tokens, audio_begin, audio_end, q_text_dev, n_queries, st, &out);
+  if (rc != WNW_OK) return rc;
+  if (n_comp == 0 || T_a == 0) return out ? send_mirror(c, seq, layer, st) : WNW_OK;
+  DeviceGuard guard(c->cfg.device);
   SeqHost &s = c->seqs[seq];
   if (!c->fixed_tok) {
     int fmax = 0;
@@ -1209,14 +1222,14 @@ extern "C" wnw_status_t wnw_place_prefill_tokens(wnw_cache_t *c, int32_t seq, in
                        cudaMemcpyHostToDevice, st));
   CK(launch_token_compress(c->cv, seq, layer, n_comp, n_tidal_base, c->stage, (const bf16 *)q_text_dev, n_queries, s.T_t, T_a,
                            segment_tokens, c->tok_ret, variant, c->tok_work, c->tok_p, c->tok_flags, c->tok_p_stride,
-                           c->fixed_tok, c->tok_cap, c->tok_n, st));
+                           c->fixed_tok, c->tok_cap, c->tok_n, out, st));
   CK(cudaEventRecord(c->ev_place, st));
   if (s.fixed_blocks.empty()) s.fixed_blocks.assign((size_t)G.L * G.Hkv, -1);
   if (s.tok_m.empty()) s.tok_m.assign((size_t)G.L * G.Hkv, make_int2(0, 0));
   for (int h = 0; h < G.Hkv; ++h) { s.fixed_blocks[layer * G.Hkv + h] = blocks[h]; s.tok_m[layer * G.Hkv + h] = m_host[h]; }
   c->wl_layers.clear();
   c->tok_last_seq = seq; c->tok_last_layer = layer;
-  return WNW_OK;
+  return out ? send_mirror(c, seq, layer, st) : WNW_OK;
 }
 
 // Index of a head's compact store among the sequence's (fixed heads first, then tidal token bases), -1 if it has none;
@@ -1509,6 +1522,8 @@ static wnw_status_t issue_side_work(wnw_cache *c, int layer, bool tiered, bool c
     CK(launch_select(c->cv, sa, c->sel_smem[layer], select_groups(li), ss));
     c->count_launch(1, 1, capturing);
     if (li.upd_count > 0 && !c->cap_external_recall && !defer) {
+      wnw_status_t ms = capturing ? WNW_OK : wait_for_mirror(c, ss);   // a replayed step waits as a whole
+      if (ms != WNW_OK) return ms;
       CK(launch_recall(c->cv, n_active, c->d_active, c->cv.upd_list + li.upd_first, li.upd_count,
                        c->cfg.recall_mode == WNW_RECALL_SKIP, RecallSignal{nullptr, nullptr, nullptr, 0}, ss));
       c->count_launch(2, 1, capturing);
@@ -1560,7 +1575,6 @@ static wnw_status_t decode_layer_impl(wnw_cache *c, int want_mode, int32_t layer
     a.order = c->d_sched + lw.order_off; a.cta_ranges = c->d_sched + c->sched_ranges_base + lw.ranges_off; a.n_ctas = lw.n_ctas;
     a.xpref = lw.packed;
   }
-  a.head_items = c->d_head_items + lw.head_items_off;
   a.q = (const bf16 *)q; a.k_new = (const bf16 *)k_new; a.v_new = (const bf16 *)v_new;
   a.head_done = c->head_done + (size_t)layer * G.max_batch * G.Hkv; a.head_mz = head_mz_l; a.out = (bf16 *)out;
   a.anchor_base = c->cv.anchor; a.anchor_seq_stride = G.anchor_seq_stride;
@@ -1665,6 +1679,8 @@ extern "C" wnw_status_t wnw_import_prefill_tidal(wnw_cache_t *c, int32_t seq, in
   DeviceGuard guard(c->cfg.device);
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (c->place_recorded) CK(cudaStreamWaitEvent(st, c->ev_place, 0));
+  wnw_status_t ms = wait_for_mirror(c, st);
+  if (ms != WNW_OK) return ms;
   if (c->layers[layer].n_tidal > 0 && c->seqs[seq].C > 0) CK(launch_prefill_retable(c->cv, seq, layer, (const float *)sums_dev, st));
   CK(cudaEventRecord(c->ev_place, st));
   c->place_recorded = true;
@@ -1701,6 +1717,8 @@ extern "C" wnw_status_t wnw_step_end(wnw_cache_t *c, void *cuda_stream) {
       stp.n_active = (int)c->active.size(); stp.active = c->d_active; stp.do_score = 0; stp.do_update = 1;
       CK(select_all(c, c->sel_map_update, stp, st));
       c->count_launch(1, 1, false);
+      wnw_status_t ms = wait_for_mirror(c, st);
+      if (ms != WNW_OK) return ms;
       CK(launch_recall(c->cv, (int)c->active.size(), c->d_active, c->cv.upd_list, (int)c->upd_list.size(),
                        c->cfg.recall_mode == WNW_RECALL_SKIP, RecallSignal{nullptr, nullptr, nullptr, 0}, st));
       c->count_launch(2, 1, false);
@@ -1795,6 +1813,13 @@ extern "C" wnw_status_t wnw_graph_launch(wnw_cache_t *c, void *cuda_stream) {
   // side-stream work of earlier eager steps touches the tables and slots the graph reads
   for (int l = 0; l < c->geo.L; ++l)
     if (c->side_recorded[l]) { CK(cudaStreamWaitEvent(st, c->ev_side_done[l], 0)); c->side_recorded[l] = 0; }
+  // Mirror copies of the last placement may still be under way.  A step whose recall follows it outside the graph can run
+  // beside them, the first one only: the next one's CTAs would sit on their SMs waiting for that recall.
+  if (c->mirror_pending && (!c->graph_external_recall || c->mirror_step_issued)) {
+    wnw_status_t ms = wait_for_mirror(c, st);
+    if (ms != WNW_OK) return ms;
+  }
+  c->mirror_step_issued = true;
   CK(cudaGraphLaunch(c->graph_exec, st));
   for (int k = 0; k < 4; ++k) c->launches[k] += c->cap_launches[k];  // the kernels of the captured step
   if (c->graph_external_recall && !c->upd_list.empty()) {
@@ -1803,6 +1828,8 @@ extern "C" wnw_status_t wnw_graph_launch(wnw_cache_t *c, void *cuda_stream) {
     // CTAs wait on the per-layer epoch words it publishes.
     CK(cudaEventRecord(c->ev_graph_done, st));
     CK(cudaStreamWaitEvent(c->side[0], c->ev_graph_done, 0));
+    wnw_status_t ms = wait_for_mirror(c, c->side[0]);
+    if (ms != WNW_OK) return ms;
     CK(launch_recall(c->cv, (int)c->graph_active.size(), c->d_active, c->cv.upd_list, (int)c->upd_list.size(),
                      c->cfg.recall_mode == WNW_RECALL_SKIP, RecallSignal{c->d_recall_epoch, c->d_recall_ctr, c->d_empty_ctr, c->host_epoch},
                      c->side[0]));
@@ -1824,6 +1851,8 @@ extern "C" wnw_status_t wnw_graph_launch(wnw_cache_t *c, void *cuda_stream) {
 static wnw_status_t drain(wnw_cache *c) {
   CK(cudaStreamSynchronize(c->last_stream));
   for (auto sd : c->side) CK(cudaStreamSynchronize(sd));
+  if (c->copy_stream) CK(cudaStreamSynchronize(c->copy_stream));
+  c->mirror_pending = false;
   return WNW_OK;
 }
 

@@ -196,11 +196,11 @@ __global__ void __launch_bounds__(128) wnw_token_gather_kernel(const __grid_cons
 }
 
 // grid (segments, tidal heads of the layer); block 128.  Token-granular tidal base: rewrites segment blockIdx.x of the
-// head's host mirror with the positions that are NOT in the base first (ascending), the kept ones after them, so that
+// head in the layer's outgoing mirror image with the positions that are NOT in the base first (ascending), the kept ones after them, so that
 // the first (length - kept) rows of a fetched segment are exactly its complement.
 __global__ void __launch_bounds__(128) wnw_token_mirror_kernel(const __grid_constant__ CacheView cv, int b, int layer,
                                                                const bf16 *stage, const int32_t *flags, long long p_stride,
-                                                               int T_a) {
+                                                               int T_a, bf16 *mirror_out) {
   const Geometry &G = cv.geo;
   extern __shared__ int mirror_dst[];   // [nc] destination row of every position of the segment
   const LayerInfo li = cv.layers[layer];
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(128) wnw_token_mirror_kernel(const __grid_cons
   const int pieces = G.d / 8;
   for (int kv = 0; kv < 2; ++kv) {
     const uint4 *src = reinterpret_cast<const uint4 *>(stage + anchor_off(G, 0, 0, h, kv) + (long long)c * G.ncp * G.d);
-    uint4 *dst = reinterpret_cast<uint4 *>(cv.mirror[b] + mirror_off(G, li, mirror_chunks_of(G, cv.C[b]), c, t, kv));
+    uint4 *dst = reinterpret_cast<uint4 *>(mirror_out + mirror_block_off(G, li, c, t, kv));
     for (int v = threadIdx.x; v < len * pieces; v += blockDim.x) {
       const int r = v / pieces, piece = v - r * pieces;
       dst[(long long)mirror_dst[r] * pieces + piece] = src[v];
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(128) wnw_token_mirror_kernel(const __grid_cons
 cudaError_t launch_token_compress(const CacheView &cv, int b, int layer, int n_comp, int n_tidal_base, const bf16 *stage,
                                   const bf16 *q_text, int n_q, int T_t, int T_a, int seg, const float *retention_dev,
                                   int variant, float *work, float *p_tok, int32_t *flags, long long p_stride,
-                                  int32_t *fixed_tok, int tok_cap, int32_t *tok_n, cudaStream_t st) {
+                                  int32_t *fixed_tok, int tok_cap, int32_t *tok_n, bf16 *mirror_out, cudaStream_t st) {
   if (n_comp <= 0 || T_a <= 0) return cudaSuccess;
   const size_t smem = (size_t)(cv.geo.d + TOK_THREADS / 32) * sizeof(float);
   wnw_token_score_kernel<<<n_comp, TOK_THREADS, smem, st>>>(cv, b, layer, stage, q_text, n_q, T_t, T_a, work, p_tok, p_stride);
@@ -243,7 +243,7 @@ cudaError_t launch_token_compress(const CacheView &cv, int b, int layer, int n_c
   if (n_tidal_base > 0) {
     const int C_b = (T_a + cv.geo.nc - 1) / cv.geo.nc;
     wnw_token_mirror_kernel<<<dim3(C_b, n_tidal_base), 128, (size_t)cv.geo.nc * sizeof(int), st>>>(cv, b, layer, stage, flags,
-                                                                                                  p_stride, T_a);
+                                                                                                  p_stride, T_a, mirror_out);
   }
   return cudaGetLastError();
 }
