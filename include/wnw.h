@@ -375,12 +375,12 @@ wnw_status_t wnw_sync(wnw_cache_t *cache);
  * Result: out = softmax(q K^T * scale) V per query head, the same computation wnw_decode_layer_full performs for
  * one sequence.  Limits (beyond them the call returns WNW_ERR_CAPACITY and does nothing): at most 64 KV heads,
  * 128 query heads, group size 16, 1,048,576 padded tokens; head_dim 64 or 128 (else WNW_ERR_UNSUPPORTED).
- * Each call queues two kernels on cuda_stream: a small one that clears the counters, then the attention kernel.
+ * Each call queues one kernel on cuda_stream.
  *
  * The first call on a device looks up the array's device address and opts the kernels into their shared-memory
  * size; make that first call before any stream capture on that device.  Every call shares the one array, which
- * keeps the previous call's contents (the call clears what must start at zero): two calls whose GPU work overlaps
- * in time - different streams, or different threads - race on it.  Calls on one stream are safe back to back.
+ * keeps the previous call's contents: two calls whose GPU work overlaps in time - different streams, or different
+ * threads - race on it.  Calls on one stream are safe back to back.
  *
  * Every device-side wait of the kernel is bounded.  If one ever runs out (a copy that never lands), the kernel
  * finishes on what it has, the output is incomplete, and a sticky bit is set in the array's status word;
