@@ -243,7 +243,7 @@ struct SelectArgs {
 // Completion signalling of a recall launch that runs outside the captured step (all null for in-step launches).
 struct RecallSignal {
   int32_t *epoch_words;       // [L] epoch of the last completed recall of each layer's table
-  int32_t *counters;          // [L] finished-CTA counters (self-resetting)
+  int32_t *counters;          // [L] finished-warp counters (self-resetting)
   int32_t *empty_ctr;         // [L] the selection kernels' empty-plan counters, reset here
   int32_t publish_epoch;      // epoch to publish: the number of replayed steps that have ended with this one (the host counts
                               // them; the device word may already be further when this kernel runs late)
@@ -267,7 +267,7 @@ cudaError_t launch_select_all_params(const CacheView &cv, const SelectArgs *laye
 cudaError_t launch_step_end(const CacheView &cv, int n_active, const int32_t *active, int appended, int32_t *bump_epoch,
                             cudaStream_t st);
 cudaError_t launch_recall(const CacheView &cv, int n_active, const int32_t *active, const int32_t *layers_dev, int n_layers,
-                          int skip_copy, RecallSignal sig, cudaStream_t st);
+                          int skip_copy, bool crowded, RecallSignal sig, cudaStream_t st);   // crowded: attention launches overlap
 cudaError_t launch_place_scatter(const CacheView &cv, int b, int layer, int full_mode, const bf16 *k, const bf16 *v, int ab, int ae,
                                  int T_t, int C_b, int S_b, int S_base, bf16 *stage, cudaStream_t st);
 // np: pieces a head was cut into by the scoring launch; n_q text queries; first, last: whether the placement begins, ends with them

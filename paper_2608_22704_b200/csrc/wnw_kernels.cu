@@ -314,96 +314,104 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 }
 
 // ------------------------------------------------------------------------------------------------
-// Recall: copies every planned chunk block pinned host -> slot pool.  A NARROW kernel: RECALL_CTAS CTAs in up to
-// RECALL_GROUPS groups; group g walks the layers g, g + groups, ... (earlier layers first), every CTA of the group taking
-// its stripe of each block, so several layers' transfers are in flight at once.  The host link needs little in flight
-// (32 CTAs x 256 threads x four 16-byte loads = 512 KB); CTAs that wait on the link must not sit on the SMs the
-// attention kernels need (40 registers, one CTA per SM, fits beside a resident attention CTA).
+// Recall: copies every planned chunk block pinned host -> slot pool, reading the mapped host memory from the SMs.
+//
+// What bounds it is the host link (51.4 GB/s for this access pattern), and what it must not do is queue up on it: 128 KB in
+// flight reach the full rate (64 KB: 39.5 GB/s), every further request only waits in the link's queue, and so does whatever
+// else crosses the link meanwhile, the GPU's own command fetches among them (a small copy or kernel on another stream,
+// host round trip: 11 us alone, 18 us beside 128 KB, 61 us beside 512 KB, 116 us beside 2 MB in flight).  So the grid is
+// a few CTAs of 8 warps with RECALL_U 16-byte loads in flight per lane, whatever there is to copy, and the warps work
+// independently: the blocks of a launch are cut into pieces of a warp's batch and dealt round robin ACROSS block and layer
+// borders, so that all warps have work and nothing waits at a barrier.
+// 40 registers a thread: a CTA fits beside a resident 8-warp attention CTA.
+// 8 CTAs where layers wait for one another: the copies have the whole next step's time (config 1, 30 chained layers, recall
+// and the step's own small copies: 254 us a step with the former 128 CTAs, 238.7 with 8, 241 with 12, 243 with 16).  24 CTAs
+// where layers overlap: attention then fills the memory system, a host read takes several times as long and the step waits for
+// it (4 x 3000 tokens: 225 us a step with 8, 197 with 16, 193 with 24, 194 with 32, 198 with 48; formerly 206).
+//
 // With `sig` set (replayed steps, where this kernel runs outside the captured graph and overlaps the next step) the
-// CTA that finishes a layer last publishes the layer's recall epoch, which the next step's tidal CTAs acquire.
+// warp that finishes a layer last publishes the layer's recall epoch, which the next step's tidal CTAs acquire.
 // ------------------------------------------------------------------------------------------------
-constexpr int RECALL_CTAS = 32, RECALL_GROUPS = 8;
-__global__ void __launch_bounds__(256, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
-                                                            const int32_t *active, const int32_t *layers, int n_layers,
-                                                            int n_groups, int skip_copy, RecallSignal sig) {
+constexpr int RECALL_CTAS = 8, RECALL_CTAS_CROWDED = 24, RECALL_WARPS = 8, RECALL_U = 4;
+__global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
+                                                                          const int32_t *active, const int32_t *layers,
+                                                                          int n_layers, int skip_copy, RecallSignal sig) {
   const Geometry &G = cv.geo;
-  constexpr int U = 4;
-  const int cpg = gridDim.x / n_groups, grp = blockIdx.x / cpg, rank = blockIdx.x - grp * cpg;
-  const int stride = cpg * blockDim.x;
-  for (int x = grp; x < n_layers; x += n_groups) {
-    const int l = layers[x];
-    if (sig.epoch_words) {
-      // Already published for this step (by the selection kernel: no sequence planned a copy for this layer).  Its
-      // plans must not be read then: the next step's selection may be rewriting them by now.
+  const int lane = threadIdx.x & 31, n_warps = gridDim.x * RECALL_WARPS, w = blockIdx.x * RECALL_WARPS + (threadIdx.x >> 5);
+  int turn = 0;   // the warp that takes the next piece (the same on every warp: plans do not change under this kernel)
+  for (int x0 = 0; x0 < n_layers; x0 += 32) {
+    // a lane looks up one layer: whether its epoch is out already (the selection kernel publishes it when no sequence planned
+    // a copy for the layer; its plans must not be read then, the next step's selection may be rewriting them by now)
+    const int my_l = x0 + lane < n_layers ? layers[x0 + lane] : -1;
+    bool todo = my_l >= 0;
+    if (todo && sig.epoch_words) {
       int seen;
-      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(seen) : "l"(sig.epoch_words + l) : "memory");
-      if (seen >= sig.publish_epoch) continue;
+      asm volatile("ld.acquire.gpu.global.s32 %0, [%1];\n" : "=r"(seen) : "l"(sig.epoch_words + my_l) : "memory");
+      todo = seen < sig.publish_epoch;
     }
-    const LayerInfo &li = cv.layers[l];
-    const int n = li.n_tidal * 2 * G.ncp * G.d * tidal_elem_bytes(G) / 16;  // 16-byte vectors per chunk block (far below 2^31)
-    bool copies = false;                             // uniform over the whole grid: the plans do not change under this kernel
-    for (int i = 0; i < n_active; ++i) {
-      const int b = active[i];
-      const long long bl = (long long)b * G.L + l;
-      const int n_plan = cv.n_plan[bl];
-      for (int r = 0; r < n_plan && r < G.plan_cap; ++r) {
-        const int c = cv.plan[(bl * G.plan_cap + r) * 2], slot = cv.plan[(bl * G.plan_cap + r) * 2 + 1];
-        if (rank == 0 && threadIdx.x == 0) atomicAdd(cv.stats + (long long)b * 4 + 3, (unsigned long long)n * 16ull);
-        if (skip_copy) continue;
-        copies = true;
-        if (c < 0 || c >= cv.C[b] || slot < 0 || slot >= cv.S[b]) {
-          if (threadIdx.x == 0) atomicOr(cv.status, STATUS_BAD_TABLE);
-          continue;
-        }
-        const uint4 *src = reinterpret_cast<const uint4 *>(tier_ptr(G, cv.mirror[b], mirror_off(G, li, mirror_chunks_of(G, cv.C[b]), c, 0, 0)));
-        uint4 *dst = reinterpret_cast<uint4 *>(tier_ptr(G, cv.pool, pool_off(G, li, b, slot, 0, 0)));
-        for (int v0 = rank * blockDim.x + threadIdx.x; v0 < n; v0 += stride * U) {
-          uint4 t[U];
+    for (unsigned left = __ballot_sync(0xffffffffu, todo); left; left &= left - 1) {
+      const int l = __shfl_sync(0xffffffffu, my_l, __ffs(left) - 1);
+      const int n_tidal = cv.layers[l].n_tidal;
+      const int n = n_tidal * 2 * G.ncp * G.d * tidal_elem_bytes(G) / 16;   // 16-byte vectors per chunk block (far below 2^31)
+      const int n_piece = (n + 32 * RECALL_U - 1) / (32 * RECALL_U);
+      for (int i0 = 0; i0 < n_active; i0 += 32) {
+        const int my_b = i0 + lane < n_active ? active[i0 + lane] : -1;
+        const int my_n = my_b >= 0 ? min(cv.n_plan[(long long)my_b * G.L + l], G.plan_cap) : 0;
+        for (unsigned seqs = __ballot_sync(0xffffffffu, my_n > 0); seqs; seqs &= seqs - 1) {
+          const int b = __shfl_sync(0xffffffffu, my_b, __ffs(seqs) - 1), n_plan = __shfl_sync(0xffffffffu, my_n, __ffs(seqs) - 1);
+          if (w == 0 && lane == 0) atomicAdd(cv.stats + (long long)b * 4 + 3, (unsigned long long)n_plan * n * 16ull);
+          if (skip_copy) continue;
+          // all plan entries of the sequence in one round trip (at most 2 * MAX_TOPK of them)
+          const int *plan = cv.plan + ((long long)b * G.L + l) * G.plan_cap * 2;
+          const int my_c = lane < n_plan ? plan[2 * lane] : 0, my_slot = lane < n_plan ? plan[2 * lane + 1] : 0;
+          const int C_b = cv.C[b], S_b = cv.S[b];
+          bf16 *mirror = cv.mirror[b];
+          for (int r = 0; r < n_plan; ++r) {
+            const int c = __shfl_sync(0xffffffffu, my_c, r), slot = __shfl_sync(0xffffffffu, my_slot, r);
+            if (c < 0 || c >= C_b || slot < 0 || slot >= S_b) {
+              if (lane == 0) atomicOr(cv.status, STATUS_BAD_TABLE);
+              continue;
+            }
+            int p = w - turn;
+            if (p < 0) p += n_warps;
+            turn = (turn + n_piece) % n_warps;
+            if (p >= n_piece) continue;
+            const uint4 *src = reinterpret_cast<const uint4 *>(tier_ptr(G, mirror, mirror_off(G, cv.layers[l], mirror_chunks_of(G, C_b), c, 0, 0)));
+            uint4 *dst = reinterpret_cast<uint4 *>(tier_ptr(G, cv.pool, pool_off(G, cv.layers[l], b, slot, 0, 0)));
+            for (; p < n_piece; p += n_warps) {
+              const int v0 = p * 32 * RECALL_U + lane;
+              uint4 t[RECALL_U];
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int v = v0 + u * stride;
-            if (v < n) t[u] = __ldcs(src + v);
-          }
+              for (int u = 0; u < RECALL_U; ++u)
+                if (v0 + u * 32 < n) t[u] = __ldcs(src + v0 + u * 32);
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const int v = v0 + u * stride;
-            if (v < n) dst[v] = t[u];
+              for (int u = 0; u < RECALL_U; ++u)
+                if (v0 + u * 32 < n) dst[v0 + u * 32] = t[u];
+            }
           }
         }
       }
-    }
-    if (sig.epoch_words && !copies) {
-      // nothing was written for this layer: its epoch goes out at once, without the round of fences and counting
-      if (rank == 0 && threadIdx.x == 0) {
-        sig.empty_ctr[l] = 0;
-        asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(sig.epoch_words + l), "r"(sig.publish_epoch) : "memory");
-      }
-    } else if (sig.epoch_words) {  // completion of this layer's recall: counted per CTA, published by the last one
-      __threadfence();
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        const int prev = atomicAdd(sig.counters + l, 1);
-        if (prev == cpg - 1) {
-          sig.counters[l] = 0;
-          sig.empty_ctr[l] = 0;
+      if (sig.epoch_words) {   // completion of this layer's recall: counted per warp, published by the last one
+        __syncwarp();
+        if (lane == 0) {
           __threadfence();
-          asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(sig.epoch_words + l), "r"(sig.publish_epoch) : "memory");
+          if (atomicAdd(sig.counters + l, 1) == n_warps - 1) {
+            sig.counters[l] = 0;
+            sig.empty_ctr[l] = 0;
+            __threadfence();
+            asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(sig.epoch_words + l), "r"(sig.publish_epoch) : "memory");
+          }
         }
+        __syncwarp();
       }
     }
   }
 }
 
 cudaError_t launch_recall(const CacheView &cv, int n_active, const int32_t *active, const int32_t *layers_dev, int n_layers,
-                          int skip_copy, RecallSignal sig, cudaStream_t st) {
+                          int skip_copy, bool crowded, RecallSignal sig, cudaStream_t st) {
   if (n_layers <= 0 || n_active <= 0) return cudaSuccess;
-  // A few tables (one short sequence or two): what counts is when the last block lands, and the link's latency grows
-  // several times while attention saturates the memory system, so four times the CTAs keep four times the loads in
-  // flight (config 1 back to back: 56 -> 53 us per step).  Many tables: the link's rate counts and more CTAs only take
-  // SM resources from attention (batch-32 ragged, link-bound: 2.56 -> 2.88 ms per step with the wide launch).
-  const int n_groups = RECALL_GROUPS, n_ctas = sig.epoch_words && (long long)n_active * n_layers <= 64 ? 4 * RECALL_CTAS : RECALL_CTAS;
-  const int groups = n_layers < n_groups ? n_layers : n_groups;   // few layers: all CTAs on each block
-  wnw_recall_kernel<<<n_ctas / groups * groups, 256, 0, st>>>(cv, n_active, active, layers_dev, n_layers, groups, skip_copy, sig);
+  wnw_recall_kernel<<<crowded ? RECALL_CTAS_CROWDED : RECALL_CTAS, RECALL_WARPS * 32, 0, st>>>(cv, n_active, active, layers_dev, n_layers, skip_copy, sig);
   return cudaGetLastError();
 }
 

@@ -65,6 +65,8 @@ struct wnw_cache {
   int tid_total = 0, n_sm = 148;
   std::vector<SeqHost> seqs;
   std::vector<void *> dev_allocs;
+  char *small_block = nullptr;      // where the next small device array goes
+  size_t small_used = 0;
   std::vector<bf16 *> mirror_ptrs;  // host copy of cv.mirror
   bf16 *stage = nullptr;
   TmaMaps maps_decode, maps_prefill;  // TMA descriptors: cache stores; prefill scoring reads the staging copy as `anchor`
@@ -170,6 +172,11 @@ struct wnw_cache {
     }                                            \
   } while (0)
 
+// Layers whose attention launches run over one another (as opposed to chained or serial ones).
+static bool layers_overlap(const wnw_cache *c) {
+  return c->layer_dependency == WNW_LAYERS_INDEPENDENT || c->layer_dependency == WNW_LAYERS_BATCHED;
+}
+
 // CTAs per sequence of a layer's selection kernel: one per eight tables to update.
 static int select_groups(const LayerInfo &li) { return std::max(1, std::min(8, (li.upd_count + 7) / 8)); }
 
@@ -200,9 +207,24 @@ static int compact_blocks(const wnw_config_t &cfg, int C) {
   return base + std::min(2 * cfg.topk * (cfg.evict_lag + 1), C - base);
 }
 
+// Small arrays share zeroed blocks (an allocation of its own costs a cache some 0.1 ms to create).
 template <typename T>
 static wnw_status_t dev_alloc(wnw_cache *c, T **p, size_t count, bool zero = true) {
+  constexpr size_t small = 64 << 10, block = 1 << 20;
   const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
+  if (bytes <= small) {
+    const size_t take = (bytes + 255) / 256 * 256;
+    if (!c->small_block || c->small_used + take > block) {
+      c->small_block = nullptr;
+      CK(cudaMalloc((void **)&c->small_block, block));
+      c->dev_allocs.push_back((void *)c->small_block);
+      CK(cudaMemset(c->small_block, 0, block));
+      c->small_used = 0;
+    }
+    *p = reinterpret_cast<T *>(c->small_block + c->small_used);
+    c->small_used += take;
+    return WNW_OK;
+  }
   CK(cudaMalloc((void **)p, bytes));
   c->dev_allocs.push_back((void *)*p);
   if (zero) CK(cudaMemset(*p, 0, bytes));
@@ -488,9 +510,10 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
     if (!full && tid_max > 0 && G.C_max > 0) {
       CKE(cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking));
       CKE(cudaEventCreateWithFlags(&c->ev_mirror, cudaEventDisableTiming));
+      const size_t elems = (size_t)G.C_max * tid_max * 2 * G.ncp * d / (G.kv8 ? 2 : 1);
+      CKC(dev_alloc(c, &c->mst[0], elems * wnw_cache::MIRROR_RING, false));
       for (int r = 0; r < wnw_cache::MIRROR_RING; ++r) {
-        const size_t elems = (size_t)G.C_max * tid_max * 2 * G.ncp * d;
-        CKC(dev_alloc(c, &c->mst[r], G.kv8 ? (elems + 1) / 2 : elems, false));
+        c->mst[r] = c->mst[0] + elems * r;
         CKE(cudaEventCreateWithFlags(&c->ev_mst_ready[r], cudaEventDisableTiming));
         CKE(cudaEventCreateWithFlags(&c->ev_mst_free[r], cudaEventDisableTiming));
       }
@@ -775,7 +798,7 @@ static void build_layer_items(const wnw_cache *c, int layer, int mode, const std
     }
   }
   bool throughput = false;
-  const bool overlapped = c->layer_dependency == WNW_LAYERS_INDEPENDENT || c->layer_dependency == WNW_LAYERS_BATCHED;
+  const bool overlapped = layers_overlap(c);
   int gpi = granules_per_item(c, total, longest, (int)seq_ids.size() * G.Hkv, overlapped, &throughput);
   // BATCHED layers share one launch: the work of the whole step is cut for one wave of CTAs, long heads into pieces as
   // fat as a pack of short ones, short heads packed whole
@@ -1525,7 +1548,7 @@ static wnw_status_t issue_side_work(wnw_cache *c, int layer, bool tiered, bool c
       wnw_status_t ms = capturing ? WNW_OK : wait_for_mirror(c, ss);   // a replayed step waits as a whole
       if (ms != WNW_OK) return ms;
       CK(launch_recall(c->cv, n_active, c->d_active, c->cv.upd_list + li.upd_first, li.upd_count,
-                       c->cfg.recall_mode == WNW_RECALL_SKIP, RecallSignal{nullptr, nullptr, nullptr, 0}, ss));
+                       c->cfg.recall_mode == WNW_RECALL_SKIP, layers_overlap(c), RecallSignal{nullptr, nullptr, nullptr, 0}, ss));
       c->count_launch(2, 1, capturing);
     }
     if (!inline_mode) {
@@ -1720,7 +1743,7 @@ extern "C" wnw_status_t wnw_step_end(wnw_cache_t *c, void *cuda_stream) {
       wnw_status_t ms = wait_for_mirror(c, st);
       if (ms != WNW_OK) return ms;
       CK(launch_recall(c->cv, (int)c->active.size(), c->d_active, c->cv.upd_list, (int)c->upd_list.size(),
-                       c->cfg.recall_mode == WNW_RECALL_SKIP, RecallSignal{nullptr, nullptr, nullptr, 0}, st));
+                       c->cfg.recall_mode == WNW_RECALL_SKIP, layers_overlap(c), RecallSignal{nullptr, nullptr, nullptr, 0}, st));
       c->count_launch(2, 1, false);
     }
   }
@@ -1831,7 +1854,7 @@ extern "C" wnw_status_t wnw_graph_launch(wnw_cache_t *c, void *cuda_stream) {
     wnw_status_t ms = wait_for_mirror(c, c->side[0]);
     if (ms != WNW_OK) return ms;
     CK(launch_recall(c->cv, (int)c->graph_active.size(), c->d_active, c->cv.upd_list, (int)c->upd_list.size(),
-                     c->cfg.recall_mode == WNW_RECALL_SKIP, RecallSignal{c->d_recall_epoch, c->d_recall_ctr, c->d_empty_ctr, c->host_epoch},
+                     c->cfg.recall_mode == WNW_RECALL_SKIP, layers_overlap(c), RecallSignal{c->d_recall_epoch, c->d_recall_ctr, c->d_empty_ctr, c->host_epoch},
                      c->side[0]));
     c->count_launch(2, 1, false);
     CK(cudaEventRecord(c->ev_recall_all, c->side[0]));
@@ -2162,7 +2185,7 @@ extern "C" wnw_status_t wnw_measure_host_link(int32_t device, int64_t bytes, int
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) { rc = WNW_ERR_CUDA; break; }
     if (r > 0) best_copy = std::min(best_copy, ms);
     cudaEventRecord(e0, st);
-    if (launch_copy_plan((const uint4 *)hd, (uint4 *)d, bytes / 16, 32, st) != cudaSuccess) { rc = WNW_ERR_CUDA; break; }
+    if (launch_copy_plan((const uint4 *)hd, (uint4 *)d, bytes / 16, 8, st) != cudaSuccess) { rc = WNW_ERR_CUDA; break; }
     cudaEventRecord(e1, st);
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) { rc = WNW_ERR_CUDA; break; }
     if (r > 0) best_kernel = std::min(best_kernel, ms);
