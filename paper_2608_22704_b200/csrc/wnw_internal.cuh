@@ -277,9 +277,11 @@ cudaError_t launch_prefill_select(const CacheView &cv, int b, int layer, int np,
 cudaError_t launch_place_gather(const CacheView &cv, int b, int layer, const bf16 *stage, int C_b, bf16 *mirror_out,
                                 cudaStream_t st);
 // token-granular compression of the layer's fixed heads (after the chunk-granular placement staged the prefix)
+struct TokenRetention { float r[MAX_AQ]; };   // per KV head, by value
+constexpr int TOK_QR = 16;                       // query rows (text query x q-head) of one scoring pass, at least MAX_G
 cudaError_t launch_token_compress(const CacheView &cv, int b, int layer, int n_comp, int n_tidal_base, const bf16 *stage,
-                                  const bf16 *q_text, int n_q, int T_t, int T_a, int seg, const float *retention_dev,
-                                  int variant, float *work, float *p_tok, int32_t *flags, long long p_stride,
+                                  const bf16 *q_text, int n_q, int T_t, int T_a, int seg, const TokenRetention &ret,
+                                  int variant, float *work, float2 *tile_ml, float *p_tok, int32_t *flags, long long p_stride,
                                   int32_t *fixed_tok, int tok_cap, int32_t *tok_n, bf16 *mirror_out, cudaStream_t st);
 cudaError_t launch_append_audio(const CacheView &cv, int b, int layer, int full_mode, const bf16 *k, const bf16 *v, int n_tokens,
                                 int T_a_old, int S_old, int set_dims, int T_a_new, int C_new, int S_new, cudaStream_t st);

@@ -152,7 +152,8 @@ struct wnw_cache {
   cudaEvent_t ev_place = nullptr, ev_step = nullptr;
   bool place_recorded = false, step_recorded = false;
   // token-granular compression of fixed heads (allocated by the first wnw_place_prefill_tokens)
-  float *tok_work = nullptr, *tok_p = nullptr, *tok_ret = nullptr;
+  float *tok_work = nullptr, *tok_p = nullptr;
+  float2 *tok_ml = nullptr;
   int32_t *tok_flags = nullptr, *fixed_tok = nullptr, *tok_n = nullptr;
   int tok_cap = 0, tok_fixed_max = 0, tok_last_seq = -1, tok_last_layer = -1;
   long long tok_p_stride = 0;
@@ -1230,21 +1231,20 @@ extern "C" wnw_status_t wnw_place_prefill_tokens(wnw_cache_t *c, int32_t seq, in
     c->tok_fixed_max = fmax; c->tok_cap = tok_cap;
     c->tok_p_stride = c->cfg.max_audio_tokens;
     const size_t B = G.max_batch;
-    if ((rc = dev_alloc(c, &c->tok_work, (size_t)fmax * ((size_t)c->cfg.max_text_tokens + c->cfg.max_audio_tokens))) != WNW_OK) return rc;
+    const size_t n_max = (size_t)c->cfg.max_text_tokens + c->cfg.max_audio_tokens;
+    if ((rc = dev_alloc(c, &c->tok_work, (size_t)fmax * TOK_QR * n_max, false)) != WNW_OK) return rc;
+    if ((rc = dev_alloc(c, &c->tok_ml, (size_t)fmax * TOK_QR * (n_max / 128 + 1), false)) != WNW_OK) return rc;
     if ((rc = dev_alloc(c, &c->tok_p, (size_t)fmax * c->tok_p_stride)) != WNW_OK) return rc;
     if ((rc = dev_alloc(c, &c->tok_flags, (size_t)fmax * c->tok_p_stride)) != WNW_OK) return rc;
-    if ((rc = dev_alloc(c, &c->tok_ret, (size_t)G.Hkv)) != WNW_OK) return rc;
     if ((rc = dev_alloc(c, &c->tok_n, B * std::max(G.F_tot, 1))) != WNW_OK) return rc;
     if ((rc = dev_alloc(c, &c->fixed_tok, B * std::max(G.F_tot, 1) * (size_t)std::max(tok_cap, 1))) != WNW_OK) return rc;
   }
   // the scratch is shared with earlier placements on other streams: the chunk placement above already ordered this
-  // stream after them; the retention values travel through a pageable copy, complete on the host side at return
-  CK(cudaMemcpyAsync(c->tok_ret, retention, (size_t)G.Hkv * sizeof(float), cudaMemcpyHostToDevice, st));
-  if (n_tidal_base > 0)
-    CK(cudaMemcpyAsync(c->cv.tok_m + ((size_t)seq * G.L + layer) * G.Hkv, m_host.data(), (size_t)G.Hkv * sizeof(int2),
-                       cudaMemcpyHostToDevice, st));
+  // stream after them
+  TokenRetention ret{};
+  for (int h = 0; h < G.Hkv; ++h) ret.r[h] = retention[h];
   CK(launch_token_compress(c->cv, seq, layer, n_comp, n_tidal_base, c->stage, (const bf16 *)q_text_dev, n_queries, s.T_t, T_a,
-                           segment_tokens, c->tok_ret, variant, c->tok_work, c->tok_p, c->tok_flags, c->tok_p_stride,
+                           segment_tokens, ret, variant, c->tok_work, c->tok_ml, c->tok_p, c->tok_flags, c->tok_p_stride,
                            c->fixed_tok, c->tok_cap, c->tok_n, out, st));
   CK(cudaEventRecord(c->ev_place, st));
   if (s.fixed_blocks.empty()) s.fixed_blocks.assign((size_t)G.L * G.Hkv, -1);

@@ -3,15 +3,17 @@
 //
 // Runs once per (sequence, layer) at placement, after the chunk-granular placement has staged the prefix: the staging
 // buffer holds every head's audio K,V in the chunk-padded row layout and the text store holds the text rows.
-//   1. wnw_token_score_kernel : p[tau] = sum over the text queries and the head's q-heads of the softmax weight of audio
-//                               position tau (softmax over the whole prefix), fp32, one CTA per fixed head, passes in a
-//                               fixed order so that the sums are reproducible;
+//   1. wnw_token_logits_kernel, wnw_token_mass_kernel: p[tau] = sum over the text queries and the head's q-heads of the
+//                               softmax weight of audio position tau (softmax over the whole prefix), fp32, sums in a
+//                               fixed order so that they are reproducible;
 //   2. wnw_token_select_kernel: per segment of n_s tokens the floor(retention * length) positions with the largest p
 //                               (equal p: the earlier position), or the same total from the whole head (the ablation's
 //                               global top-k); kept positions in ascending order; block table of the compact store;
 //   3. wnw_token_gather_kernel: K,V rows of the kept positions from staging into the head's compact fixed store.
 // The decode kernel then reads a fixed head as blocks of nc rows whose table entries carry their row count (-(2 + rows))
 // instead of a chunk id.
+#include <algorithm>
+
 #include "wnw_internal.cuh"
 
 namespace wnw {
@@ -19,6 +21,7 @@ namespace wnw {
 namespace {
 
 constexpr int TOK_THREADS = 512;
+constexpr int TOK_TILE = 128;
 
 // Compressed head x of a layer: the fixed heads first, then (token-granular tidal bases) the tidal heads.  Returns the
 // KV-head, and in `head` its index among the sequence's compact stores.
@@ -32,86 +35,107 @@ __device__ __forceinline__ int comp_head(const CacheView &cv, int layer, int x, 
   return -1;
 }
 
-__device__ __forceinline__ float block_max(float v, float *red) {
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  float r = red[0];
-  for (int i = 1; i < TOK_THREADS / 32; ++i) r = fmaxf(r, red[i]);
-  return r;
-}
-__device__ __forceinline__ float block_sum(float v, float *red) {   // fixed tree: the same bits on every run
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  float r = red[0];
-  for (int i = 1; i < TOK_THREADS / 32; ++i) r += red[i];
-  return r;
-}
-
 }  // namespace
 
-// grid: fixed heads of the layer; block: TOK_THREADS.  work: [n_fixed][T_t + T_a] fp32; p_tok: [n_fixed][p_stride] fp32.
-__global__ void __launch_bounds__(TOK_THREADS) wnw_token_score_kernel(const __grid_constant__ CacheView cv, int b, int layer,
-                                                                     const bf16 *stage, const bf16 *q_text, int n_q, int T_t,
-                                                                     int T_a, float *work, float *p_tok, long long p_stride) {
+// Scores in two kernels over tiles of TOK_TILE positions, so that the tiles of all heads fill the machine (one CTA per head, as
+// it was, left 141 of 148 SMs idle: 523 us a layer at 3064 positions, 7 heads, 4 queries of 4 heads; now 21 + 10 us).
+//
+// (1) grid (tiles, compressed heads), a thread per position: its logits for up to TOK_QR query rows (a row = one q-head of one
+// text query).  The position's K row passes through registers once, 16 bytes at a time, the query rows sit in shared memory
+// (broadcast reads).  Bound by the fp32 multiply-adds of the warps in flight, 128 x TOK_QR per position.  A tile also leaves
+// each row's (max, sum of 2^(logit - max)).
+__global__ void __launch_bounds__(TOK_TILE) wnw_token_logits_kernel(const __grid_constant__ CacheView cv, int b, int layer,
+                                                                   const bf16 *stage, const bf16 *q_rows, int n_q, int T_t, int T_a,
+                                                                   float *work, float2 *tile_ml) {
   const Geometry &G = cv.geo;
-  extern __shared__ float tok_smem[];
-  float *qf = tok_smem, *red = tok_smem + G.d;
+  extern __shared__ float tok_smem[];   // [n_q * g][d] query rows, then [n_q * g][warps] (max, sum)
+  const int n = T_t + T_a, d = G.d, g = G.g, n_row = n_q * g, i = blockIdx.x * TOK_TILE + threadIdx.x;
   int head;
-  const int f = blockIdx.x, h = comp_head(cv, layer, f, head);
+  const int f = blockIdx.y, h = comp_head(cv, layer, f, head);
   if (h < 0) return;
-  const int n = T_t + T_a, d = G.d, pieces = d / 8;
-  float *lg = work + (long long)f * (T_t + T_a), *p = p_tok + (long long)f * p_stride;
-  const bf16 *tK = cv.text + text_off(G, b, layer, h, 0), *aK = stage + anchor_off(G, 0, 0, h, 0);
-  for (int t = threadIdx.x; t < T_a; t += TOK_THREADS) p[t] = 0.f;
-  for (int qi = 0; qi < n_q; ++qi)
-    for (int j = 0; j < G.g; ++j) {
-      __syncthreads();
-      const bf16 *q = q_text + ((long long)qi * G.Hq + h * G.g + j) * d;
-      for (int x = threadIdx.x; x < d; x += TOK_THREADS) qf[x] = __bfloat162float(q[x]);
-      __syncthreads();
-      float mx = -INFINITY;
-      for (int i = threadIdx.x; i < n; i += TOK_THREADS) {
-        const bf16 *row;
-        if (i < T_t) row = tK + (long long)i * d;
-        else { const int tau = i - T_t; row = aK + ((long long)(tau / G.nc) * G.ncp + tau % G.nc) * d; }
-        const uint4 *r4 = reinterpret_cast<const uint4 *>(row);
-        float acc = 0.f;
-        for (int v = 0; v < pieces; ++v) {
-          const uint4 u = r4[v];
-          const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(&u);
+  float2 *red = reinterpret_cast<float2 *>(tok_smem + n_row * d);
+  for (int x = threadIdx.x; x < n_row * d; x += TOK_TILE) {
+    const int r = x / d;
+    tok_smem[x] = __bfloat162float(q_rows[((long long)(r / g) * G.Hq + h * g + r % g) * d + (x - r * d)]);
+  }
+  __syncthreads();
+  float acc[TOK_QR];
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 kf = __bfloat1622float2(h2[e]);
-            acc = fmaf(qf[v * 8 + 2 * e], kf.x, acc);
-            acc = fmaf(qf[v * 8 + 2 * e + 1], kf.y, acc);
-          }
+  for (int r = 0; r < TOK_QR; ++r) acc[r] = 0.f;
+  if (i < n) {
+    const bf16 *row;
+    if (i < T_t) row = cv.text + text_off(G, b, layer, h, 0) + (long long)i * d;
+    else { const int tau = i - T_t; row = stage + anchor_off(G, 0, 0, h, 0) + ((long long)(tau / G.nc) * G.ncp + tau % G.nc) * d; }
+    const uint4 *r4 = reinterpret_cast<const uint4 *>(row);
+#pragma unroll 2
+    for (int v = 0; v < d / 8; ++v) {
+      const uint4 u = r4[v];
+      const __nv_bfloat162 *h2 = reinterpret_cast<const __nv_bfloat162 *>(&u);
+      float kf[8];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) { const float2 x = __bfloat1622float2(h2[e]); kf[2 * e] = x.x; kf[2 * e + 1] = x.y; }
+#pragma unroll
+      for (int r = 0; r < TOK_QR; ++r)
+        if (r < n_row) {
+          const float4 qa = *reinterpret_cast<const float4 *>(tok_smem + r * d + v * 8), qb = *reinterpret_cast<const float4 *>(tok_smem + r * d + v * 8 + 4);
+          acc[r] = fmaf(qa.x, kf[0], acc[r]); acc[r] = fmaf(qa.y, kf[1], acc[r]); acc[r] = fmaf(qa.z, kf[2], acc[r]); acc[r] = fmaf(qa.w, kf[3], acc[r]);
+          acc[r] = fmaf(qb.x, kf[4], acc[r]); acc[r] = fmaf(qb.y, kf[5], acc[r]); acc[r] = fmaf(qb.z, kf[6], acc[r]); acc[r] = fmaf(qb.w, kf[7], acc[r]);
         }
-        const float l2 = acc * G.scale_log2;
-        lg[i] = l2;
-        mx = fmaxf(mx, l2);
-      }
-      mx = block_max(mx, red);
-      float z = 0.f;
-      for (int i = threadIdx.x; i < n; i += TOK_THREADS) {
-        const float e = exp2f(lg[i] - mx);
-        lg[i] = e;
-        z += e;
-      }
-      z = block_sum(z, red);
-      for (int t = threadIdx.x; t < T_a; t += TOK_THREADS) p[t] += __fdiv_rn(lg[T_t + t], z);
     }
+  }
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int r = 0; r < TOK_QR; ++r)
+    if (r < n_row) {
+      const float l2 = i < n ? acc[r] * G.scale_log2 : -INFINITY;
+      if (i < n) work[((long long)f * TOK_QR + r) * n + i] = l2;
+      float m = l2;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      float z = m > -INFINITY ? exp2f(l2 - m) : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      if (lane == 0) red[r * (TOK_TILE / 32) + w] = make_float2(m, z);
+    }
+  __syncthreads();
+  for (int r = threadIdx.x; r < n_row; r += TOK_TILE) {
+    float M = -INFINITY, Z = 0.f;
+    for (int x = 0; x < TOK_TILE / 32; ++x) M = fmaxf(M, red[r * (TOK_TILE / 32) + x].x);
+    for (int x = 0; x < TOK_TILE / 32; ++x) Z += red[r * (TOK_TILE / 32) + x].y * exp2f(red[r * (TOK_TILE / 32) + x].x - M);
+    tile_ml[((long long)f * TOK_QR + r) * gridDim.x + blockIdx.x] = make_float2(M, Z);
+  }
+}
+
+// (2) grid (tiles of the audio, compressed heads): the rows' final (max, denominator) from the tiles' (a warp per row, fixed
+// tree), then p[tau] += 2^(logit - max) / denominator, row by row in order.
+__global__ void __launch_bounds__(TOK_TILE) wnw_token_mass_kernel(const __grid_constant__ CacheView cv, int n_q, int T_t, int T_a,
+                                                                 int n_tiles, const float *work, const float2 *tile_ml, float *p_tok,
+                                                                 long long p_stride, int first) {
+  const int n = T_t + T_a, n_row = n_q * cv.geo.g, f = blockIdx.y, lane = threadIdx.x & 31;
+  __shared__ float2 mz[TOK_QR];
+  for (int r = threadIdx.x >> 5; r < n_row; r += TOK_TILE / 32) {
+    const float2 *ml = tile_ml + ((long long)f * TOK_QR + r) * n_tiles;
+    float M = -INFINITY, Z = 0.f;
+    for (int x = lane; x < n_tiles; x += 32) M = fmaxf(M, ml[x].x);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    for (int x = lane; x < n_tiles; x += 32) Z += ml[x].y * exp2f(ml[x].x - M);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, o);
+    if (lane == 0) mz[r] = make_float2(M, Z);
+  }
+  __syncthreads();
+  const int tau = blockIdx.x * TOK_TILE + threadIdx.x;
+  if (tau >= T_a) return;
+  float p = first ? 0.f : p_tok[(long long)f * p_stride + tau];
+  for (int r = 0; r < n_row; ++r) p += __fdiv_rn(exp2f(work[((long long)f * TOK_QR + r) * n + T_t + tau] - mz[r].x), mz[r].y);
+  p_tok[(long long)f * p_stride + tau] = p;
 }
 
 // grid: fixed heads of the layer; block: TOK_THREADS.  flags: [n_fixed][p_stride] int32 scratch.
 __global__ void __launch_bounds__(TOK_THREADS) wnw_token_select_kernel(const __grid_constant__ CacheView cv, int b, int layer,
                                                                       const float *p_tok, long long p_stride, int T_a, int seg,
-                                                                      const float *retention, int variant, int32_t *flags,
+                                                                      const __grid_constant__ TokenRetention ret_h, int variant, int32_t *flags,
                                                                       int32_t *fixed_tok, int tok_cap, int32_t *tok_n) {
   const Geometry &G = cv.geo;
   __shared__ int counts[TOK_THREADS + 1];
@@ -121,7 +145,7 @@ __global__ void __launch_bounds__(TOK_THREADS) wnw_token_select_kernel(const __g
   const long long fh = (long long)b * G.F_tot + head;
   const float *key = p_tok + (long long)f * p_stride;
   int32_t *fl = flags + (long long)f * p_stride, *out = fixed_tok + fh * tok_cap;
-  const double ret = (double)retention[h];
+  const double ret = (double)ret_h.r[h];
   int total = 0;
   if (variant != 0)
     for (int lo = 0; lo < T_a; lo += seg) total += (int)floor(ret * (double)min(seg, T_a - lo));
@@ -157,6 +181,11 @@ __global__ void __launch_bounds__(TOK_THREADS) wnw_token_select_kernel(const __g
     cv.fixed_chunks[fh * G.FB + s] = s < n_blk ? -(2 + min(G.nc, n - s * G.nc)) : -1;
   if (threadIdx.x == 0) { cv.fixed_n[fh] = n_blk; tok_n[fh] = n; }
   const LayerInfo &li = cv.layers[layer];
+  if (f >= li.n_fixed && threadIdx.x == 0) {   // (the global variant keeps a different number per segment: the table below says)
+    const int tail_len = T_a - (T_a - 1) / G.nc * G.nc;
+    cv.tok_m[((long long)b * G.L + layer) * G.Hkv + h] =
+        variant != 0 ? make_int2(-1, -1) : make_int2((int)floor(ret * (double)G.nc), (int)floor(ret * (double)tail_len));
+  }
   if (f >= li.n_fixed) {   // a tidal head's base: how many positions of every segment it holds (what a fetched segment must skip)
     int32_t *sk = cv.seg_kept + ((long long)b * cv.tid_total + li.tid_prefix + (f - li.n_fixed)) * G.C_max;
     for (int c = threadIdx.x; c * G.nc < T_a; c += TOK_THREADS) {
@@ -231,13 +260,21 @@ __global__ void __launch_bounds__(128) wnw_token_mirror_kernel(const __grid_cons
 
 // n_comp: compressed heads of the layer (its fixed heads, then its tidal heads when they keep a token base)
 cudaError_t launch_token_compress(const CacheView &cv, int b, int layer, int n_comp, int n_tidal_base, const bf16 *stage,
-                                  const bf16 *q_text, int n_q, int T_t, int T_a, int seg, const float *retention_dev,
-                                  int variant, float *work, float *p_tok, int32_t *flags, long long p_stride,
+                                  const bf16 *q_text, int n_q, int T_t, int T_a, int seg, const TokenRetention &ret,
+                                  int variant, float *work, float2 *tile_ml, float *p_tok, int32_t *flags, long long p_stride,
                                   int32_t *fixed_tok, int tok_cap, int32_t *tok_n, bf16 *mirror_out, cudaStream_t st) {
   if (n_comp <= 0 || T_a <= 0) return cudaSuccess;
-  const size_t smem = (size_t)(cv.geo.d + TOK_THREADS / 32) * sizeof(float);
-  wnw_token_score_kernel<<<n_comp, TOK_THREADS, smem, st>>>(cv, b, layer, stage, q_text, n_q, T_t, T_a, work, p_tok, p_stride);
-  wnw_token_select_kernel<<<n_comp, TOK_THREADS, 0, st>>>(cv, b, layer, p_tok, p_stride, T_a, seg, retention_dev, variant, flags,
+  const Geometry &G = cv.geo;
+  const int n_tiles = (T_t + T_a + TOK_TILE - 1) / TOK_TILE, per = TOK_QR / G.g;   // whole queries per pass
+  for (int q0 = 0; q0 < n_q; q0 += per) {
+    const int nq = std::min(per, n_q - q0);
+    const size_t smem = (size_t)nq * G.g * (G.d + 2 * (TOK_TILE / 32)) * sizeof(float);
+    wnw_token_logits_kernel<<<dim3(n_tiles, n_comp), TOK_TILE, smem, st>>>(cv, b, layer, stage, q_text + (size_t)q0 * G.Hq * G.d, nq, T_t,
+                                                                          T_a, work, tile_ml);
+    wnw_token_mass_kernel<<<dim3((T_a + TOK_TILE - 1) / TOK_TILE, n_comp), TOK_TILE, 0, st>>>(cv, nq, T_t, T_a, n_tiles, work, tile_ml, p_tok,
+                                                                                            p_stride, q0 == 0);
+  }
+  wnw_token_select_kernel<<<n_comp, TOK_THREADS, 0, st>>>(cv, b, layer, p_tok, p_stride, T_a, seg, ret, variant, flags,
                                                          fixed_tok, tok_cap, tok_n);
   wnw_token_gather_kernel<<<dim3(cv.geo.FB, n_comp), 128, 0, st>>>(cv, b, layer, stage, fixed_tok, tok_cap, tok_n);
   if (n_tidal_base > 0) {
