@@ -131,11 +131,20 @@ def _ptr(t) -> Optional[int]:
     return int(t.data_ptr())
 
 
+_raw_stream = None    # torch's current stream of the current device as an integer, without building a Stream object
+
+
 def _stream(stream) -> Optional[int]:
-    if stream is None:
+    if stream is not None:
+        return int(stream.cuda_stream) or None
+    global _raw_stream
+    if _raw_stream is None:
         import torch
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream) or None
+        get_raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        torch.cuda.current_stream()    # initialises CUDA
+        _raw_stream = ((lambda: get_raw(torch._C._cuda_getDevice())) if get_raw else
+                       (lambda: int(torch.cuda.current_stream().cuda_stream)))
+    return _raw_stream() or None
 
 
 def wnw_create(n_layers, n_q_heads, n_kv_heads, head_dim, max_batch, max_audio_tokens, max_text_tokens, chunk_tokens,
