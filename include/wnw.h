@@ -148,7 +148,7 @@ typedef struct {
   int64_t steps;            /* decode steps completed (sum over sequences) */
   int64_t hits, misses;     /* selected chunks found resident / recalled */
   int64_t evictions;        /* residents displaced */
-  int64_t recall_bytes;     /* bytes copied host -> slot pool */
+  int64_t recall_bytes;     /* recalled chunk blocks, in bytes as stored (rows that only pad a chunk count, though they stay where they are) */
   int64_t resident_audio_tokens; /* audio tokens on the GPU now, all heads (r_GPU numerator, Audio KV retention paragraph) */
   int64_t host_audio_tokens;     /* audio tokens of tidal heads held in host memory and not on the GPU */
   int64_t full_audio_tokens;     /* L * H_kv * T_a summed over placed sequences (denominator) */

@@ -323,7 +323,7 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // a few CTAs of 8 warps with RECALL_U 16-byte loads in flight per lane, whatever there is to copy, and the warps work
 // independently: the blocks of a launch are cut into pieces of a warp's batch and dealt round robin ACROSS block and layer
 // borders, so that all warps have work and nothing waits at a barrier.
-// 40 registers a thread: a CTA fits beside a resident 8-warp attention CTA.
+// At most 48 registers a thread: a CTA fits beside a resident 8-warp attention CTA (208 registers).
 // 8 CTAs where layers wait for one another: the copies have the whole next step's time (config 1, 30 chained layers, recall
 // and the step's own small copies: 254 us a step with the former 128 CTAs, 238.7 with 8, 241 with 12, 243 with 16).  24 CTAs
 // where layers overlap: attention then fills the memory system, a host read takes several times as long and the step waits for
@@ -333,7 +333,7 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // warp that finishes a layer last publishes the layer's recall epoch, which the next step's tidal CTAs acquire.
 // ------------------------------------------------------------------------------------------------
 constexpr int RECALL_CTAS = 8, RECALL_CTAS_CROWDED = 24, RECALL_WARPS = 8, RECALL_U = 4;
-__global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
+__global__ void __launch_bounds__(RECALL_WARPS * 32, 5) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
                                                                           const int32_t *active, const int32_t *layers,
                                                                           int n_layers, int skip_copy, RecallSignal sig) {
   const Geometry &G = cv.geo;
@@ -352,14 +352,16 @@ __global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const 
     for (unsigned left = __ballot_sync(0xffffffffu, todo); left; left &= left - 1) {
       const int l = __shfl_sync(0xffffffffu, my_l, __ffs(left) - 1);
       const int n_tidal = cv.layers[l].n_tidal;
-      const int n = n_tidal * 2 * G.ncp * G.d * tidal_elem_bytes(G) / 16;   // 16-byte vectors per chunk block (far below 2^31)
+      // 16-byte vectors of a chunk block (far below 2^31): its n_tidal x (K, V) runs of nc rows, without the rows that pad a run
+      // to whole granules (25-token segments: 22 % of the block)
+      const int run = G.nc * G.d * tidal_elem_bytes(G) / 16, run_pad = G.ncp * G.d * tidal_elem_bytes(G) / 16 - run, n = n_tidal * 2 * run;
       const int n_piece = (n + 32 * RECALL_U - 1) / (32 * RECALL_U);
       for (int i0 = 0; i0 < n_active; i0 += 32) {
         const int my_b = i0 + lane < n_active ? active[i0 + lane] : -1;
         const int my_n = my_b >= 0 ? min(cv.n_plan[(long long)my_b * G.L + l], G.plan_cap) : 0;
         for (unsigned seqs = __ballot_sync(0xffffffffu, my_n > 0); seqs; seqs &= seqs - 1) {
           const int b = __shfl_sync(0xffffffffu, my_b, __ffs(seqs) - 1), n_plan = __shfl_sync(0xffffffffu, my_n, __ffs(seqs) - 1);
-          if (w == 0 && lane == 0) atomicAdd(cv.stats + (long long)b * 4 + 3, (unsigned long long)n_plan * n * 16ull);
+          if (w == 0 && lane == 0) atomicAdd(cv.stats + (long long)b * 4 + 3, (unsigned long long)n_plan * (n + n_tidal * 2 * run_pad) * 16ull);   // blocks as stored
           if (skip_copy) continue;
           // all plan entries of the sequence in one round trip (at most 2 * MAX_TOPK of them)
           const int *plan = cv.plan + ((long long)b * G.L + l) * G.plan_cap * 2;
@@ -381,12 +383,16 @@ __global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const 
             for (; p < n_piece; p += n_warps) {
               const int v0 = p * 32 * RECALL_U + lane;
               uint4 t[RECALL_U];
+              int at[RECALL_U];
+#pragma unroll
+              for (int u = 0; u < RECALL_U; ++u) {
+                at[u] = v0 + u * 32;
+                if (run_pad) at[u] += at[u] / run * run_pad;
+                if (v0 + u * 32 < n) t[u] = __ldcs(src + at[u]);
+              }
 #pragma unroll
               for (int u = 0; u < RECALL_U; ++u)
-                if (v0 + u * 32 < n) t[u] = __ldcs(src + v0 + u * 32);
-#pragma unroll
-              for (int u = 0; u < RECALL_U; ++u)
-                if (v0 + u * 32 < n) dst[v0 + u * 32] = t[u];
+                if (v0 + u * 32 < n) dst[at[u]] = t[u];
             }
           }
         }

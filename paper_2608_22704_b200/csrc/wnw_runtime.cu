@@ -1028,8 +1028,11 @@ static wnw_status_t send_mirror(wnw_cache_t *c, int seq, int layer, cudaStream_t
   const size_t eb = tidal_elem_bytes(G);
   CK(cudaEventRecord(c->ev_mst_ready[r], st));
   CK(cudaStreamWaitEvent(c->copy_stream, c->ev_mst_ready[r], 0));
-  CK(cudaMemcpyAsync(reinterpret_cast<char *>(s.mirror) + mirror_off(G, li, mirror_chunks_of(G, s.C), 0, 0, 0) * eb, c->mst[r],
-                     (size_t)s.C * li.n_tidal * 2 * G.ncp * G.d * eb, cudaMemcpyDeviceToHost, c->copy_stream));
+  char *dst = reinterpret_cast<char *>(s.mirror) + mirror_off(G, li, mirror_chunks_of(G, s.C), 0, 0, 0) * eb;
+  const size_t runs = (size_t)s.C * li.n_tidal * 2, pitch = (size_t)G.ncp * G.d * eb, width = (size_t)G.nc * G.d * eb;
+  // the rows that pad a chunk's run to whole granules stay here
+  if (width == pitch) CK(cudaMemcpyAsync(dst, c->mst[r], runs * pitch, cudaMemcpyDeviceToHost, c->copy_stream));
+  else CK(cudaMemcpy2DAsync(dst, pitch, c->mst[r], pitch, width, runs, cudaMemcpyDeviceToHost, c->copy_stream));
   CK(cudaEventRecord(c->ev_mst_free[r], c->copy_stream));
   CK(cudaEventRecord(c->ev_mirror, c->copy_stream));
   c->mst_used[r] = true;
