@@ -84,6 +84,12 @@ struct wnw_cache {
   size_t d_sched_cap = 0, sched_ranges_base = 0;
   std::vector<WorkItem> h_items;  // host copy (short lists are inlined into kernel parameters)
   size_t d_items_cap = 0;
+  // the lists on their way to the device: pinned, one copy queued by the first call that has a stream
+  std::vector<int32_t> h_order, h_ranges;
+  bool wl_dirty = false, upload_recorded = false;
+  char *h_upload = nullptr;
+  size_t h_upload_cap = 0;
+  cudaEvent_t ev_upload = nullptr;
   // partial buffers
   float *part_o = nullptr;
   float2 *part_ml = nullptr, *gran_em = nullptr, *head_mz = nullptr;
@@ -147,9 +153,11 @@ struct wnw_cache {
   std::vector<int> graph_active, graph_prepared;
   long long wl_epoch = 0, graph_epoch = -1;  // work-list generation the graph was captured against
   int graph_appended = 0;
+  bool graph_fresh = false;   // not replayed since its capture
+  bool graph_launched = false;   // ev_graph_done follows a replay
   int last_side_layer[N_SIDE] = {-1, -1, -1, -1, -1, -1, -1, -1};
 
-  cudaEvent_t ev_place = nullptr, ev_step = nullptr;
+  cudaEvent_t ev_place = nullptr, ev_step = nullptr, last_step = nullptr;   // last_step: ev_step or, after a replay, ev_graph_done
   bool place_recorded = false, step_recorded = false;
   // token-granular compression of fixed heads (allocated by the first wnw_place_prefill_tokens)
   float *tok_work = nullptr, *tok_p = nullptr;
@@ -253,6 +261,8 @@ static void destroy_impl(wnw_cache *c) {
     if (c->ev_mst_free[r]) cudaEventDestroy(c->ev_mst_free[r]);
   }
   if (c->ev_mirror) cudaEventDestroy(c->ev_mirror);
+  if (c->ev_upload) cudaEventDestroy(c->ev_upload);
+  if (c->h_upload) cudaFreeHost(c->h_upload);
   for (auto e : c->ev_layer_done) cudaEventDestroy(e);
   for (auto e : c->ev_side_done) cudaEventDestroy(e);
   for (auto e : c->ev_layer_done_cap) cudaEventDestroy(e);
@@ -537,6 +547,7 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
     }
   }
   CKE(cudaEventCreateWithFlags(&c->ev_place, cudaEventDisableTiming));
+  CKE(cudaEventCreateWithFlags(&c->ev_upload, cudaEventDisableTiming));
   CKE(cudaEventCreateWithFlags(&c->ev_step, cudaEventDisableTiming));
   CKE(cudaEventCreateWithFlags(&c->ev_graph_done, cudaEventDisableTiming));
   CKE(cudaEventCreateWithFlags(&c->ev_recall_all, cudaEventDisableTiming));
@@ -958,8 +969,6 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
     c->wl_layers[l].part_off = part_total;
     part_total += (size_t)c->wl_layers[l].n_items;
   }
-  // the previous lists may still be read by queued kernels
-  CK(cudaDeviceSynchronize());
   if (part_total > c->part_cap_total) {  // one partial region per layer
     float *po = nullptr; float2 *pm = nullptr;
     CK(cudaMalloc((void **)&po, part_total * G.g * G.d * sizeof(float)));
@@ -968,28 +977,53 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
     c->dev_allocs.push_back(pm);
     c->part_o = po; c->part_ml = pm; c->part_cap_total = part_total;
   }
-  if (items.size() > c->d_items_cap) {
-    CK(cudaMalloc((void **)&c->d_items, items.size() * sizeof(WorkItem)));
-    c->dev_allocs.push_back(c->d_items);
-    c->d_items_cap = items.size();
-  }
-  if (order.size() + ranges.size() > c->d_sched_cap) {
-    CK(cudaMalloc((void **)&c->d_sched, (order.size() + ranges.size()) * sizeof(int32_t)));
-    c->dev_allocs.push_back(c->d_sched);
-    c->d_sched_cap = order.size() + ranges.size();
-  }
-  if (!order.empty()) {
-    CK(cudaMemcpy(c->d_sched, order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(c->d_sched + order.size(), ranges.data(), ranges.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-  }
-  c->sched_ranges_base = order.size();
-  CK(cudaMemcpy(c->d_items, items.data(), items.size() * sizeof(WorkItem), cudaMemcpyHostToDevice));
-  std::vector<int32_t> act(c->active.begin(), c->active.end());
-  CK(cudaMemcpy(c->d_active, act.data(), act.size() * sizeof(int32_t), cudaMemcpyHostToDevice));
-  c->h_items = items;
+  c->h_items.swap(items); c->h_order.swap(order); c->h_ranges.swap(ranges);
+  c->wl_dirty = true;
   ++c->wl_epoch;
   c->wl_active = c->active;
   c->wl_T_a = T_a;
+  return WNW_OK;
+}
+
+// Queues the copy of freshly built lists on `st`, behind everything that may still read the lists they replace.  The host
+// waits for nothing (but the previous such copy): a placement's kernels and transfers go on while the step that follows it is
+// built and captured.
+static wnw_status_t upload_worklists(wnw_cache *c, cudaStream_t st) {
+  if (!c->wl_dirty) return WNW_OK;
+  const size_t n_items = c->h_items.size(), n_sched = c->h_order.size() + c->h_ranges.size(), n_act = c->active.size();
+  if (n_items > c->d_items_cap) {
+    CK(cudaMalloc((void **)&c->d_items, n_items * sizeof(WorkItem)));
+    c->dev_allocs.push_back(c->d_items);
+    c->d_items_cap = n_items;
+  }
+  if (n_sched > c->d_sched_cap) {
+    CK(cudaMalloc((void **)&c->d_sched, n_sched * sizeof(int32_t)));
+    c->dev_allocs.push_back(c->d_sched);
+    c->d_sched_cap = n_sched;
+  }
+  const size_t at_sched = n_items * sizeof(WorkItem), at_act = at_sched + n_sched * sizeof(int32_t), total = at_act + n_act * sizeof(int32_t);
+  if (c->upload_recorded) CK(cudaEventSynchronize(c->ev_upload));
+  if (total > c->h_upload_cap) {
+    if (c->h_upload) cudaFreeHost(c->h_upload);
+    c->h_upload = nullptr; c->h_upload_cap = 0;
+    if (cudaHostAlloc((void **)&c->h_upload, 2 * total, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_OOM_HOST; }
+    c->h_upload_cap = 2 * total;
+  }
+  memcpy(c->h_upload, c->h_items.data(), at_sched);
+  if (!c->h_order.empty()) memcpy(c->h_upload + at_sched, c->h_order.data(), c->h_order.size() * sizeof(int32_t));
+  if (!c->h_ranges.empty()) memcpy(c->h_upload + at_sched + c->h_order.size() * sizeof(int32_t), c->h_ranges.data(), c->h_ranges.size() * sizeof(int32_t));
+  memcpy(c->h_upload + at_act, c->active.data(), n_act * sizeof(int32_t));
+  if (c->step_recorded) CK(cudaStreamWaitEvent(st, c->last_step, 0));
+  for (int l = 0; l < c->geo.L; ++l)
+    if (c->side_recorded[l]) CK(cudaStreamWaitEvent(st, c->ev_side_done[l], 0));
+  if (c->recall_all_pending) CK(cudaStreamWaitEvent(st, c->ev_recall_all, 0));
+  CK(cudaMemcpyAsync(c->d_items, c->h_upload, at_sched, cudaMemcpyHostToDevice, st));
+  if (n_sched) CK(cudaMemcpyAsync(c->d_sched, c->h_upload + at_sched, n_sched * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+  CK(cudaMemcpyAsync(c->d_active, c->h_upload + at_act, n_act * sizeof(int32_t), cudaMemcpyHostToDevice, st));
+  CK(cudaEventRecord(c->ev_upload, st));
+  c->upload_recorded = true;
+  c->sched_ranges_base = c->h_order.size();
+  c->wl_dirty = false;
   return WNW_OK;
 }
 
@@ -1099,7 +1133,7 @@ static wnw_status_t place_multi(wnw_cache_t *c, int32_t seq, int32_t layer, cons
   }
   // the staging buffer and the partial buffers are shared: order after earlier placements and steps
   if (c->place_recorded) CK(cudaStreamWaitEvent(st, c->ev_place, 0));
-  if (c->step_recorded) CK(cudaStreamWaitEvent(st, c->ev_step, 0));
+  if (c->step_recorded) CK(cudaStreamWaitEvent(st, c->last_step, 0));
   if (c->recall_all_pending) CK(cudaStreamWaitEvent(st, c->ev_recall_all, 0));
   CK(launch_place_scatter(c->cv, seq, layer, full ? 1 : 0, (const bf16 *)k_dev, (const bf16 *)v_dev, audio_begin, audio_end, T_t,
                           C_b, S_b, S_base_b, c->stage, st));
@@ -1307,26 +1341,27 @@ extern "C" wnw_status_t wnw_get_fixed_tokens(wnw_cache_t *c, int32_t seq, int32_
   return WNW_OK;
 }
 
-// One selection launch for the map entries [range[0], range[0] + range[1]); small stacks carry the layers' arguments in
-// the kernel parameters.
-static cudaError_t select_all(wnw_cache *c, const int *range, const SelectArgs &stp, cudaStream_t st) {
-  if (c->geo.L <= SELECT_TABLE_LAYERS && range[1] <= SELECT_TABLE_ENTRIES && !c->h_sel_args.empty())
+// One selection launch for the map entries [range[0], range[0] + range[1]).  A captured step of a small stack carries the layers'
+// arguments in the kernel parameters (nothing is loaded before a CTA knows its work); a launch that the host makes anew on
+// every step reads them from memory instead: copying some 20 KB of parameters costs the host more than the GPU gains.
+static cudaError_t select_all(wnw_cache *c, const int *range, const SelectArgs &stp, bool capturing, cudaStream_t st) {
+  if (capturing && c->geo.L <= SELECT_TABLE_LAYERS && range[1] <= SELECT_TABLE_ENTRIES && !c->h_sel_args.empty())
     return launch_select_all_params(c->cv, c->h_sel_args.data(), c->geo.L, c->h_sel_map.data() + range[0], range[1], stp,
                                     c->sel_all_smem, st);
   return launch_select_all(c->cv, c->d_sel_args, c->d_sel_map + range[0], range[1], stp, c->sel_all_smem, st);
 }
 
-// The selection work of a captured step in one launch (two when a layer ranks by another layer's scores).  overlapped:
+// The selection work of a step in one launch (two when a layer ranks by another layer's scores).  overlapped:
 // it runs beside the step's tidal attention and leaves the step's bookkeeping to a step-end kernel.
-static wnw_status_t launch_step_selection(wnw_cache *c, bool overlapped, cudaStream_t st) {
+static wnw_status_t launch_step_selection(wnw_cache *c, bool overlapped, bool capturing, cudaStream_t st) {
   SelectArgs stp{};
   stp.n_active = (int)c->active.size(); stp.active = c->d_active;
   stp.epoch_words = c->d_recall_epoch; stp.empty_ctr = c->d_empty_ctr; stp.step_epoch = c->d_step_epoch;
   stp.overlapped = overlapped ? 1 : 0;
   if (!c->select_single_ok) {   // first every anchor layer's scores, then every table update
     stp.do_score = 1; stp.do_update = 0;
-    CK(select_all(c, c->sel_map_score, stp, st));
-    if (c->sel_map_score[1] > 0) c->count_launch(1, 1, true);
+    CK(select_all(c, c->sel_map_score, stp, capturing, st));
+    if (c->sel_map_score[1] > 0) c->count_launch(1, 1, capturing);
   }
   const int *range = c->select_single_ok ? c->sel_map_single : c->sel_map_update;
   stp.do_score = c->select_single_ok ? 1 : 0; stp.do_update = 1;
@@ -1334,8 +1369,8 @@ static wnw_status_t launch_step_selection(wnw_cache *c, bool overlapped, cudaStr
     stp.fold_total = range[1] * stp.n_active; stp.fold_appended = c->appended == 1;
     stp.fold_counter = c->d_fold_ctr; stp.fold_bump_epoch = c->d_step_epoch;
   }
-  CK(select_all(c, range, stp, st));
-  c->count_launch(1, 1, true);
+  CK(select_all(c, range, stp, capturing, st));
+  c->count_launch(1, 1, capturing);
   return WNW_OK;
 }
 
@@ -1390,27 +1425,25 @@ static SelectArgs static_select_args(const wnw_cache *c, int layer) {
   return sa;
 }
 
-// Decided once per step, at its first layer: how a captured step issues its selection, recall and attention launches.
+// Decided once per step, at its first layer: how the step issues its selection, recall and attention launches.
 static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   const Geometry &G = c->geo;
-  // Replayed steps of small launches take their recall out of the captured graph, so that it can overlap the next
-  // replay.  Where a launch could fill the machine, its attention CTAs would sit on their SMs while they wait for
-  // it, so recall stays inside the step there.
+  // Steps of small launches take their recall out of the step, so that it can overlap the next one.  Where a launch could
+  // fill the machine, its attention CTAs would sit on their SMs while they wait for it, so recall stays inside the step
+  // there.  (A caller's own capture of an eager step keeps everything inside, too: nothing could be issued behind it.)
   bool small = true;   // no launch can fill the machine with CTAs that wait
   for (const LayerWork &w : c->wl_layers) small = small && !w.throughput && (w.n_ctas > 0 ? w.n_ctas : w.n_items) <= c->n_sm / 2;
+  const bool ours = tiered && c->cfg.recall_mode != WNW_RECALL_INLINE && !c->cfg.defer_selection && (!capturing || c->graph_capturing);
+  const int n_select = c->select_single_ok ? c->sel_map_single[1] : c->sel_map_update[1];
+  // With the recall outside, nothing inside the step needs a layer's selection before the step ends: all of it goes into one
+  // launch (or two) behind the last attention kernel, and its last CTA closes the step.  An eager step without any selection
+  // has nothing to gain from it.
+  c->cap_external_recall = ours && small && (capturing || n_select > 0);
+  c->cap_select_all = c->cap_external_recall && n_select > 0;
   // the selection kernel of the last layer starts after every attention kernel of the step has completed, so the
   // selection CTA that finishes last in the step may update what those kernels read
   const LayerInfo &last = c->layers[G.L - 1];
-  c->cap_fold = capturing && c->graph_capturing && tiered && c->cfg.recall_mode != WNW_RECALL_INLINE &&
-                (last.n_anchor > 0 || last.upd_count > 0);
-  c->cap_select_all = false;
-  c->cap_external_recall = capturing && c->graph_capturing && tiered && c->cfg.recall_mode != WNW_RECALL_INLINE &&
-                           small;
-  // With the recall outside the graph nothing inside it needs a layer's selection before the step ends: all of it
-  // goes into one launch (or two) behind the last attention kernel.
-  c->cap_select_all = c->cap_external_recall && small &&
-                      (c->select_single_ok ? c->sel_map_single[1] : c->sel_map_update[1]) > 0;
-  if (c->cap_select_all) c->cap_fold = true;
+  c->cap_fold = c->cap_select_all || (capturing && ours && (last.n_anchor > 0 || last.upd_count > 0));
   // BATCHED layers: one launch for the whole step where nothing inside the step needs a layer's result earlier
   bool one_shot = G.L <= MULTI_LAYERS_MAX;
   for (const LayerWork &w : c->wl_layers) one_shot = one_shot && !w.throughput;
@@ -1435,10 +1468,24 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
 // An eager layer waits for what earlier work on other streams has to have finished: placements, the recall launch that
 // followed the last replayed step, and the previous step's side-stream work on this layer's partials, table and slots.
 static wnw_status_t wait_for_earlier_steps(wnw_cache *c, int layer, bool tiered, cudaStream_t st) {
-  if (layer == 0 && c->place_recorded) CK(cudaStreamWaitEvent(st, c->ev_place, 0));
-  if (layer == 0 && c->recall_all_pending) {  // the recall launch that followed the last replayed step
-    CK(cudaStreamWaitEvent(st, c->ev_recall_all, 0));
-    c->recall_all_pending = false;
+  if (layer == 0) {
+    if (c->place_recorded) CK(cudaStreamWaitEvent(st, c->ev_place, 0));
+    if (c->last_stream != st && c->step_recorded) CK(cudaStreamWaitEvent(st, c->last_step, 0));
+    // the recall launch that followed the last step: as a whole, unless this step's tidal CTAs wait for it layer by layer
+    if (c->recall_all_pending && !c->cap_external_recall) {
+      CK(cudaStreamWaitEvent(st, c->ev_recall_all, 0));
+      c->recall_all_pending = false;
+    }
+    if (c->cap_external_recall) {
+      // beside the mirror copies of a placement runs one such step (see wnw_graph_launch)
+      if (c->mirror_pending && c->mirror_step_issued) {
+        wnw_status_t ms = wait_for_mirror(c, st);
+        if (ms != WNW_OK) return ms;
+      }
+      c->mirror_step_issued = true;
+    }
+    wnw_status_t us = upload_worklists(c, st);
+    if (us != WNW_OK) return us;
   }
   // side-stream work of the previous step that this layer depends on must have landed: the selection kernel that
   // read this layer's partial buffers, and the recall that refreshed this layer's slots
@@ -1486,7 +1533,7 @@ static wnw_status_t issue_batched_step(wnw_cache *c, bool tiered, bool capturing
       c->appended = has_new;
       CK(cudaEventRecord(c->ev_sel_fork, st));
       CK(cudaStreamWaitEvent(c->side[0], c->ev_sel_fork, 0));
-      wnw_status_t rs = launch_step_selection(c, true, c->side[0]);
+      wnw_status_t rs = launch_step_selection(c, true, capturing, c->side[0]);
       if (rs != WNW_OK) return rs;
       CK(cudaEventRecord(c->ev_sel_join, c->side[0]));
     }
@@ -1583,7 +1630,10 @@ static wnw_status_t decode_layer_impl(wnw_cache *c, int want_mode, int32_t layer
   const bool capturing = stream_is_capturing(st);
   if (layer == 0) c->step_capturing = capturing;
   else if (capturing != c->step_capturing) return WNW_ERR_STATE;
-  if (layer == 0) plan_step(c, capturing, tiered);
+  if (layer == 0) {
+    if (capturing && c->wl_dirty) return WNW_ERR_STATE;   // a caller's own capture: the lists of the set must be in place
+    plan_step(c, capturing, tiered);
+  }
   if (!capturing) {
     wnw_status_t ws = wait_for_earlier_steps(c, layer, tiered, st);
     if (ws != WNW_OK) return ws;
@@ -1714,6 +1764,22 @@ extern "C" wnw_status_t wnw_import_prefill_tidal(wnw_cache_t *c, int32_t seq, in
   return WNW_OK;
 }
 
+// The recall of the step that ended with c->last_step, for every layer's table at once, outside the step: it overlaps the next
+// step, whose tidal CTAs wait on the per-layer epoch words it publishes.
+static wnw_status_t launch_step_recall(wnw_cache *c, int n_active) {
+  if (c->upd_list.empty()) return WNW_OK;
+  ++c->host_epoch;
+  CK(cudaStreamWaitEvent(c->side[0], c->last_step, 0));
+  wnw_status_t ms = wait_for_mirror(c, c->side[0]);
+  if (ms != WNW_OK) return ms;
+  CK(launch_recall(c->cv, n_active, c->d_active, c->cv.upd_list, (int)c->upd_list.size(), c->cfg.recall_mode == WNW_RECALL_SKIP,
+                   layers_overlap(c), RecallSignal{c->d_recall_epoch, c->d_recall_ctr, c->d_empty_ctr, c->host_epoch}, c->side[0]));
+  c->count_launch(2, 1, false);
+  CK(cudaEventRecord(c->ev_recall_all, c->side[0]));
+  c->recall_all_pending = true;
+  return WNW_OK;
+}
+
 extern "C" wnw_status_t wnw_step_end(wnw_cache_t *c, void *cuda_stream) {
   if (!c) return WNW_ERR_INVALID_ARG;
   if (!c->in_step || c->next_layer != c->geo.L) return WNW_ERR_STATE;
@@ -1725,11 +1791,11 @@ extern "C" wnw_status_t wnw_step_end(wnw_cache_t *c, void *cuda_stream) {
     for (int ls : c->last_side_layer)  // join the forked side streams into the graph
       if (ls >= 0) CK(cudaStreamWaitEvent(st, c->ev_side_done_cap[ls], 0));
 
-  if (capturing && c->cap_select_all) {
+  if (c->cap_select_all) {
     if (c->cap_sel_overlap) {   // forked behind the first part of the attention launch: join it
       CK(cudaStreamWaitEvent(st, c->ev_sel_join, 0));
     } else {
-      wnw_status_t rs = launch_step_selection(c, false, st);
+      wnw_status_t rs = launch_step_selection(c, false, capturing, st);
       if (rs != WNW_OK) return rs;
     }
   }
@@ -1741,7 +1807,7 @@ extern "C" wnw_status_t wnw_step_end(wnw_cache_t *c, void *cuda_stream) {
     if (c->sel_map_update[1] > 0) {
       SelectArgs stp{};
       stp.n_active = (int)c->active.size(); stp.active = c->d_active; stp.do_score = 0; stp.do_update = 1;
-      CK(select_all(c, c->sel_map_update, stp, st));
+      CK(select_all(c, c->sel_map_update, stp, false, st));
       c->count_launch(1, 1, false);
       wnw_status_t ms = wait_for_mirror(c, st);
       if (ms != WNW_OK) return ms;
@@ -1750,16 +1816,18 @@ extern "C" wnw_status_t wnw_step_end(wnw_cache_t *c, void *cuda_stream) {
       c->count_launch(2, 1, false);
     }
   }
-  if (!(capturing && c->cap_fold)) {
-    CK(launch_step_end(c->cv, (int)c->active.size(), c->d_active, c->appended == 1,
-                       (capturing && c->cap_external_recall) ? c->d_step_epoch : nullptr, st));
+  if (!c->cap_fold) {
+    CK(launch_step_end(c->cv, (int)c->active.size(), c->d_active, c->appended == 1, c->cap_external_recall ? c->d_step_epoch : nullptr, st));
     c->count_launch(3, 1, capturing);
   }
   if (!capturing) {
     CK(cudaEventRecord(c->ev_step, st));
-    c->step_recorded = true;
-  }
-  if (!capturing) {
+    c->last_step = c->ev_step; c->step_recorded = true;
+    if (c->cap_external_recall) {
+      wnw_status_t rs = launch_step_recall(c, (int)c->active.size());
+      if (rs != WNW_OK) return rs;
+    }
+    c->cap_external_recall = false;
     for (int b : c->active)
       if (c->appended == 1) c->seqs[b].T_t += 1;
   } else if (c->graph_capturing) {
@@ -1784,17 +1852,15 @@ extern "C" wnw_status_t wnw_graph_begin(wnw_cache_t *c, const int32_t *active, i
   }
   DeviceGuard guard(c->cfg.device);
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  // work lists are built and uploaded now: nothing may allocate or synchronise once the capture has begun
+  // work lists are built and their upload is queued now: nothing may allocate or be ordered against earlier work once the
+  // capture has begun (the first replay waits for what earlier work is still under way: wnw_graph_launch)
   c->active.assign(active, active + n_active);
   {
     wnw_status_t ws = ensure_worklists(c);
+    if (ws == WNW_OK) ws = upload_worklists(c, st);
     if (ws != WNW_OK) return ws;
   }
   c->graph_prepared = c->active;
-  // everything queued so far must be ordered before the first replay: drain now, the capture cannot wait on it
-  for (auto sd : c->side) CK(cudaStreamSynchronize(sd));
-  if (c->last_stream != st) CK(cudaStreamSynchronize(c->last_stream));
-  CK(cudaStreamSynchronize(st));
   for (long long &x : c->cap_launches) x = 0;
   CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
   c->graph_capturing = true;
@@ -1814,10 +1880,21 @@ extern "C" wnw_status_t wnw_graph_end(wnw_cache_t *c, void *cuda_stream) {
   c->in_step = false;
   if (e != cudaSuccess || !g) { c->last_cuda = e; cudaGetLastError(); return WNW_ERR_CUDA; }
   if (!complete) { cudaGraphDestroy(g); return WNW_ERR_STATE; }  // the capture must hold exactly one whole step
-  if (c->graph_exec) { cudaGraphExecDestroy(c->graph_exec); c->graph_exec = nullptr; }
+  // A new capture of the same shape (the next request of a serving loop, as a rule) updates the executable graph, which leaves
+  // replays under way alone; otherwise the old one goes once its last replay has run.
+  if (c->graph_exec) {
+    cudaGraphExecUpdateResultInfo info;
+    if (cudaGraphExecUpdate(c->graph_exec, g, &info) != cudaSuccess) {
+      cudaGetLastError();
+      if (c->graph_launched) CK(cudaEventSynchronize(c->ev_graph_done));
+      cudaGraphExecDestroy(c->graph_exec);
+      c->graph_exec = nullptr;
+    }
+  }
   if (c->graph) { cudaGraphDestroy(c->graph); c->graph = nullptr; }
   c->graph = g;
-  CK(cudaGraphInstantiate(&c->graph_exec, g, 0));
+  if (!c->graph_exec) CK(cudaGraphInstantiate(&c->graph_exec, g, 0));
+  c->graph_fresh = true;
   c->graph_epoch = c->wl_epoch;
   c->graph_external_recall = c->cap_external_recall;
   c->cap_external_recall = false;
@@ -1836,6 +1913,16 @@ extern "C" wnw_status_t wnw_graph_launch(wnw_cache_t *c, void *cuda_stream) {
   DeviceGuard guard(c->cfg.device);
   cudaStream_t st = (cudaStream_t)cuda_stream;
   if (c->place_recorded) CK(cudaStreamWaitEvent(st, c->ev_place, 0));
+  if (c->graph_fresh || c->last_stream != st) {   // what the lists were uploaded behind, an earlier step on another stream
+    if (c->upload_recorded) CK(cudaStreamWaitEvent(st, c->ev_upload, 0));
+    if (c->step_recorded) CK(cudaStreamWaitEvent(st, c->last_step, 0));
+  }
+  // the recall behind an earlier replay: replays of one graph wait for it inside, layer by layer
+  if (c->recall_all_pending && (c->graph_fresh || !c->graph_external_recall)) {
+    CK(cudaStreamWaitEvent(st, c->ev_recall_all, 0));
+    c->recall_all_pending = false;
+  }
+  c->graph_fresh = false;
   // side-stream work of earlier eager steps touches the tables and slots the graph reads
   for (int l = 0; l < c->geo.L; ++l)
     if (c->side_recorded[l]) { CK(cudaStreamWaitEvent(st, c->ev_side_done[l], 0)); c->side_recorded[l] = 0; }
@@ -1848,23 +1935,13 @@ extern "C" wnw_status_t wnw_graph_launch(wnw_cache_t *c, void *cuda_stream) {
   c->mirror_step_issued = true;
   CK(cudaGraphLaunch(c->graph_exec, st));
   for (int k = 0; k < 4; ++k) c->launches[k] += c->cap_launches[k];  // the kernels of the captured step
-  if (c->graph_external_recall && !c->upd_list.empty()) {
-    ++c->host_epoch;
-    // This step's recall, for every layer's table at once, outside the graph: it overlaps the next replay, whose tidal
-    // CTAs wait on the per-layer epoch words it publishes.
-    CK(cudaEventRecord(c->ev_graph_done, st));
-    CK(cudaStreamWaitEvent(c->side[0], c->ev_graph_done, 0));
-    wnw_status_t ms = wait_for_mirror(c, c->side[0]);
-    if (ms != WNW_OK) return ms;
-    CK(launch_recall(c->cv, (int)c->graph_active.size(), c->d_active, c->cv.upd_list, (int)c->upd_list.size(),
-                     c->cfg.recall_mode == WNW_RECALL_SKIP, layers_overlap(c), RecallSignal{c->d_recall_epoch, c->d_recall_ctr, c->d_empty_ctr, c->host_epoch},
-                     c->side[0]));
-    c->count_launch(2, 1, false);
-    CK(cudaEventRecord(c->ev_recall_all, c->side[0]));
-    c->recall_all_pending = true;
+  CK(cudaEventRecord(c->ev_graph_done, st));
+  c->graph_launched = true;
+  c->last_step = c->ev_graph_done; c->step_recorded = true;
+  if (c->graph_external_recall) {
+    wnw_status_t rs = launch_step_recall(c, (int)c->graph_active.size());
+    if (rs != WNW_OK) return rs;
   }
-  CK(cudaEventRecord(c->ev_step, st));
-  c->step_recorded = true;
   for (int b : c->graph_active)
     if (c->graph_appended) c->seqs[b].T_t += 1;
   c->last_stream = st;
