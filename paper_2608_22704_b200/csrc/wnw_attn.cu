@@ -118,6 +118,16 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     if (clock64() - t0 > 2000000000ll) return false;
   return true;
 }
+// The same for bytes that other CTAs of the cluster send, eight times as long (their own waits may have run out before).
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
+  for (const long long t0 = clock64();;) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (ok) return true;
+    if (clock64() - t0 > 16000000000ll) return false;
+  }
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t bar) {
   asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n"
                ::"r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
@@ -139,6 +149,13 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t *>(&v);
+}
+
+// 2^x in one instruction (results below the normal range come out as 0; exp2f spends three more on them)
+__device__ __forceinline__ float ex2(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
+  return r;
 }
 
 // Two e4m3 bytes (low 16 bits of x) as two fp16 numbers: one instruction, exact (every e4m3 value is an fp16 value).
@@ -228,7 +245,8 @@ __device__ __forceinline__ GranDesc decode_granule(const CacheView &cv, const At
 //   The default path (VAR 0) carries none of any variant's branches.
 // bid: the CTA's index within its layer's launch (a launch may carry the CTAs of several layers back to back);
 // inl: the layer's work items when they travel in the kernel parameters, else null (read from a.items).
-template <int D, bool G16, int NW, int VAR>
+// CL: one-shot CTAs in thread-block clusters, all pieces of a head inside one cluster (see the exchange at the end of the body).
+template <int D, bool G16, int NW, int VAR, bool CL = false>
 __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a, const InlineItems *inl, const TmaMaps &maps,
                                           const int bid) {
   extern __shared__ unsigned char smem_raw[];
@@ -266,6 +284,10 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   __shared__ int2 ring[NW][NSTAGE];                              // per stage: visible rows | loaded << 8, score index
   __shared__ __align__(8) unsigned long long bars[NW][NSTAGE];   // one mbarrier per stage, producer = consumer = this warp
   __shared__ int s_flag;
+  __shared__ __align__(16) float2 cl_ml[CL ? NW * 16 : 1];   // (max, denominator) of every warp and head
+  __shared__ __align__(8) unsigned long long cl_bar;         // bytes of the head's pieces arriving at this one
+  constexpr int QROW = D * 2 + 16;                            // a query row, padded: ldmatrix reads eight of them without conflicts
+  __shared__ __align__(16) unsigned char cl_q[CL ? (G16 ? 16 : 8) * QROW : 16];
   if (VAR == 3) asm volatile("griddepcontrol.wait;\n" ::: "memory");   // the caller's buffer may be what the preceding work wrote
   const uint32_t my_base = smem_u32(smem + (size_t)warp * NSTAGE * STAGEB);
   if (lane == 0) {
@@ -273,6 +295,15 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
     for (int st = 0; st < NSTAGE; ++st) mbar_init(smem_u32(&bars[warp][st]), 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     fence_proxy_async();
+  }
+  if constexpr (CL) {
+    if (threadIdx.x == 0) {
+      mbar_init(smem_u32(&cl_bar), 1);
+      asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncwarp();
+    // the pieces' barriers exist before anything is sent to them: waited for ahead of the first send, long after
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");
   }
   __syncwarp();
   uint32_t phase_bits = 0;   // parity of each stage's barrier (carried across the CTA's work items)
@@ -470,6 +501,11 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   }
   const WorkItem &it = cc.it;
   const int item_idx = cc.item_idx;
+  if constexpr (CL)
+    if (it.hd_count == 0) {   // a place in the cluster without work
+      asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+      continue;
+    }
   if (!UNI && it.h == 0 && it.g0 == 0 && threadIdx.x == 0) cv.step_snap[(long long)it.b * G.L + a.layer] = cv.steps[it.b];
   const int b = it.b, ridx = it.ridx, T_t = cc.T_t;
   const int first = cc.first, n_my = cc.n_my;
@@ -490,7 +526,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   // Chained layers: while the preceding work still runs, this warp resolves the metadata of the granules it has queued,
   // waits for their bytes and clears masked V rows; none of it depends on that work.  What is left behind the wait is the
   // query load, the arithmetic and the merge.
-  const bool early = arm && a.wait_inputs && qi == q_begin;
+  const bool early = CL || (arm && a.wait_inputs && qi == q_begin);
   if (early) {
 #pragma unroll
     for (int n = 0; n < NSTAGE; ++n)
@@ -521,6 +557,101 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       for (int n = n_pro; n < NSTAGE; ++n) produce();
   }
 
+  const int new_j = a.has_new ? (T_t - 1) / GR : -1;   // the text granule that takes the row of the token being generated
+  // Up to two granules per step, from n on: waits for their bytes (bounded) and clears masked V rows; a granule with nothing
+  // visible (an empty slot, text capacity not yet written) is passed over.  u_new: which of them takes the new token's row.
+  uint32_t sKs[2] = {0u, 0u}, sVs[2] = {0u, 0u};
+  int valids[2] = {0, 0}, sidxs[2] = {-1, -1}, fmt[2] = {0, 0};
+  int cnt = 0, nu = 0, adv = 0, u_new = -1;
+  auto collect = [&](int n) {
+    cnt = n + 1 < n_my ? 2 : 1;
+    nu = 0; adv = 0; u_new = -1;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (u < cnt && n < n_my && !timed_out) {
+        const int stage = (int)((seq_c + u) % NSTAGE);
+        const int2 rg = ring[warp][stage];
+        const int valid = rg.x & 255;
+        const bool pre = (prewaited >> stage) & 1u;   // waited for (and masked rows cleared) ahead of the inputs
+        prewaited &= ~(1u << stage);
+        if ((rg.x & 256) && !pre) {  // a copy was queued for this stage: wait for its bytes (bounded)
+          if (!mbar_wait(smem_u32(&bars[warp][stage]), (phase_bits >> stage) & 1u)) timed_out = true;
+          else phase_bits ^= 1u << stage;
+        }
+        if (!timed_out) ++adv;
+        if (valid > 0 && !timed_out) {
+          const uint32_t sK = my_base + stage * STAGEB, sV = sK + TILEB;
+          if (first + (n + u) * NW == new_j) u_new = nu;
+          if (!KO && valid < GR && !pre) {
+            // rows past the visible ones get probability 0, but 0 x NaN is NaN and a caller-owned buffer (the allocation-free
+            // entry) may hold anything there: clear those V rows (a masked K row only spoils logits that are replaced anyway)
+            for (int r = valid + (lane >> 3); r < GR; r += 4)
+#pragma unroll
+              for (int hf = 0; hf < HALVES; ++hf)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};\n" ::"r"(sV + hf * HALFB + r * 128 + ((lane & 7) << 4)), "r"(0u) : "memory");
+          }
+          if (nu == 0) { sKs[0] = sK; sVs[0] = sV; valids[0] = valid; sidxs[0] = rg.y; fmt[0] = rg.x >> 9; }
+          else { sKs[1] = sK; sVs[1] = sV; valids[1] = valid; sidxs[1] = rg.y; fmt[1] = rg.x >> 9; }
+          ++nu;
+        }
+      }
+    }
+    // the cluster kernel has one form of the step: a single granule goes with a copy of itself, fully masked
+    if (CL && nu == 1) { sKs[1] = sKs[0]; sVs[1] = sVs[0]; valids[1] = 0; sidxs[1] = -1; fmt[1] = fmt[0]; }
+  };
+  // The row of the token being generated: from k_new / v_new to the text region and into the collected granule.
+  auto load_new = [&]() {
+    const int kv = lane / PPR, pc = lane - kv * PPR;
+    return lane < 2 * PPR ? __ldcg(reinterpret_cast<const uint4 *>((kv ? a.v_new : a.k_new) + ((long long)it.i * G.Hkv + it.h) * D + pc * 8))
+                          : make_uint4(0, 0, 0, 0);
+  };
+  auto place_new = [&](const uint4 &val) {
+    const int nr = (T_t - 1) - new_j * GR;
+    if (lane < 2 * PPR) {
+      const int kv = lane / PPR, pc = lane - kv * PPR;
+      *reinterpret_cast<uint4 *>(cv.text + text_off(G, b, a.layer, it.h, kv) + (long long)(T_t - 1) * D + pc * 8) = val;
+      const uint32_t sK = u_new ? sKs[1] : sKs[0], sV = u_new ? sVs[1] : sVs[0];
+      const uint32_t dst = (kv ? sV : sK) + (pc >> 3) * HALFB + nr * 128 + (((pc & 7) ^ (nr & 7)) << 4);
+      asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst), "r"(val.x), "r"(val.y), "r"(val.z), "r"(val.w) : "memory");
+    }
+  };
+  // What the exchange between the pieces of a head needs, all of it ahead of the inputs (see there)
+  int cl_np = 1, cl_piece = 0, cl_slots = 0;
+  uint32_t cl_recv = 0, cl_dst[G16 ? 4 : 2] = {}, cl_dbar[G16 ? 4 : 2] = {}, cl_mldst = 0, cl_mlbar = 0;
+  const int GP = (g + 1) / 2, U = GP * (D / 2);
+  if constexpr (CL) {
+    cl_np = it.hd_count; cl_piece = item_idx - it.hd_first;
+    cl_slots = (U - cl_piece + cl_np - 1) / cl_np;
+    cl_recv = smem_u32(smem + (size_t)NW * NSTAGE * STAGEB);
+    const uint32_t rank0 = (uint32_t)(it.hd_first % a.cluster), bar = smem_u32(&cl_bar);
+    auto peer = [&](uint32_t addr, int piece) {
+      uint32_t r;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank0 + piece));
+      return r;
+    };
+    if (cl_np > 1) {
+#pragma unroll
+      for (int y = 0; y < (G16 ? 4 : 2); ++y) {
+        const int u = (threadIdx.x + y * NW * 32) >> 1;
+        if (u < U) {
+          const int slot = u / cl_np, dest = u - slot * cl_np;
+          cl_dst[y] = peer(cl_recv + (uint32_t)(slot * cl_np + cl_piece) * 16, dest);
+          cl_dbar[y] = peer(bar, dest);
+        }
+      }
+      const int td = (threadIdx.x >> 1) % (D / 2);
+      if (td < cl_np) {
+        cl_mldst = peer(cl_recv + (uint32_t)(U + 16) * 16 + (uint32_t)cl_piece * 16, td);   // + p * 256 for head pair p
+        cl_mlbar = peer(bar, td);
+      }
+      if (threadIdx.x == 0) mbar_expect_tx(bar, (uint32_t)(cl_np * 16 * (cl_slots + GP)));
+    }
+    for (int x = threadIdx.x; x < ((G16 ? 16 : 8) - g) * PPR; x += NW * 32)   // query heads beyond the group
+      *reinterpret_cast<uint4 *>(cl_q + (g + x / PPR) * QROW + (x % PPR) * 16) = make_uint4(0, 0, 0, 0);
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    collect(0);
+  }
+
   // Chained layers: the cache loads above never depend on the preceding work, the query and the new token's K/V do.
   // Their lines are asked into L2 ahead of the wait (L2 is where the preceding work's stores land, so nothing stale can
   // be read from it); the loads after the wait go past L1.
@@ -538,7 +669,26 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   // ---- Q fragments (the B operand of S^T = K q^T; heads >= g are zero columns); loaded after the first K/V copies are in flight ----
   const int r0 = lane >> 2, cq = (lane & 3) * 2;
   uint32_t qa[KK][NQ];
-  {
+  if constexpr (CL) {
+    // One read of the query per CTA, not one per warp: the pieces of an anchor head are 14 CTAs that ask the same few lines
+    // at the same moment (each warp its own: 0.4 to 1.2 us, queueing at the lines' L2 slices)
+    uint4 new_val = make_uint4(0, 0, 0, 0);
+    if (u_new >= 0) new_val = load_new();
+    if (threadIdx.x < g * PPR) {
+      const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(a.q + ((long long)it.i * G.Hq + (long long)it.h * g) * D) + threadIdx.x);
+      *reinterpret_cast<uint4 *>(cl_q + (threadIdx.x / PPR) * QROW + (threadIdx.x % PPR) * 16) = v;
+    }
+    if (u_new >= 0) place_new(new_val);
+    __syncthreads();
+#pragma unroll
+    for (int kk = 0; kk < KK; kk += 2)
+#pragma unroll
+      for (int nt = 0; nt < NQ / 2; ++nt) {
+        uint32_t r[4];
+        ldsm_x4(r, smem_u32(cl_q) + (uint32_t)((nt * 8 + (lane & 7)) * QROW + (kk * 2 + (lane >> 3)) * 16));
+        qa[kk][2 * nt] = r[0]; qa[kk][2 * nt + 1] = r[1]; qa[kk + 1][2 * nt] = r[2]; qa[kk + 1][2 * nt + 1] = r[3];
+      }
+  } else {
     const bf16 *qb = a.q + ((long long)(KO ? blockIdx.y : it.i) * G.Hq + (long long)it.h * g) * D;
 #pragma unroll
     for (int kk = 0; kk < KK; ++kk) {
@@ -603,9 +753,9 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
     for (int u = 0; u < NU; ++u) {
       scu[u] = sc; vshift[u] = 0.f; vinv[u] = 1.f;
       if (F8 && (fmt[u] & 1)) {
-        scu[u] = sc * exp2f((float)(int8_t)((fmt[u] >> 7) & 0xff));
+        scu[u] = sc * ex2((float)(int8_t)((fmt[u] >> 7) & 0xff));
         vshift[u] = (float)(int8_t)((fmt[u] >> 15) & 0xff);
-        vinv[u] = exp2f(-vshift[u]);
+        vinv[u] = ex2(-vshift[u]);
       }
     }
     {
@@ -686,13 +836,13 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
         mxB = fmaxf(mxB, __shfl_xor_sync(0xffffffffu, mxB, sh));
       }
       const float mnA = fmaxf(mrun[nt][0], mxA), mnB = fmaxf(mrun[nt][1], mxB);   // finite: the step has a visible token
-      const float alA = exp2f(mrun[nt][0] - mnA), alB = exp2f(mrun[nt][1] - mnB);
+      const float alA = ex2(mrun[nt][0] - mnA), alB = ex2(mrun[nt][1] - mnB);
       mrun[nt][0] = mnA; mrun[nt][1] = mnB;
       float addA = 0.f, addB = 0.f;
 #pragma unroll
       for (int u = 0; u < NU; ++u) {
-        v[u][0] = exp2f(v[u][0] - mnA); v[u][2] = exp2f(v[u][2] - mnA);
-        v[u][1] = exp2f(v[u][1] - mnB); v[u][3] = exp2f(v[u][3] - mnB);
+        v[u][0] = ex2(v[u][0] - mnA); v[u][2] = ex2(v[u][2] - mnA);
+        v[u][1] = ex2(v[u][1] - mnB); v[u][3] = ex2(v[u][3] - mnB);
         float eA = v[u][0] + v[u][2], eB = v[u][1] + v[u][3];
         if constexpr (F8) { addA += eA * vinv[u]; addB += eB * vinv[u]; }
         else { addA += eA; addB += eB; }
@@ -767,69 +917,36 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   };
 
   STAMP(17);
-  const int new_j = a.has_new ? (T_t - 1) / GR : -1;   // the text granule that takes the row of the token being generated
-  for (int n = 0; n < n_my && !timed_out;) {
-    __syncwarp();
-    // up to two granules per step; a granule with nothing visible (an empty slot, text capacity not yet written) is passed over
-    const int cnt = n + 1 < n_my ? 2 : 1;
-    uint32_t sKs[2] = {0u, 0u}, sVs[2] = {0u, 0u};
-    int valids[2] = {0, 0}, sidxs[2] = {-1, -1}, fmt[2] = {0, 0};
-    int nu = 0, adv = 0;
-    if (n == 0) STAMP(18);
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      if (u < cnt && !timed_out) {
-        const int stage = (int)((seq_c + u) % NSTAGE);
-        const int2 rg = ring[warp][stage];
-        const int valid = rg.x & 255;
-        const bool pre = (prewaited >> stage) & 1u;   // waited for (and masked rows cleared) ahead of the inputs
-        prewaited &= ~(1u << stage);
-        if ((rg.x & 256) && !pre) {  // a copy was queued for this stage: wait for its bytes (bounded)
-          if (!mbar_wait(smem_u32(&bars[warp][stage]), (phase_bits >> stage) & 1u)) timed_out = true;
-          else phase_bits ^= 1u << stage;
-        }
-        if (!timed_out) ++adv;
-        if (n == 0 && u == 0) STAMP(24);
-        if (valid > 0 && !timed_out) {
-          const uint32_t sK = my_base + stage * STAGEB, sV = sK + TILEB;
-          // the row of the token being generated: take it from k_new/v_new and store it into the text region
-          const int j = first + (n + u) * NW;
-          if (j == new_j) {
-            const int nr = (T_t - 1) - j * GR;
-            if (lane < 2 * PPR) {
-              const int kv = lane / PPR, pc = lane - kv * PPR;
-              const long long noff = ((long long)it.i * G.Hkv + it.h) * D + pc * 8;
-              const uint4 val = __ldcg(reinterpret_cast<const uint4 *>((kv ? a.v_new : a.k_new) + noff));
-              *reinterpret_cast<uint4 *>(cv.text + text_off(G, b, a.layer, it.h, kv) + (long long)(T_t - 1) * D + pc * 8) = val;
-              const uint32_t dst = (kv ? sV : sK) + (pc >> 3) * HALFB + nr * 128 + (((pc & 7) ^ (nr & 7)) << 4);
-              asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst), "r"(val.x), "r"(val.y), "r"(val.z), "r"(val.w) : "memory");
-            }
-          }
-          if (!KO && valid < GR && !pre) {
-            // rows past the visible ones get probability 0, but 0 x NaN is NaN and a caller-owned buffer (the allocation-free
-            // entry) may hold anything there: clear those V rows (a masked K row only spoils logits that are replaced anyway)
-            for (int r = valid + (lane >> 3); r < GR; r += 4)
-#pragma unroll
-              for (int hf = 0; hf < HALVES; ++hf)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};\n" ::"r"(sV + hf * HALFB + r * 128 + ((lane & 7) << 4)), "r"(0u) : "memory");
-          }
-          if (nu == 0) { sKs[0] = sK; sVs[0] = sV; valids[0] = valid; sidxs[0] = rg.y; fmt[0] = rg.x >> 9; }
-          else { sKs[1] = sK; sVs[1] = sV; valids[1] = valid; sidxs[1] = rg.y; fmt[1] = rg.x >> 9; }
-          ++nu;
-        }
-      }
+  if constexpr (CL) {
+    // the first granules are collected; more than two a warp are the exception
+    for (int n = 0;;) {
+      if (timed_out) { seq_c += adv; break; }   // the stages whose bytes never came are drained (bounded) before the CTA ends
+      if (nu > 0) step(std::integral_constant<int, 2>{}, sKs, sVs, valids, sidxs, fmt);
+      STAMP(8);
+      n += cnt; seq_c += cnt;
+      if (__builtin_expect(n >= n_my, 1)) break;
+      __syncwarp();
+      for (int u = 0; u < cnt; ++u) produce();
+      collect(n);
+      if (u_new >= 0) place_new(load_new());
+      __syncwarp();
     }
-    __syncwarp();
-    if (n == 0) STAMP(7);
-    if (timed_out) { seq_c += adv; break; }   // the stages whose bytes never came are drained (bounded) before the CTA ends
-    {
+  } else {
+    for (int n = 0; n < n_my && !timed_out;) {
+      __syncwarp();
+      if (n == 0) STAMP(18);
+      collect(n);
+      if (u_new >= 0 && !timed_out) place_new(load_new());
+      __syncwarp();
+      if (n == 0) STAMP(7);
+      if (timed_out) { seq_c += adv; break; }   // the stages whose bytes never came are drained (bounded) before the CTA ends
       if (nu == 2) step(std::integral_constant<int, 2>{}, sKs, sVs, valids, sidxs, fmt);
       else if (nu == 1) step(std::integral_constant<int, 1>{}, sKs, sVs, valids, sidxs, fmt);
+      __syncwarp();
+      if (n == 0) STAMP(8);
+      n += cnt; seq_c += cnt;
+      for (int u = 0; u < cnt; ++u) produce();
     }
-    __syncwarp();
-    if (n == 0) STAMP(8);
-    n += cnt; seq_c += cnt;
-    for (int u = 0; u < cnt; ++u) produce();
   }
   STAMP(9);
   if (timed_out && lane == 0 && cv.status) atomicOr(cv.status, STATUS_TIMEOUT);
@@ -841,6 +958,132 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       lrun[nt][0] += __shfl_xor_sync(0xffffffffu, lrun[nt][0], sh);
       lrun[nt][1] += __shfl_xor_sync(0xffffffffu, lrun[nt][1], sh);
     }
+  if constexpr (CL) {
+    // ---- chained layers, one wave: what counts is the span of the kernel, and a head's pieces meet inside a cluster ----
+    // A piece merges its warps, then every piece of the head sends every other one the share of the accumulators that one
+    // finishes (and its (max, denominator) pairs) straight into the other's shared memory (st.async, completion counted in
+    // bytes by the receiver's mbarrier), and each finishes its share: no partials in global memory, no fence, no counter, no
+    // last CTA that reads all partials back.  From the end of the last product to the output, config 1 (14 and 4 pieces):
+    // CL_BEFORE -> CL_AFTER us; a chained layer 7.1 -> CL_LAYER us.
+    //
+    // The accumulators travel as units of four values as they sit in a lane: heads 2p and 2p + 1 at d = 16 t + r and 16 t + r + 8.
+    // Unit u = p * D / 2 + 8 t + r; piece u % np finishes it, in place u / np of its receive buffer.
+    // All addresses were made before the inputs were waited for; what is left is one barrier, the merge of the warps, the
+    // flight of the bytes and the last sums.
+    constexpr int US = D / 2 + 2;   // units of a head pair in a warp's scratch, padded: the lanes of a store fall in different banks
+    if (r0 == 0) {
+#pragma unroll
+      for (int nt = 0; nt < NTN; ++nt)
+        *reinterpret_cast<float4 *>(&cl_ml[warp * 16 + nt * 8 + cq]) = make_float4(mrun[nt][0], lrun[nt][0], mrun[nt][1], lrun[nt][1]);
+    }
+#pragma unroll
+    for (int nt = 0; nt < NTN; ++nt) {
+      const int p = nt * 4 + (lane & 3);
+      if (p < GP)
+#pragma unroll
+        for (int t = 0; t < D / 16; ++t)   // the warp's own stages are idle by now
+          asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};\n" ::"r"(my_base + (p * US + t * 8 + r0) * 16), "f"(oT[nt][t][0]), "f"(oT[nt][t][1]),
+                       "f"(oT[nt][t][2]), "f"(oT[nt][t][3]) : "memory");
+    }
+    __syncthreads();
+    STAMP(2);
+    bf16 *ob = a.out + ((long long)it.i * G.Hq + (long long)it.h * g) * D;
+    auto send = [&](uint32_t dst, uint32_t bar, float x, float y, float z, float w) {
+      asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n" ::"r"(dst), "f"(x), "f"(y), "f"(z),
+                   "f"(w), "r"(bar) : "memory");
+    };
+    // merge of the warps: two threads per unit, four warps each
+#pragma unroll
+    for (int y = 0; y < (G16 ? 4 : 2); ++y) {
+      const int u = (threadIdx.x + y * NW * 32) >> 1, hf = threadIdx.x & 1, p = u / (D / 2), td = u % (D / 2);
+      if (u < U) {   // uniform over a warp: a warp's 16 units belong to one head pair
+        float4 ml[NW], o[NW / 2];
+#pragma unroll
+        for (int w = 0; w < NW; ++w) ml[w] = *reinterpret_cast<const float4 *>(&cl_ml[w * 16 + 2 * p]);
+#pragma unroll
+        for (int x = 0; x < NW / 2; ++x)
+          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(o[x].x), "=f"(o[x].y), "=f"(o[x].z), "=f"(o[x].w)
+                       : "r"(smem_u32(smem) + (uint32_t)((hf * (NW / 2) + x) * NSTAGE * STAGEB + (p * US + td) * 16)));
+        float MA = -INFINITY, MB = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) { MA = fmaxf(MA, ml[w].x); MB = fmaxf(MB, ml[w].z); }
+        // a warp without keys has max -inf and weight 0; without any key in the piece all weights are 0
+        const float MA0 = MA > -INFINITY ? MA : 0.f, MB0 = MB > -INFINITY ? MB : 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float LA = 0.f, LB = 0.f;
+#pragma unroll
+        for (int x = 0; x < NW / 2; ++x) {
+          const float4 m = hf ? ml[NW / 2 + x] : ml[x];
+          const float fA = ex2(m.x - MA0), fB = ex2(m.z - MB0);
+          acc.x += o[x].x * fA; acc.y += o[x].y * fB; acc.z += o[x].z * fA; acc.w += o[x].w * fB;
+          LA += m.y * fA; LB += m.w * fB;
+        }
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 1); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 1);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 1); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 1);
+        LA += __shfl_xor_sync(0xffffffffu, LA, 1); LB += __shfl_xor_sync(0xffffffffu, LB, 1);
+        if (cl_np > 1) {
+          if (hf == 0) send(cl_dst[y], cl_dbar[y], acc.x, acc.y, acc.z, acc.w);
+          else if (td < cl_np) send(cl_mldst + (uint32_t)p * 256, cl_mlbar, MA, LA, MB, LB);
+        } else {   // the whole head is here: finish it
+          const float L = hf ? LB : LA, inv = L > 0.f ? 1.f / L : 0.f;
+          const int hq = 2 * p + hf, dd = (td >> 3) * 16 + (td & 7);
+          if (hq < g) {
+            ob[hq * D + dd] = __float2bfloat16_rn((hf ? acc.y : acc.x) * inv);
+            ob[hq * D + dd + 8] = __float2bfloat16_rn((hf ? acc.w : acc.z) * inv);
+            if (td == 0) a.head_mz[(long long)it.i * G.Hq + it.h * g + hq] = make_float2(hf ? MB : MA, L);
+          }
+        }
+      }
+    }
+    STAMP(3);
+    if (cl_np == 1) continue;
+    // a peer may be late by its own bounded waits; this wait is long enough for all of them, so that nobody sends to a CTA that has left
+    if (!mbar_wait_cluster(smem_u32(&cl_bar), 0) && threadIdx.x == 0) atomicOr(cv.status, STATUS_TIMEOUT);
+    STAMP(4);
+    // finish this piece's share: four lanes per unit, each adds up every fourth piece
+    const int src = threadIdx.x & 3;
+    for (int s0 = 0; s0 < cl_slots; s0 += NW * 8) {
+      const int slot = s0 + (threadIdx.x >> 2), u = slot * cl_np + cl_piece, p = u / (D / 2), td = u % (D / 2);
+      float4 o[4], ml[4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        o[x] = make_float4(0.f, 0.f, 0.f, 0.f); ml[x] = make_float4(-INFINITY, 0.f, -INFINITY, 0.f);
+        if (slot < cl_slots && src + 4 * x < cl_np) {
+          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(o[x].x), "=f"(o[x].y), "=f"(o[x].z), "=f"(o[x].w)
+                       : "r"(cl_recv + (uint32_t)(slot * cl_np + src + 4 * x) * 16) : "memory");
+          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(ml[x].x), "=f"(ml[x].y), "=f"(ml[x].z), "=f"(ml[x].w)
+                       : "r"(cl_recv + (uint32_t)(U + 16) * 16 + (uint32_t)(p * 16 + src + 4 * x) * 16) : "memory");
+        }
+      }
+      float MA = fmaxf(fmaxf(ml[0].x, ml[1].x), fmaxf(ml[2].x, ml[3].x)), MB = fmaxf(fmaxf(ml[0].z, ml[1].z), fmaxf(ml[2].z, ml[3].z));
+#pragma unroll
+      for (int sh = 2; sh > 0; sh >>= 1) { MA = fmaxf(MA, __shfl_xor_sync(0xffffffffu, MA, sh)); MB = fmaxf(MB, __shfl_xor_sync(0xffffffffu, MB, sh)); }
+      const float MA0 = MA > -INFINITY ? MA : 0.f, MB0 = MB > -INFINITY ? MB : 0.f;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float LA = 0.f, LB = 0.f;
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const float fA = ex2(ml[x].x - MA0), fB = ex2(ml[x].z - MB0);
+        acc.x += o[x].x * fA; acc.y += o[x].y * fB; acc.z += o[x].z * fA; acc.w += o[x].w * fB;
+        LA += ml[x].y * fA; LB += ml[x].w * fB;
+      }
+#pragma unroll
+      for (int sh = 2; sh > 0; sh >>= 1) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, sh); acc.y += __shfl_xor_sync(0xffffffffu, acc.y, sh);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, sh); acc.w += __shfl_xor_sync(0xffffffffu, acc.w, sh);
+        LA += __shfl_xor_sync(0xffffffffu, LA, sh); LB += __shfl_xor_sync(0xffffffffu, LB, sh);
+      }
+      // lane e of the four stores value e of the unit
+      const int hq = 2 * p + (src & 1), dd = (td >> 3) * 16 + (td & 7) + (src >> 1) * 8;
+      if (slot < cl_slots && hq < g) {
+        const float L = (src & 1) ? LB : LA, inv = L > 0.f ? 1.f / L : 0.f;
+        ob[hq * D + dd] = __float2bfloat16_rn((src == 0 ? acc.x : src == 1 ? acc.y : src == 2 ? acc.z : acc.w) * inv);
+        if (td == 0 && src < 2) a.head_mz[(long long)it.i * G.Hq + it.h * g + hq] = make_float2(src ? MB : MA, L);
+      }
+    }
+    STAMP(5);
+    continue;
+  }
   __syncthreads();
   STAMP(2);
 
@@ -868,7 +1111,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       for (int w = 0; w < NW; ++w) M = fmaxf(M, red_ml[w * 16 + threadIdx.x].x);
       if (M > -INFINITY)
 #pragma unroll
-        for (int w = 0; w < NW; ++w) L += red_ml[w * 16 + threadIdx.x].y * exp2f(red_ml[w * 16 + threadIdx.x].x - M);
+        for (int w = 0; w < NW; ++w) L += red_ml[w * 16 + threadIdx.x].y * ex2(red_ml[w * 16 + threadIdx.x].x - M);
       a.part_ml[((long long)blockIdx.y * gridDim.x + item_idx) * g + threadIdx.x] = make_float2(M, L);
     }
     continue;
@@ -905,7 +1148,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
 #pragma unroll
       for (int w = 0; w < NW; ++w) {
         const float2 ml = red_ml[w * 16 + row];
-        const float f = exp2f(ml.x - M);   // a warp without work has m = -inf -> factor 0
+        const float f = ex2(ml.x - M);   // a warp without work has m = -inf -> factor 0
         const float2 x = *reinterpret_cast<const float2 *>(red_o + ((size_t)w * g + row) * RS + (idx - row * D));
         a0 += x.x * f; a1 += x.y * f;
         L += ml.y * f;
@@ -973,11 +1216,11 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
 #pragma unroll
         for (int j = 0; j < MB; ++j) Mb = fmaxf(Mb, ml[j].x);
         if (Mb > -INFINITY) {
-          const float sc0 = exp2f(M - Mb);  // M = -inf on the first batch -> 0
+          const float sc0 = ex2(M - Mb);  // M = -inf on the first batch -> 0
           acc.x *= sc0; acc.y *= sc0; acc.z *= sc0; acc.w *= sc0; Z *= sc0;
 #pragma unroll
           for (int j = 0; j < MB; ++j) {
-            const float w = exp2f(ml[j].x - Mb);  // empty split: m = -inf -> 0
+            const float w = ex2(ml[j].x - Mb);  // empty split: m = -inf -> 0
             acc.x += x[j].x * w; acc.y += x[j].y * w; acc.z += x[j].z * w; acc.w += x[j].w * w;
             Z += ml[j].y * w;
           }
@@ -1015,6 +1258,15 @@ __global__ void __launch_bounds__(NW * 32, NW == NW_THR ? (G16 ? 2 : WNW_THR_CTA
                                                            const __grid_constant__ InlineItems inl,
                                                            const __grid_constant__ TmaMaps maps) {
   attn_body<D, G16, NW, VAR>(cv, a, &inl, maps, (int)blockIdx.x);
+}
+
+// Chained or serial layers of one wave: the pieces of a head in one cluster.
+template <int D, bool G16, int VAR>
+__global__ void __launch_bounds__(NW_LAT * 32, 1) wnw_attn_cluster_kernel(const __grid_constant__ CacheView cv,
+                                                                         const __grid_constant__ AttnArgs a,
+                                                                         const __grid_constant__ InlineItems inl,
+                                                                         const __grid_constant__ TmaMaps maps) {
+  attn_body<D, G16, NW_LAT, VAR, true>(cv, a, &inl, maps, (int)blockIdx.x);
 }
 
 // All heads cut alike (VAR 3, 4): the item list is in the launch shape.
@@ -1107,6 +1359,51 @@ cudaError_t launch_attn_uniform(const CacheView &cv, const AttnArgs &a, int n_he
   return g16 ? launch_uniform_t<64, true, 3>(cv, a, n, 1, st) : launch_uniform_t<64, false, 3>(cv, a, n, 1, st);
 }
 
+// Receive buffers of a piece: units of its share from every piece, (max, denominator) pairs
+static size_t cluster_smem(int g, int d) { return uniform_smem(d) + (size_t)((g + 1) / 2 * (d / 2) + 16) * 16 + 8 * 16 * 16; }
+static void cluster_attrs(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int g, int d, int n_ctas, int cluster, bool pdl, cudaStream_t st) {
+  cfg.gridDim = dim3((unsigned)n_ctas, 1, 1);
+  cfg.blockDim = dim3(NW_LAT * 32, 1, 1);
+  cfg.dynamicSmemBytes = cluster_smem(g, d);
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cluster; attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = pdl ? 2 : 1;
+}
+template <int D, bool G16, int VAR>
+static cudaError_t launch_cluster_t(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
+  if (!a.maps || a.n_items % a.cluster) return cudaErrorInvalidValue;
+  InlineItems inl;
+  if (a.n_items <= INLINE_ITEMS_MAX) memcpy(inl.it, a.items_host, sizeof(WorkItem) * a.n_items);
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[2];
+  cluster_attrs(cfg, attr, cv.geo.g, D, a.n_items, a.cluster, a.pdl, st);
+  return cudaLaunchKernelEx(&cfg, wnw_attn_cluster_kernel<D, G16, VAR>, cv, a, inl, *a.maps);
+}
+template <int D, bool G16>
+static cudaError_t launch_cluster(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
+  if constexpr (D == 128)
+    if (cv.geo.kv8) return launch_cluster_t<D, G16, 2>(cv, a, st);
+  if (cv.geo.kv8) return cudaErrorInvalidValue;
+  return cv.geo.token_base ? launch_cluster_t<D, G16, 1>(cv, a, st) : launch_cluster_t<D, G16, 0>(cv, a, st);
+}
+// Clusters of the given size that the GPU holds at once (0 if it takes none)
+template <int D, bool G16>
+static int cluster_room_t(int g, int cluster) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[2];
+  cluster_attrs(cfg, attr, g, D, cluster, cluster, false, nullptr);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, wnw_attn_cluster_kernel<D, G16, 0>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return n;
+}
+int attn_cluster_room(int g, int d, int cluster) {
+  if (d == 128) return g > 8 ? cluster_room_t<128, true>(g, cluster) : cluster_room_t<128, false>(g, cluster);
+  return g > 8 ? cluster_room_t<64, true>(g, cluster) : cluster_room_t<64, false>(g, cluster);
+}
+
 template <int D, bool G16, int NW>
 static cudaError_t launch_t(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
   if constexpr (D == 128)
@@ -1171,7 +1468,15 @@ static cudaError_t configure_t() {
   if ((e = cudaFuncSetAttribute(wnw_attn_multi_kernel<D, G16, NW, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(wnw_attn_multi_kernel<D, G16, NW, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) != cudaSuccess) return e;
   if constexpr (NW == NW_LAT) {
-    const int ub = (int)uniform_smem(D);
+    const int ub = (int)uniform_smem(D), cb = (int)cluster_smem(G16 ? 16 : 8, D);
+    auto cluster = [&](auto *k) {
+      const cudaError_t r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, cb);
+      return r != cudaSuccess ? r : cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // up to 16 CTAs
+    };
+    if ((e = cluster(wnw_attn_cluster_kernel<D, G16, 0>)) != cudaSuccess) return e;
+    if ((e = cluster(wnw_attn_cluster_kernel<D, G16, 1>)) != cudaSuccess) return e;
+    if constexpr (D == 128)
+      if ((e = cluster(wnw_attn_cluster_kernel<D, G16, 2>)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(wnw_attn_uniform_kernel<D, G16, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, ub)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(wnw_attn_uniform_kernel<D, G16, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, ub)) != cudaSuccess) return e;
   }
@@ -1197,7 +1502,10 @@ cudaError_t configure_attn_kernels() {
 cudaError_t launch_attn(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
   if (a.n_items <= 0) return cudaSuccess;
   const bool g16 = cv.geo.g > 8;
-  if (a.throughput) {
+  if (a.cluster) {
+    if (cv.geo.d == 128) return g16 ? launch_cluster<128, true>(cv, a, st) : launch_cluster<128, false>(cv, a, st);
+    if (cv.geo.d == 64) return g16 ? launch_cluster<64, true>(cv, a, st) : launch_cluster<64, false>(cv, a, st);
+  } else if (a.throughput) {
     if (cv.geo.d == 128) return g16 ? launch_t<128, true, NW_THR>(cv, a, st) : launch_t<128, false, NW_THR>(cv, a, st);
     if (cv.geo.d == 64) return g16 ? launch_t<64, true, NW_THR>(cv, a, st) : launch_t<64, false, NW_THR>(cv, a, st);
   } else {

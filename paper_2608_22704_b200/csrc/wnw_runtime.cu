@@ -36,6 +36,7 @@ struct LayerWork {
   int n_ctas = 0, order_off = 0, ranges_off = 0;   // items per CTA (persistent schedule, or packed short heads): offsets
   int n_ctas_free = 0;   // BATCHED layers: the first n_ctas_free CTAs hold no tidal head (they need no recall epoch) ...
   int n_ctas_anchor = 0; // ... and the first n_ctas_anchor of those hold the anchor heads (what the step's selection waits for)
+  int cluster = 0;                                 // chained layers of one wave: CTAs per cluster
   bool packed = false;                             // one-shot CTAs that serve several short heads each
   int head_items_off = 0;                          // offset in the list's HeadItems
 };
@@ -63,6 +64,7 @@ struct wnw_cache {
   std::vector<uint8_t> anchor_layer;   // [L] the layer has an anchor head (on any shard, when the cache holds one shard of the heads)
   bool scores_exported = false, scores_imported = false;   // head-sharded step: where the exchange stands
   int tid_total = 0, n_sm = 148;
+  int cluster_room[3] = {0, 0, 0};   // attention clusters of 4, 8 and 16 CTAs that fit the GPU at once
   std::vector<SeqHost> seqs;
   std::vector<void *> dev_allocs;
   char *small_block = nullptr;      // where the next small device array goes
@@ -353,6 +355,7 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
   cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
   CKE(configure_attn_kernels());
   CKE(configure_select_kernel());
+  for (int k = 0; k < 3; ++k) c->cluster_room[k] = attn_cluster_room(cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim, 4 << k);
   const int L = cfg->n_layers, Hkv = cfg->n_kv_heads, d = cfg->head_dim, nc = cfg->chunk_tokens;
   const bool full = cfg->mode == WNW_MODE_FULL;
   c->roles.assign(cfg->roles, cfg->roles + (size_t)L * Hkv);
@@ -657,6 +660,10 @@ static void head_granules(const wnw_cache *c, int layer, int mode, const SeqHost
 // single piece of the same size).  So heads are cut as little as the balance allows: for a piece size T a head becomes
 // round(work / T) even pieces (at least one), the pieces go longest-first to the least loaded CTA, and T is the candidate
 // between 0.3 and three even shares of the launch that gives the shortest longest CTA under that cost model.
+#ifndef WNW_CLUSTER_MAX_PER_WARP
+#define WNW_CLUSTER_MAX_PER_WARP 8
+#endif
+constexpr int CLUSTER_MAX_PER_WARP = WNW_CLUSTER_MAX_PER_WARP;
 struct CutMemo {   // piece sizes found for one work list, by the launch's head sizes
   struct Entry { std::vector<int> sizes; double T; };
   std::vector<Entry> entries;
@@ -789,6 +796,57 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   lw.packed = true;   // the pipeline runs across a CTA's items (its merge scratch sits behind the stages)
 }
 
+// Chained or serial layers whose work fits one wave: the pieces of a head form (part of) a cluster and merge inside it, which
+// costs little however many there are, so heads are cut as fine as fits: two granules a warp (all bytes of a piece in flight
+// before the layer's inputs are there, one softmax step behind them), more where that would not fit one wave or where a head
+// would need more than the 16 pieces a cluster holds.  Heads are packed into clusters, most pieces first; places left over stay empty.
+static bool build_cluster_items(const wnw_cache *c, int layer, int mode, const std::vector<int> &seq_ids,
+                                const std::vector<int> &n_gran, const std::vector<int> &n_work, std::vector<WorkItem> &items,
+                                std::vector<HeadItems> &heads, LayerWork &lw) {
+  const Geometry &G = c->geo;
+  const int n_heads = (int)seq_ids.size() * G.Hkv, nw = attn_warps(false);
+  std::vector<int> np(n_heads), by(n_heads), first(n_heads), room;
+  for (int per = 2; per <= CLUSTER_MAX_PER_WARP; ++per) {
+    int most = 1;
+    for (int hd = 0; hd < n_heads; ++hd) {
+      np[hd] = std::max(1, std::min(16, (n_work[hd] + per * nw - 1) / (per * nw)));
+      most = std::max(most, np[hd]);
+      by[hd] = hd;
+    }
+    const int k = most <= 4 ? 0 : most <= 8 ? 1 : 2, size = 4 << k;
+    std::stable_sort(by.begin(), by.end(), [&](int x, int y) { return np[x] > np[y]; });
+    room.clear();
+    for (int hd : by) {
+      size_t x = 0;
+      while (x < room.size() && room[x] < np[hd]) ++x;
+      if (x == room.size()) room.push_back(size);
+      first[hd] = (int)x * size + size - room[x];
+      room[x] -= np[hd];
+    }
+    if ((int)room.size() > c->cluster_room[k]) continue;
+    lw.cluster = size;
+    items.resize(lw.first_item + room.size() * size, WorkItem{0, -1, 0, 0, seq_ids[0], ROLE_ANCHOR, 0, 0, 0, 0, 0, 0, 0});
+    for (int hd = 0; hd < n_heads; ++hd) {
+      const int i = hd / G.Hkv, h = hd % G.Hkv, n = n_gran[hd];
+      const SeqHost &sq = c->seqs[seq_ids[i]];
+      const int role = mode == ATTN_DECODE ? c->roles[layer * G.Hkv + h] : ROLE_ANCHOR;
+      const int ridx = mode == ATTN_DECODE ? c->role_idx[layer * G.Hkv + h] : h;
+      const int perm = (G.token_base && role == ROLE_TIDAL && !sq.fixed_blocks.empty()) ? std::max(sq.fixed_blocks[layer * G.Hkv + h], 0)
+                                                                                       : sq.S_base;
+      for (int x = 0; x < np[hd]; ++x)
+        items[lw.first_item + first[hd] + x] =
+            WorkItem{i, h, (int)((long long)n * x / np[hd]), (int)((long long)n * (x + 1) / np[hd]), seq_ids[i], role, ridx,
+                     role == ROLE_FIXED ? sq.T_a_fixed : sq.T_a, sq.C, perm, sq.T_t, first[hd], np[hd]};
+      heads.push_back(HeadItems{first[hd], np[hd]});
+      lw.max_count = std::max(lw.max_count, np[hd]);
+    }
+    lw.n_items = (int)(room.size() * size);
+    lw.n_ctas = 0; lw.packed = false; lw.throughput = false;
+    return true;
+  }
+  return false;
+}
+
 // Appends the items of one layer for the given sequences.
 static void build_layer_items(const wnw_cache *c, int layer, int mode, const std::vector<int> &seq_ids,
                               std::vector<WorkItem> &items, std::vector<HeadItems> &heads, LayerWork &lw,
@@ -830,6 +888,7 @@ static void build_layer_items(const wnw_cache *c, int layer, int mode, const std
   lw.first_item = (int)items.size();
   lw.head_items_off = (int)heads.size();
   lw.max_count = 0;
+  if (!overlapped && build_cluster_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw)) return;
   if (throughput) {
     build_throughput_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw, order, ranges, memo);
     return;
@@ -1646,7 +1705,7 @@ static wnw_status_t decode_layer_impl(wnw_cache *c, int want_mode, int32_t layer
   a.mode = tiered ? ATTN_DECODE : ATTN_FULL; a.layer = layer; a.li = li; a.n_active = n_active; a.has_new = has_new;
   a.score_on = tiered && li.n_anchor > 0;
   a.active = c->d_active; a.items = c->d_items + lw.first_item; a.items_host = c->h_items.data() + lw.first_item;
-  a.n_items = lw.n_items; a.maps = &c->maps_decode; a.throughput = lw.throughput;
+  a.n_items = lw.n_items; a.maps = &c->maps_decode; a.throughput = lw.throughput; a.cluster = lw.cluster;
   if (lw.n_ctas > 0) {
     a.order = c->d_sched + lw.order_off; a.cta_ranges = c->d_sched + c->sched_ranges_base + lw.ranges_off; a.n_ctas = lw.n_ctas;
     a.xpref = lw.packed;
