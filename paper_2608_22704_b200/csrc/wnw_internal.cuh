@@ -159,8 +159,7 @@ __host__ __device__ inline size_t select_ws_bytes(int C, int S) {
 // ---- attention launch ----
 enum { ATTN_DECODE = 0, ATTN_FULL = 1, ATTN_PREFILL = 2 };
 
-// TMA descriptors of the K/V stores, each viewed as a 2-D bf16 tensor [rows][d] with 16 x 64-element boxes and the
-// 128-byte swizzle.  `anchor` is whichever store plays the contiguous full-audio role in the launch.
+// TMA descriptors of the K/V stores; a box is a granule, K and V (encode_store_map).  `anchor` is whichever store plays the contiguous full-audio role in the launch.
 struct TmaMaps { CUtensorMap text, anchor, pool, fixed; };
 
 struct AttnArgs {
@@ -296,10 +295,11 @@ cudaError_t configure_attn_kernels();
 // what precedes it in the stream
 cudaError_t launch_attn_multi(const CacheView &cv, const AttnArgs *args, int n, const int *first, const int *count, bool pdl,
                               cudaStream_t st);
-// Encodes the descriptor of one store: base (device), rows, head_dim.  Returns false if the driver refuses.
-bool encode_store_map(CUtensorMap *map, const void *base, unsigned long long rows, int d);
-// the slot pool as e4m3: rows of 128 bytes, boxes of 16 rows, 128-byte swizzle
-bool encode_store_map_e4m3(CUtensorMap *map, const void *base, unsigned long long rows);
+// Encodes the descriptor of one store: base (device), rows, head_dim, rows from a K row to its V row, 2 for K and V / 1 for K
+// alone in a box.  Returns false if the driver refuses.
+bool encode_store_map(CUtensorMap *map, const void *base, unsigned long long rows, int d, long long v_rows, int kv);
+// the slot pool as e4m3: rows of 128 bytes
+bool encode_store_map_e4m3(CUtensorMap *map, const void *base, unsigned long long rows, long long v_rows);
 // e4m3 tidal tier, at placement: per (chunk, tidal head, K|V) the scale exponent from the staged rows, which are then
 // replaced by the values their bytes decode to
 cudaError_t launch_quantise_stage(const CacheView &cv, int b, int layer, bf16 *stage, int C_b, cudaStream_t st);

@@ -509,13 +509,15 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
                              r_pool = B * (unsigned long long)G.pool_seq_stride / d, r_fixed = B * (unsigned long long)G.fixed_seq_stride / d,
                              r_stage = (unsigned long long)Hkv * 2 * G.T_a_pad;
     if (std::max({r_text, r_anchor, r_pool, r_fixed}) >= (1ull << 31)) return fail(WNW_ERR_UNSUPPORTED);  // rows are 32-bit TMA coordinates
-    bool ok = encode_store_map(&c->maps_decode.text, cv.text, r_text, d);
-    ok = ok && encode_store_map(&c->maps_decode.anchor, cv.anchor, r_anchor, d);
-    if (G.kv8 && r_pool) ok = ok && encode_store_map_e4m3(&c->maps_decode.pool, cv.pool, r_pool);
-    else ok = ok && encode_store_map(&c->maps_decode.pool, r_pool ? (void *)cv.pool : (void *)cv.text, r_pool ? r_pool : r_text, d);
-    ok = ok && encode_store_map(&c->maps_decode.fixed, r_fixed ? (void *)cv.fixed : (void *)cv.text, r_fixed ? r_fixed : r_text, d);
-    c->maps_prefill = c->maps_decode;
-    if (!full) ok = ok && encode_store_map(&c->maps_prefill.anchor, c->stage, r_stage, d);
+    // a store that the cache does not have is never read: its descriptor stands on the text store
+    auto store = [&](CUtensorMap *m, const void *base, unsigned long long rows, long long v_rows, int kv) {
+      return rows ? encode_store_map(m, base, rows, d, v_rows, kv) : encode_store_map(m, cv.text, r_text, d, G.T_cap_pad, kv);
+    };
+    bool ok = store(&c->maps_decode.text, cv.text, r_text, G.T_cap_pad, 2) && store(&c->maps_decode.anchor, cv.anchor, r_anchor, G.T_a_pad, 2) &&
+              store(&c->maps_decode.fixed, cv.fixed, r_fixed, (long long)G.FB * G.ncp, 2);
+    ok = ok && (G.kv8 && r_pool ? encode_store_map_e4m3(&c->maps_decode.pool, cv.pool, r_pool, G.ncp) : store(&c->maps_decode.pool, cv.pool, r_pool, G.ncp, 2));
+    c->maps_prefill = c->maps_decode;   // the scoring pass reads K alone, the staging copy as the anchor store
+    ok = ok && store(&c->maps_prefill.text, cv.text, r_text, G.T_cap_pad, 1) && (full || store(&c->maps_prefill.anchor, c->stage, r_stage, G.T_a_pad, 1));
     if (!ok) return fail(WNW_ERR_CUDA);
   }
   {

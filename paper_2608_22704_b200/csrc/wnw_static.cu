@@ -121,7 +121,7 @@ extern "C" wnw_status_t wnw_attend_static(const void *kv_dev, int32_t n_tokens, 
 
   // descriptor of the caller's buffer (a host-side encode, no allocation); every role points at it
   TmaMaps maps;
-  if (!encode_store_map(&maps.anchor, kv_dev, (unsigned long long)n_kv_heads * 2 * padded_tokens, head_dim)) return WNW_ERR_CUDA;
+  if (!encode_store_map(&maps.anchor, kv_dev, (unsigned long long)n_kv_heads * 2 * padded_tokens, head_dim, padded_tokens, 2)) return WNW_ERR_CUDA;
   maps.text = maps.pool = maps.fixed = maps.anchor;
   AttnArgs a{};
   a.maps = &maps;
