@@ -162,6 +162,16 @@ __device__ __forceinline__ float ex2(float x) {
   return r;
 }
 
+// The first product of a chain: the accumulator starts at zero
+__device__ __forceinline__ void mma16816_z(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};\n"
+               : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+// (x, y) *= (a, b) in one instruction
+__device__ __forceinline__ void mul2(float &x, float &y, float a, float b) {
+  asm("{\n .reg .b64 p, q;\n mov.b64 p, {%0, %1};\n mov.b64 q, {%2, %3};\n mul.rn.f32x2 p, p, q;\n mov.b64 {%0, %1}, p;\n}\n" : "+f"(x), "+f"(y) : "f"(a), "f"(b));
+}
+
 // Two e4m3 bytes (low 16 bits of x) as two fp16 numbers: one instruction, exact (every e4m3 value is an fp16 value).
 __device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t x) {
   uint32_t h;
@@ -188,7 +198,9 @@ struct GranDesc {
   int off;         // token offset of the granule inside its chunk
   int score_idx;   // audio granule index for score partials, -1 = none
   int ex;          // e4m3 tidal tier: K scale exponent | V scale exponent << 8 | 1 << 16 for a slot granule (filled with the metadata)
-  bool loaded;     // a copy has been queued
+  bool loaded;     // a copy has been (or will be) queued
+  uint32_t word;   // the granule's ring entry, once its metadata is resolved
+  const CUtensorMap *map;
   int vis;         // visible rows, resolved with the first metadata of the descriptor's block of 32 granules
 };
 
@@ -199,7 +211,7 @@ __device__ __forceinline__ GranDesc decode_granule(const CacheView &cv, const At
                                                    const WorkItem &it, int j, int table_parity) {
   const Geometry &G = cv.geo;
   GranDesc r;
-  r.cid = -1; r.off = 0; r.score_idx = -1; r.ex = 0; r.vis = 0; r.loaded = false;
+  r.cid = -1; r.off = 0; r.score_idx = -1; r.ex = 0; r.vis = 0; r.loaded = false; r.word = 0; r.map = nullptr;
   if (j < G.n_tg) {
     const int tok0 = j * GR;
     r.row = (int)(text_off(G, it.b, a.layer, it.h, 0) / D) + tok0;
@@ -294,7 +306,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   constexpr int QROW = D * 2 + 16;                            // a query row, padded: ldmatrix reads eight of them without conflicts
   __shared__ __align__(16) unsigned char cl_q[CL ? (G16 ? 16 : 8) * QROW : 16];
   if (VAR == 3) asm volatile("griddepcontrol.wait;\n" ::: "memory");   // the caller's buffer may be what the preceding work wrote
-  const uint32_t my_base = smem_u32(smem + (size_t)warp * NSTAGE * STAGEB);
+  const uint32_t my_base = smem_u32(smem + (size_t)warp * NSTAGE * STAGEB), bar0 = smem_u32(&bars[warp][0]);
   if (lane == 0) {
 #pragma unroll
     for (int st = 0; st < NSTAGE; ++st) mbar_init(smem_u32(&bars[warp][st]), 1);
@@ -390,9 +402,9 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   Ctx prod;
   prod.n_my = 0;   // loaded by the first work item before anything is produced
   int p_n = 0;
-  uint32_t seq_p = 0, seq_c = 0;
+  uint32_t seq_p = 0, seq_c = 0, st_p = 0;   // st_p: seq_p % NSTAGE
   GranDesc blk;  // descriptor this lane decoded for the producer's current block of 32 granules
-  blk.row = 0; blk.meta = 0; blk.cid = -1; blk.off = 0; blk.score_idx = -1; blk.ex = 0; blk.vis = 0; blk.loaded = false;
+  blk.row = 0; blk.meta = 0; blk.cid = -1; blk.off = 0; blk.score_idx = -1; blk.ex = 0; blk.vis = 0; blk.loaded = false; blk.word = 0; blk.map = nullptr;
 
   // Visible rows of a granule once its metadata has arrived.
   auto visible = [&](const Ctx &c, int meta, int cid, int off, int j) -> int {
@@ -411,6 +423,13 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       len -= off;
     }
     return len <= 0 ? 0 : (len < GR ? len : GR);
+  };
+  // By the lane that holds the descriptor.  f8g: an e4m3 granule, half the bytes.
+  auto queue_copy = [&](uint32_t stage, bool f8g) {
+    const uint32_t bar = bar0 + stage * 8;
+    fence_proxy_async();  // the stage was last read through the generic proxy (ldmatrix)
+    mbar_expect_tx(bar, f8g ? 2 * HALFB : STAGEB);
+    tma_load_granule(my_base + stage * STAGEB, blk.map, blk.row, bar);
   };
   // Queues the copies of granules n .. n + k - 1 of item c (one box each: K and V, all 16 rows) into the stages of the
   // sequence numbers from seq on; the granules lie in one block of 32, and the lane that holds a granule's descriptor queues
@@ -436,13 +455,8 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       if (blk.meta == -1) load = visible(c, -1, 0, 0, j) > 0;   // waits for the text length
       if (blk.meta == -3) load = blk.cid >= 0;                  // waits for the table entry
       blk.loaded = load;
-      if (load) {
-        const uint32_t stage = (seq + o) % NSTAGE, bar = smem_u32(&bars[warp][stage]);
-        const bool f8g = F8 && !is_text && c.it.role == ROLE_TIDAL;   // an e4m3 granule: half the bytes
-        fence_proxy_async();  // the stage was last read through the generic proxy (ldmatrix)
-        mbar_expect_tx(bar, f8g ? 2 * HALFB : STAGEB);
-        tma_load_granule(my_base + stage * STAGEB, is_text ? &maps.text : (base_blk ? &maps.fixed : c.map_audio), blk.row, bar);
-      }
+      blk.map = is_text ? &maps.text : (base_blk ? &maps.fixed : c.map_audio);
+      if (load) queue_copy((seq + o) % NSTAGE, F8 && !is_text && c.it.role == ROLE_TIDAL);
     }
   };
   // Publishes (visible rows, loaded, score index) of the same granules for the compute step; may wait for the metadata loads.
@@ -458,14 +472,35 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       }
     }
     const int o = lane - (n & 31);
-    // x: visible rows | copy queued << 8 | e4m3 granule << 9 | K exponent << 16 | V exponent << 24
-    if (o >= 0 && o < k)
-      ring[warp][(seq + o) % NSTAGE] = make_int2(blk.vis | (blk.loaded ? 256 : 0) | ((blk.ex >> 16) << 9) | (int)(((unsigned)blk.ex & 0xffffu) << 16), blk.score_idx);
+    if (o >= 0 && o < k) {
+      // visible rows | copy queued << 8 | e4m3 granule << 9 | K exponent << 16 | V exponent << 24
+      blk.word = (uint32_t)blk.vis | (blk.loaded ? 256u : 0u) | (uint32_t)((blk.ex >> 16) << 9) | (((uint32_t)blk.ex & 0xffffu) << 16);
+      ring[warp][(seq + o) % NSTAGE] = make_int2((int)blk.word, blk.score_idx);
+    }
   };
   // Fetches the producer's next `want` granules, moving on to the CTA's next work item when this warp has none left in the
   // current one (only when the pipeline runs across items).
   int p_qi = q_begin;
   auto produce = [&](int want) {
+    // The common case, a pair of granules inside a resolved block: everything is in the owner lanes' registers.
+    const int o = lane - (p_n & 31);
+    if (want == 2 && p_n + 2 <= prod.n_my && (p_n & 31) != 0 && (p_n & 31) != 31 && !epoch_pending) {
+      if ((unsigned)o < 2u) {
+        const int j = prod.first + (p_n + o) * NW;
+        const bool is_text = j < G.n_tg, base_blk = TB && blk.score_idx == -2;
+        blk.map = is_text ? &maps.text : (base_blk ? &maps.fixed : prod.map_audio);
+        blk.loaded = blk.meta == -3 ? blk.cid >= 0 : blk.meta == -1 ? blk.vis > 0 : blk.meta != 0;
+        uint32_t stage = st_p + (uint32_t)o;
+        if (stage >= NSTAGE) stage -= NSTAGE;
+        if (blk.loaded) queue_copy(stage, F8 && !is_text && prod.it.role == ROLE_TIDAL);
+        blk.word = (uint32_t)blk.vis | (blk.loaded ? 256u : 0u) | (uint32_t)((blk.ex >> 16) << 9) | (((uint32_t)blk.ex & 0xffffu) << 16);
+        ring[warp][stage] = make_int2((int)blk.word, blk.score_idx);
+      }
+      p_n += 2; seq_p += 2;
+      st_p += 2;
+      if (st_p >= NSTAGE) st_p -= NSTAGE;
+      return;
+    }
     while (want > 0) {
       while (p_n >= prod.n_my) {
         if (!xpref || p_qi + 1 >= q_end) return;
@@ -477,6 +512,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
       issue_copy(prod, p_n, k, seq_p);
       issue_meta(prod, p_n, k, seq_p);
       p_n += k; seq_p += k; want -= k;
+      st_p = seq_p % NSTAGE;
     }
   };
 
@@ -538,7 +574,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
               asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};\n" ::"r"(sVz + hf * HALFB + r * 128 + ((lane & 7) << 4)), "r"(0u) : "memory");
         }
       }
-    p_n = n_pro; seq_p += n_pro;
+    p_n = n_pro; seq_p += n_pro; st_p = seq_p % NSTAGE;
     // the consumer takes two granules at a time and counts on the producer being a full ring ahead: an item shorter than
     // the pipeline is topped up from the items that follow, here as on the ordinary path
     if (xpref) produce(NSTAGE - n_pro);
@@ -553,6 +589,21 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   auto collect = [&](int n) {
     cnt = n + 1 < n_my ? 2 : 1;
     nu = 0; adv = 0; u_new = -1;
+    if constexpr (!CL && !F8) {   // the common case: two granules, all rows visible, neither takes the new row
+      const uint32_t sa = seq_c % NSTAGE, sb = sa + 1 == NSTAGE ? 0 : sa + 1;
+      const int2 ra = ring[warp][sa], rb = ring[warp][sb];
+      const int j0 = first + n * NW;
+      if (cnt == 2 && (ra.x & rb.x & 511) == 256 + GR && ((ra.x | rb.x) & 255) == GR && !prewaited && j0 != new_j && j0 + NW != new_j) {
+        if (mbar_wait(bar0 + sa * 8, (phase_bits >> sa) & 1u)) { phase_bits ^= 1u << sa; adv = 1; }
+        if (adv == 1 && mbar_wait(bar0 + sb * 8, (phase_bits >> sb) & 1u)) { phase_bits ^= 1u << sb; adv = 2; }
+        if (adv < 2) timed_out = true;
+        sKs[0] = my_base + sa * STAGEB; sKs[1] = my_base + sb * STAGEB;
+        sVs[0] = sKs[0] + TILEB; sVs[1] = sKs[1] + TILEB;
+        valids[0] = valids[1] = GR; sidxs[0] = ra.y; sidxs[1] = rb.y;
+        nu = 2;
+        return;
+      }
+    }
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       if (u < cnt && n < n_my && !timed_out) {
@@ -700,7 +751,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   if (arm && !early) {
     if (n_pro > 0) issue_meta(prod, 0, n_pro, seq_p);
     STAMP(23);
-    p_n = n_pro; seq_p += n_pro;
+    p_n = n_pro; seq_p += n_pro; st_p = seq_p % NSTAGE;
     if (xpref) produce(NSTAGE - n_pro);   // an item shorter than the pipeline: top up from the items that follow
   }
 
@@ -743,12 +794,14 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
     }
     {
       float sO[NU][NTN][4];   // odd k-steps: shorter dependent mma chains
+      if constexpr (F8) {
 #pragma unroll
-      for (int u = 0; u < NU; ++u)
+        for (int u = 0; u < NU; ++u)
 #pragma unroll
-        for (int nt = 0; nt < NTN; ++nt)
+          for (int nt = 0; nt < NTN; ++nt)
 #pragma unroll
-          for (int e = 0; e < 4; ++e) sT[u][nt][e] = sO[u][nt][e] = 0.f;
+            for (int e = 0; e < 4; ++e) sT[u][nt][e] = sO[u][nt][e] = 0.f;
+      }
       const int mtx = lane >> 3;
       // A lane's ldmatrix row address inside a 16 x 128-byte box with the 128-byte swizzle: row * 128 + ((piece ^ row % 8) << 4),
       // piece = 2 * kk + (0 or 1 by lane).  The lane's part, row * 128 + (((0 or 1) ^ row % 8) << 4), is a constant of the
@@ -758,8 +811,10 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
         uint32_t bk[4];   // K rows 0-7 | 8-15 of the granule x d 0-7 | 8-15 of the k-step: the A operand's four quadrants
         ldsm_x4(bk, ((sKs[u] + lane_k) ^ (uint32_t)(((2 * kk) & 7) << 4)) + (kk >> 2) * HALFB);
 #pragma unroll
-        for (int nt = 0; nt < NTN; ++nt)
-          mma16816((kk & 1) ? sO[u][nt] : sT[u][nt], bk[0], bk[2], bk[1], bk[3], qa[kk][2 * nt], qa[kk][2 * nt + 1]);
+        for (int nt = 0; nt < NTN; ++nt) {
+          if (kk < 2) mma16816_z((kk & 1) ? sO[u][nt] : sT[u][nt], bk[0], bk[2], bk[1], bk[3], qa[kk][2 * nt], qa[kk][2 * nt + 1]);
+          else mma16816((kk & 1) ? sO[u][nt] : sT[u][nt], bk[0], bk[2], bk[1], bk[3], qa[kk][2 * nt], qa[kk][2 * nt + 1]);
+        }
       };
       if constexpr (!F8) {
 #pragma unroll
@@ -853,8 +908,10 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
         asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(pb[u][nt][1]) : "r"(p23));
       }
       lrun[nt][0] = lrun[nt][0] * alA + addA; lrun[nt][1] = lrun[nt][1] * alB + addB;
+      if (__any_sync(0xffffffffu, alA != 1.f || alB != 1.f)) {   // rarely, once the head's largest logit has been seen
 #pragma unroll
-      for (int t = 0; t < D / 16; ++t) { oT[nt][t][0] *= alA; oT[nt][t][1] *= alB; oT[nt][t][2] *= alA; oT[nt][t][3] *= alB; }
+        for (int t = 0; t < D / 16; ++t) { mul2(oT[nt][t][0], oT[nt][t][1], alA, alB); mul2(oT[nt][t][2], oT[nt][t][3], alA, alB); }
+      }
     }
     STAMP(26);
     if constexpr (!KO) {
@@ -1381,6 +1438,24 @@ static int cluster_room_t(int g, int cluster) {
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, wnw_attn_cluster_kernel<D, G16, 0>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
   return n;
+}
+template <int D, bool G16, int VAR>
+static bool recall_room_t(int g, bool cluster) {
+  cudaFuncAttributes at;
+  if ((cluster ? cudaFuncGetAttributes(&at, wnw_attn_cluster_kernel<D, G16, VAR>) : cudaFuncGetAttributes(&at, wnw_attn_kernel<D, G16, NW_THR, VAR>)) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  const int threads = cluster ? NW_LAT * 32 : attn_persistent_ctas_per_sm(g, D) * NW_THR * 32;
+  return 65536 - threads * ((at.numRegs + 7) / 8 * 8) >= RECALL_REGS;
+}
+bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, bool cluster) {
+  if (d == 128) {
+    if (g > 8) return kv8 ? recall_room_t<128, true, 2>(g, cluster) : token_base ? recall_room_t<128, true, 1>(g, cluster) : recall_room_t<128, true, 0>(g, cluster);
+    return kv8 ? recall_room_t<128, false, 2>(g, cluster) : token_base ? recall_room_t<128, false, 1>(g, cluster) : recall_room_t<128, false, 0>(g, cluster);
+  }
+  if (g > 8) return token_base ? recall_room_t<64, true, 1>(g, cluster) : recall_room_t<64, true, 0>(g, cluster);
+  return token_base ? recall_room_t<64, false, 1>(g, cluster) : recall_room_t<64, false, 0>(g, cluster);
 }
 int attn_cluster_room(int g, int d, int cluster) {
   if (d == 128) return g > 8 ? cluster_room_t<128, true>(g, cluster) : cluster_room_t<128, false>(g, cluster);
