@@ -92,10 +92,10 @@ __device__ __forceinline__ void select_body(const CacheView &cv, const SelectArg
     __threadfence();
     for (int j = threadIdx.x; j < a.n_active; j += NT) {
       const int bj = a.active[j];
-      cv.steps[bj] += 1;
-      if (a.fold_appended) cv.text_len[bj] += 1;
+      atomicAdd(reinterpret_cast<unsigned long long *>(cv.steps + bj), 1ull);   // (reductions: nothing is waited for)
+      if (a.fold_appended) atomicAdd(cv.text_len + bj, 1);
     }
-    if (threadIdx.x == 0 && a.fold_bump_epoch) *a.fold_bump_epoch += 1;
+    if (threadIdx.x == 0 && a.fold_bump_epoch) atomicAdd(a.fold_bump_epoch, 1);
   };
   if (em_room < 0 || (scored && tile_c < 1)) {  // beyond what the host sized the launch for
     if (threadIdx.x == 0) atomicOr(cv.status, STATUS_BAD_TABLE);
@@ -141,15 +141,21 @@ __device__ __forceinline__ void select_body(const CacheView &cv, const SelectArg
         cp_async_commit_wait_all();
         __syncthreads();
       }
+      // a thread per (query head, chunk): its share, left in the place of the chunk's first partial; then a thread per chunk adds
+      // the heads up in order
+      const int n_c = c1 - c0;
+      for (int x = threadIdx.x; x < n_aq * n_c; x += NT) {
+        const int aq = x / n_c;
+        const float2 mz = mz_s[aq];
+        float2 *p = em_s + (size_t)aq * span + (size_t)(x - aq * n_c) * G.gpc;
+        float sum_h = 0.f;
+        for (int gi = 0; gi < G.gpc; ++gi) sum_h += p[gi].x * exp2f(p[gi].y - mz.x);
+        p[0].x = mz.y > 0.f ? sum_h / mz.y : 0.f;
+      }
+      __syncthreads();
       for (int c = c0 + threadIdx.x; c < c1; c += NT) {
         float total = 0.f;
-        for (int aq = 0; aq < n_aq; ++aq) {
-          const float2 mz = mz_s[aq];
-          const float2 *p = em_s + (size_t)aq * span + (size_t)(c - c0) * G.gpc;
-          float sum_h = 0.f;
-          for (int gi = 0; gi < G.gpc; ++gi) sum_h += p[gi].x * exp2f(p[gi].y - mz.x);
-          total += mz.y > 0.f ? sum_h / mz.y : 0.f;
-        }
+        for (int aq = 0; aq < n_aq; ++aq) total += em_s[(size_t)aq * span + (size_t)(c - c0) * G.gpc].x;
         if (!(total >= 0.f) || isinf(total)) atomicOr(cv.status, STATUS_NONFINITE);
         dst[c] = total;
         sc_s[c] = total;
@@ -323,7 +329,7 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // a few CTAs of 8 warps with RECALL_U 16-byte loads in flight per lane, whatever there is to copy, and the warps work
 // independently: the blocks of a launch are cut into pieces of a warp's batch and dealt round robin ACROSS block and layer
 // borders, so that all warps have work and nothing waits at a barrier.
-// At most 48 registers a thread: a CTA fits beside a resident 8-warp attention CTA (208 registers).
+// 40 registers a thread: a CTA fits beside a resident 8-warp attention CTA, or two of four warps, of up to 216 registers.
 // 8 CTAs where layers wait for one another: the copies have the whole next step's time (config 1, 30 chained layers, recall
 // and the step's own small copies: 254 us a step with the former 128 CTAs, 238.7 with 8, 241 with 12, 243 with 16).  24 CTAs
 // where layers overlap: attention then fills the memory system, a host read takes several times as long and the step waits for
@@ -333,7 +339,7 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // warp that finishes a layer last publishes the layer's recall epoch, which the next step's tidal CTAs acquire.
 // ------------------------------------------------------------------------------------------------
 constexpr int RECALL_CTAS = 8, RECALL_CTAS_CROWDED = 24, RECALL_WARPS = 8, RECALL_U = 4;
-__global__ void __launch_bounds__(RECALL_WARPS * 32, 5) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
+__global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
                                                                           const int32_t *active, const int32_t *layers,
                                                                           int n_layers, int skip_copy, RecallSignal sig) {
   const Geometry &G = cv.geo;
