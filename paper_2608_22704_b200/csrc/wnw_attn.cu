@@ -589,7 +589,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   auto collect = [&](int n) {
     cnt = n + 1 < n_my ? 2 : 1;
     nu = 0; adv = 0; u_new = -1;
-    if constexpr (!CL && !F8) {   // the common case: two granules, all rows visible, neither takes the new row
+    if constexpr (!CL) {   // the common case: two granules, all rows visible, neither takes the new row
       const uint32_t sa = seq_c % NSTAGE, sb = sa + 1 == NSTAGE ? 0 : sa + 1;
       const int2 ra = ring[warp][sa], rb = ring[warp][sb];
       const int j0 = first + n * NW;
@@ -598,7 +598,8 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
         if (adv == 1 && mbar_wait(bar0 + sb * 8, (phase_bits >> sb) & 1u)) { phase_bits ^= 1u << sb; adv = 2; }
         if (adv < 2) timed_out = true;
         sKs[0] = my_base + sa * STAGEB; sKs[1] = my_base + sb * STAGEB;
-        sVs[0] = sKs[0] + TILEB; sVs[1] = sKs[1] + TILEB;
+        sVs[0] = sKs[0] + (F8 && (ra.x & 512) ? HALFB : TILEB); sVs[1] = sKs[1] + (F8 && (rb.x & 512) ? HALFB : TILEB);
+        fmt[0] = ra.x >> 9; fmt[1] = rb.x >> 9;
         valids[0] = valids[1] = GR; sidxs[0] = ra.y; sidxs[1] = rb.y;
         nu = 2;
         return;
@@ -1004,7 +1005,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
     // finishes (and its (max, denominator) pairs) straight into the other's shared memory (st.async, completion counted in
     // bytes by the receiver's mbarrier), and each finishes its share: no partials in global memory, no fence, no counter, no
     // last CTA that reads all partials back.  From the end of the last product to the output, config 1 (14 and 4 pieces):
-    // CL_BEFORE -> CL_AFTER us; a chained layer 7.1 -> CL_LAYER us.
+    // 3.4 -> 1.5 us; a chained layer 7.3 -> 4.2 us.
     //
     // The accumulators travel as units of four values as they sit in a lane: heads 2p and 2p + 1 at d = 16 t + r and 16 t + r + 8.
     // Unit u = p * D / 2 + 8 t + r; piece u % np finishes it, in place u / np of its receive buffer.
@@ -1300,13 +1301,13 @@ __global__ void __launch_bounds__(NW * 32, NW == NW_THR ? (G16 ? 2 : WNW_THR_CTA
   attn_body<D, G16, NW, VAR>(cv, a, &inl, maps, (int)blockIdx.x);
 }
 
-// Chained or serial layers of one wave: the pieces of a head in one cluster.
+// Chained or serial layers of one wave: the pieces of a head in one cluster.  (Items come from memory, ahead of the inputs: 5 KB less of
+// parameters for the host to copy on every launch.)
 template <int D, bool G16, int VAR>
 __global__ void __launch_bounds__(NW_LAT * 32, 1) wnw_attn_cluster_kernel(const __grid_constant__ CacheView cv,
                                                                          const __grid_constant__ AttnArgs a,
-                                                                         const __grid_constant__ InlineItems inl,
                                                                          const __grid_constant__ TmaMaps maps) {
-  attn_body<D, G16, NW_LAT, VAR, true>(cv, a, &inl, maps, (int)blockIdx.x);
+  attn_body<D, G16, NW_LAT, VAR, true>(cv, a, nullptr, maps, (int)blockIdx.x);
 }
 
 // All heads cut alike (VAR 3, 4): the item list is in the launch shape.
@@ -1415,12 +1416,10 @@ static void cluster_attrs(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2
 template <int D, bool G16, int VAR>
 static cudaError_t launch_cluster_t(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
   if (!a.maps || a.n_items % a.cluster) return cudaErrorInvalidValue;
-  InlineItems inl;
-  if (a.n_items <= INLINE_ITEMS_MAX) memcpy(inl.it, a.items_host, sizeof(WorkItem) * a.n_items);
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[2];
   cluster_attrs(cfg, attr, cv.geo.g, D, a.n_items, a.cluster, a.pdl, st);
-  return cudaLaunchKernelEx(&cfg, wnw_attn_cluster_kernel<D, G16, VAR>, cv, a, inl, *a.maps);
+  return cudaLaunchKernelEx(&cfg, wnw_attn_cluster_kernel<D, G16, VAR>, cv, a, *a.maps);
 }
 template <int D, bool G16>
 static cudaError_t launch_cluster(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
@@ -1567,7 +1566,7 @@ cudaError_t launch_attn(const CacheView &cv, const AttnArgs &a, cudaStream_t st)
   if (a.cluster) {
     if (cv.geo.d == 128) return g16 ? launch_cluster<128, true>(cv, a, st) : launch_cluster<128, false>(cv, a, st);
     if (cv.geo.d == 64) return g16 ? launch_cluster<64, true>(cv, a, st) : launch_cluster<64, false>(cv, a, st);
-  } else if (a.throughput) {
+  } else if (a.throughput || a.narrow) {
     if (cv.geo.d == 128) return g16 ? launch_t<128, true, NW_THR>(cv, a, st) : launch_t<128, false, NW_THR>(cv, a, st);
     if (cv.geo.d == 64) return g16 ? launch_t<64, true, NW_THR>(cv, a, st) : launch_t<64, false, NW_THR>(cv, a, st);
   } else {

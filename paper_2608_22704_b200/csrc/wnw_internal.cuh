@@ -180,6 +180,7 @@ struct AttnArgs {
   int32_t throughput;            // items were cut for the 4-warp, 2-CTAs-per-SM variant (more than one wave of work)
   const int32_t *wait_epoch;     // replayed steps: tidal CTAs wait until *wait_epoch >= *expect_epoch (this layer's recall of the
   const int32_t *expect_epoch;   //   previous step, which runs outside the captured graph, has landed); null otherwise
+  int32_t narrow;                // one-shot CTAs of four warps, two per SM, instead of eight
   int32_t cluster;               // > 0: CTAs in clusters of this size, item x is CTA x, all items of a head in one cluster
   int32_t pdl;                   // launch with programmatic stream serialization (previous stream op is a layer kernel)
   int xpref;        // the CTAs serve several work items each and keep their copy pipeline running across them
@@ -308,7 +309,7 @@ constexpr int SELECT_SMEM_CAP = 200 * 1024;  // dynamic shared memory the select
 bool attn_xpref_fits(int g, int d);  // a one-shot CTA can hold its merge scratch behind the copy stages
 // whether an SM that holds all the persistent attention CTAs (or the cluster kernel's CTA) it can take has registers left for a recall CTA
 bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, bool cluster);
-constexpr int RECALL_REGS = 256 * 48;       // registers of a recall CTA
+constexpr int RECALL_REGS = 256 * 40;       // registers of a recall CTA
 int attn_cluster_room(int g, int d, int cluster);   // clusters of that size that fit the GPU at once
 int attn_warps(bool throughput);  // warps per attention CTA in the latency / throughput variant
 int attn_persistent_ctas_per_sm(int g, int d);  // persistent (throughput-variant) CTAs that fit one SM

@@ -36,6 +36,7 @@ struct LayerWork {
   int n_ctas = 0, order_off = 0, ranges_off = 0;   // items per CTA (persistent schedule, or packed short heads): offsets
   int n_ctas_free = 0;   // BATCHED layers: the first n_ctas_free CTAs hold no tidal head (they need no recall epoch) ...
   int n_ctas_anchor = 0; // ... and the first n_ctas_anchor of those hold the anchor heads (what the step's selection waits for)
+  bool narrow = false;                             // one-shot CTAs of four warps, two per SM
   int cluster = 0;                                 // chained layers of one wave: CTAs per cluster
   bool packed = false;                             // one-shot CTAs that serve several short heads each
   int head_items_off = 0;                          // offset in the list's HeadItems
@@ -943,6 +944,10 @@ static void build_layer_items(const wnw_cache *c, int layer, int mode, const std
   lw.n_items = (int)items.size() - lw.first_item;
   lw.n_ctas = 0;
   lw.packed = false;
+  // Unpacked one-shot CTAs of overlapping layers: four warps, two CTAs to an SM, so that one streams while the other starts or
+  // merges (4 x 3000 tokens, 30 layers: 165 -> 150 us a step, full cache 277 -> 265, two sequences 114 -> 105, one of 15000
+  // tokens 121 -> 116); a single short sequence keeps eight warps (94 against 96 us: there the span of a head's CTA counts).
+  lw.narrow = overlapped && !batched && lw.n_items <= c->n_sm && (seq_ids.size() > 1 || longest > 4 * c->direct_max_granules);
   if (big_single_wave && lw.n_items <= c->n_sm) {   // see above: the persistent two-per-SM cut instead
     items.resize(lw.first_item);
     heads.resize(lw.head_items_off);
@@ -1737,7 +1742,7 @@ static wnw_status_t decode_layer_impl(wnw_cache *c, int want_mode, int32_t layer
   a.mode = tiered ? ATTN_DECODE : ATTN_FULL; a.layer = layer; a.li = li; a.n_active = n_active; a.has_new = has_new;
   a.score_on = tiered && li.n_anchor > 0;
   a.active = c->d_active; a.items = c->d_items + lw.first_item; a.items_host = c->h_items.data() + lw.first_item;
-  a.n_items = lw.n_items; a.maps = &c->maps_decode; a.throughput = lw.throughput; a.cluster = lw.cluster;
+  a.n_items = lw.n_items; a.maps = &c->maps_decode; a.throughput = lw.throughput; a.cluster = lw.cluster; a.narrow = lw.narrow;
   if (lw.n_ctas > 0) {
     a.order = c->d_sched + lw.order_off; a.cta_ranges = c->d_sched + c->sched_ranges_base + lw.ranges_off; a.n_ctas = lw.n_ctas;
     a.xpref = lw.packed;
