@@ -236,8 +236,8 @@ wnw_status_t wnw_get_fixed_tokens(wnw_cache_t *cache, int32_t seq, int32_t layer
  *   fixed heads   keep the subset chosen at placement, which is final: they never see a position that arrived later,
  *                 not even inside a chunk they keep.
  * Layers must be given in order 0..n_layers-1, all with the same n_tokens, outside a step; the grown clip is in force
- * once the last layer has been appended (wnw_step_begin is refused in between).  The first layer's call waits for all
- * queued work of the cache.  Work lists are rebuilt by the next step and a captured step must be captured again.
+ * once the last layer has been appended (wnw_step_begin is refused in between).  The work is queued behind all earlier
+ * work of the cache; the call does not wait for it.  Work lists are rebuilt by the next step and a captured step must be captured again.
  * Needs streaming_audio = 1 at creation and the HARD_BUDGET residency (or FULL mode, where every head is stored in
  * full): WNW_ERR_UNSUPPORTED otherwise; WNW_ERR_CAPACITY beyond max_audio_tokens; WNW_ERR_STATE out of order. */
 wnw_status_t wnw_append_audio(wnw_cache_t *cache, int32_t seq, int32_t layer, const void *k_dev, const void *v_dev,

@@ -200,7 +200,9 @@ def wnw_import_prefill_tidal(cache, seq, layer, sums, stream=None):
 
 def wnw_append_audio(cache, seq, layer, k, v, stream=None):
     """k, v: [n_tokens, n_kv_heads, head_dim] bf16 CUDA tensors, the new audio positions of one layer."""
-    _ck(lib().wnw_append_audio(cache, seq, layer, _ptr(k), _ptr(v), k.shape[0], _stream(stream)), "wnw_append_audio")
+    rc = (_lib or lib()).wnw_append_audio(cache, seq, layer, k.data_ptr(), v.data_ptr(), k.shape[0], _stream(stream))
+    if rc:
+        raise WnwError(rc, "wnw_append_audio")
 
 
 def wnw_place_prefill_multi(cache, seq, layer, k, v, audio_begin, audio_end, q_text, stream=None):
@@ -229,13 +231,19 @@ def wnw_step_begin(cache, active: Sequence[int]):
     _ck(lib().wnw_step_begin(cache, a, len(active)), "wnw_step_begin")
 
 
+# The calls of a decode loop go to the library directly: a step issued call by call is bound by what each costs the host.
 def wnw_decode_layer(cache, layer, q, k_new, v_new, out, stream=None):
-    _ck(lib().wnw_decode_layer(cache, layer, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out), _stream(stream)), "wnw_decode_layer")
+    rc = (_lib or lib()).wnw_decode_layer(cache, layer, q.data_ptr(), None if k_new is None else k_new.data_ptr(),
+                                          None if v_new is None else v_new.data_ptr(), out.data_ptr(), _stream(stream))
+    if rc:
+        raise WnwError(rc, "wnw_decode_layer")
 
 
 def wnw_decode_layer_full(cache, layer, q, k_new, v_new, out, stream=None):
-    _ck(lib().wnw_decode_layer_full(cache, layer, _ptr(q), _ptr(k_new), _ptr(v_new), _ptr(out), _stream(stream)),
-        "wnw_decode_layer_full")
+    rc = (_lib or lib()).wnw_decode_layer_full(cache, layer, q.data_ptr(), None if k_new is None else k_new.data_ptr(),
+                                               None if v_new is None else v_new.data_ptr(), out.data_ptr(), _stream(stream))
+    if rc:
+        raise WnwError(rc, "wnw_decode_layer_full")
 
 
 def wnw_step_end(cache, stream=None):

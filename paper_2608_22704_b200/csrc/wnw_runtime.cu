@@ -1270,11 +1270,17 @@ extern "C" wnw_status_t wnw_append_audio(wnw_cache_t *c, int32_t seq, int32_t la
   if (!s.fixed_blocks.empty()) return WNW_ERR_UNSUPPORTED;   // heads compacted token by token have no chunk geometry to grow
   DeviceGuard guard(c->cfg.device);
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  if (layer == 0) {   // selections and recalls of earlier steps read and write the tables and slots this touches
-    wnw_status_t ds = drain(c);
-    if (ds != WNW_OK) return ds;
-    CK(cudaStreamSynchronize(st));
+  if (layer == 0) {   // behind the placements, steps, selections and recalls that read and write the tables, slots and mirrors this touches
+    if (c->place_recorded) CK(cudaStreamWaitEvent(st, c->ev_place, 0));
+    if (c->step_recorded) CK(cudaStreamWaitEvent(st, c->last_step, 0));
+    for (int l = 0; l < G.L; ++l)
+      if (c->side_recorded[l]) CK(cudaStreamWaitEvent(st, c->ev_side_done[l], 0));
+    if (c->recall_all_pending) CK(cudaStreamWaitEvent(st, c->ev_recall_all, 0));
+    wnw_status_t ms = wait_for_mirror(c, st);
+    if (ms != WNW_OK) return ms;
     s.append_n = n_tokens;
+  } else if (c->last_stream != st && c->place_recorded) {
+    CK(cudaStreamWaitEvent(st, c->ev_place, 0));   // an earlier layer went to another stream
   }
   const int T_new = s.T_a + n_tokens, C_new = (T_new + G.nc - 1) / G.nc;
   const int S_new = full ? 0 : slots_total(c->cfg, C_new);
