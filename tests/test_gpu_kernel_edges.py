@@ -1,0 +1,140 @@
+"""The attention, scoring, token-compression and recall kernels at the sizes where their cuts change: edges of granules, tiles,
+pieces and clusters, groups with padding heads, more text queries than a launch takes (needs a B200)."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2608_22704_b200 as wnw
+from helpers import bf16_bits_to_f64, dense_attention
+from workloads import ROLE_ANCHOR as A, ROLE_FIXED as F, ROLE_TIDAL as T, Synth, tiny_custom
+from workloads.synth import bf16_bits
+
+pytestmark = pytest.mark.gpu
+
+
+# audio tokens: one granule; a head of one piece and one of two (256 keys a piece); 16 pieces; more than 16 pieces' worth
+@pytest.mark.parametrize("n_q,n_kv,d,audio", [(2, 2, 64, (16, 17)), (6, 2, 128, (255, 256, 257)), (16, 2, 128, (500,)), (18, 2, 128, (270,)),
+                                              (32, 2, 64, (4097, 31)), (14, 2, 128, (3900, 4200))])
+@pytest.mark.parametrize("mode", [wnw.WNW_LAYERS_CHAINED, wnw.WNW_LAYERS_SERIAL])
+def test_chained_layers_clustered_pieces(n_q, n_kv, d, audio, mode):
+    from parity_harness import Lockstep
+    w = tiny_custom(n_layers=3, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=d, n_text=14, audio_lens=audio, chunk=16, budget=0.25, n_steps=5,
+                    roles=[[A, T], [T, F], [F, A]], region=16, jump_every=2)
+    ls = Lockstep(w, seed=41)
+    try:
+        wnw.wnw_set_layer_dependency(ls.h, mode)
+        ls.prefill()
+        for t in range(5):          # the new token's row crosses into a second text granule (14 + 2)
+            ls.decode_step(t, graph=t >= 2, check_slots=(t == 4))
+        ls.check_stats()
+        assert ls.max_out_err <= 2e-2
+    finally:
+        ls.close()
+
+
+@pytest.mark.parametrize("n_q,n_kv,d", [(8, 4, 64), (16, 1, 128), (9, 3, 128), (128, 64, 64)])
+def test_static_attention_edges(n_q, n_kv, d):
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device="cpu").manual_seed(n_q + d)
+    for n in (1, 15, 16, 17, 127, 128, 129, 2400, 2401):
+        padded = (n + 15) // 16 * 16
+        kv = torch.randn(n_kv, 2, padded, d, generator=gen).to(torch.bfloat16).to(dev)
+        q = (torch.randn(n_q, d, generator=gen) * 1.5).to(torch.bfloat16).to(dev)
+        out = torch.full((n_q, d), float("nan"), dtype=torch.bfloat16, device=dev)
+        wnw.wnw_attend_static(kv, n, q, out)
+        K, V, Q = (bf16_bits_to_f64(bf16_bits(x.cpu().contiguous())) for x in (kv[:, 0, :n], kv[:, 1, :n], q))
+        want = np.stack([dense_attention(Q[h], K[h * n_kv // n_q], V[h * n_kv // n_q], 1.0 / np.sqrt(d))[0] for h in range(n_q)])
+        assert np.abs(out.float().cpu().numpy() - want).max() <= 2e-2, n
+    assert not wnw.wnw_attend_static_status()
+
+
+@pytest.mark.parametrize("n_queries", [8, 9, 17])
+def test_scoring_takes_several_queries_per_launch(n_queries):
+    from parity_harness import Lockstep
+    w = tiny_custom(n_layers=2, n_q_heads=6, n_kv_heads=3, head_dim=128, n_text=3, audio_lens=(127, 400), chunk=25, budget=0.3, n_steps=2,
+                    roles=[[A, T, F], [F, T, T]], region=25)
+    w.n_prefill_queries = n_queries
+    ls = Lockstep(w, seed=42)
+    try:
+        ls.prefill()                # scores, sets, tables and slots against the oracle
+        ls.decode_step(0, check_slots=True)
+        ls.decode_step(1, check_slots=True)
+        ls.check_stats()
+    finally:
+        ls.close()
+
+
+# tiles of 128 positions, 16 query rows a pass: one, two and three passes
+@pytest.mark.parametrize("n_queries,audio", [(1, (123, 124)), (8, (125, 252)), (9, (1024,)), (20, (300,))])
+def test_token_scores_over_tiles_and_passes(n_queries, audio):
+    from parity_harness import Lockstep
+    w = tiny_custom(n_layers=2, n_q_heads=8, n_kv_heads=4, head_dim=64, n_text=4, audio_lens=audio, chunk=32, budget=0.5, n_steps=2,
+                    roles=[[A, T, F, F], [T, F, T, F]], region=32)
+    w.n_prefill_queries = n_queries
+    ret = np.array([[1.0, 1.0, 0.4, 0.25], [1.0, 0.3, 1.0, 0.5]], np.float32)
+    ls = Lockstep(w, seed=43, token_retention=ret, token_seg=25)
+    try:
+        ls.prefill()                # per-position scores and kept positions against the oracle
+        ls.decode_step(0)
+        ls.decode_step(1)
+        assert ls.max_out_err <= 2e-2
+    finally:
+        ls.close()
+
+
+@pytest.mark.parametrize("chunk,n_kv,batch", [(1, 2, 1), (25, 3, 3), (33, 4, 40)])
+def test_recall_moves_chunks_without_their_padding(chunk, n_kv, batch):
+    """Chunks that fill their granules partly, many sequences (more than a warp looks up at once): slots stay bit-exact."""
+    from parity_harness import Lockstep
+    w = tiny_custom(n_layers=2, n_q_heads=n_kv, n_kv_heads=n_kv, head_dim=64, n_text=3, audio_lens=(6 * chunk + chunk // 2 + 1,) * batch, chunk=chunk,
+                    budget=0.5, n_steps=4, roles=[[A] + [T] * (n_kv - 1), [T] * n_kv], region=max(chunk, 2), jump_every=1)
+    ls = Lockstep(w, seed=44, oracle_seqs=[0, batch - 1] if batch > 1 else [0])
+    try:
+        ls.prefill()
+        for t in range(4):
+            ls.decode_step(t, graph=t >= 2, check_slots=True)
+        assert ls.max_out_err <= 2e-2
+    finally:
+        ls.close()
+
+
+def test_appends_queue_behind_steps_without_a_wait():
+    """Audio arriving between eager and replayed steps with nothing drained: the outputs of the drained run."""
+    w = tiny_custom(n_layers=3, n_q_heads=4, n_kv_heads=2, head_dim=64, n_text=4, audio_lens=(200,), chunk=16, budget=0.25, n_steps=8,
+                    roles=[[A, T], [T, T], [A, T]], region=16, jump_every=2)
+    syn, dev = Synth(w, seed=45, device="cuda:0"), torch.device("cuda:0")
+    dec = [syn.decode(0, l) for l in range(3)]
+    extra = torch.randn(2, 3, 4, 10, 2, 64, generator=torch.Generator(device=dev).manual_seed(5), device=dev).to(torch.bfloat16)
+
+    def run(drained):
+        h = wnw.wnw_create(3, 4, 2, 64, 1, 240, w.text_capacity, 16, 0.25, w.roles, streaming_audio=1)
+        try:
+            st = torch.cuda.Stream()
+            for l in range(3):
+                p = syn.prefill(0, l)
+                wnw.wnw_place_prefill(h, 0, l, p["k"], p["v"], p["audio_begin"], p["audio_end"], p["q_last"])
+                torch.cuda.synchronize()
+            outs = []
+            with torch.cuda.stream(st):
+                for t in range(8):
+                    if t % 2 == 0:
+                        for l in range(3):
+                            wnw.wnw_append_audio(h, 0, l, extra[0, l, t // 2], extra[1, l, t // 2], stream=st)
+                    out = torch.zeros(3, 1, 4, 64, dtype=torch.bfloat16, device=dev)
+                    wnw.wnw_step_begin(h, [0])
+                    for l in range(3):
+                        wnw.wnw_decode_layer(h, l, dec[l]["q"][t:t + 1], dec[l]["k_new"][t:t + 1], dec[l]["v_new"][t:t + 1], out[l], stream=st)
+                    wnw.wnw_step_end(h, stream=st)
+                    outs.append(out)
+                    if drained:
+                        wnw.wnw_sync(h)
+            wnw.wnw_sync(h)
+            return outs, [wnw.wnw_get_residency(h, 0, l) for l in range(3)]
+        finally:
+            wnw.wnw_destroy(h)
+
+    a, b = run(True), run(False)
+    for x, y in zip(a[0], b[0]):
+        assert torch.equal(x, y)
+    for (t1, s1), (t2, s2) in zip(a[1], b[1]):
+        assert np.array_equal(t1, t2) and np.array_equal(s1, s2)
