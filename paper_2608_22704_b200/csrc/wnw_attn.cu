@@ -21,6 +21,9 @@
 // Chunk scoring, selection and recall are not needed by whatever consumes the attention output next, so they run
 // in wnw_select_kernel / wnw_recall_kernel on a side stream (wnw_kernels.cu), off the critical path.
 #include <cstring>
+#include <map>
+#include <mutex>
+#include <tuple>
 #include <type_traits>
 
 #include <cuda_fp16.h>
@@ -1456,9 +1459,17 @@ bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, bool clust
   if (g > 8) return token_base ? recall_room_t<64, true, 1>(g, cluster) : recall_room_t<64, true, 0>(g, cluster);
   return token_base ? recall_room_t<64, false, 1>(g, cluster) : recall_room_t<64, false, 0>(g, cluster);
 }
-int attn_cluster_room(int g, int d, int cluster) {
-  if (d == 128) return g > 8 ? cluster_room_t<128, true>(g, cluster) : cluster_room_t<128, false>(g, cluster);
-  return g > 8 ? cluster_room_t<64, true>(g, cluster) : cluster_room_t<64, false>(g, cluster);
+int attn_cluster_room(int device, int g, int d, int cluster) {   // (an occupancy query takes some 0.2 ms: asked once per shape)
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, int, int>, int> known;
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = known.find({device, g, d, cluster});
+  if (it != known.end()) return it->second;
+  int n;
+  if (d == 128) n = g > 8 ? cluster_room_t<128, true>(g, cluster) : cluster_room_t<128, false>(g, cluster);
+  else n = g > 8 ? cluster_room_t<64, true>(g, cluster) : cluster_room_t<64, false>(g, cluster);
+  if (n > 0) known[{device, g, d, cluster}] = n;
+  return n;
 }
 
 template <int D, bool G16, int NW>

@@ -310,7 +310,7 @@ bool attn_xpref_fits(int g, int d);  // a one-shot CTA can hold its merge scratc
 // whether an SM that holds all the persistent attention CTAs (or the cluster kernel's CTA) it can take has registers left for a recall CTA
 bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, bool cluster);
 constexpr int RECALL_REGS = 256 * 40;       // registers of a recall CTA
-int attn_cluster_room(int g, int d, int cluster);   // clusters of that size that fit the GPU at once
+int attn_cluster_room(int device, int g, int d, int cluster);   // clusters of that size that fit the GPU at once
 int attn_warps(bool throughput);  // warps per attention CTA in the latency / throughput variant
 int attn_persistent_ctas_per_sm(int g, int d);  // persistent (throughput-variant) CTAs that fit one SM
 

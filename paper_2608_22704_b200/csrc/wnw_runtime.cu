@@ -369,7 +369,7 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
     c->recall_fits_beside[k] = attn_leaves_recall_room(cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim,
                                                        cfg->mode == WNW_MODE_TIERED && cfg->tidal_kv_format == WNW_TIDAL_KV_FP8_E4M3,
                                                        cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE, k == 1);
-  for (int k = 0; k < 3; ++k) c->cluster_room[k] = attn_cluster_room(cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim, 4 << k);
+  for (int k = 0; k < 3; ++k) c->cluster_room[k] = attn_cluster_room(cfg->device, cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim, 4 << k);
   const int L = cfg->n_layers, Hkv = cfg->n_kv_heads, d = cfg->head_dim, nc = cfg->chunk_tokens;
   const bool full = cfg->mode == WNW_MODE_FULL;
   c->roles.assign(cfg->roles, cfg->roles + (size_t)L * Hkv);
