@@ -34,10 +34,7 @@
 namespace wnw {
 
 constexpr int NW_LAT = 8;  // warps of a one-shot CTA (one work item each): 1 CTA per SM
-#ifndef WNW_NW_THR
-#define WNW_NW_THR 4
-#endif
-constexpr int NW_THR = WNW_NW_THR;  // warps of a persistent CTA (launches of more than one wave): several per SM, whose phases drift apart,
+constexpr int NW_THR = 4;  // warps of a persistent CTA (launches of more than one wave): several per SM, whose phases drift apart,
                            // so one CTA's prologue and merge overlap the others' streaming
 // Granules in flight per warp, and persistent CTAs per SM.  Three stages and two 4-warp CTAs per SM are what was kept after
 // measuring the alternative that shared memory allows, two-stage rings (exactly the pair a softmax step consumes) with
@@ -1560,7 +1557,11 @@ static cudaError_t configure_t() {
 }
 // Opt-in shared-memory sizes, set once per device at cache creation (never during a stream capture).
 cudaError_t configure_attn_kernels() {
+  // (some hundred calls: the kernel configured last tells whether this device has them behind it)
   cudaError_t e;
+  cudaFuncAttributes at;
+  if ((e = cudaFuncGetAttributes(&at, wnw_attn_kernel<64, false, NW_THR, 1>)) != cudaSuccess) return e;
+  if (at.maxDynamicSharedSizeBytes > 48 * 1024) return cudaSuccess;
   if ((e = configure_t<128, true, NW_LAT>()) != cudaSuccess) return e;
   if ((e = configure_t<128, false, NW_LAT>()) != cudaSuccess) return e;
   if ((e = configure_t<64, true, NW_LAT>()) != cudaSuccess) return e;

@@ -676,10 +676,7 @@ static void head_granules(const wnw_cache *c, int layer, int mode, const SeqHost
 // single piece of the same size).  So heads are cut as little as the balance allows: for a piece size T a head becomes
 // round(work / T) even pieces (at least one), the pieces go longest-first to the least loaded CTA, and T is the candidate
 // between 0.3 and three even shares of the launch that gives the shortest longest CTA under that cost model.
-#ifndef WNW_CLUSTER_MAX_PER_WARP
-#define WNW_CLUSTER_MAX_PER_WARP 8
-#endif
-constexpr int CLUSTER_MAX_PER_WARP = WNW_CLUSTER_MAX_PER_WARP;
+constexpr int CLUSTER_MAX_PER_WARP = 8;   // granules: with more, persistent CTAs are the better cut (8 x 3000 tokens, 12 layers: 206 us at 8, 234 at 4)
 struct CutMemo {   // piece sizes found for one work list, by the launch's head sizes
   struct Entry { std::vector<int> sizes; double T; };
   std::vector<Entry> entries;
@@ -696,10 +693,7 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   const int nw = attn_warps(true), n_heads = (int)seq_ids.size() * G.Hkv;
   const double cost_whole = 5.0, cost_piece = 16.0;   // fixed cost of an item in granules' worth: finished in the CTA / left as a partial
   const double mean_weight = 1.0;                     // weight of the mean CTA load beside the longest one in the objective
-#ifndef WNW_THR_CHAINED_PER_SM
-#define WNW_THR_CHAINED_PER_SM 2
-#endif
-  const int per_sm = layers_overlap(c) ? attn_persistent_ctas_per_sm(G.g, G.d) : std::min(WNW_THR_CHAINED_PER_SM, attn_persistent_ctas_per_sm(G.g, G.d));
+  const int per_sm = attn_persistent_ctas_per_sm(G.g, G.d);   // persistent 4-warp CTAs an SM holds
   double total = 0.0;
   for (int hd = 0; hd < n_heads; ++hd) total += n_work[hd];
   const int P = (int)std::min<double>(per_sm * c->n_sm, std::max(1.0, total / (2.0 * nw)));   // at least two granules per warp and CTA
