@@ -248,6 +248,8 @@ struct RecallSignal {
   int32_t *empty_ctr;         // [L] the selection kernels' empty-plan counters, reset here
   int32_t publish_epoch;      // epoch to publish: the number of replayed steps that have ended with this one (the host counts
                               // them; the device word may already be further when this kernel runs late)
+  const int32_t *landed;      // [n_landed] layers whose recall the step itself did, before this kernel started: their epoch is
+  int32_t n_landed;           //   published too, nothing else is left to do for them
 };
 
 // kernels' host launchers (defined in the .cu files)

@@ -335,8 +335,10 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // where layers overlap: attention then fills the memory system, a host read takes several times as long and the step waits for
 // it (4 x 3000 tokens: 225 us a step with 8, 197 with 16, 193 with 24, 194 with 32, 198 with 48; formerly 206).
 //
-// With `sig` set (replayed steps, where this kernel runs outside the captured graph and overlaps the next step) the
-// warp that finishes a layer last publishes the layer's recall epoch, which the next step's tidal CTAs acquire.
+// With `sig` set (this kernel runs behind its step and overlaps the next one) the warp that finishes a layer last publishes the
+// layer's recall epoch, which the next step's tidal CTAs acquire.  Every step that raises the step epoch ends with EVERY layer's
+// word raised, also those of layers that recalled inside the step (`landed`): which layers a step's tidal CTAs wait for depends
+// on how that step is issued, and the next one may be issued another way.
 // ------------------------------------------------------------------------------------------------
 constexpr int RECALL_CTAS = 8, RECALL_CTAS_CROWDED = 24, RECALL_WARPS = 8, RECALL_U = 4;
 __global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
@@ -344,6 +346,9 @@ __global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const 
                                                                           int n_layers, int skip_copy, RecallSignal sig) {
   const Geometry &G = cv.geo;
   const int lane = threadIdx.x & 31, n_warps = gridDim.x * RECALL_WARPS, w = blockIdx.x * RECALL_WARPS + (threadIdx.x >> 5);
+  if (sig.epoch_words && w == 0)   // copies that landed before this kernel started
+    for (int x = lane; x < sig.n_landed; x += 32)
+      asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(sig.epoch_words + sig.landed[x]), "r"(sig.publish_epoch) : "memory");
   int turn = 0;   // the warp that takes the next piece (the same on every warp: plans do not change under this kernel)
   for (int x0 = 0; x0 < n_layers; x0 += 32) {
     // a lane looks up one layer: whether its epoch is out already (the selection kernel publishes it when no sequence planned

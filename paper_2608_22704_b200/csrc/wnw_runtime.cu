@@ -1536,9 +1536,11 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   // 8 x 3000, 12 layers: 201 -> 191 us; with recall at speech rate as before.
   bool fits = true;
   for (const LayerWork &w : c->wl_layers) fits = fits && (w.throughput ? c->recall_fits_beside[0] : w.cluster > 0 && c->recall_fits_beside[1]);
-  if (c->cap_fold && capturing && !small && !layers_overlap(c) && fits && G.L > 1) {
+  const int half = (G.L + 1) / 2;
+  if (c->cap_fold && capturing && !small && !layers_overlap(c) && fits && half < G.L &&
+      c->layers[half].upd_first < (int)c->upd_list.size()) {   // (some layer is recalled behind the step)
     c->cap_external_recall = true;
-    c->cap_ext_from = (G.L + 1) / 2;
+    c->cap_ext_from = half;
   }
   // BATCHED layers: one launch for the whole step where nothing inside the step needs a layer's result earlier
   bool one_shot = G.L <= MULTI_LAYERS_MAX;
@@ -1694,7 +1696,7 @@ static wnw_status_t issue_side_work(wnw_cache *c, int layer, bool tiered, bool c
       wnw_status_t ms = capturing ? WNW_OK : wait_for_mirror(c, ss);   // a replayed step waits as a whole
       if (ms != WNW_OK) return ms;
       CK(launch_recall(c->cv, n_active, c->d_active, c->cv.upd_list + li.upd_first, li.upd_count,
-                       c->cfg.recall_mode == WNW_RECALL_SKIP, recall_crowded(c), RecallSignal{nullptr, nullptr, nullptr, 0}, ss));
+                       c->cfg.recall_mode == WNW_RECALL_SKIP, recall_crowded(c), RecallSignal{}, ss));
       c->count_launch(2, 1, capturing);
     }
     if (!inline_mode) {
@@ -1860,8 +1862,9 @@ extern "C" wnw_status_t wnw_import_prefill_tidal(wnw_cache_t *c, int32_t seq, in
   return WNW_OK;
 }
 
-// The recall of the step that ended with c->last_step, for every layer's table at once, outside the step: it overlaps the next
-// step, whose tidal CTAs wait on the per-layer epoch words it publishes.
+// The recall of the step that ended with c->last_step, outside the step, for the tables updated from layer ext_from's tail on at
+// once: it overlaps the next step, whose tidal CTAs wait on the per-layer epoch words it publishes.  The tables before those
+// were recalled inside the step; their words are raised with the others.
 static wnw_status_t launch_step_recall(wnw_cache *c, int n_active, int ext_from) {
   if (c->upd_list.empty()) return WNW_OK;
   const int first = c->layers[ext_from].upd_first, n = (int)c->upd_list.size() - first;   // (the list is in the order of the layers' tails)
@@ -1870,7 +1873,7 @@ static wnw_status_t launch_step_recall(wnw_cache *c, int n_active, int ext_from)
   wnw_status_t ms = wait_for_mirror(c, c->side[0]);
   if (ms != WNW_OK) return ms;
   CK(launch_recall(c->cv, n_active, c->d_active, c->cv.upd_list + first, n, c->cfg.recall_mode == WNW_RECALL_SKIP,
-                   recall_crowded(c), RecallSignal{c->d_recall_epoch, c->d_recall_ctr, c->d_empty_ctr, c->host_epoch}, c->side[0]));
+                   recall_crowded(c), RecallSignal{c->d_recall_epoch, c->d_recall_ctr, c->d_empty_ctr, c->host_epoch, c->cv.upd_list, first}, c->side[0]));
   c->count_launch(2, 1, false);
   CK(cudaEventRecord(c->ev_recall_all, c->side[0]));
   c->recall_all_pending = true;
@@ -1909,7 +1912,7 @@ extern "C" wnw_status_t wnw_step_end(wnw_cache_t *c, void *cuda_stream) {
       wnw_status_t ms = wait_for_mirror(c, st);
       if (ms != WNW_OK) return ms;
       CK(launch_recall(c->cv, (int)c->active.size(), c->d_active, c->cv.upd_list, (int)c->upd_list.size(),
-                       c->cfg.recall_mode == WNW_RECALL_SKIP, recall_crowded(c), RecallSignal{nullptr, nullptr, nullptr, 0}, st));
+                       c->cfg.recall_mode == WNW_RECALL_SKIP, recall_crowded(c), RecallSignal{}, st));
       c->count_launch(2, 1, false);
     }
   }

@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import paper_2608_22704_b200 as wnw
-from workloads import ROLE_ANCHOR, ROLE_FIXED, ROLE_TIDAL, tiny_custom
+from workloads import ROLE_ANCHOR, ROLE_FIXED, ROLE_TIDAL, config4, tiny_custom
 from workloads.synth import bf16_bits
 
 pytestmark = pytest.mark.gpu
@@ -73,5 +73,51 @@ def test_graph_is_recaptured_when_the_active_set_changes():
             if t in (3, 4, 6):
                 ls._graph = None                                      # capture again for the new set
             ls.decode_step(t, active=act, graph=True, check_slots=True)
+    finally:
+        ls.close()
+
+
+def _split_recall_launches(w):
+    """Recall launches of a replayed chained step that fills the machine: one inside the step for every layer of the first half
+    whose tail updates tables, one behind the step for all the others."""
+    L = w.n_layers
+    anchor = [l for l in range(L) if (w.roles[l] == A).any()]
+    tails = {max(l, min(anchor, key=lambda a: (abs(a - l), a))) for l in range(L) if (w.roles[l] == T).any()}
+    half = (L + 1) // 2
+    inside = sum(t < half for t in tails)
+    assert 0 < inside < len(tails)
+    return inside + 1
+
+
+@pytest.mark.parametrize("dependency", [wnw.WNW_LAYERS_CHAINED, wnw.WNW_LAYERS_BATCHED])
+def test_few_sequences_decode_on_after_steps_that_filled_the_machine(dependency):
+    """Chained replays of twelve long sequences recall half of their layers inside the step and half behind it.  Most requests
+    finish; the steps of the ones that are left are small, recall behind the step altogether, and their tidal heads wait for
+    every layer's epoch: call by call, newly captured, and (all layers issued together) with the selection waiting too."""
+    from parity_harness import Lockstep
+    w = config4(budget=0.1, batch=12, n_steps=12)
+    w.n_layers = 4; w.roles = w.roles[:4]; w.jump_every = 2
+    ls = Lockstep(w, seed=17, gen_device="cuda:0", oracle_seqs=[0, 7])
+    everyone, left = list(range(12)), [7]
+
+    def steps(ts, active, graph):
+        before = wnw.wnw_get_launch_counts(ls.h)[2]
+        ls._graph = None
+        for t in ts:
+            ls.decode_step(t, active=active, graph=graph, check_slots=True)
+        return wnw.wnw_get_launch_counts(ls.h)[2] - before
+
+    try:
+        wnw.wnw_set_layer_dependency(ls.h, wnw.WNW_LAYERS_CHAINED)
+        ls.prefill(check_slots=False)
+        assert steps([0, 1, 2], everyone, True) == 3 * _split_recall_launches(w)     # the form that the first half takes part in
+        assert steps([3], left, False) == 1
+        wnw.wnw_set_layer_dependency(ls.h, dependency)
+        assert steps([4, 5], left, True) == 2
+        assert steps([6], left, False) == 1
+        wnw.wnw_set_layer_dependency(ls.h, wnw.WNW_LAYERS_CHAINED)
+        assert steps([7, 8], everyone, True) == 2 * _split_recall_launches(w)
+        wnw.wnw_set_layer_dependency(ls.h, dependency)
+        assert steps([9, 10], left, True) == 2
     finally:
         ls.close()

@@ -166,3 +166,56 @@ def test_undrained_batched_config1_full_stack():
     b = _run(w, False, 64, dependency=3)
     _same(a, b)
     assert a[2]["misses"] > 0
+
+
+def test_undrained_replays_of_changing_sets():
+    """Twelve long sequences (half of the recall inside the step, half behind it), then one of them, then all again, each set
+    newly captured, nothing drained in between: bit for bit what the drained run gives."""
+    w = config4(budget=0.1, batch=12, n_steps=15)
+    w.n_layers = 4; w.roles = w.roles[:4]
+    dev = torch.device("cuda:0")
+
+    def run(drained):
+        syn = Synth(w, seed=6, device="cuda:0")
+        h = wnw.wnw_create(w.n_layers, w.n_q_heads, w.n_kv_heads, w.head_dim, w.batch, max(w.audio_lens), w.text_capacity, w.chunk,
+                           w.budget, w.roles, topk=w.topk)
+        try:
+            wnw.wnw_set_layer_dependency(h, wnw.WNW_LAYERS_CHAINED)
+            for b in range(w.batch):
+                for l in range(w.n_layers):
+                    p = syn.prefill(b, l)
+                    wnw.wnw_place_prefill(h, b, l, p["k"], p["v"], p["audio_begin"], p["audio_end"], p["q_last"])
+                    torch.cuda.synchronize()
+            dec = [[syn.decode(b, l) for b in range(w.batch)] for l in range(w.n_layers)]
+            st = torch.cuda.Stream(device=dev)
+            torch.cuda.synchronize()
+            outs = []
+            with torch.cuda.stream(st):
+                for first, act in ((0, list(range(12))), (5, [3]), (10, list(range(12)))):
+                    part = lambda name, t: torch.stack([torch.stack([dec[l][b][name][t] for b in act]) for l in range(w.n_layers)])  # noqa: E731
+                    ins = [[part(name, t) for name in ("q", "k_new", "v_new")] for t in range(first, first + 5)]
+                    buf = [torch.empty_like(x) for x in ins[0]]
+                    out = torch.zeros_like(buf[0])
+                    wnw.wnw_graph_begin(h, act, st)
+                    wnw.wnw_step_begin(h, act)
+                    for l in range(w.n_layers):
+                        wnw.wnw_decode_layer(h, l, buf[0][l], buf[1][l], buf[2][l], out[l], stream=st)
+                    wnw.wnw_step_end(h, stream=st)
+                    wnw.wnw_graph_end(h, st)
+                    for x in ins:
+                        for dst, src in zip(buf, x):
+                            dst.copy_(src)
+                        wnw.wnw_graph_launch(h, st)
+                        outs.append(out.clone())
+                        if drained:
+                            wnw.wnw_sync(h)
+            torch.cuda.synchronize()
+            wnw.wnw_sync(h)
+            tabs = [wnw.wnw_get_residency(h, b, l) for b in range(w.batch) for l in range(w.n_layers) if (w.roles[l] == ROLE_TIDAL).any()]
+            return outs, tabs, wnw.wnw_get_stats(h)
+        finally:
+            wnw.wnw_destroy(h)
+
+    a = run(True)
+    _same(a, run(False))
+    assert a[2]["misses"] > 0
