@@ -1438,23 +1438,37 @@ static int cluster_room_t(int g, int cluster) {
   if (cudaOccupancyMaxActiveClusters(&n, wnw_attn_cluster_kernel<D, G16, 0>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
   return n;
 }
-template <int D, bool G16, int VAR>
-static bool recall_room_t(int g, bool cluster) {
+// An SM has 64 K registers, 228 KB of shared memory (1 KB of it kept for every CTA) and 2 048 threads.
+template <class K>
+static bool recall_room(K *kernel, int threads, size_t dynamic_smem) {
   cudaFuncAttributes at;
-  if ((cluster ? cudaFuncGetAttributes(&at, wnw_attn_cluster_kernel<D, G16, VAR>) : cudaFuncGetAttributes(&at, wnw_attn_kernel<D, G16, NW_THR, VAR>)) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  const int threads = cluster ? NW_LAT * 32 : attn_persistent_ctas_per_sm(g, D) * NW_THR * 32;
-  return 65536 - threads * ((at.numRegs + 7) / 8 * 8) >= RECALL_REGS;
+  if (cudaFuncGetAttributes(&at, kernel) != cudaSuccess) { cudaGetLastError(); return false; }
+  const int regs = threads * ((at.numRegs + 7) / 8 * 8), smem = (int)((dynamic_smem + at.sharedSizeBytes + 127) / 128 * 128) + 1024;
+  const int n = std::min(std::min(65536 / regs, 228 * 1024 / smem), 2048 / threads);
+  return 65536 - n * regs >= RECALL_REGS && 228 * 1024 - n * smem >= 1024 && 2048 - n * threads >= RECALL_THREADS;
 }
-bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, bool cluster) {
-  if (d == 128) {
-    if (g > 8) return kv8 ? recall_room_t<128, true, 2>(g, cluster) : token_base ? recall_room_t<128, true, 1>(g, cluster) : recall_room_t<128, true, 0>(g, cluster);
-    return kv8 ? recall_room_t<128, false, 2>(g, cluster) : token_base ? recall_room_t<128, false, 1>(g, cluster) : recall_room_t<128, false, 0>(g, cluster);
+template <int D, bool G16, int VAR>
+static bool recall_room_t(int g, AttnForm form) {
+  const size_t lat = uniform_smem(D), thr = (size_t)NW_THR * nstage_of(NW_THR) * 2 * GR * D * 2 + 1024;
+  const size_t lat_scratch = attn_scratch_bytes(NW_LAT, g, D), thr_scratch = attn_scratch_bytes(NW_THR, g, D);
+  switch (form) {
+    case FORM_PERSISTENT: return recall_room(wnw_attn_kernel<D, G16, NW_THR, VAR>, NW_THR * 32, thr + thr_scratch);
+    case FORM_NARROW: return recall_room(wnw_attn_kernel<D, G16, NW_THR, VAR>, NW_THR * 32, thr);
+    case FORM_CLUSTER: return recall_room(wnw_attn_cluster_kernel<D, G16, VAR>, NW_LAT * 32, cluster_smem(g, D));
+    case FORM_ONE_SHOT: return recall_room(wnw_attn_kernel<D, G16, NW_LAT, VAR>, NW_LAT * 32, lat);
+    case FORM_PACKED: return recall_room(wnw_attn_kernel<D, G16, NW_LAT, VAR>, NW_LAT * 32, lat + lat_scratch);
+    default:   // a launch of all layers takes the scratch if one of them does
+      return recall_room(wnw_attn_multi_kernel<D, G16, NW_LAT, VAR>, NW_LAT * 32, lat) &&
+             recall_room(wnw_attn_multi_kernel<D, G16, NW_LAT, VAR>, NW_LAT * 32, lat + lat_scratch);
   }
-  if (g > 8) return token_base ? recall_room_t<64, true, 1>(g, cluster) : recall_room_t<64, true, 0>(g, cluster);
-  return token_base ? recall_room_t<64, false, 1>(g, cluster) : recall_room_t<64, false, 0>(g, cluster);
+}
+bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, AttnForm form) {
+  if (d == 128) {
+    if (g > 8) return kv8 ? recall_room_t<128, true, 2>(g, form) : token_base ? recall_room_t<128, true, 1>(g, form) : recall_room_t<128, true, 0>(g, form);
+    return kv8 ? recall_room_t<128, false, 2>(g, form) : token_base ? recall_room_t<128, false, 1>(g, form) : recall_room_t<128, false, 0>(g, form);
+  }
+  if (g > 8) return token_base ? recall_room_t<64, true, 1>(g, form) : recall_room_t<64, true, 0>(g, form);
+  return token_base ? recall_room_t<64, false, 1>(g, form) : recall_room_t<64, false, 0>(g, form);
 }
 int attn_cluster_room(int device, int g, int d, int cluster) {   // (an occupancy query takes some 0.2 ms: asked once per shape)
   static std::mutex mu;

@@ -309,9 +309,12 @@ cudaError_t launch_quantise_stage(const CacheView &cv, int b, int layer, bf16 *s
 cudaError_t configure_select_kernel();
 constexpr int SELECT_SMEM_CAP = 200 * 1024;  // dynamic shared memory the selection kernel may be launched with
 bool attn_xpref_fits(int g, int d);  // a one-shot CTA can hold its merge scratch behind the copy stages
-// whether an SM that holds all the persistent attention CTAs (or the cluster kernel's CTA) it can take has registers left for a recall CTA
-bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, bool cluster);
-constexpr int RECALL_REGS = 256 * 40;       // registers of a recall CTA
+// The attention kernels as a step launches them: persistent CTAs, one-shot CTAs in clusters, of eight warps, of four, of eight
+// with several heads packed into a CTA, the CTAs of all layers together.
+enum AttnForm { FORM_PERSISTENT, FORM_CLUSTER, FORM_ONE_SHOT, FORM_NARROW, FORM_PACKED, FORM_TOGETHER, N_ATTN_FORMS };
+// whether an SM that holds as many CTAs of that form as it can has room left for a recall CTA
+bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, AttnForm form);
+constexpr int RECALL_THREADS = 256, RECALL_REGS = RECALL_THREADS * 40;   // of a recall CTA
 int attn_cluster_room(int device, int g, int d, int cluster);   // clusters of that size that fit the GPU at once
 int attn_warps(bool throughput);  // warps per attention CTA in the latency / throughput variant
 int attn_persistent_ctas_per_sm(int g, int d);  // persistent (throughput-variant) CTAs that fit one SM

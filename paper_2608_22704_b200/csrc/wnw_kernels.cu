@@ -340,7 +340,7 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // word raised, also those of layers that recalled inside the step (`landed`): which layers a step's tidal CTAs wait for depends
 // on how that step is issued, and the next one may be issued another way.
 // ------------------------------------------------------------------------------------------------
-constexpr int RECALL_CTAS = 8, RECALL_CTAS_CROWDED = 24, RECALL_WARPS = 8, RECALL_U = 4;
+constexpr int RECALL_CTAS = 8, RECALL_CTAS_CROWDED = 24, RECALL_WARPS = RECALL_THREADS / 32, RECALL_U = 4;
 __global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
                                                                           const int32_t *active, const int32_t *layers,
                                                                           int n_layers, int skip_copy, RecallSignal sig) {

@@ -147,7 +147,7 @@ struct wnw_cache {
   int32_t *d_recall_epoch = nullptr, *d_recall_ctr = nullptr, *d_step_epoch = nullptr;
   bool cap_external_recall = false, graph_external_recall = false, recall_all_pending = false;
   int cap_ext_from = 0, graph_ext_from = 0;   // first layer whose table updates are recalled outside the step
-  bool recall_fits_beside[2] = {false, false};   // a recall CTA has room on an SM full of persistent / of clustered attention CTAs
+  bool recall_fits_beside[N_ATTN_FORMS] = {};   // a recall CTA has room on an SM full of attention CTAs of that form
   cudaEvent_t ev_graph_done = nullptr, ev_recall_all = nullptr;
   static constexpr int direct_max_granules = 64;   // scale of the one-CTA rule: a head of up to 2x (overlapping layers) or x/2
                                                    // (chained layers) this many granules (text capacity included) is not split
@@ -189,6 +189,10 @@ struct wnw_cache {
 // Layers whose attention launches run over one another (as opposed to chained or serial ones).
 static bool layers_overlap(const wnw_cache *c) {
   return c->layer_dependency == WNW_LAYERS_INDEPENDENT || c->layer_dependency == WNW_LAYERS_BATCHED;
+}
+
+static AttnForm form_of(const LayerWork &w) {
+  return w.cluster > 0 ? FORM_CLUSTER : w.throughput ? FORM_PERSISTENT : w.narrow ? FORM_NARROW : w.packed ? FORM_PACKED : FORM_ONE_SHOT;
 }
 
 // Whether attention keeps the memory system busy while recalls run.
@@ -365,10 +369,10 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
   cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
   CKE(configure_attn_kernels());
   CKE(configure_select_kernel());
-  for (int k = 0; k < 2; ++k)
+  for (int k = 0; k < N_ATTN_FORMS; ++k)
     c->recall_fits_beside[k] = attn_leaves_recall_room(cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim,
                                                        cfg->mode == WNW_MODE_TIERED && cfg->tidal_kv_format == WNW_TIDAL_KV_FP8_E4M3,
-                                                       cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE, k == 1);
+                                                       cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE, (AttnForm)k);
   for (int k = 0; k < 3; ++k) c->cluster_room[k] = attn_cluster_room(cfg->device, cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim, 4 << k);
   const int L = cfg->n_layers, Hkv = cfg->n_kv_heads, d = cfg->head_dim, nc = cfg->chunk_tokens;
   const bool full = cfg->mode == WNW_MODE_FULL;
@@ -1510,11 +1514,29 @@ static SelectArgs static_select_args(const wnw_cache *c, int layer) {
 // Decided once per step, at its first layer: how the step issues its selection, recall and attention launches.
 static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   const Geometry &G = c->geo;
+  // BATCHED layers: one launch for the whole step where nothing inside the step needs a layer's result earlier
+  bool one_shot = G.L <= MULTI_LAYERS_MAX;
+  for (const LayerWork &w : c->wl_layers) one_shot = one_shot && !w.throughput;
+  const bool together = c->layer_dependency == WNW_LAYERS_BATCHED && c->batched_target > 0 && capturing && c->graph_capturing && one_shot;
   // Steps of small launches take their recall out of the step, so that it can overlap the next one.  Where a launch could
   // fill the machine, its attention CTAs would sit on their SMs while they wait for it, so recall stays inside the step
   // there.  (A caller's own capture of an eager step keeps everything inside, too: nothing could be issued behind it.)
+  // Small launches add up: a layer's CTAs start beside its predecessors', and while the first layer's tidal CTAs wait for the
+  // recall the later ones can take every SM.  The recall starts all the same where one of its CTAs has room beside the attention
+  // CTAs, or where the CTAs that can be there at once (all layers'; one layer's in plain stream order; the tidal part of a launch
+  // of all layers, the others end by themselves) are fewer than the SMs.  Elsewhere it stays inside the step: kernels of eight
+  // warps and more than 216 registers a thread (groups of more than 8 query heads, as a rule), packed CTAs of 8 heads of 128
+  // elements (all of the shared memory).
   bool small = true;   // no launch can fill the machine with CTAs that wait
-  for (const LayerWork &w : c->wl_layers) small = small && !w.throughput && (w.n_ctas > 0 ? w.n_ctas : w.n_items) <= c->n_sm / 2;
+  bool beside = true;
+  int there = 0;
+  for (const LayerWork &w : c->wl_layers) {
+    const int n = w.n_ctas > 0 ? w.n_ctas : w.n_items, wait = together && w.packed ? n - w.n_ctas_free : n;
+    small = small && !w.throughput && n <= c->n_sm / 2;
+    beside = beside && c->recall_fits_beside[together ? FORM_TOGETHER : form_of(w)];
+    there = c->layer_dependency == WNW_LAYERS_SERIAL ? std::max(there, wait) : there + wait;
+  }
+  small = small && (beside || there < c->n_sm);
   const bool ours = tiered && c->cfg.recall_mode != WNW_RECALL_INLINE && !c->cfg.defer_selection && (!capturing || c->graph_capturing);
   const int n_select = c->select_single_ok ? c->sel_map_single[1] : c->sel_map_update[1];
   // With the recall outside, nothing inside the step needs a layer's selection before the step ends: all of it goes into one
@@ -1534,22 +1556,20 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   // CTAs that wait for it: recall_fits_beside.)
   // Measured, back to back: 16 ragged sequences, 6 layers, 10 MB of recall a step: 320 -> 273 us; 16 x 7500 e4m3, 4 MB: 219 -> 198 us;
   // 8 x 3000, 12 layers: 201 -> 191 us; with recall at speech rate as before.
-  bool fits = true;
-  for (const LayerWork &w : c->wl_layers) fits = fits && (w.throughput ? c->recall_fits_beside[0] : w.cluster > 0 && c->recall_fits_beside[1]);
+  bool fits = beside;
+  for (const LayerWork &w : c->wl_layers) fits = fits && (w.throughput || w.cluster > 0);
   const int half = (G.L + 1) / 2;
   if (c->cap_fold && capturing && !small && !layers_overlap(c) && fits && half < G.L &&
       c->layers[half].upd_first < (int)c->upd_list.size()) {   // (some layer is recalled behind the step)
     c->cap_external_recall = true;
     c->cap_ext_from = half;
   }
-  // BATCHED layers: one launch for the whole step where nothing inside the step needs a layer's result earlier
-  bool one_shot = G.L <= MULTI_LAYERS_MAX;
-  for (const LayerWork &w : c->wl_layers) one_shot = one_shot && !w.throughput;
-  c->cap_batched = c->layer_dependency == WNW_LAYERS_BATCHED && c->batched_target > 0 && capturing && c->graph_capturing &&
-                   one_shot && (!tiered || c->cap_select_all);
+  c->cap_batched = together && (!tiered || c->cap_select_all);
   if (c->cap_batched) c->batch_args.assign(G.L, AttnArgs{});
   // Two parts (slot-free CTAs, then the tidal heads'): every anchor head is in the first, so the step's selection can
-  // run beside the second; the step's bookkeeping then waits for both (a step-end kernel instead of the fold).
+  // run beside the second; the step's bookkeeping then waits for both (a step-end kernel instead of the fold).  Selection CTAs
+  // wait for the recall as well, and two of them (120 registers a thread) leave an SM no room for it: the same rule with them
+  // counted, one to an SM where attention leaves no room either.
   c->cap_sel_overlap = false;
   if (c->cap_batched && tiered && c->cap_external_recall && c->cap_select_all) {
     bool any_free = false, any_tidal = false;
@@ -1558,7 +1578,8 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
       any_free = any_free || n_free > 0;
       any_tidal = any_tidal || n_free < (w.n_ctas > 0 ? w.n_ctas : w.n_items);
     }
-    c->cap_sel_overlap = any_free && any_tidal;
+    const int n_wait = n_select * (int)c->active.size();
+    c->cap_sel_overlap = any_free && any_tidal && (beside ? n_wait < 2 * c->n_sm : there + n_wait < c->n_sm);
     if (c->cap_sel_overlap) c->cap_fold = false;
   }
 }

@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import paper_2608_22704_b200 as wnw
-from workloads import ROLE_ANCHOR, ROLE_TIDAL, Synth, config1, config4
+from workloads import ROLE_ANCHOR, ROLE_FIXED, ROLE_TIDAL, Synth, config1, config4, tiny_custom
 
 pytestmark = pytest.mark.gpu
 
@@ -219,3 +219,42 @@ def test_undrained_replays_of_changing_sets():
     a = run(True)
     _same(a, run(False))
     assert a[2]["misses"] > 0
+
+
+def _replays(w, dependency, n, seed):
+    """n lock-step replays after an eager step; launches (attention, selection, recall, step end) of the eager step and of them."""
+    from parity_harness import Lockstep
+    ls = Lockstep(w, seed=seed, gen_device="cuda:0", oracle_seqs=[0, w.batch - 1] if w.batch > 1 else [0])
+    try:
+        wnw.wnw_set_layer_dependency(ls.h, dependency)
+        ls.prefill(check_slots=False)
+        ls.decode_step(0, check_slots=True)
+        eager = wnw.wnw_get_launch_counts(ls.h)
+        for t in range(1, n + 1):
+            ls.decode_step(t, graph=True, check_slots=True)
+        ls.check_stats()
+        assert ls.max_out_err <= 2e-2
+        return eager, tuple(x - y for x, y in zip(wnw.wnw_get_launch_counts(ls.h), eager))
+    finally:
+        ls.close()
+
+
+@pytest.mark.parametrize("n_q,dependency,outside", [(32, wnw.WNW_LAYERS_CHAINED, False), (32, wnw.WNW_LAYERS_INDEPENDENT, False),
+                                                    (32, wnw.WNW_LAYERS_SERIAL, True), (16, wnw.WNW_LAYERS_CHAINED, True)])
+def test_recall_leaves_the_step_where_it_can_start(n_q, dependency, outside):
+    """Sixteen query heads a KV head: no recall CTA has room beside the attention CTAs, and the layers' CTAs together outnumber
+    the SMs.  Recall then stays inside the step, replayed or not (in plain stream order one layer's CTAs leave SMs free)."""
+    w = tiny_custom(n_layers=12, n_q_heads=n_q, n_kv_heads=2, head_dim=128, n_text=14, audio_lens=(4200, 3900), chunk=64, budget=0.25,
+                    n_steps=5, roles=[[ROLE_ANCHOR, ROLE_TIDAL], [ROLE_TIDAL, ROLE_TIDAL]] * 6, region=64, jump_every=2)
+    eager, replayed = _replays(w, dependency, 4, 11)
+    assert (eager[2], replayed[2]) == ((1, 4) if outside else (12, 48))
+
+
+def test_selection_waits_for_the_recall_only_beside_free_sms():
+    """All layers together, eight query heads a KV head (packed CTAs take all of an SM's shared memory): with as many selection
+    and tidal CTAs as SMs the selection follows the attention instead of waiting beside it: two attention launches a step (three
+    with the selection forked between them), no step-end kernel."""
+    w = tiny_custom(n_layers=12, n_q_heads=16, n_kv_heads=2, head_dim=128, n_text=14, audio_lens=(9000, 8000, 9000, 7000), chunk=64, budget=0.25,
+                    n_steps=5, roles=[[ROLE_ANCHOR, ROLE_TIDAL], [ROLE_TIDAL, ROLE_FIXED]] * 6, region=64, jump_every=2)
+    _, (attention, _, recall, step_end) = _replays(w, wnw.WNW_LAYERS_BATCHED, 4, 12)
+    assert (attention, recall, step_end) == (2 * 4, 4, 0)
