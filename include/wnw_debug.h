@@ -19,6 +19,15 @@ extern "C" {
  * The cache's results are meaningless afterwards; destroy it.  Not for production use. */
 wnw_status_t wnw_debug_advance_step_epoch(wnw_cache_t *cache, int32_t delta);
 
+/* Chunks of a size that is no multiple of 16 tokens are stored padded to whole granules of 16 rows.  On the device the
+ * padding rows of a slot are zero; those of the pinned host mirror are neither written nor read.  Test hooks for that:
+ * fill sets every byte of the mirror's padding rows of a placed sequence; get copies the padding rows of one slot, head
+ * and K|V (which = 0|1) as stored: (chunk_tokens rounded up to 16, minus chunk_tokens) rows of head_dim elements, two
+ * bytes each (one in an e4m3 tidal tier).  Both drain the cache's work. */
+wnw_status_t wnw_debug_fill_mirror_padding(wnw_cache_t *cache, int32_t seq, int32_t byte);
+wnw_status_t wnw_debug_get_slot_padding(wnw_cache_t *cache, int32_t seq, int32_t layer, int32_t kv_head, int32_t slot,
+                                        int32_t which, void *rows);
+
 /* Optional per-kernel timing: when enabled the library brackets its attention-kernel launches with CUDA events
  * on the launching stream; wnw_get_kernel_time returns the accumulated milliseconds and launch count since the
  * last call (drains the stream).  Off by default. */

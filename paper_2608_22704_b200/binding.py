@@ -80,6 +80,8 @@ _SIGNATURES = {
     "wnw_set_layer_dependency": [_vp, _i32],
     "wnw_get_launch_counts": [_vp, C.POINTER(C.c_int64)],
     "wnw_debug_advance_step_epoch": [_vp, _i32],
+    "wnw_debug_fill_mirror_padding": [_vp, _i32, _i32],
+    "wnw_debug_get_slot_padding": [_vp, _i32, _i32, _i32, _i32, _i32, _vp],
     "wnw_get_base_slots": [_vp, _i32, C.POINTER(_i32)],
     "wnw_set_kernel_timing": [_vp, _i32],
     "wnw_get_kernel_time": [_vp, C.POINTER(C.c_float), C.POINTER(_i32)],
@@ -352,6 +354,17 @@ def wnw_get_stats(cache) -> dict:
 
 def wnw_debug_advance_step_epoch(cache, delta: int):
     _ck(lib().wnw_debug_advance_step_epoch(cache, int(delta)), "wnw_debug_advance_step_epoch")
+
+
+def wnw_debug_fill_mirror_padding(cache, seq: int, byte: int):
+    _ck(lib().wnw_debug_fill_mirror_padding(cache, seq, byte), "wnw_debug_fill_mirror_padding")
+
+
+def wnw_debug_get_slot_padding(cache, seq, layer, kv_head, slot, which, chunk_tokens, head_dim, elem_bytes=2) -> np.ndarray:
+    """The rows that pad a slot's chunk to whole granules, as the bytes stored."""
+    out = np.zeros((-chunk_tokens % 16, head_dim * elem_bytes), np.uint8)
+    _ck(lib().wnw_debug_get_slot_padding(cache, seq, layer, kv_head, slot, which, out.ctypes.data_as(_vp)), "wnw_debug_get_slot_padding")
+    return out
 
 
 def wnw_get_launch_counts(cache):

@@ -714,17 +714,21 @@ __global__ void __launch_bounds__(512) wnw_prefill_retable_kernel(const __grid_c
     }
   }
 }
-// ... (3) and its slots filled from the host mirror: one CTA per slot copies the chunk's block (all tidal heads, K and V).
+// ... (3) and its slots filled from the host mirror: one CTA per slot copies the chunk's block (all tidal heads, K and V) without
+// the rows that pad a run to whole granules: nobody writes those in the mirror, and in the slots they are zero.
 __global__ void wnw_refill_slots_kernel(const __grid_constant__ CacheView cv, int b, int layer) {
   const Geometry &G = cv.geo;
   const LayerInfo li = cv.layers[layer];
   const long long bl = (long long)b * G.L + layer;
   const int slot = blockIdx.x, c = cv.slot_chunk[slot_table_off(G, (int)(cv.steps[b] & 1), bl) + slot];
   if (c < 0 || li.n_tidal == 0) return;
-  const long long n_vec = (long long)li.n_tidal * 2 * G.ncp * G.d * tidal_elem_bytes(G) / 16;
+  const int run = G.nc * G.d * tidal_elem_bytes(G) / 16, run_pad = G.ncp * G.d * tidal_elem_bytes(G) / 16 - run, n_vec = li.n_tidal * 2 * run;
   const uint4 *src = reinterpret_cast<const uint4 *>(tier_ptr(G, cv.mirror[b], mirror_off(G, li, mirror_chunks_of(G, cv.C[b]), c, 0, 0)));
   uint4 *dst = reinterpret_cast<uint4 *>(tier_ptr(G, cv.pool, pool_off(G, li, b, slot, 0, 0)));
-  for (long long i = threadIdx.x; i < n_vec; i += blockDim.x) dst[i] = src[i];
+  for (int i = threadIdx.x; i < n_vec; i += blockDim.x) {
+    const int at = i + i / run * run_pad;
+    dst[at] = src[at];
+  }
 }
 // Head-sharded step: grid (active sequence, layer).  Out: the cache's own partial sums of the layer's chunk scores, a zero
 // row where none of the layer's anchor heads is the cache's own (the row may still hold the sums taken back in an earlier

@@ -2242,6 +2242,35 @@ extern "C" wnw_status_t wnw_get_slot_kv(wnw_cache_t *c, int32_t seq, int32_t lay
   return WNW_OK;
 }
 
+extern "C" wnw_status_t wnw_debug_fill_mirror_padding(wnw_cache_t *c, int32_t seq, int32_t byte) {
+  wnw_status_t s = check_seq_layer(c, seq, 0);
+  if (s != WNW_OK) return s;
+  const Geometry &G = c->geo;
+  if (!c->seqs[seq].mirror) return WNW_OK;
+  DeviceGuard guard(c->cfg.device);
+  if ((s = drain(c)) != WNW_OK) return s;
+  const size_t row = (size_t)G.d * tidal_elem_bytes(G), runs = (size_t)mirror_chunks_of(G, c->seqs[seq].C) * c->tid_total * 2;
+  char *base = reinterpret_cast<char *>(c->seqs[seq].mirror);
+  for (size_t x = 0; x < runs; ++x) memset(base + (x * G.ncp + G.nc) * row, byte, (G.ncp - G.nc) * row);
+  return WNW_OK;
+}
+
+extern "C" wnw_status_t wnw_debug_get_slot_padding(wnw_cache_t *c, int32_t seq, int32_t layer, int32_t kv_head, int32_t slot,
+                                                   int32_t which, void *rows) {
+  wnw_status_t s = check_seq_layer(c, seq, layer);
+  if (s != WNW_OK) return s;
+  if (!rows || kv_head < 0 || kv_head >= c->geo.Hkv || which < 0 || which > 1) return WNW_ERR_INVALID_ARG;
+  if (c->cfg.mode != WNW_MODE_TIERED || c->roles[layer * c->geo.Hkv + kv_head] != ROLE_TIDAL) return WNW_ERR_INVALID_ARG;
+  if (slot < 0 || slot >= c->seqs[seq].S) return WNW_ERR_INVALID_ARG;
+  const Geometry &G = c->geo;
+  DeviceGuard guard(c->cfg.device);
+  if ((s = drain(c)) != WNW_OK) return s;
+  const long long off = pool_off(G, c->layers[layer], seq, slot, c->role_idx[layer * G.Hkv + kv_head], which) + (long long)G.nc * G.d;
+  const size_t eb = tidal_elem_bytes(G);
+  if (G.ncp > G.nc) CK(cudaMemcpy(rows, reinterpret_cast<const char *>(c->cv.pool) + off * eb, (size_t)(G.ncp - G.nc) * G.d * eb, cudaMemcpyDeviceToHost));
+  return WNW_OK;
+}
+
 extern "C" wnw_status_t wnw_get_stats(wnw_cache_t *c, wnw_stats_t *out) {
   if (!c || !out) return WNW_ERR_INVALID_ARG;
   DeviceGuard guard(c->cfg.device);

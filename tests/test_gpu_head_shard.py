@@ -161,3 +161,49 @@ def test_one_shard_with_deferred_selection_is_the_ordinary_cache():
     finally:
         wnw.wnw_destroy(h)
         o.close()
+
+
+@pytest.mark.parametrize("kv_fp8", [False, True])
+def test_padding_rows_of_the_mirror_stay_out_of_the_slots(kv_fp8):
+    """25-token chunks fill two granules partly.  The mirror's rows behind them hold whatever the pinned page held (here: NaN);
+    slots refilled after the exchange of the prefill sums, and slots recalled while decoding, keep their zero rows."""
+    d = 128 if kv_fp8 else 64
+    w = tiny_custom(n_layers=2, n_q_heads=8, n_kv_heads=4, head_dim=d, n_text=6, audio_lens=(260,), chunk=25, budget=0.3, n_steps=4,
+                    roles=[[A, T, T, F], [T, F, T, T]], region=25, jump_every=1)
+    dev = torch.device("cuda:0")
+    syn = Synth(w, seed=23)
+    sh = shard_plan(w.roles, w.n_q_heads, 1)[0]
+    h = create_shard_cache(sh, w.n_q_heads, w.n_kv_heads, d, 1, 260, w.text_capacity, w.chunk, w.budget, topk=w.topk,
+                           tidal_kv_format=wnw.WNW_TIDAL_KV_FP8_E4M3 if kv_fp8 else wnw.WNW_TIDAL_KV_BF16)
+    n_chunks, n_slots = 11, 3
+
+    def check_padding():
+        for l in range(2):
+            for head in np.nonzero(w.roles[l] == T)[0]:
+                for slot in range(n_slots):
+                    for which in (0, 1):
+                        assert not wnw.wnw_debug_get_slot_padding(h, 0, l, head, slot, which, 25, d, 1 if kv_fp8 else 2).any(), (l, head, slot, which)
+
+    try:
+        for l in range(2):
+            p = syn.prefill(0, l)
+            wnw.wnw_place_prefill(h, 0, l, p["k"].to(dev), p["v"].to(dev), p["audio_begin"], p["audio_end"], p["q_last"].to(dev))
+        wnw.wnw_debug_fill_mirror_padding(h, 0, 0xff)
+        check_padding()
+        for l in range(2):      # sums that no shard's own ranking would give: the last chunks first
+            before = wnw.wnw_get_residency(h, 0, l)[0].tolist()
+            wnw.wnw_import_prefill_tidal(h, 0, l, torch.arange(n_chunks, dtype=torch.float32, device=dev))
+            assert wnw.wnw_get_residency(h, 0, l)[0].tolist() != before
+        check_padding()
+        dec = [syn.decode(0, l) for l in range(2)]
+        scores = torch.zeros((1, 2, n_chunks), dtype=torch.float32, device=dev)
+        for t in range(w.n_steps):
+            q, kn, vn = ([dec[l][name][t][None].to(dev) for l in range(2)] for name in ("q", "k_new", "v_new"))
+            out = [torch.empty_like(x) for x in q]
+            sharded_step(h, [0], q, kn, vn, out, scores, all_reduce=lambda x: x)
+            wnw.wnw_sync(h)
+            assert all(torch.isfinite(x.float()).all() for x in out)
+        assert wnw.wnw_get_stats(h)["misses"] > 0
+        check_padding()
+    finally:
+        wnw.wnw_destroy(h)
