@@ -681,6 +681,13 @@ static void head_granules(const wnw_cache *c, int layer, int mode, const SeqHost
 // round(work / T) even pieces (at least one), the pieces go longest-first to the least loaded CTA, and T is the candidate
 // between 0.3 and three even shares of the launch that gives the shortest longest CTA under that cost model.
 constexpr int CLUSTER_MAX_PER_WARP = 8;   // granules: with more, persistent CTAs are the better cut (8 x 3000 tokens, 12 layers: 206 us at 8, 234 at 4)
+// Granules a warp of the longest head: a cluster holds 16 pieces, so a long head's warps walk ever more granules one after
+// another, where the cuts that merge through global memory (one-shot: 32 pieces a head; persistent) take half as many and pay
+// some 2.5 us for the merge.  Chained, one sequence, us a layer, cluster / other cut: 2 KV heads of 128 elements (anchor and
+// tidal) at 8 000 tokens 9.0 / 11.9, 20 000 (10 granules) 15.3 / 16.0, 24 000 (12) 18.0 / 17.7, 32 000 (16) 22.1 / 19.9, 60 000
+// 37.3 / 28.7; 8 KV heads at 20 000 15.3 / 15.8, 24 000 17.4 / 16.2, 32 000 21.4 / 18.6; 4 KV heads of 64 at 20 000 11.5 / 11.8,
+// 24 000 13.1 / 12.6.  The lines cross between 9 (e4m3) and 14 (full cache, 2 KV heads).
+constexpr int CLUSTER_LONGEST_PER_WARP = 11;
 struct CutMemo {   // piece sizes found for one work list, by the launch's head sizes
   struct Entry { std::vector<int> sizes; double T; };
   std::vector<Entry> entries;
@@ -816,13 +823,15 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
 // Chained or serial layers whose work fits one wave: the pieces of a head form (part of) a cluster and merge inside it, which
 // costs little however many there are, so heads are cut as fine as fits: two granules a warp (all bytes of a piece in flight
 // before the layer's inputs are there, one softmax step behind them), more where that would not fit one wave or where a head
-// would need more than the 16 pieces a cluster holds.  Heads are packed into clusters, most pieces first; places left over stay empty.
+// would need more than the 16 pieces a cluster holds (up to CLUSTER_LONGEST_PER_WARP).  Heads are packed into clusters, most pieces first; places left over stay empty.
 static bool build_cluster_items(const wnw_cache *c, int layer, int mode, const std::vector<int> &seq_ids,
                                 const std::vector<int> &n_gran, const std::vector<int> &n_work, std::vector<WorkItem> &items,
                                 std::vector<HeadItems> &heads, LayerWork &lw) {
   const Geometry &G = c->geo;
   const int n_heads = (int)seq_ids.size() * G.Hkv, nw = attn_warps(false);
   std::vector<int> np(n_heads), by(n_heads), first(n_heads), room;
+  for (int hd = 0; hd < n_heads; ++hd)
+    if (n_work[hd] > 16 * nw * CLUSTER_LONGEST_PER_WARP) return false;
   for (int per = 2; per <= CLUSTER_MAX_PER_WARP; ++per) {
     int most = 1;
     for (int hd = 0; hd < n_heads; ++hd) {
@@ -1556,10 +1565,8 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   // CTAs that wait for it: recall_fits_beside.)
   // Measured, back to back: 16 ragged sequences, 6 layers, 10 MB of recall a step: 320 -> 273 us; 16 x 7500 e4m3, 4 MB: 219 -> 198 us;
   // 8 x 3000, 12 layers: 201 -> 191 us; with recall at speech rate as before.
-  bool fits = beside;
-  for (const LayerWork &w : c->wl_layers) fits = fits && (w.throughput || w.cluster > 0);
   const int half = (G.L + 1) / 2;
-  if (c->cap_fold && capturing && !small && !layers_overlap(c) && fits && half < G.L &&
+  if (c->cap_fold && capturing && !small && !layers_overlap(c) && beside && half < G.L &&
       c->layers[half].upd_first < (int)c->upd_list.size()) {   // (some layer is recalled behind the step)
     c->cap_external_recall = true;
     c->cap_ext_from = half;

@@ -32,6 +32,24 @@ def test_chained_layers_clustered_pieces(n_q, n_kv, d, audio, mode):
         ls.close()
 
 
+# 1408 granules, 3 of them text, are the longest head whose pieces share a cluster; layers without a long head stay clustered
+@pytest.mark.parametrize("audio,d", [((22480,), 64), ((22481,), 64), ((22600, 500), 128), ((40000,), 128)])
+def test_chained_layers_around_the_longest_clustered_head(audio, d):
+    from parity_harness import Lockstep
+    w = tiny_custom(n_layers=4, n_q_heads=8, n_kv_heads=2, head_dim=d, n_text=27, audio_lens=audio, chunk=16, budget=0.1, n_steps=6,
+                    roles=[[A, T], [T, F], [T, A], [T, T]], region=16, jump_every=2)
+    ls = Lockstep(w, seed=47, gen_device="cuda:0")
+    try:
+        wnw.wnw_set_layer_dependency(ls.h, wnw.WNW_LAYERS_CHAINED)
+        ls.prefill(check_slots=False)
+        for t in range(6):
+            ls.decode_step(t, graph=t >= 2, check_slots=(t == 5))
+        ls.check_stats()
+        assert ls.max_out_err <= 2e-2
+    finally:
+        ls.close()
+
+
 @pytest.mark.parametrize("n_q,n_kv,d", [(8, 4, 64), (16, 1, 128), (9, 3, 128), (128, 64, 64)])
 def test_static_attention_edges(n_q, n_kv, d):
     dev = torch.device("cuda:0")
