@@ -39,14 +39,8 @@ constexpr int NW_THR = 4;  // warps of a persistent CTA (launches of more than o
 // Granules in flight per warp, and persistent CTAs per SM.  Three stages and two 4-warp CTAs per SM are what was kept after
 // measuring the alternative that shared memory allows, two-stage rings (exactly the pair a softmax step consumes) with
 // three CTAs, i.e. twelve warps, per SM: 16 x 7500 tokens chained 0.417 -> 0.402 ms and overlapped 0.344 -> 0.360 ms,
-// batch-32 ragged chained 1.31 -> 1.41 ms; two stages with two CTAs: 0.445, 0.355, 1.28 ms.  The macros are the sweep's.
-#ifndef WNW_THR_CTAS_PER_SM
-#define WNW_THR_CTAS_PER_SM 2
-#endif
-#ifndef WNW_NSTAGE_THR
-#define WNW_NSTAGE_THR 3
-#endif
-constexpr int nstage_of(int nw) { return nw == NW_THR ? WNW_NSTAGE_THR : 3; }
+// batch-32 ragged chained 1.31 -> 1.41 ms; two stages with two CTAs: 0.445, 0.355, 1.28 ms.
+constexpr int THR_CTAS_PER_SM = 2, STAGES = 3;
 
 int attn_warps(bool throughput) { return throughput ? NW_THR : NW_LAT; }
 // Merge scratch of a CTA when it sits behind the stages instead of aliasing them: (m, l) and o of every warp.
@@ -54,14 +48,13 @@ static size_t attn_scratch_bytes(int nw, int g, int d) { return (size_t)nw * 128
 // Persistent CTAs an SM holds: what the shared memory allows (stages, alignment slack, merge scratch behind the stages,
 // 1 KB the system keeps per CTA) up to what the kernel's register bound was compiled for.
 int attn_persistent_ctas_per_sm(int g, int d) {
-  const size_t per_cta = (size_t)NW_THR * nstage_of(NW_THR) * 2 * GR * d * 2 + 1024 + attn_scratch_bytes(NW_THR, g, d) + 512 + 1024;
+  const size_t per_cta = (size_t)NW_THR * STAGES * 2 * GR * d * 2 + 1024 + attn_scratch_bytes(NW_THR, g, d) + 512 + 1024;
   const int fit = (int)((228 * 1024) / per_cta);
-  const int cap = g > 8 ? 2 : WNW_THR_CTAS_PER_SM;   // registers: the two-tile variant is compiled for two CTAs per SM
-  return fit < 1 ? 1 : (fit > cap ? cap : fit);
+  return fit < 1 ? 1 : (fit > THR_CTAS_PER_SM ? THR_CTAS_PER_SM : fit);
 }
 // One-shot 8-warp CTAs can keep it there while everything fits the 227 KB a CTA may have.
 bool attn_xpref_fits(int g, int d) {
-  return (size_t)NW_LAT * nstage_of(NW_LAT) * 2 * GR * d * 2 + 1024 + attn_scratch_bytes(NW_LAT, g, d) + 512 <= 227 * 1024;
+  return (size_t)NW_LAT * STAGES * 2 * GR * d * 2 + 1024 + attn_scratch_bytes(NW_LAT, g, d) + 512 <= 227 * 1024;
 }
 
 
@@ -155,7 +148,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// 2^x in one instruction (results below the normal range come out as 0; exp2f spends three more on them)
+// 2^x in one instruction; results below the normal range come out as 0
 __device__ __forceinline__ float ex2(float x) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(r) : "f"(x));
@@ -277,7 +270,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   constexpr int KK = D / 16;              // k16 steps of QK^T; also pairs of n8 tiles of PV
   constexpr int NQ = G16 ? 4 : 2;
   constexpr bool TB = VAR == 1, F8 = VAR == 2, UNI = VAR == 3 || VAR == 4, KO = VAR == 4;
-  constexpr int NSTAGE = KO ? 2 * nstage_of(NW) : nstage_of(NW);
+  constexpr int NSTAGE = KO ? 2 * STAGES : STAGES;
   constexpr int STAGEB = KO ? TILEB : 2 * TILEB;   // a stage holds a granule's K rows, then its V rows
   static_assert(!F8 || D == 128, "an e4m3 row must fill one 128-byte swizzle atom");
 
@@ -1228,10 +1221,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
   {
     // Each thread owns four output columns of one query head.  The partials of up to MB splits are fetched in one
     // batch of independent loads (one L2 round trip); longer heads continue with an online log-sum-exp merge.
-#ifndef WNW_MERGE_BATCH
-#define WNW_MERGE_BATCH 16
-#endif
-    constexpr int MB = WNW_MERGE_BATCH;
+    constexpr int MB = 16;
     const int nvec = g * D / 4;
     const float4 *po = reinterpret_cast<const float4 *>(a.part_o + (long long)hi.first * g * D);
     const float2 *pml = a.part_ml + (long long)hi.first * g;
@@ -1294,7 +1284,7 @@ __device__ __forceinline__ void attn_body(const CacheView &cv, const AttnArgs &a
 }
 
 template <int D, bool G16, int NW, int VAR>
-__global__ void __launch_bounds__(NW * 32, NW == NW_THR ? (G16 ? 2 : WNW_THR_CTAS_PER_SM) : 1) wnw_attn_kernel(const __grid_constant__ CacheView cv,
+__global__ void __launch_bounds__(NW * 32, NW == NW_THR ? THR_CTAS_PER_SM : 1) wnw_attn_kernel(const __grid_constant__ CacheView cv,
                                                            const __grid_constant__ AttnArgs a,
                                                            const __grid_constant__ InlineItems inl,
                                                            const __grid_constant__ TmaMaps maps) {
@@ -1354,7 +1344,7 @@ static cudaError_t launch_multi_tb(const CacheView &cv, const MultiArgs &m, size
 template <int D, bool G16, int NW, int VAR>
 static cudaError_t launch_tb(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
   // stages + slack to align them to the swizzle atom + the merge scratch when it does not alias the stages
-  const size_t smem = (size_t)NW * nstage_of(NW) * 2 * GR * D * 2 + 1024 + (a.xpref ? attn_scratch_bytes(NW, cv.geo.g, D) : 0);
+  const size_t smem = (size_t)NW * STAGES * 2 * GR * D * 2 + 1024 + (a.xpref ? attn_scratch_bytes(NW, cv.geo.g, D) : 0);
   if (!a.maps) return cudaErrorInvalidValue;
   InlineItems inl;
   if (a.n_items <= INLINE_ITEMS_MAX && a.items_host) memcpy(inl.it, a.items_host, sizeof(WorkItem) * a.n_items);
@@ -1372,7 +1362,7 @@ static cudaError_t launch_tb(const CacheView &cv, const AttnArgs &a, cudaStream_
   }
   return cudaLaunchKernelEx(&cfg, wnw_attn_kernel<D, G16, NW, VAR>, cv, a, inl, *a.maps);
 }
-static size_t uniform_smem(int d) { return (size_t)NW_LAT * nstage_of(NW_LAT) * 2 * GR * d * 2 + 1024; }
+static size_t uniform_smem(int d) { return (size_t)NW_LAT * STAGES * 2 * GR * d * 2 + 1024; }
 template <int D, bool G16, int VAR>
 static cudaError_t launch_uniform_t(const CacheView &cv, const AttnArgs &a, int n_ctas, int n_rows, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
@@ -1449,7 +1439,7 @@ static bool recall_room(K *kernel, int threads, size_t dynamic_smem) {
 }
 template <int D, bool G16, int VAR>
 static bool recall_room_t(int g, AttnForm form) {
-  const size_t lat = uniform_smem(D), thr = (size_t)NW_THR * nstage_of(NW_THR) * 2 * GR * D * 2 + 1024;
+  const size_t lat = uniform_smem(D), thr = (size_t)NW_THR * STAGES * 2 * GR * D * 2 + 1024;
   const size_t lat_scratch = attn_scratch_bytes(NW_LAT, g, D), thr_scratch = attn_scratch_bytes(NW_THR, g, D);
   switch (form) {
     case FORM_PERSISTENT: return recall_room(wnw_attn_kernel<D, G16, NW_THR, VAR>, NW_THR * 32, thr + thr_scratch);
@@ -1544,7 +1534,7 @@ bool encode_store_map_e4m3(CUtensorMap *map, const void *base, unsigned long lon
 
 template <int D, bool G16, int NW>
 static cudaError_t configure_t() {
-  const size_t want = (size_t)NW * nstage_of(NW) * 2 * GR * D * 2 + 1024 + attn_scratch_bytes(NW, G16 ? 16 : 8, D);
+  const size_t want = (size_t)NW * STAGES * 2 * GR * D * 2 + 1024 + attn_scratch_bytes(NW, G16 ? 16 : 8, D);
   const int bytes = (int)std::min<size_t>(want, 227 * 1024 - 512);   // what a CTA may have, less this kernel's static shared memory
   cudaError_t e = cudaFuncSetAttribute(wnw_attn_kernel<D, G16, NW, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
@@ -1625,7 +1615,7 @@ cudaError_t launch_attn_multi(const CacheView &cv, const AttnArgs *args, int n, 
     m.l[n_used].pdl = 0; m.l[n_used].wait_inputs = 0;
     ++n_used;
     ctas += count;
-    smem = std::max(smem, (size_t)NW_LAT * nstage_of(NW_LAT) * 2 * GR * d * 2 + 1024 + (a.xpref ? attn_scratch_bytes(NW_LAT, cv.geo.g, d) : 0));
+    smem = std::max(smem, (size_t)NW_LAT * STAGES * 2 * GR * d * 2 + 1024 + (a.xpref ? attn_scratch_bytes(NW_LAT, cv.geo.g, d) : 0));
   }
   if (n_used == 0) return cudaSuccess;
   m.n = n_used; m.cta_prefix[n_used] = ctas;

@@ -270,7 +270,7 @@ cudaError_t launch_select_all_params(const CacheView &cv, const SelectArgs *laye
 cudaError_t launch_step_end(const CacheView &cv, int n_active, const int32_t *active, int appended, int32_t *bump_epoch,
                             cudaStream_t st);
 cudaError_t launch_recall(const CacheView &cv, int n_active, const int32_t *active, const int32_t *layers_dev, int n_layers,
-                          int skip_copy, bool crowded, RecallSignal sig, cudaStream_t st);   // crowded: attention launches overlap
+                          int skip_copy, bool crowded, RecallSignal sig, cudaStream_t st);   // crowded: attention keeps the memory system busy
 cudaError_t launch_place_scatter(const CacheView &cv, int b, int layer, int full_mode, const bf16 *k, const bf16 *v, int ab, int ae,
                                  int T_t, int C_b, int S_b, int S_base, bf16 *stage, cudaStream_t st);
 // np: pieces a head was cut into by the scoring launch; n_q text queries; first, last: whether the placement begins, ends with them

@@ -332,8 +332,9 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // 40 registers a thread: a CTA fits beside a resident 8-warp attention CTA, or two of four warps, of up to 216 registers.
 // 8 CTAs where layers wait for one another: the copies have the whole next step's time (config 1, 30 chained layers, recall
 // and the step's own small copies: 254 us a step with the former 128 CTAs, 238.7 with 8, 241 with 12, 243 with 16).  24 CTAs
-// where layers overlap: attention then fills the memory system, a host read takes several times as long and the step waits for
-// it (4 x 3000 tokens: 225 us a step with 8, 197 with 16, 193 with 24, 194 with 32, 198 with 48; formerly 206).
+// where attention keeps the memory system busy (overlapping layers, persistent CTAs): a host read takes several times as long
+// then and the step waits for it (4 x 3000 tokens, overlapping: 225 us a step with 8, 197 with 16, 193 with 24, 194 with 32, 198
+// with 48; formerly 206).
 //
 // With `sig` set (this kernel runs behind its step and overlaps the next one) the warp that finishes a layer last publishes the
 // layer's recall epoch, which the next step's tidal CTAs acquire.  Every step that raises the step epoch ends with EVERY layer's

@@ -150,7 +150,7 @@ struct wnw_cache {
   bool recall_fits_beside[N_ATTN_FORMS] = {};   // a recall CTA has room on an SM full of attention CTAs of that form
   cudaEvent_t ev_graph_done = nullptr, ev_recall_all = nullptr;
   static constexpr int direct_max_granules = 64;   // scale of the one-CTA rule: a head of up to 2x (overlapping layers) or x/2
-                                                   // (chained layers) this many granules (text capacity included) is not split
+                                                   // (chained layers outside clusters) this many granules (text included) is not split
   // captured step
   bool graph_capturing = false;
   cudaGraph_t graph = nullptr;
@@ -195,7 +195,7 @@ static AttnForm form_of(const LayerWork &w) {
   return w.cluster > 0 ? FORM_CLUSTER : w.throughput ? FORM_PERSISTENT : w.narrow ? FORM_NARROW : w.packed ? FORM_PACKED : FORM_ONE_SHOT;
 }
 
-// Whether attention keeps the memory system busy while recalls run.
+// Whether attention keeps the memory system busy while recalls run: overlapping layers, persistent CTAs.
 static bool recall_crowded(const wnw_cache *c) {
   bool crowded = layers_overlap(c);
   for (const LayerWork &w : c->wl_layers) crowded = crowded || w.throughput;
@@ -638,9 +638,10 @@ extern "C" wnw_status_t wnw_destroy(wnw_cache_t *c) {
 // the block scheduler and the next layers' CTAs fill the SMs that short heads free early.  Measured against the
 // persistent schedule on the batched workloads: 77 % vs 71 % and 85 % vs 82 % of the copy bandwidth.
 //
-// Layers that wait for one another (chained or serial): the span of one kernel counts.  Little work (fits one wave of
-// CTAs): small items (two granules per warp), so nearly every byte is in flight at once and the merge stays short.  Otherwise persistent 4-warp CTAs, two per
-// SM, over items sized for about one item per CTA and placed longest-first by the host.
+// Layers that wait for one another (chained or serial): the span of one kernel counts.  What fits the cluster cut takes it
+// (build_cluster_items).  What does not: one wave of one-shot CTAs where that is enough (two granules a warp or more, a head in
+// at most 32 pieces, merged through global memory: single very long sequences), else persistent 4-warp CTAs, two per SM, over
+// items sized for about one item per CTA and placed longest-first by the host.
 static int granules_per_item(const wnw_cache *c, long long total_granules, int longest_head, int n_heads, bool overlapped,
                              bool *throughput) {
   const int nw = attn_warps(false), min_gpi = nw;
@@ -651,9 +652,7 @@ static int granules_per_item(const wnw_cache *c, long long total_granules, int l
     per = std::max<long long>(per, (total_granules + cap - 1) / cap);
     return (int)((per + nw - 1) / nw * nw);
   }
-  // two granules per warp: all of an item's bytes are in flight at once and few partials are left to merge (measured on
-  // config 1, chained: 212 us per step; one granule per warp 259 us, three 237 us)
-  long long per = std::max<long long>(2 * min_gpi, (longest_head + 31) / 32);
+  long long per = std::max<long long>(2 * min_gpi, (longest_head + 31) / 32);   // two granules a warp: all of a piece's bytes in flight
   per = (per + nw - 1) / nw * nw;
   *throughput = (total_granules + per - 1) / per + n_heads > c->n_sm;   // more than one wave: build_throughput_items cuts the work
   return (int)per;
@@ -929,7 +928,7 @@ static void build_layer_items(const wnw_cache *c, int layer, int mode, const std
       const int nw_ = n_work[i * G.Hkv + h];
       int n_cta = std::max(1, (nw_ + gpi - 1) / gpi);
       // a short head stays in one CTA: up to 128 granules when layers overlap (work per launch counts), 32 when the
-      // kernel's span counts (measured, chained config 1: 298 -> 240 us per step against a threshold of 64)
+      // kernel's span counts
       if (!throughput && nw_ <= (overlapped ? 2 * c->direct_max_granules : c->direct_max_granules / 2)) n_cta = 1;
       if (batched) {   // long heads in pieces as fat as a CTA of their part of the launch
         const int nwp = attn_warps(false);
@@ -1205,7 +1204,7 @@ static wnw_status_t place_multi(wnw_cache_t *c, int32_t seq, int32_t layer, cons
         cudaGetLastError();
         return WNW_ERR_OOM_HOST;
       }
-      if (G.mirror_chunks) memset(p, 0, need);   // chunks that have not arrived yet must read as padding
+      if (G.mirror_chunks) memset(p, 0, need);   // rows that have not arrived yet are recalled with their chunk, and masked
       void *dp = nullptr;
       CK(cudaHostGetDevicePointer(&dp, p, 0));
       s.mirror = (bf16 *)p; s.mirror_cap = need;

@@ -121,14 +121,18 @@ def test_undrained_mix_of_eager_steps_and_replays(residency):
 
 @pytest.mark.parametrize("dependency,residency", [(0, 0), (1, 0), (0, 1), (1, 1)])
 def test_undrained_replays_large_launches(dependency, residency):
-    """Launches too large for the out-of-graph recall (recall stays inside the captured step); chained layers run the
-    persistent schedule.  Eager steps mixed in."""
+    """Launches that fill the machine.  Overlapping layers keep their recall inside the captured step; chained layers run the
+    persistent schedule and recall the first half of the layers inside the step, the second half behind it.  Eager steps, which
+    recall inside, mixed in."""
     w = config4(budget=0.1, chunk=25 if residency else 64, batch=12, n_steps=8)
     w.n_layers = 4; w.roles = w.roles[:4]
     a = _run(w, True, 8, dependency=dependency, residency=residency, eager_steps=(2, 5))
     b = _run(w, False, 8, dependency=dependency, residency=residency, eager_steps=(2, 5))
     _same(a, b)
-    assert b[3][2] > 8      # recall launches per layer, not one per step
+    n_recalled = sum((r == ROLE_TIDAL).any() for r in w.roles)      # (every layer of the stack has an anchor: its own tail)
+    assert all((r == ROLE_ANCHOR).any() for r in w.roles) and n_recalled == 4
+    inside = 2 if dependency == 1 else 4                              # ... of a replayed step, and one launch behind it
+    assert b[3][2] == 2 * n_recalled + 6 * (inside + (dependency == 1))
 
 
 @pytest.mark.parametrize("budget,chunk,batch,residency", [(0.2, 64, 1, 0), (0.4, 64, 2, 0), (0.2, 25, 2, 1), (0.4, 256, 3, 0)])
