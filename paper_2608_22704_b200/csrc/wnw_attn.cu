@@ -1452,13 +1452,22 @@ static bool recall_room_t(int g, AttnForm form) {
              recall_room(wnw_attn_multi_kernel<D, G16, NW_LAT, VAR>, NW_LAT * 32, lat + lat_scratch);
   }
 }
-bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, AttnForm form) {
+static bool find_recall_room(int g, int d, bool kv8, bool token_base, AttnForm form) {
   if (d == 128) {
     if (g > 8) return kv8 ? recall_room_t<128, true, 2>(g, form) : token_base ? recall_room_t<128, true, 1>(g, form) : recall_room_t<128, true, 0>(g, form);
     return kv8 ? recall_room_t<128, false, 2>(g, form) : token_base ? recall_room_t<128, false, 1>(g, form) : recall_room_t<128, false, 0>(g, form);
   }
   if (g > 8) return token_base ? recall_room_t<64, true, 1>(g, form) : recall_room_t<64, true, 0>(g, form);
   return token_base ? recall_room_t<64, false, 1>(g, form) : recall_room_t<64, false, 0>(g, form);
+}
+bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, AttnForm form) {   // (a function's attributes take some 30 us: asked once)
+  static std::mutex mu;
+  static std::map<std::tuple<int, int, bool, bool, int>, bool> known;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto key = std::make_tuple(g, d, kv8, token_base, (int)form);
+  auto it = known.find(key);
+  if (it == known.end()) it = known.emplace(key, find_recall_room(g, d, kv8, token_base, form)).first;
+  return it->second;
 }
 int attn_cluster_room(int device, int g, int d, int cluster) {   // (an occupancy query takes some 0.2 ms: asked once per shape)
   static std::mutex mu;
