@@ -35,3 +35,14 @@ def test_both_arms_use_the_same_config_keys():
     assert ours == bench.method_config(w)
     assert isinstance(ours["layers"], int) and ours["tidal_kv"] == "bf16" and ours["score_scope"] == "per layer"
     assert bench.method_config(w, 3, 1, 1, True)["layer_issue"] == "all_layers_together"
+
+
+def test_roofline_names_the_kernel_that_the_step_launches():
+    sys.path.insert(0, ROOT)
+    import bench
+    one, many = bench.make_workload("cfg1", 4, 0), bench.make_workload("hbm", 4, 0)
+    assert [bench.attention_kernel(one, dep, False) for dep in (0, 1, 2, 3)] == [
+        "wnw_attn_kernel", "wnw_attn_cluster_kernel", "wnw_attn_cluster_kernel", "wnw_attn_multi_kernel"]
+    assert bench.attention_kernel(many, 1, False) == "wnw_attn_kernel" == bench.attention_kernel(one, 3, True)
+    traffic = json.load(open(os.path.join(ROOT, "profiles", "attn_traffic.json")))
+    assert bench.attention_kernel(one, 1, False) in traffic["source"] and traffic[one.name] > 0
