@@ -39,6 +39,7 @@ struct LayerWork {
   bool narrow = false;                             // one-shot CTAs of four warps, two per SM
   int cluster = 0;                                 // chained layers of one wave: CTAs per cluster
   bool packed = false;                             // one-shot CTAs that serve several short heads each
+  int n_tidal_items = 0;                           // items of tidal heads
   int head_items_off = 0;                          // offset in the list's HeadItems
 };
 
@@ -1056,6 +1057,10 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
     build_layer_items(c, l, mode, c->active, items, heads, c->wl_layers[l], order, ranges, &memo);
     c->wl_layers[l].part_off = part_total;
     part_total += (size_t)c->wl_layers[l].n_items;
+    for (int x = 0; x < c->wl_layers[l].n_items; ++x) {
+      const WorkItem &it = items[c->wl_layers[l].first_item + x];
+      c->wl_layers[l].n_tidal_items += it.role == ROLE_TIDAL && it.h >= 0;
+    }
   }
   if (part_total > c->part_cap_total) {  // one partial region per layer
     float *po = nullptr; float2 *pm = nullptr;
@@ -1531,15 +1536,17 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   // there.  (A caller's own capture of an eager step keeps everything inside, too: nothing could be issued behind it.)
   // Small launches add up: a layer's CTAs start beside its predecessors', and while the first layer's tidal CTAs wait for the
   // recall the later ones can take every SM.  The recall starts all the same where one of its CTAs has room beside the attention
-  // CTAs, or where the CTAs that can be there at once (all layers'; one layer's in plain stream order; the tidal part of a launch
-  // of all layers, the others end by themselves) are fewer than the SMs.  Elsewhere it stays inside the step: kernels of eight
+  // CTAs, or where the CTAs that can wait there at once are fewer than the SMs: with chained layers everybody's, in plain stream
+  // order one layer's, with overlapping layers the tidal heads' (and of each launch the one that waits for its predecessor to end),
+  // in a launch of all layers its tidal part; the others end by themselves.  Elsewhere it stays inside the step: kernels of eight
   // warps and more than 216 registers a thread (groups of more than 8 query heads, as a rule), packed CTAs of 8 heads of 128
   // elements (all of the shared memory).
   bool small = true;   // no launch can fill the machine with CTAs that wait
   bool beside = true;
   int there = 0;
   for (const LayerWork &w : c->wl_layers) {
-    const int n = w.n_ctas > 0 ? w.n_ctas : w.n_items, wait = together && w.packed ? n - w.n_ctas_free : n;
+    const int n = w.n_ctas > 0 ? w.n_ctas : w.n_items;
+    const int wait = together ? n - (w.packed ? w.n_ctas_free : 0) : layers_overlap(c) ? std::min(n, w.n_tidal_items + 1) : n;
     small = small && !w.throughput && n <= c->n_sm / 2;
     beside = beside && c->recall_fits_beside[together ? FORM_TOGETHER : form_of(w)];
     there = c->layer_dependency == WNW_LAYERS_SERIAL ? std::max(there, wait) : there + wait;

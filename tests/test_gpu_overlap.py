@@ -243,15 +243,26 @@ def _replays(w, dependency, n, seed):
         ls.close()
 
 
-@pytest.mark.parametrize("n_q,dependency,outside", [(32, wnw.WNW_LAYERS_CHAINED, False), (32, wnw.WNW_LAYERS_INDEPENDENT, False),
-                                                    (32, wnw.WNW_LAYERS_SERIAL, True), (16, wnw.WNW_LAYERS_CHAINED, True)])
-def test_recall_leaves_the_step_where_it_can_start(n_q, dependency, outside):
-    """Sixteen query heads a KV head: no recall CTA has room beside the attention CTAs, and the layers' CTAs together outnumber
-    the SMs.  Recall then stays inside the step, replayed or not (in plain stream order one layer's CTAs leave SMs free)."""
-    w = tiny_custom(n_layers=12, n_q_heads=n_q, n_kv_heads=2, head_dim=128, n_text=14, audio_lens=(4200, 3900), chunk=64, budget=0.25,
-                    n_steps=5, roles=[[ROLE_ANCHOR, ROLE_TIDAL], [ROLE_TIDAL, ROLE_TIDAL]] * 6, region=64, jump_every=2)
+@pytest.mark.parametrize("n_q,batch,dependency,outside", [(32, 2, wnw.WNW_LAYERS_CHAINED, False), (32, 8, wnw.WNW_LAYERS_INDEPENDENT, False),
+                                                          (32, 2, wnw.WNW_LAYERS_INDEPENDENT, True), (32, 2, wnw.WNW_LAYERS_SERIAL, True),
+                                                          (16, 2, wnw.WNW_LAYERS_CHAINED, True)])
+def test_recall_leaves_the_step_where_it_can_start(n_q, batch, dependency, outside):
+    """Sixteen query heads a KV head: no recall CTA has room beside the attention CTAs.  Recall stays inside the step, replayed or
+    not, where the CTAs that can wait for it at once outnumber the SMs: all layers' of a chained step, the tidal heads' (144 and
+    one a launch for eight sequences) of overlapping ones; in plain stream order one layer's leave SMs free."""
+    w = tiny_custom(n_layers=12, n_q_heads=n_q, n_kv_heads=2, head_dim=128, n_text=14, audio_lens=(4200, 3900) * (batch // 2), chunk=64,
+                    budget=0.25, n_steps=5, roles=[[ROLE_ANCHOR, ROLE_TIDAL], [ROLE_TIDAL, ROLE_TIDAL]] * 6, region=64, jump_every=2)
     eager, replayed = _replays(w, dependency, 4, 11)
     assert (eager[2], replayed[2]) == ((1, 4) if outside else (12, 48))
+
+
+def test_chained_one_shot_launches_that_fill_the_machine_split_their_recall():
+    """One very long sequence: its heads are too long for clusters, a layer's one-shot CTAs take more than half the SMs.  Replayed,
+    half of the four layers recalls inside the step and half behind it; an eager step recalls inside."""
+    w = tiny_custom(n_layers=4, n_q_heads=32, n_kv_heads=8, head_dim=128, n_text=14, audio_lens=(24000,), chunk=64, budget=0.2, n_steps=6,
+                    roles=[[ROLE_ANCHOR] + [ROLE_TIDAL] * 5 + [ROLE_FIXED] * 2] * 4, region=64, jump_every=2)
+    eager, replayed = _replays(w, wnw.WNW_LAYERS_CHAINED, 5, 13)
+    assert (eager[2], replayed[2]) == (4, 5 * 3)
 
 
 def test_selection_waits_for_the_recall_only_beside_free_sms():
