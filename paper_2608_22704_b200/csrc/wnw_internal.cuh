@@ -173,6 +173,7 @@ struct AttnArgs {
   const WorkItem *items;         // device copy of the items
   const WorkItem *items_host;    // host copy (the launcher inlines short lists into the kernel parameters)
   const TmaMaps *maps;           // host pointer; passed to the kernel by value
+  const TmaMaps *maps_rows;      // the same with boxes of K or V rows alone
   int32_t n_items;
   const int32_t *order;          // persistent schedule (throughput regime), else null: order[cta_ranges[c] .. cta_ranges[c+1]) are
   const int32_t *cta_ranges;     //   the item indices CTA c processes; n_ctas CTAs are launched
@@ -182,6 +183,7 @@ struct AttnArgs {
   const int32_t *expect_epoch;   //   previous step, which runs outside the captured graph, has landed); null otherwise
   int32_t narrow;                // one-shot CTAs of four warps, two per SM, instead of eight
   int32_t cluster;               // > 0: CTAs in clusters of this size, item x is CTA x, all items of a head in one cluster
+  int32_t short_pieces;          // ... and no item of more than SHORT_GRANULES granules: SHORT_*, else 0
   int32_t pdl;                   // launch with programmatic stream serialization (previous stream op is a layer kernel)
   int xpref;        // the CTAs serve several work items each and keep their copy pipeline running across them
   int wait_inputs;  // q/k_new/v_new come from the preceding work on the stream: wait for it before reading them
@@ -293,6 +295,14 @@ cudaError_t launch_prefill_tidal_sum(const CacheView &cv, int b, int layer, floa
 cudaError_t launch_prefill_retable(const CacheView &cv, int b, int layer, const float *sums, cudaStream_t st);
 cudaError_t launch_copy_plan(const uint4 *src_host_mapped, uint4 *dst, long long n_vec, int n_ctas, cudaStream_t st);
 cudaError_t configure_attn_kernels();
+// clustered layers of short pieces (wnw_attn_short.cu)
+constexpr int SHORT_GRANULES = 16;   // two granules for each of eight warps
+enum { SHORT_WIDE = 1, SHORT_DENSE = 2 };   // one CTA to an SM; two
+cudaError_t launch_attn_short(const CacheView &cv, const AttnArgs &a, cudaStream_t st);
+cudaError_t configure_short_kernels();
+int short_cluster_room(int g, int d, bool dense, int cluster);
+bool short_leaves_recall_room(int g, int d, bool token_base, bool dense, int recall_threads);
+bool recall_room(const void *kernel, int threads, size_t dynamic_smem, int recall_threads);   // room for a recall CTA on an SM full of that kernel's CTAs
 // the CTAs of several layers' launches (one-shot variant) in one launch
 // CTAs [first[l], first[l] + count[l]) of every layer l (null: all of them); pdl: launched programmatically dependent on
 // what precedes it in the stream
@@ -309,13 +319,13 @@ cudaError_t launch_quantise_stage(const CacheView &cv, int b, int layer, bf16 *s
 cudaError_t configure_select_kernel();
 constexpr int SELECT_SMEM_CAP = 200 * 1024;  // dynamic shared memory the selection kernel may be launched with
 bool attn_xpref_fits(int g, int d);  // a one-shot CTA can hold its merge scratch behind the copy stages
-// The attention kernels as a step launches them: persistent CTAs, one-shot CTAs in clusters, of eight warps, of four, of eight
+// The attention kernels as a step launches them: persistent CTAs, one-shot CTAs in clusters, the same of short pieces, of eight warps, of four, of eight
 // with several heads packed into a CTA, the CTAs of all layers together.
-enum AttnForm { FORM_PERSISTENT, FORM_CLUSTER, FORM_ONE_SHOT, FORM_NARROW, FORM_PACKED, FORM_TOGETHER, N_ATTN_FORMS };
+enum AttnForm { FORM_PERSISTENT, FORM_CLUSTER, FORM_SHORT, FORM_SHORT_DENSE, FORM_ONE_SHOT, FORM_NARROW, FORM_PACKED, FORM_TOGETHER, N_ATTN_FORMS };
 // whether an SM that holds as many CTAs of that form as it can has room left for a recall CTA
-bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, AttnForm form);
-constexpr int RECALL_THREADS = 256, RECALL_REGS = RECALL_THREADS * 40;   // of a recall CTA
-int attn_cluster_room(int device, int g, int d, int cluster);   // clusters of that size that fit the GPU at once
+bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, AttnForm form, bool crowded);
+constexpr int RECALL_THREADS = 64, RECALL_THREADS_CROWDED = 256, RECALL_REGS_PER_THREAD = 40;   // of a recall CTA (crowded: see launch_recall)
+int attn_cluster_room(int device, int g, int d, int cluster, int short_pieces);   // clusters of that size that fit the GPU at once
 int attn_warps(bool throughput);  // warps per attention CTA in the latency / throughput variant
 int attn_persistent_ctas_per_sm(int g, int d);  // persistent (throughput-variant) CTAs that fit one SM
 

@@ -326,27 +326,27 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // flight reach the full rate (64 KB: 39.5 GB/s), every further request only waits in the link's queue, and so does whatever
 // else crosses the link meanwhile, the GPU's own command fetches among them (a small copy or kernel on another stream,
 // host round trip: 11 us alone, 18 us beside 128 KB, 61 us beside 512 KB, 116 us beside 2 MB in flight).  So the grid is
-// a few CTAs of 8 warps with RECALL_U 16-byte loads in flight per lane, whatever there is to copy, and the warps work
+// 64 warps with RECALL_U 16-byte loads in flight per lane, whatever there is to copy, and the warps work
 // independently: the blocks of a launch are cut into pieces of a warp's batch and dealt round robin ACROSS block and layer
 // borders, so that all warps have work and nothing waits at a barrier.
-// 40 registers a thread: a CTA fits beside a resident 8-warp attention CTA, or two of four warps, of up to 216 registers.
-// 8 CTAs where layers wait for one another: the copies have the whole next step's time (config 1, 30 chained layers, recall
-// and the step's own small copies: 254 us a step with the former 128 CTAs, 238.7 with 8, 241 with 12, 243 with 16).  24 CTAs
-// where attention keeps the memory system busy (overlapping layers, persistent CTAs): a host read takes several times as long
-// then and the step waits for it (4 x 3000 tokens, overlapping: 225 us a step with 8, 197 with 16, 193 with 24, 194 with 32, 198
-// with 48; formerly 206).
+// 40 registers a thread.  64 warps, two to a CTA (one fits beside an 8-warp attention CTA of up to 240 registers, two of up to 120),
+// where layers wait for one another: the copies have the whole next step's time (config 1, 30 chained layers, recall and the step's
+// own small copies: 254 us a step with 1 024 warps, 238.7 with 64, 241 with 96, 243 with 128).  192 warps, eight to a CTA (on 96 SMs
+// instead of 24 they disturb attention: 16 ragged sequences 49.7 -> 50.4 ms a request), where attention keeps the memory system busy
+// (overlapping layers, persistent CTAs): a host read takes several times as long then and the step waits for it (4 x 3000 tokens,
+// overlapping: 225 us a step with 64, 197 with 128, 193 with 192, 194 with 256, 198 with 384; 206 with 1 024).
 //
 // With `sig` set (this kernel runs behind its step and overlaps the next one) the warp that finishes a layer last publishes the
 // layer's recall epoch, which the next step's tidal CTAs acquire.  Every step that raises the step epoch ends with EVERY layer's
 // word raised, also those of layers that recalled inside the step (`landed`): which layers a step's tidal CTAs wait for depends
 // on how that step is issued, and the next one may be issued another way.
 // ------------------------------------------------------------------------------------------------
-constexpr int RECALL_CTAS = 8, RECALL_CTAS_CROWDED = 24, RECALL_WARPS = RECALL_THREADS / 32, RECALL_U = 4;
-__global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
+constexpr int RECALL_CTAS = 32, RECALL_CTAS_CROWDED = 24, RECALL_U = 4;
+__global__ void __launch_bounds__(RECALL_THREADS_CROWDED, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
                                                                           const int32_t *active, const int32_t *layers,
                                                                           int n_layers, int skip_copy, RecallSignal sig) {
   const Geometry &G = cv.geo;
-  const int lane = threadIdx.x & 31, n_warps = gridDim.x * RECALL_WARPS, w = blockIdx.x * RECALL_WARPS + (threadIdx.x >> 5);
+  const int lane = threadIdx.x & 31, warps = blockDim.x >> 5, n_warps = gridDim.x * warps, w = blockIdx.x * warps + (threadIdx.x >> 5);
   if (sig.epoch_words && w == 0)   // copies that landed before this kernel started
     for (int x = lane; x < sig.n_landed; x += 32)
       asm volatile("st.release.gpu.global.s32 [%0], %1;\n" ::"l"(sig.epoch_words + sig.landed[x]), "r"(sig.publish_epoch) : "memory");
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(RECALL_WARPS * 32, 6) wnw_recall_kernel(const 
 cudaError_t launch_recall(const CacheView &cv, int n_active, const int32_t *active, const int32_t *layers_dev, int n_layers,
                           int skip_copy, bool crowded, RecallSignal sig, cudaStream_t st) {
   if (n_layers <= 0 || n_active <= 0) return cudaSuccess;
-  wnw_recall_kernel<<<crowded ? RECALL_CTAS_CROWDED : RECALL_CTAS, RECALL_WARPS * 32, 0, st>>>(cv, n_active, active, layers_dev, n_layers, skip_copy, sig);
+  wnw_recall_kernel<<<crowded ? RECALL_CTAS_CROWDED : RECALL_CTAS, crowded ? RECALL_THREADS_CROWDED : RECALL_THREADS, 0, st>>>(cv, n_active, active, layers_dev, n_layers, skip_copy, sig);
   return cudaGetLastError();
 }
 

@@ -38,6 +38,7 @@ struct LayerWork {
   int n_ctas_anchor = 0; // ... and the first n_ctas_anchor of those hold the anchor heads (what the step's selection waits for)
   bool narrow = false;                             // one-shot CTAs of four warps, two per SM
   int cluster = 0;                                 // chained layers of one wave: CTAs per cluster
+  int short_pieces = 0;                            // ... of at most SHORT_GRANULES granules each: SHORT_*
   bool packed = false;                             // one-shot CTAs that serve several short heads each
   int n_tidal_items = 0;                           // items of tidal heads
   int head_items_off = 0;                          // offset in the list's HeadItems
@@ -66,7 +67,7 @@ struct wnw_cache {
   std::vector<uint8_t> anchor_layer;   // [L] the layer has an anchor head (on any shard, when the cache holds one shard of the heads)
   bool scores_exported = false, scores_imported = false;   // head-sharded step: where the exchange stands
   int tid_total = 0, n_sm = 148;
-  int cluster_room[3] = {0, 0, 0};   // attention clusters of 4, 8 and 16 CTAs that fit the GPU at once
+  int cluster_room[3][3] = {};   // attention clusters of 4, 8 and 16 CTAs that fit the GPU at once; [SHORT_*]: of short pieces
   std::vector<SeqHost> seqs;
   std::vector<void *> dev_allocs;
   char *small_block = nullptr;      // where the next small device array goes
@@ -74,6 +75,7 @@ struct wnw_cache {
   std::vector<bf16 *> mirror_ptrs;  // host copy of cv.mirror
   bf16 *stage = nullptr;
   TmaMaps maps_decode, maps_prefill;  // TMA descriptors: cache stores; prefill scoring reads the staging copy as `anchor`
+  TmaMaps maps_rows;                  // the cache stores, K and V rows apart (short pieces)
   int32_t *d_iota = nullptr, *d_active = nullptr;
   // step state
   std::vector<int> active;
@@ -148,7 +150,7 @@ struct wnw_cache {
   int32_t *d_recall_epoch = nullptr, *d_recall_ctr = nullptr, *d_step_epoch = nullptr;
   bool cap_external_recall = false, graph_external_recall = false, recall_all_pending = false;
   int cap_ext_from = 0, graph_ext_from = 0;   // first layer whose table updates are recalled outside the step
-  bool recall_fits_beside[N_ATTN_FORMS] = {};   // a recall CTA has room on an SM full of attention CTAs of that form
+  bool recall_fits_beside[2][N_ATTN_FORMS] = {};   // [crowded]: a recall CTA has room on an SM full of attention CTAs of that form
   cudaEvent_t ev_graph_done = nullptr, ev_recall_all = nullptr;
   static constexpr int direct_max_granules = 64;   // scale of the one-CTA rule: a head of up to 2x (overlapping layers) or x/2
                                                    // (chained layers outside clusters) this many granules (text included) is not split
@@ -193,7 +195,7 @@ static bool layers_overlap(const wnw_cache *c) {
 }
 
 static AttnForm form_of(const LayerWork &w) {
-  return w.cluster > 0 ? FORM_CLUSTER : w.throughput ? FORM_PERSISTENT : w.narrow ? FORM_NARROW : w.packed ? FORM_PACKED : FORM_ONE_SHOT;
+  return w.cluster > 0 ? (w.short_pieces == SHORT_DENSE ? FORM_SHORT_DENSE : w.short_pieces ? FORM_SHORT : FORM_CLUSTER) : w.throughput ? FORM_PERSISTENT : w.narrow ? FORM_NARROW : w.packed ? FORM_PACKED : FORM_ONE_SHOT;
 }
 
 // Whether attention keeps the memory system busy while recalls run: overlapping layers, persistent CTAs.
@@ -370,11 +372,12 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
   cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
   CKE(configure_attn_kernels());
   CKE(configure_select_kernel());
-  for (int k = 0; k < N_ATTN_FORMS; ++k)
-    c->recall_fits_beside[k] = attn_leaves_recall_room(cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim,
+  for (int k = 0; k < 2 * N_ATTN_FORMS; ++k)
+    c->recall_fits_beside[k / N_ATTN_FORMS][k % N_ATTN_FORMS] = attn_leaves_recall_room(cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim,
                                                        cfg->mode == WNW_MODE_TIERED && cfg->tidal_kv_format == WNW_TIDAL_KV_FP8_E4M3,
-                                                       cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE, (AttnForm)k);
-  for (int k = 0; k < 3; ++k) c->cluster_room[k] = attn_cluster_room(cfg->device, cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim, 4 << k);
+                                                       cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE, (AttnForm)(k % N_ATTN_FORMS), k >= N_ATTN_FORMS);
+  for (int s = 0; s < 3; ++s)
+    for (int k = 0; k < 3; ++k) c->cluster_room[s][k] = attn_cluster_room(cfg->device, cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim, 4 << k, s);
   const int L = cfg->n_layers, Hkv = cfg->n_kv_heads, d = cfg->head_dim, nc = cfg->chunk_tokens;
   const bool full = cfg->mode == WNW_MODE_FULL;
   c->roles.assign(cfg->roles, cfg->roles + (size_t)L * Hkv);
@@ -535,6 +538,8 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
     bool ok = store(&c->maps_decode.text, cv.text, r_text, G.T_cap_pad, 2) && store(&c->maps_decode.anchor, cv.anchor, r_anchor, G.T_a_pad, 2) &&
               store(&c->maps_decode.fixed, cv.fixed, r_fixed, (long long)G.FB * G.ncp, 2);
     ok = ok && (G.kv8 && r_pool ? encode_store_map_e4m3(&c->maps_decode.pool, cv.pool, r_pool, G.ncp) : store(&c->maps_decode.pool, cv.pool, r_pool, G.ncp, 2));
+    ok = ok && store(&c->maps_rows.text, cv.text, r_text, G.T_cap_pad, 1) && store(&c->maps_rows.anchor, cv.anchor, r_anchor, G.T_a_pad, 1) &&
+         store(&c->maps_rows.fixed, cv.fixed, r_fixed, (long long)G.FB * G.ncp, 1) && (G.kv8 || store(&c->maps_rows.pool, cv.pool, r_pool, G.ncp, 1));
     c->maps_prefill = c->maps_decode;   // the scoring pass reads K alone, the staging copy as the anchor store
     ok = ok && store(&c->maps_prefill.text, cv.text, r_text, G.T_cap_pad, 1) && (full || store(&c->maps_prefill.anchor, c->stage, r_stage, G.T_a_pad, 1));
     if (!ok) return fail(WNW_ERR_CUDA);
@@ -820,6 +825,12 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   lw.packed = true;   // the pipeline runs across a CTA's items (its merge scratch sits behind the stages)
 }
 
+// Short pieces: a head of at most 256 granules in pieces of 16, wnw_attn_short_kernel, as wide CTAs (one to an SM, all fragments ahead
+// of the query) where the clusters of two layers fit the GPU side by side, so that a layer's bytes land while its predecessor runs;
+// else dense ones, two to an SM.  Chained, us a replayed step of 30 layers, 32 query heads on 8 KV heads of 128, wide / dense / the
+// cut below: 3000 tokens (3 clusters of 16) 140 / 146 / 154; 2 x 3000 (6) 206 / 157 / 225; 4 x 1000 196 / 163 / 211; the paper's form
+// (4) 182 / 154 / 204; 1000 tokens, full cache (8 clusters of 8) 117 / 127 / 132.
+//
 // Chained or serial layers whose work fits one wave: the pieces of a head form (part of) a cluster and merge inside it, which
 // costs little however many there are, so heads are cut as fine as fits: two granules a warp (all bytes of a piece in flight
 // before the layer's inputs are there, one softmax step behind them), more where that would not fit one wave or where a head
@@ -832,10 +843,14 @@ static bool build_cluster_items(const wnw_cache *c, int layer, int mode, const s
   std::vector<int> np(n_heads), by(n_heads), first(n_heads), room;
   for (int hd = 0; hd < n_heads; ++hd)
     if (n_work[hd] > 16 * nw * CLUSTER_LONGEST_PER_WARP) return false;
-  for (int per = 2; per <= CLUSTER_MAX_PER_WARP; ++per) {
+  // per = 1: pieces of at most SHORT_GRANULES granules whatever they hold, which wnw_attn_short_kernel takes (bf16 tiers)
+  bool may_be_short = !G.kv8;
+  for (int hd = 0; hd < n_heads; ++hd) may_be_short = may_be_short && n_gran[hd] <= 16 * SHORT_GRANULES;
+  for (int per = may_be_short ? 1 : 2; per <= CLUSTER_MAX_PER_WARP; ++per) {
     int most = 1;
     for (int hd = 0; hd < n_heads; ++hd) {
-      np[hd] = std::max(1, std::min(16, (n_work[hd] + per * nw - 1) / (per * nw)));
+      np[hd] = per == 1 ? std::max(1, (n_gran[hd] + SHORT_GRANULES - 1) / SHORT_GRANULES)
+                        : std::max(1, std::min(16, (n_work[hd] + per * nw - 1) / (per * nw)));
       most = std::max(most, np[hd]);
       by[hd] = hd;
     }
@@ -849,8 +864,11 @@ static bool build_cluster_items(const wnw_cache *c, int layer, int mode, const s
       first[hd] = (int)x * size + size - room[x];
       room[x] -= np[hd];
     }
-    if ((int)room.size() > c->cluster_room[k]) continue;
+    const int n_cl = (int)room.size();
+    const int form = per > 1 ? 0 : 2 * n_cl <= c->cluster_room[SHORT_WIDE][k] ? SHORT_WIDE : SHORT_DENSE;
+    if (n_cl > c->cluster_room[form][k]) continue;
     lw.cluster = size;
+    lw.short_pieces = form;
     items.resize(lw.first_item + room.size() * size, WorkItem{0, -1, 0, 0, seq_ids[0], ROLE_ANCHOR, 0, 0, 0, 0, 0, 0, 0});
     for (int hd = 0; hd < n_heads; ++hd) {
       const int i = hd / G.Hkv, h = hd % G.Hkv, n = n_gran[hd];
@@ -1539,8 +1557,9 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   // CTAs, or where the CTAs that can wait there at once are fewer than the SMs: with chained layers everybody's, in plain stream
   // order one layer's, with overlapping layers the tidal heads' (and of each launch the one that waits for its predecessor to end),
   // in a launch of all layers its tidal part; the others end by themselves.  Elsewhere it stays inside the step: kernels of eight
-  // warps and more than 216 registers a thread (groups of more than 8 query heads, as a rule), packed CTAs of 8 heads of 128
-  // elements (all of the shared memory).
+  // warps and more than 240 registers a thread (groups of more than 8 query heads of 128 elements outside short pieces; 216 where
+  // attention crowds the memory system and recall CTAs are larger), packed CTAs of 8 heads of 128 elements (all of the shared memory).
+  const bool crowded = recall_crowded(c);
   bool small = true;   // no launch can fill the machine with CTAs that wait
   bool beside = true;
   int there = 0;
@@ -1548,7 +1567,7 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
     const int n = w.n_ctas > 0 ? w.n_ctas : w.n_items;
     const int wait = together ? n - (w.packed ? w.n_ctas_free : 0) : layers_overlap(c) ? std::min(n, w.n_tidal_items + 1) : n;
     small = small && !w.throughput && n <= c->n_sm / 2;
-    beside = beside && c->recall_fits_beside[together ? FORM_TOGETHER : form_of(w)];
+    beside = beside && c->recall_fits_beside[crowded][together ? FORM_TOGETHER : form_of(w)];
     there = c->layer_dependency == WNW_LAYERS_SERIAL ? std::max(there, wait) : there + wait;
   }
   small = small && (beside || there < c->n_sm);
@@ -1778,7 +1797,7 @@ static wnw_status_t decode_layer_impl(wnw_cache *c, int want_mode, int32_t layer
   a.mode = tiered ? ATTN_DECODE : ATTN_FULL; a.layer = layer; a.li = li; a.n_active = n_active; a.has_new = has_new;
   a.score_on = tiered && li.n_anchor > 0;
   a.active = c->d_active; a.items = c->d_items + lw.first_item; a.items_host = c->h_items.data() + lw.first_item;
-  a.n_items = lw.n_items; a.maps = &c->maps_decode; a.throughput = lw.throughput; a.cluster = lw.cluster; a.narrow = lw.narrow;
+  a.n_items = lw.n_items; a.maps = &c->maps_decode; a.throughput = lw.throughput; a.cluster = lw.cluster; a.short_pieces = lw.short_pieces; a.maps_rows = &c->maps_rows; a.narrow = lw.narrow;
   if (lw.n_ctas > 0) {
     a.order = c->d_sched + lw.order_off; a.cta_ranges = c->d_sched + c->sched_ranges_base + lw.ranges_off; a.n_ctas = lw.n_ctas;
     a.xpref = lw.packed;

@@ -32,6 +32,28 @@ def test_chained_layers_clustered_pieces(n_q, n_kv, d, audio, mode):
         ls.close()
 
 
+# Short pieces of one and of two CTAs to an SM (the fourth cluster of 16 decides): one piece and 16 of 16 granules exactly, one granule
+# more, groups with padding heads, the new token's row in either half of a granule and across two; chunks that fill granules partly
+@pytest.mark.parametrize("n_q,n_kv,d,chunk,audio,n_text", [
+    (8, 2, 128, 16, (224,), 6), (8, 2, 128, 16, (4064,), 14), (8, 2, 128, 16, (4065,), 14),                  # wide; 16 pieces; beyond
+    (12, 4, 128, 16, (4000, 3900, 17), 6), (8, 4, 64, 16, (4064, 4064, 900, 60), 15), (64, 4, 128, 16, (2000,) * 4, 7),   # dense
+    (64, 4, 64, 25, (1500, 2500, 1700, 26), 13), (10, 2, 128, 25, (1990,) * 8, 7), (5, 5, 64, 16, (300,), 0)])
+def test_chained_layers_of_short_pieces(n_q, n_kv, d, chunk, audio, n_text):
+    from parity_harness import Lockstep
+    roles = [[(A, T, F, T, A)[(h + l) % 5] for h in range(n_kv)] for l in range(3)]
+    w = tiny_custom(n_layers=3, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=d, n_text=n_text, audio_lens=audio, chunk=chunk, budget=0.25, n_steps=6,
+                    roles=roles, region=chunk, jump_every=2)
+    ls = Lockstep(w, seed=53, oracle_seqs=[0, len(audio) - 1] if len(audio) > 1 else [0])
+    try:
+        wnw.wnw_set_layer_dependency(ls.h, wnw.WNW_LAYERS_CHAINED)
+        ls.prefill()
+        for t in range(6):
+            ls.decode_step(t, graph=t >= 2)
+        assert ls.max_out_err <= 2e-2
+    finally:
+        ls.close()
+
+
 # 1408 granules, 3 of them text, are the longest head whose pieces share a cluster; layers without a long head stay clustered
 @pytest.mark.parametrize("audio,d", [((22480,), 64), ((22481,), 64), ((22600, 500), 128), ((40000,), 128)])
 def test_chained_layers_around_the_longest_clustered_head(audio, d):
