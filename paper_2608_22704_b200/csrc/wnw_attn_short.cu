@@ -1,5 +1,5 @@
-// Chained or serial layers whose heads are cut into pieces of at most two granules a warp, all pieces of a head in one
-// thread-block cluster: the layer's span is what counts (sm_100a).
+// Chained or serial layers whose heads are cut into pieces of at most two granules a warp, the pieces of a head in one
+// thread-block cluster or, of long heads, in several (PARTS): the layer's span is what counts (sm_100a).
 //
 // What bounds such a layer is a chain of latencies, not bytes (config 1 moves 4 MB a layer, 0.6 us of HBM): inputs visible, query
 // into registers, K q^T, softmax, P V, merge over the warps, merge over the head's pieces, output.  wnw_attn_cluster_kernel gives
@@ -47,7 +47,7 @@ struct ShortShape {
 
 // tokens x heads accumulators in units of four values as a lane holds them: heads 2p and 2p + 1 at d = 16 t + r and 16 t + r + 8.
 // Unit u = p * D / 2 + 8 t + r; piece u % np finishes it, in place u / np of its receive buffer.
-template <int D, bool G16, bool TB, bool DENSE>
+template <int D, bool G16, bool TB, bool DENSE, bool PARTS>
 __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
                                                                        const __grid_constant__ TmaMaps maps) {
   typedef ShortShape<D, G16, DENSE> X;
@@ -408,6 +408,7 @@ __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __gri
   timed_out = __any_sync(0xffffffffu, timed_out);
   if (timed_out && lane == 0 && cv.status) atomicOr(cv.status, STATUS_TIMEOUT);
 
+  const ItemPart pt = PARTS ? a.parts[bid] : ItemPart{0, 1, 0, 0};
   // ---- finish this piece's share: four lanes per unit, each adds up every fourth source ----
   // a peer may be late by its own bounded waits; these waits are long enough for all of them, so that nobody sends to a CTA that has left
   bool late = !mbar_wait_cluster(ml_bar, 0);
@@ -459,12 +460,69 @@ __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __gri
     k1 += __shfl_xor_sync(0xffffffffu, up ? acc.y : acc.w, 2);
     const float val = (odd ? k1 : k0) + __shfl_xor_sync(0xffffffffu, odd ? k0 : k1, 1);
     const int hq = 2 * p + (src & 1), dd = (td >> 3) * 16 + (td & 7) + (src >> 1) * 8;
-    if (on && hq < g) {
+    if (PARTS && pt.n > 1) {
+      if (on && hq < g) {
+        const long long row = (long long)(pt.base + pt.part) * g + hq;
+        a.part_o[row * D + dd] = val;
+        if (td == 0 && src < 2) a.part_ml[row] = make_float2(src ? MB : MA, L);
+      }
+    } else if (on && hq < g) {
       ob[hq * D + dd] = __float2bfloat16_rn(val * inv);
       if (td == 0 && src < 2) a.head_mz[(long long)it.i * G.Hq + it.h * g + hq] = make_float2(src ? MB : MA, L);
     }
   }
   if (late && threadIdx.x == 0 && cv.status) atomicOr(cv.status, STATUS_TIMEOUT);
+  // ---- a head of several clusters: the piece that comes last adds up what the clusters left in global memory ----
+  // (No cluster waits for another: two steps on two streams may hold a part of the machine each.)  Every thread's stores are ordered
+  // before the barrier, thread 0's fence makes them visible device-wide before the head's counter moves.
+  if (PARTS && pt.n > 1) {
+    __shared__ int s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      int *ctr = a.head_done + it.i * G.Hkv + it.h;
+      __threadfence();
+      s_last = atomicAdd(ctr, 1) == pt.pieces - 1;
+      if (s_last) *ctr = 0;
+    }
+    __syncthreads();
+    if (s_last) {
+      constexpr int MB = 8;   // parts a batch of loads takes
+      for (int x = threadIdx.x; x < g * (D / 4); x += NW * 32) {
+        const int row = x / (D / 4), col = x % (D / 4);
+        float m = -INFINITY, z = 0.f;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int c0 = 0; c0 < pt.n; c0 += MB) {
+          float2 ml[MB];
+          float4 o[MB];
+          float mb = m;
+#pragma unroll
+          for (int c = 0; c < MB; ++c) {
+            ml[c] = make_float2(-INFINITY, 0.f); o[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (c0 + c < pt.n) {
+              const long long r = (long long)(pt.base + c0 + c) * g + row;
+              ml[c] = __ldcg(a.part_ml + r);
+              o[c] = __ldcg(reinterpret_cast<const float4 *>(a.part_o + r * D) + col);
+            }
+          }
+#pragma unroll
+          for (int c = 0; c < MB; ++c) mb = fmaxf(mb, ml[c].x);
+          if (mb == -INFINITY) continue;   // nothing visible so far
+          const float f0 = ex2(m - mb);    // (m = -inf on the first batch: 0)
+          acc.x *= f0; acc.y *= f0; acc.z *= f0; acc.w *= f0; z *= f0;
+#pragma unroll
+          for (int c = 0; c < MB; ++c) {
+            const float f = ex2(ml[c].x - mb);
+            acc.x += o[c].x * f; acc.y += o[c].y * f; acc.z += o[c].z * f; acc.w += o[c].w * f;
+            z += ml[c].y * f;
+          }
+          m = mb;
+        }
+        const float inv = z > 0.f ? 1.f / z : 0.f;
+        *reinterpret_cast<uint2 *>(ob + row * D + col * 4) = make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+        if (col == 0) a.head_mz[(long long)it.i * G.Hq + it.h * g + row] = make_float2(m, z);
+      }
+    }
+  }
   // after a timeout copies may still be in flight towards this CTA's shared memory: bounded wait before it is released
   if (timed_out && lane < 2 && loaded) mbar_wait(smem_u32(&bars[warp][lane]), X::TWICE ? 1 : 0);
   finish();
@@ -473,10 +531,10 @@ __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __gri
 // ---- host: one list of the forms there are ----
 namespace {
 
-template <int D, bool G16, bool TB, bool DENSE>
+template <int D, bool G16, bool TB, bool DENSE, bool PARTS>
 struct ShortForm {
   typedef ShortShape<D, G16, DENSE> X;
-  static auto kernel() { return wnw_attn_short_kernel<D, G16, TB, DENSE>; }
+  static auto kernel() { return wnw_attn_short_kernel<D, G16, TB, DENSE, PARTS>; }
   static size_t smem(int g) { return (size_t)X::STAGES_B + X::P_B + (size_t)((g + 1) / 2 * (D / 2) + 16) * 16 + 8 * 16 * 16 + 1024; }
   static void config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int g, int n_ctas, int cluster, bool pdl, cudaStream_t st) {
     cfg.gridDim = dim3((unsigned)n_ctas, 1, 1);
@@ -512,34 +570,39 @@ struct ShortForm {
   static bool leaves_recall_room(int g, int rt) { return recall_room((const void *)kernel(), NW_LAT * 32, smem(g), rt); }
 };
 // f: called with the form's ShortForm
-template <bool TB, bool DENSE, class F>
+template <bool TB, bool DENSE, bool PARTS, class F>
 auto with_form_t(int g, int d, F f) {
-  if (d == 128) return g > 8 ? f(ShortForm<128, true, TB, false>{}) : f(ShortForm<128, false, TB, DENSE>{});   // (two n-tiles at 128: one form)
-  return g > 8 ? f(ShortForm<64, true, TB, DENSE>{}) : f(ShortForm<64, false, TB, DENSE>{});
+  if (d == 128) return g > 8 ? f(ShortForm<128, true, TB, false, PARTS>{}) : f(ShortForm<128, false, TB, DENSE, PARTS>{});   // (two n-tiles at 128: one form)
+  return g > 8 ? f(ShortForm<64, true, TB, DENSE, PARTS>{}) : f(ShortForm<64, false, TB, DENSE, PARTS>{});
 }
 template <class F>
-auto with_form(int g, int d, bool tb, bool dense, F f) {
-  if (tb) return dense ? with_form_t<true, true>(g, d, f) : with_form_t<true, false>(g, d, f);
-  return dense ? with_form_t<false, true>(g, d, f) : with_form_t<false, false>(g, d, f);
+auto with_form(int g, int d, bool tb, bool dense, bool parts, F f) {
+  if (parts) {
+    if (tb) return dense ? with_form_t<true, true, true>(g, d, f) : with_form_t<true, false, true>(g, d, f);
+    return dense ? with_form_t<false, true, true>(g, d, f) : with_form_t<false, false, true>(g, d, f);
+  }
+  if (tb) return dense ? with_form_t<true, true, false>(g, d, f) : with_form_t<true, false, false>(g, d, f);
+  return dense ? with_form_t<false, true, false>(g, d, f) : with_form_t<false, false, false>(g, d, f);
 }
 
 }  // namespace
 
 cudaError_t launch_attn_short(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
   if (cv.geo.kv8 || (cv.geo.d != 64 && cv.geo.d != 128)) return cudaErrorInvalidValue;
-  return with_form(cv.geo.g, cv.geo.d, cv.geo.token_base != 0, a.short_pieces == SHORT_DENSE, [&](auto x) { return x.launch(cv, a, st); });
+  return with_form(cv.geo.g, cv.geo.d, cv.geo.token_base != 0, a.short_pieces == SHORT_DENSE, a.parts != nullptr, [&](auto x) { return x.launch(cv, a, st); });
 }
 cudaError_t configure_short_kernels() {
   cudaError_t e = cudaSuccess;
-  for (int k = 0; k < 16 && e == cudaSuccess; ++k)
-    e = with_form(k & 1 ? 16 : 8, k & 2 ? 64 : 128, k & 4, k & 8, [](auto x) { return x.configure(); });
+  for (int k = 0; k < 32 && e == cudaSuccess; ++k)
+    e = with_form(k & 1 ? 16 : 8, k & 2 ? 64 : 128, k & 4, k & 8, k & 16, [](auto x) { return x.configure(); });
   return e;
 }
 int short_cluster_room(int g, int d, bool dense, int cluster) {
-  return with_form(g, d, false, dense, [&](auto x) { return x.cluster_room(g, cluster); });
+  return with_form(g, d, false, dense, false, [&](auto x) { return x.cluster_room(g, cluster); });
 }
 bool short_leaves_recall_room(int g, int d, bool token_base, bool dense, int recall_threads) {
-  return with_form(g, d, token_base, dense, [&](auto x) { return x.leaves_recall_room(g, recall_threads); });
+  return with_form(g, d, token_base, dense, false, [&](auto x) { return x.leaves_recall_room(g, recall_threads); }) &&
+         with_form(g, d, token_base, dense, true, [&](auto x) { return x.leaves_recall_room(g, recall_threads); });
 }
 
 }  // namespace wnw

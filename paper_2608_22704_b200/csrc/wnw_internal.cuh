@@ -36,6 +36,10 @@ struct WorkItem {  // one CTA of the attention kernel; everything static about i
   int32_t T_hint;  // text rows known to exist when the list was built (a lower bound: text only grows)
   int32_t hd_first, hd_count;  // the work items (= split partials) of this item's head: first (relative to the layer's list), number
 };
+// Short pieces: a head of more pieces than a cluster holds has several clusters (an item's hd_first, hd_count: within its own), whose
+// results meet in the layer's partials base .. base + n - 1; part: the item's cluster; pieces: over all of them.
+struct ItemPart { int16_t part, n, base, pieces; };
+static_assert(sizeof(ItemPart) == 8, "two schedule words");
 constexpr int INLINE_ITEMS_MAX = 96;  // launches with at most this many items carry them in kernel parameters
 struct InlineItems { WorkItem it[INLINE_ITEMS_MAX]; };
 struct HeadItems { int32_t first, count; };  // work items (= split partials) of one (active seq, KV head)
@@ -171,6 +175,7 @@ struct AttnArgs {
   int32_t score_on;      // write per-granule softmax-mass partials for anchor-like heads
   const int32_t *active; // [n_active] sequence ids
   const WorkItem *items;         // device copy of the items
+  const ItemPart *parts;         // [n_items] where a head has several clusters, else null
   const WorkItem *items_host;    // host copy (the launcher inlines short lists into the kernel parameters)
   const TmaMaps *maps;           // host pointer; passed to the kernel by value
   const TmaMaps *maps_rows;      // the same with boxes of K or V rows alone

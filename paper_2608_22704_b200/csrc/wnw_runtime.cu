@@ -39,6 +39,7 @@ struct LayerWork {
   bool narrow = false;                             // one-shot CTAs of four warps, two per SM
   int cluster = 0;                                 // chained layers of one wave: CTAs per cluster
   int short_pieces = 0;                            // ... of at most SHORT_GRANULES granules each: SHORT_*
+  bool parts = false;                              // some head has several clusters: ItemParts
   bool packed = false;                             // one-shot CTAs that serve several short heads each
   int n_tidal_items = 0;                           // items of tidal heads
   int head_items_off = 0;                          // offset in the list's HeadItems
@@ -86,9 +87,10 @@ struct wnw_cache {
   std::vector<int> wl_T_a;
   std::vector<LayerWork> wl_layers;
   WorkItem *d_items = nullptr;
-  int32_t *d_sched = nullptr;  // persistent schedules: [order of all layers | ranges of all layers]
-  size_t d_sched_cap = 0, sched_ranges_base = 0;
+  int32_t *d_sched = nullptr;  // persistent schedules: [order of all layers | ranges of all layers]; item parts
+  size_t d_sched_cap = 0, sched_ranges_base = 0, sched_parts_base = 0;
   std::vector<WorkItem> h_items;  // host copy (short lists are inlined into kernel parameters)
+  std::vector<ItemPart> h_parts;  // by item, of the layers with heads of several clusters (up to the last of those); on the device behind the schedules
   size_t d_items_cap = 0;
   // the lists on their way to the device: pinned, one copy queued by the first call that has a stream
   std::vector<int32_t> h_order, h_ranges;
@@ -825,64 +827,88 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   lw.packed = true;   // the pipeline runs across a CTA's items (its merge scratch sits behind the stages)
 }
 
-// Short pieces: a head of at most 256 granules in pieces of 16, wnw_attn_short_kernel, as wide CTAs (one to an SM, all fragments ahead
+// Short pieces: heads in pieces of at most 16 granules, wnw_attn_short_kernel, as wide CTAs (one to an SM, all fragments ahead
 // of the query) where the clusters of two layers fit the GPU side by side, so that a layer's bytes land while its predecessor runs;
 // else dense ones, two to an SM.  Chained, us a replayed step of 30 layers, 32 query heads on 8 KV heads of 128, wide / dense / the
 // cut below: 3000 tokens (3 clusters of 16) 140 / 146 / 154; 2 x 3000 (6) 206 / 157 / 225; 4 x 1000 196 / 163 / 211; the paper's form
 // (4) 182 / 154 / 204; 1000 tokens, full cache (8 clusters of 8) 117 / 127 / 132.
 //
+// A head of more than 16 pieces takes several clusters, which meet in global memory (some 1 us: a fence, a counter, the last piece
+// reads).  That pays from the fourth granule on that a warp of the cut below would walk: 5000 tokens (3 a warp) 202 / 200 us a step,
+// 6000 243 / 209, 8000 245 / 210, 15000 355 / 279, 2 x 8000 355 / 268; 2 KV heads x 15000, 36 layers, 246 / 193; 4 KV heads of 64 x
+// 15000 353 / 240 (the cut below / several clusters).
+//
 // Chained or serial layers whose work fits one wave: the pieces of a head form (part of) a cluster and merge inside it, which
 // costs little however many there are, so heads are cut as fine as fits: two granules a warp (all bytes of a piece in flight
 // before the layer's inputs are there, one softmax step behind them), more where that would not fit one wave or where a head
 // would need more than the 16 pieces a cluster holds (up to CLUSTER_LONGEST_PER_WARP).  Heads are packed into clusters, most pieces first; places left over stay empty.
+constexpr int SHORT_PARTS_FROM = 3;   // granules a warp: see above
 static bool build_cluster_items(const wnw_cache *c, int layer, int mode, const std::vector<int> &seq_ids,
                                 const std::vector<int> &n_gran, const std::vector<int> &n_work, std::vector<WorkItem> &items,
-                                std::vector<HeadItems> &heads, LayerWork &lw) {
+                                std::vector<HeadItems> &heads, LayerWork &lw, std::vector<ItemPart> &item_parts) {
   const Geometry &G = c->geo;
   const int n_heads = (int)seq_ids.size() * G.Hkv, nw = attn_warps(false);
-  std::vector<int> np(n_heads), by(n_heads), first(n_heads), room;
-  for (int hd = 0; hd < n_heads; ++hd)
-    if (n_work[hd] > 16 * nw * CLUSTER_LONGEST_PER_WARP) return false;
+  // A part: the pieces of a head that share a cluster.  A head has one, in short pieces as many as it takes.
+  struct Part { int hd, part, n_parts, base, np, x0, total; };
+  std::vector<Part> parts;
+  std::vector<int> by, first, room;
+  bool longest_fits = true;
+  int longest = 0;
+  for (int hd = 0; hd < n_heads; ++hd) {
+    longest_fits = longest_fits && n_work[hd] <= 16 * nw * CLUSTER_LONGEST_PER_WARP;
+    longest = std::max(longest, n_gran[hd]);
+  }
   // per = 1: pieces of at most SHORT_GRANULES granules whatever they hold, which wnw_attn_short_kernel takes (bf16 tiers)
-  bool may_be_short = !G.kv8;
-  for (int hd = 0; hd < n_heads; ++hd) may_be_short = may_be_short && n_gran[hd] <= 16 * SHORT_GRANULES;
-  for (int per = may_be_short ? 1 : 2; per <= CLUSTER_MAX_PER_WARP; ++per) {
+  const bool short_pieces = !G.kv8 && (longest <= 16 * SHORT_GRANULES || longest > 16 * nw * SHORT_PARTS_FROM);
+  for (int per = short_pieces ? 1 : 2; per <= CLUSTER_MAX_PER_WARP; ++per) {
+    if (per > 1 && !longest_fits) return false;
     int most = 1;
+    parts.clear();
     for (int hd = 0; hd < n_heads; ++hd) {
-      np[hd] = per == 1 ? std::max(1, (n_gran[hd] + SHORT_GRANULES - 1) / SHORT_GRANULES)
-                        : std::max(1, std::min(16, (n_work[hd] + per * nw - 1) / (per * nw)));
-      most = std::max(most, np[hd]);
-      by[hd] = hd;
+      const int np = per == 1 ? std::max(1, (n_gran[hd] + SHORT_GRANULES - 1) / SHORT_GRANULES)
+                              : std::max(1, std::min(16, (n_work[hd] + per * nw - 1) / (per * nw)));
+      const int n_parts = (np + 15) / 16, base = (int)parts.size();
+      for (int y = 0; y < n_parts; ++y) {
+        const int x0 = np * y / n_parts, x1 = np * (y + 1) / n_parts;
+        parts.push_back(Part{hd, y, n_parts, base, x1 - x0, x0, np});
+        most = std::max(most, x1 - x0);
+      }
     }
     const int k = most <= 4 ? 0 : most <= 8 ? 1 : 2, size = 4 << k;
-    std::stable_sort(by.begin(), by.end(), [&](int x, int y) { return np[x] > np[y]; });
+    by.resize(parts.size()); first.resize(parts.size());
+    for (size_t x = 0; x < by.size(); ++x) by[x] = (int)x;
+    std::stable_sort(by.begin(), by.end(), [&](int x, int y) { return parts[x].np > parts[y].np; });
     room.clear();
-    for (int hd : by) {
+    for (int y : by) {
       size_t x = 0;
-      while (x < room.size() && room[x] < np[hd]) ++x;
+      while (x < room.size() && room[x] < parts[y].np) ++x;
       if (x == room.size()) room.push_back(size);
-      first[hd] = (int)x * size + size - room[x];
-      room[x] -= np[hd];
+      first[y] = (int)x * size + size - room[x];
+      room[x] -= parts[y].np;
     }
     const int n_cl = (int)room.size();
     const int form = per > 1 ? 0 : 2 * n_cl <= c->cluster_room[SHORT_WIDE][k] ? SHORT_WIDE : SHORT_DENSE;
-    if (n_cl > c->cluster_room[form][k]) continue;
+    if (n_cl > c->cluster_room[form][k] * (form == SHORT_DENSE ? 7 : 8) / 8) continue;   // (an eighth of the dense places for the next layer's first)
     lw.cluster = size;
     lw.short_pieces = form;
     items.resize(lw.first_item + room.size() * size, WorkItem{0, -1, 0, 0, seq_ids[0], ROLE_ANCHOR, 0, 0, 0, 0, 0, 0, 0});
-    for (int hd = 0; hd < n_heads; ++hd) {
-      const int i = hd / G.Hkv, h = hd % G.Hkv, n = n_gran[hd];
+    lw.parts = parts.size() > (size_t)n_heads;
+    if (lw.parts) item_parts.resize(items.size(), ItemPart{0, 1, 0, 0});
+    for (size_t y = 0; y < parts.size(); ++y) {
+      const Part &pt = parts[y];
+      const int hd = pt.hd, i = hd / G.Hkv, h = hd % G.Hkv, n = n_gran[hd];
       const SeqHost &sq = c->seqs[seq_ids[i]];
       const int role = mode == ATTN_DECODE ? c->roles[layer * G.Hkv + h] : ROLE_ANCHOR;
       const int ridx = mode == ATTN_DECODE ? c->role_idx[layer * G.Hkv + h] : h;
       const int perm = (G.token_base && role == ROLE_TIDAL && !sq.fixed_blocks.empty()) ? std::max(sq.fixed_blocks[layer * G.Hkv + h], 0)
                                                                                        : sq.S_base;
-      for (int x = 0; x < np[hd]; ++x)
-        items[lw.first_item + first[hd] + x] =
-            WorkItem{i, h, (int)((long long)n * x / np[hd]), (int)((long long)n * (x + 1) / np[hd]), seq_ids[i], role, ridx,
-                     role == ROLE_FIXED ? sq.T_a_fixed : sq.T_a, sq.C, perm, sq.T_t, first[hd], np[hd]};
-      heads.push_back(HeadItems{first[hd], np[hd]});
-      lw.max_count = std::max(lw.max_count, np[hd]);
+      for (int x = 0; x < pt.np; ++x)
+        items[lw.first_item + first[y] + x] =
+            WorkItem{i, h, (int)((long long)n * (pt.x0 + x) / pt.total), (int)((long long)n * (pt.x0 + x + 1) / pt.total), seq_ids[i], role, ridx,
+                     role == ROLE_FIXED ? sq.T_a_fixed : sq.T_a, sq.C, perm, sq.T_t, first[y], pt.np};
+      if (lw.parts) std::fill_n(item_parts.begin() + lw.first_item + first[y], pt.np, ItemPart{(int16_t)pt.part, (int16_t)pt.n_parts, (int16_t)pt.base, (int16_t)pt.total});
+      if (pt.part == 0) heads.push_back(HeadItems{first[y], pt.total});
+      lw.max_count = std::max(lw.max_count, pt.np);
     }
     lw.n_items = (int)(room.size() * size);
     lw.n_ctas = 0; lw.packed = false; lw.throughput = false;
@@ -894,7 +920,7 @@ static bool build_cluster_items(const wnw_cache *c, int layer, int mode, const s
 // Appends the items of one layer for the given sequences.
 static void build_layer_items(const wnw_cache *c, int layer, int mode, const std::vector<int> &seq_ids,
                               std::vector<WorkItem> &items, std::vector<HeadItems> &heads, LayerWork &lw,
-                              std::vector<int32_t> &order, std::vector<int32_t> &ranges, CutMemo *memo = nullptr) {
+                              std::vector<int32_t> &order, std::vector<int32_t> &ranges, std::vector<ItemPart> &item_parts, CutMemo *memo = nullptr) {
   const Geometry &G = c->geo;
   // n_gran: the head's whole virtual key space (what the items must cover); n_work: the granules expected to hold data
   // (what the items are sized by): the dynamic slots of a SEGMENT_LAG table are about half empty and cost nothing then
@@ -932,7 +958,7 @@ static void build_layer_items(const wnw_cache *c, int layer, int mode, const std
   lw.first_item = (int)items.size();
   lw.head_items_off = (int)heads.size();
   lw.max_count = 0;
-  if (!overlapped && build_cluster_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw)) return;
+  if (!overlapped && build_cluster_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw, item_parts)) return;
   if (throughput) {
     build_throughput_items(c, layer, mode, seq_ids, n_gran, n_work, items, heads, lw, order, ranges, memo);
     return;
@@ -1031,6 +1057,7 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
   std::vector<WorkItem> items;
   std::vector<HeadItems> heads;
   std::vector<int32_t> order, ranges;
+  std::vector<ItemPart> parts;
   c->wl_layers.assign(G.L, LayerWork{});
   c->batched_target = 0;
   if (c->layer_dependency == WNW_LAYERS_BATCHED) {   // the step's whole work over one wave of CTAs
@@ -1062,7 +1089,7 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
       int first_part = 0;
       for (int l = 0; l < G.L; ++l) {
         LayerWork lw_t;
-        build_layer_items(c, l, mode, c->active, it_t, hd_t, lw_t, or_t, ra_t);
+        build_layer_items(c, l, mode, c->active, it_t, hd_t, lw_t, or_t, ra_t, parts);
         first_part += lw_t.packed ? lw_t.n_ctas_free : (lw_t.n_ctas > 0 ? lw_t.n_ctas : lw_t.n_items);
       }
       if (first_part <= c->n_sm) break;
@@ -1072,7 +1099,7 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
   size_t part_total = 0;
   CutMemo memo;
   for (int l = 0; l < G.L; ++l) {
-    build_layer_items(c, l, mode, c->active, items, heads, c->wl_layers[l], order, ranges, &memo);
+    build_layer_items(c, l, mode, c->active, items, heads, c->wl_layers[l], order, ranges, parts, &memo);
     c->wl_layers[l].part_off = part_total;
     part_total += (size_t)c->wl_layers[l].n_items;
     for (int x = 0; x < c->wl_layers[l].n_items; ++x) {
@@ -1088,7 +1115,7 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
     c->dev_allocs.push_back(pm);
     c->part_o = po; c->part_ml = pm; c->part_cap_total = part_total;
   }
-  c->h_items.swap(items); c->h_order.swap(order); c->h_ranges.swap(ranges);
+  c->h_items.swap(items); c->h_parts.swap(parts); c->h_order.swap(order); c->h_ranges.swap(ranges);
   c->wl_dirty = true;
   ++c->wl_epoch;
   c->wl_active = c->active;
@@ -1101,7 +1128,10 @@ static wnw_status_t ensure_worklists(wnw_cache *c) {
 // built and captured.
 static wnw_status_t upload_worklists(wnw_cache *c, cudaStream_t st) {
   if (!c->wl_dirty) return WNW_OK;
-  const size_t n_items = c->h_items.size(), n_sched = c->h_order.size() + c->h_ranges.size(), n_act = c->active.size();
+  // schedules: order of all layers | ranges of all layers | item parts (8 bytes each, from an even index)
+  const size_t n_lists = c->h_order.size() + c->h_ranges.size(), n_parts = c->h_parts.size();
+  c->sched_parts_base = (n_lists + 1) / 2 * 2;
+  const size_t n_items = c->h_items.size(), n_sched = n_parts ? c->sched_parts_base + 2 * n_parts : n_lists, n_act = c->active.size();
   if (n_items > c->d_items_cap) {
     CK(cudaMalloc((void **)&c->d_items, n_items * sizeof(WorkItem)));
     c->dev_allocs.push_back(c->d_items);
@@ -1123,6 +1153,7 @@ static wnw_status_t upload_worklists(wnw_cache *c, cudaStream_t st) {
   memcpy(c->h_upload, c->h_items.data(), at_sched);
   if (!c->h_order.empty()) memcpy(c->h_upload + at_sched, c->h_order.data(), c->h_order.size() * sizeof(int32_t));
   if (!c->h_ranges.empty()) memcpy(c->h_upload + at_sched + c->h_order.size() * sizeof(int32_t), c->h_ranges.data(), c->h_ranges.size() * sizeof(int32_t));
+  if (n_parts) memcpy(c->h_upload + at_sched + c->sched_parts_base * sizeof(int32_t), c->h_parts.data(), n_parts * sizeof(ItemPart));
   memcpy(c->h_upload + at_act, c->active.data(), n_act * sizeof(int32_t));
   if (c->step_recorded) CK(cudaStreamWaitEvent(st, c->last_step, 0));
   for (int l = 0; l < c->geo.L; ++l)
@@ -1566,7 +1597,9 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   for (const LayerWork &w : c->wl_layers) {
     const int n = w.n_ctas > 0 ? w.n_ctas : w.n_items;
     const int wait = together ? n - (w.packed ? w.n_ctas_free : 0) : layers_overlap(c) ? std::min(n, w.n_tidal_items + 1) : n;
-    small = small && !w.throughput && n <= c->n_sm / 2;
+    // (Half the SMs; of short pieces two to an SM 5/8: chained, inside and half behind the step / all behind it, 80 CTAs a layer 203 / 195 us a
+    // step of 36 layers and 213 / 209 of 30, 96 CTAs 162 / 164, 144 CTAs 223 / 237.)
+    small = small && !w.throughput && n <= (w.short_pieces == SHORT_DENSE ? c->n_sm * 5 / 8 : c->n_sm / 2);
     beside = beside && c->recall_fits_beside[crowded][together ? FORM_TOGETHER : form_of(w)];
     there = c->layer_dependency == WNW_LAYERS_SERIAL ? std::max(there, wait) : there + wait;
   }
@@ -1798,6 +1831,7 @@ static wnw_status_t decode_layer_impl(wnw_cache *c, int want_mode, int32_t layer
   a.score_on = tiered && li.n_anchor > 0;
   a.active = c->d_active; a.items = c->d_items + lw.first_item; a.items_host = c->h_items.data() + lw.first_item;
   a.n_items = lw.n_items; a.maps = &c->maps_decode; a.throughput = lw.throughput; a.cluster = lw.cluster; a.short_pieces = lw.short_pieces; a.maps_rows = &c->maps_rows; a.narrow = lw.narrow;
+  if (lw.parts) a.parts = reinterpret_cast<const ItemPart *>(c->d_sched + c->sched_parts_base) + lw.first_item;
   if (lw.n_ctas > 0) {
     a.order = c->d_sched + lw.order_off; a.cta_ranges = c->d_sched + c->sched_ranges_base + lw.ranges_off; a.n_ctas = lw.n_ctas;
     a.xpref = lw.packed;

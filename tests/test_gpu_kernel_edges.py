@@ -54,6 +54,26 @@ def test_chained_layers_of_short_pieces(n_q, n_kv, d, chunk, audio, n_text):
         ls.close()
 
 
+# Heads of more than 384 granules take several clusters: one granule less and more, five clusters, a part of a batch; token bases
+@pytest.mark.parametrize("n_q,n_kv,d,chunk,audio,n_text,residency", [
+    (8, 2, 128, 16, (6112,), 6, 0), (8, 2, 128, 16, (6144, 40), 6, 0), (10, 2, 128, 64, (17000,), 14, 0), (32, 2, 128, 16, (6200,), 7, 0),
+    (32, 2, 64, 16, (9000, 300, 6300), 3, 0), (8, 2, 64, 25, (5000,), 15, 2), (8, 2, 128, 25, (5300, 700), 7, 2)])
+def test_chained_heads_of_several_clusters(n_q, n_kv, d, chunk, audio, n_text, residency):
+    from parity_harness import Lockstep
+    w = tiny_custom(n_layers=3, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=d, n_text=n_text, audio_lens=audio, chunk=chunk, budget=0.2, n_steps=5,
+                    roles=[[A, T], [T, F], [F, A]], region=chunk, jump_every=2)
+    extra = dict(residency=residency, evict_lag=1, token_retention=np.full((3, n_kv), 0.2, np.float32), token_seg=25) if residency else {}
+    ls = Lockstep(w, seed=59, gen_device="cuda:0", **extra)
+    try:
+        wnw.wnw_set_layer_dependency(ls.h, wnw.WNW_LAYERS_CHAINED)
+        ls.prefill(check_slots=False)
+        for t in range(5):
+            ls.decode_step(t, graph=t >= 2)
+        assert ls.max_out_err <= 2e-2
+    finally:
+        ls.close()
+
+
 # 1408 granules, 3 of them text, are the longest head whose pieces share a cluster; layers without a long head stay clustered
 @pytest.mark.parametrize("audio,d", [((22480,), 64), ((22481,), 64), ((22600, 500), 128), ((40000,), 128)])
 def test_chained_layers_around_the_longest_clustered_head(audio, d):
