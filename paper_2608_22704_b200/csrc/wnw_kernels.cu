@@ -326,12 +326,13 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // flight reach the full rate (64 KB: 39.5 GB/s), every further request only waits in the link's queue, and so does whatever
 // else crosses the link meanwhile, the GPU's own command fetches among them (a small copy or kernel on another stream,
 // host round trip: 11 us alone, 18 us beside 128 KB, 61 us beside 512 KB, 116 us beside 2 MB in flight).  So the grid is
-// 64 warps with RECALL_U 16-byte loads in flight per lane, whatever there is to copy, and the warps work
+// 48 to 192 warps with RECALL_U 16-byte loads in flight per lane, whatever there is to copy, and the warps work
 // independently: the blocks of a launch are cut into pieces of a warp's batch and dealt round robin ACROSS block and layer
 // borders, so that all warps have work and nothing waits at a barrier.
-// 40 registers a thread.  64 warps, two to a CTA (one fits beside an 8-warp attention CTA of up to 240 registers, two of up to 120),
-// where layers wait for one another: the copies have the whole next step's time (config 1, 30 chained layers, recall and the step's
-// own small copies: 254 us a step with 1 024 warps, 238.7 with 64, 241 with 96, 243 with 128).  192 warps, eight to a CTA (on 96 SMs
+// 40 registers a thread.  48 warps, two to a CTA (one fits beside an 8-warp attention CTA of up to 240 registers, two of up to 120),
+// where layers wait for one another: the copies have the whole next step's time, and the step's own small copies and launches share
+// the link (30 chained layers with the program's copies, 1 / 2 / 4 x 3000 tokens, us a step: 64 warps 139.6 / 165.6 / 221, 48 warps
+// 136.9 / 166.8 / 213, 32 warps 135.2 / 172 / 210, 24 warps 138 / 188 / 220).  192 warps, eight to a CTA (on 96 SMs
 // instead of 24 they disturb attention: 16 ragged sequences 49.7 -> 50.4 ms a request), where attention keeps the memory system busy
 // (overlapping layers, persistent CTAs): a host read takes several times as long then and the step waits for it (4 x 3000 tokens,
 // overlapping: 225 us a step with 64, 197 with 128, 193 with 192, 194 with 256, 198 with 384; 206 with 1 024).
@@ -341,7 +342,7 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // word raised, also those of layers that recalled inside the step (`landed`): which layers a step's tidal CTAs wait for depends
 // on how that step is issued, and the next one may be issued another way.
 // ------------------------------------------------------------------------------------------------
-constexpr int RECALL_CTAS = 32, RECALL_CTAS_CROWDED = 24, RECALL_U = 4;
+constexpr int RECALL_CTAS = 24, RECALL_CTAS_CROWDED = 24, RECALL_U = 4;
 __global__ void __launch_bounds__(RECALL_THREADS_CROWDED, 6) wnw_recall_kernel(const __grid_constant__ CacheView cv, int n_active,
                                                                           const int32_t *active, const int32_t *layers,
                                                                           int n_layers, int skip_copy, RecallSignal sig) {
