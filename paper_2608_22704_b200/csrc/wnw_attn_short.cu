@@ -47,9 +47,9 @@ struct ShortShape {
 
 // tokens x heads accumulators in units of four values as a lane holds them: heads 2p and 2p + 1 at d = 16 t + r and 16 t + r + 8.
 // Unit u = p * D / 2 + 8 t + r; piece u % np finishes it, in place u / np of its receive buffer.
-template <int D, bool G16, bool TB, bool DENSE, bool PARTS>
-__global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
-                                                                       const __grid_constant__ TmaMaps maps) {
+// UNI: the allocation-free call: all heads alike, one cluster each; a CTA's item follows from its index and nothing is chained.
+template <int D, bool G16, bool TB, bool DENSE, bool PARTS, bool UNI>
+__device__ __forceinline__ void short_body(const CacheView &cv, const AttnArgs &a, const TmaMaps &maps) {
   typedef ShortShape<D, G16, DENSE> X;
   constexpr int NW = X::NW, HALVES = X::HALVES, HALFB = X::HALFB, TILEB = X::TILEB, STAGEB = X::STAGEB, KK = X::KK, NTN = X::NTN, PPR = X::PPR,
                 QROW = X::QROW, TILES = X::TILES, NTV = X::NTV;
@@ -58,7 +58,14 @@ __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __gri
   const Geometry &G = cv.geo;
   const LayerInfo &li = a.li;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bid = (int)blockIdx.x, g = G.g;
-  const WorkItem it = a.items[bid];   // the first load of the chain item -> granule -> bytes: on its way before anything else
+  if (UNI) asm volatile("griddepcontrol.wait;\n" ::: "memory");   // the caller's buffer may be what the preceding work wrote
+  WorkItem it;
+  if constexpr (UNI) {
+    const int np = a.uni.hd_count, n = a.uni.g1, h = bid / a.cluster, x = bid - h * a.cluster;
+    it = a.uni;
+    it.h = it.ridx = h; it.hd_first = h * a.cluster; it.hd_count = x < np ? np : 0;
+    it.g0 = (int)((long long)n * x / np); it.g1 = (int)((long long)n * (x + 1) / np);
+  } else it = a.items[bid];           // the first load of the chain item -> granule -> bytes: on its way before anything else
   if (warp == NW - 1 && lane < 4)     // the copies' descriptors, beside it
     asm volatile("prefetch.tensormap [%0];\n" ::"l"(lane == 0 ? &maps.text : lane == 1 ? &maps.anchor : lane == 2 ? &maps.pool : &maps.fixed) : "memory");
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");   // (what later work may rely on: see attn_body)
@@ -88,8 +95,8 @@ __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __gri
     finish();
     return;
   }
-  const int T_t = cv.text_len[it.b] + a.has_new, ridx = it.ridx;
-  if (it.h == 0 && it.g0 == 0 && threadIdx.x == 0) cv.step_snap[(long long)it.b * G.L + a.layer] = cv.steps[it.b];
+  const int T_t = UNI ? 0 : cv.text_len[it.b] + a.has_new, ridx = it.ridx;
+  if (!UNI && it.h == 0 && it.g0 == 0 && threadIdx.x == 0) cv.step_snap[(long long)it.b * G.L + a.layer] = cv.steps[it.b];
   const int parity = it.role == ROLE_TIDAL ? (int)(cv.steps[it.b] & 1) : 0;   // which copy of the slot table this step reads
 
   // ---- the warp's two granules: lane n holds granule n's descriptor and queues its copy ----
@@ -144,6 +151,13 @@ __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __gri
   } else {
     queue(true);
   }
+  auto load_q = [&]() {
+    if (threadIdx.x < g * PPR) {
+      const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(a.q + ((long long)it.i * G.Hq + (long long)it.h * g) * D) + threadIdx.x);
+      *reinterpret_cast<uint4 *>(cl_q + (threadIdx.x / PPR) * QROW + (threadIdx.x % PPR) * 16) = v;
+    }
+  };
+  if (UNI) load_q();   // (nothing to wait for: beside the bytes)
   const int mtx = lane >> 3, r0 = lane >> 2, cq = (lane & 3) * 2;
   const int tile = warp % TILES, nt0 = X::SPLIT_NT ? warp / TILES : 0;   // this warp's share of the second product
   const bool pv = X::SPLIT_NT || warp < TILES;
@@ -245,10 +259,7 @@ __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __gri
   const bool new_mine = new_here && warp == new_w && lane < 2 * PPR;
   uint4 new_val = make_uint4(0, 0, 0, 0);
   if (new_mine) new_val = __ldcg(reinterpret_cast<const uint4 *>((new_kv ? a.v_new : a.k_new) + ((long long)it.i * G.Hkv + it.h) * D + new_pc * 8));
-  if (threadIdx.x < g * PPR) {
-    const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(a.q + ((long long)it.i * G.Hq + (long long)it.h * g) * D) + threadIdx.x);
-    *reinterpret_cast<uint4 *>(cl_q + (threadIdx.x / PPR) * QROW + (threadIdx.x % PPR) * 16) = v;
-  }
+  if (!UNI) load_q();
   if (new_mine) {   // the row of the token being generated: V into its granule, K beside the query, both to the text region
     // (at once: a store still under way when the kernel ends holds up the next layer)
     *reinterpret_cast<uint4 *>(cv.text + text_off(G, it.b, a.layer, it.h, new_kv) + (long long)(T_t - 1) * D + new_pc * 8) = new_val;
@@ -528,13 +539,27 @@ __global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __gri
   finish();
 }
 
+template <int D, bool G16, bool TB, bool DENSE, bool PARTS>
+__global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
+                                                                       const __grid_constant__ TmaMaps maps) {
+  short_body<D, G16, TB, DENSE, PARTS, false>(cv, a, maps);
+}
+template <int D, bool G16>
+__global__ void __maxnreg__(208) wnw_attn_short_uniform_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
+                                                               const __grid_constant__ TmaMaps maps) {
+  short_body<D, G16, false, false, false, true>(cv, a, maps);
+}
+
 // ---- host: one list of the forms there are ----
 namespace {
 
-template <int D, bool G16, bool TB, bool DENSE, bool PARTS>
+template <int D, bool G16, bool TB, bool DENSE, bool PARTS, bool UNI = false>
 struct ShortForm {
   typedef ShortShape<D, G16, DENSE> X;
-  static auto kernel() { return wnw_attn_short_kernel<D, G16, TB, DENSE, PARTS>; }
+  static auto kernel() {
+    if constexpr (UNI) return wnw_attn_short_uniform_kernel<D, G16>;
+    else return wnw_attn_short_kernel<D, G16, TB, DENSE, PARTS>;
+  }
   static size_t smem(int g) { return (size_t)X::STAGES_B + X::P_B + (size_t)((g + 1) / 2 * (D / 2) + 16) * 16 + 8 * 16 * 16 + 1024; }
   static void config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int g, int n_ctas, int cluster, bool pdl, cudaStream_t st) {
     cfg.gridDim = dim3((unsigned)n_ctas, 1, 1);
@@ -585,8 +610,21 @@ auto with_form(int g, int d, bool tb, bool dense, bool parts, F f) {
   return dense ? with_form_t<false, true, false>(g, d, f) : with_form_t<false, false, false>(g, d, f);
 }
 
+template <class F>
+auto with_uniform_form(int g, int d, F f) {
+  if (d == 128) return g > 8 ? f(ShortForm<128, true, false, false, false, true>{}) : f(ShortForm<128, false, false, false, false, true>{});
+  return g > 8 ? f(ShortForm<64, true, false, false, false, true>{}) : f(ShortForm<64, false, false, false, false, true>{});
+}
+
 }  // namespace
 
+// a.uni as for launch_attn_uniform, pieces of at most SHORT_GRANULES granules, a cluster of a.cluster CTAs a head
+cudaError_t launch_attn_short_uniform(const CacheView &cv, AttnArgs a, int n_heads, cudaStream_t st) {
+  const int np = a.uni.hd_count;
+  if (np < 1 || np > a.cluster || a.cluster > 16 || a.uni.g1 > np * SHORT_GRANULES || n_heads < 1 || (cv.geo.d != 64 && cv.geo.d != 128)) return cudaErrorInvalidValue;
+  a.n_items = n_heads * a.cluster;
+  return with_uniform_form(cv.geo.g, cv.geo.d, [&](auto x) { return x.launch(cv, a, st); });
+}
 cudaError_t launch_attn_short(const CacheView &cv, const AttnArgs &a, cudaStream_t st) {
   if (cv.geo.kv8 || (cv.geo.d != 64 && cv.geo.d != 128)) return cudaErrorInvalidValue;
   return with_form(cv.geo.g, cv.geo.d, cv.geo.token_base != 0, a.short_pieces == SHORT_DENSE, a.parts != nullptr, [&](auto x) { return x.launch(cv, a, st); });
@@ -595,6 +633,7 @@ cudaError_t configure_short_kernels() {
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < 32 && e == cudaSuccess; ++k)
     e = with_form(k & 1 ? 16 : 8, k & 2 ? 64 : 128, k & 4, k & 8, k & 16, [](auto x) { return x.configure(); });
+  for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = with_uniform_form(k & 1 ? 16 : 8, k & 2 ? 64 : 128, [](auto x) { return x.configure(); });
   return e;
 }
 int short_cluster_room(int g, int d, bool dense, int cluster) {

@@ -1,5 +1,5 @@
 // wnw_attend_static: one-query full attention over a caller-owned K/V buffer, with every byte of scratch taken
-// from a fixed array inside the library image.  It reuses the split-K attention kernel of wnw_attn.cu unchanged;
+// from a fixed array inside the library image.  It reuses the attention kernels of wnw_attn.cu and wnw_attn_short.cu;
 // what differs from the cache-based entry points is only where the split partials, the completion counters and
 // the per-head split table live.
 //
@@ -136,6 +136,18 @@ extern "C" wnw_status_t wnw_attend_static(const void *kv_dev, int32_t n_tokens, 
   a.head_done = reinterpret_cast<int32_t *>(scr + OFF_COUNTERS);
   a.head_mz = reinterpret_cast<float2 *>(scr + OFF_HEAD_MZ);
   a.out = (bf16 *)out_dev;
-  if (launch_attn_uniform(cv, a, n_kv_heads, 1, st) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
+  // Where a head would be split and its pieces of 16 granules fit a cluster, all heads' clusters on the GPU at once: they meet inside
+  // the cluster instead of in global memory.  us a call among others, through global memory / in clusters: 4 KV heads of 64 (8 query
+  // heads), 129 tokens 5.6 / 4.2, 777 5.6 / 4.3, 4096 8.9 / 4.4; 2 of 128 (16 query heads) 777 6.8 / 5.1, 4096 10.3 / 5.0.  Not one
+  // piece a head (16 tokens 3.4 / 4.1), nor a second wave of clusters (8 KV heads of 128, 4096 tokens 8.6 / 9.7; 64 of 64 7.7 / 8.5).
+  const int n_short = (n_gran + SHORT_GRANULES - 1) / SHORT_GRANULES, size = n_short <= 4 ? 4 : n_short <= 8 ? 8 : 16;
+  cudaError_t e;
+  if (n_gran > nw && n_short <= 16 && n_kv_heads <= attn_cluster_room(device, G.g, head_dim, size, SHORT_WIDE)) {
+    a.uni.hd_count = n_short; a.cluster = size;
+    e = launch_attn_short_uniform(cv, a, n_kv_heads, st);
+  } else {
+    e = launch_attn_uniform(cv, a, n_kv_heads, 1, st);
+  }
+  if (e != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
   return WNW_OK;
 }

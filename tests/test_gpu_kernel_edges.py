@@ -108,6 +108,23 @@ def test_static_attention_edges(n_q, n_kv, d):
     assert not wnw.wnw_attend_static_status()
 
 
+# a cluster a head: 2, 4, 5, 8, 9 and 16 pieces of 16 granules and one granule more; rows behind the clip hold NaN
+@pytest.mark.parametrize("n_q,n_kv,d", [(8, 4, 64), (3, 1, 128), (32, 2, 128), (48, 3, 64)])
+def test_static_attention_in_clusters(n_q, n_kv, d):
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device="cpu").manual_seed(n_q * d)
+    for n in (130, 257, 1024, 1025, 2048, 2049, 4095, 4096, 4097):
+        kv = torch.full((n_kv, 2, (n + 47) // 16 * 16, d), float("nan"), dtype=torch.bfloat16)
+        kv[:, :, :n] = torch.randn(n_kv, 2, n, d, generator=gen).to(torch.bfloat16)
+        q = (torch.randn(n_q, d, generator=gen) * 1.5).to(torch.bfloat16)
+        out = torch.full((n_q, d), float("nan"), dtype=torch.bfloat16, device=dev)
+        wnw.wnw_attend_static(kv.to(dev), n, q.to(dev), out)
+        K, V, Q = (bf16_bits_to_f64(bf16_bits(x.contiguous())) for x in (kv[:, 0, :n], kv[:, 1, :n], q))
+        want = np.stack([dense_attention(Q[h], K[h * n_kv // n_q], V[h * n_kv // n_q], 1.0 / np.sqrt(d))[0] for h in range(n_q)])
+        assert np.abs(out.float().cpu().numpy() - want).max() <= 2e-2, n   # bf16 weights and outputs of O(1)
+    assert not wnw.wnw_attend_static_status()
+
+
 @pytest.mark.parametrize("n_queries", [8, 9, 17])
 def test_scoring_takes_several_queries_per_launch(n_queries):
     from parity_harness import Lockstep
