@@ -1415,7 +1415,6 @@ cudaError_t configure_attn_kernels() {
   if ((e = configure_t<128, true, NW_THR>()) != cudaSuccess) return e;
   if ((e = configure_t<128, false, NW_THR>()) != cudaSuccess) return e;
   if ((e = configure_t<64, true, NW_THR>()) != cudaSuccess) return e;
-  if ((e = configure_short_kernels()) != cudaSuccess) return e;
   return configure_t<64, false, NW_THR>();
 }
 

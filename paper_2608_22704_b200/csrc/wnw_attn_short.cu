@@ -2,7 +2,7 @@
 // thread-block cluster or, of long heads, in several (PARTS): the layer's span is what counts (sm_100a).
 //
 // What bounds such a layer is a chain of latencies, not bytes (config 1 moves 4 MB a layer, 0.6 us of HBM): inputs visible, query
-// into registers, K q^T, softmax, P V, merge over the warps, merge over the head's pieces, output.  wnw_attn_cluster_kernel gives
+// into registers, K q^T, softmax, P V, merge over the warps, merge over the head's pieces, output.  The kernel of longer pieces (wnw_attn.cu) gives
 // every warp the whole head_dim of its own tokens and merges eight warps' accumulators through shared memory.  Here the tokens are
 // split over the warps for the first product alone and head_dim for the second, and what does not depend on the query is done
 // ahead of it:
@@ -18,7 +18,9 @@
 // program's copies: 154 -> 140 us a step; 16 query heads a KV head 235 -> 174; the paper's form 204 -> 154.
 // tcgen05 does not pay here: with 8 to 16 query heads its M = 128, N = 16, K = 16 steps take 50 to 59 cycles each (485 to 567 for
 // 128 tokens), where mma.sync needs 256 for 256 tokens with its operands in registers.
-#include <cstring>
+#include <mutex>
+#include <set>
+#include <tuple>
 
 #include "wnw_attn_dev.cuh"
 #include "wnw_internal.cuh"
@@ -539,16 +541,20 @@ __device__ __forceinline__ void short_body(const CacheView &cv, const AttnArgs &
   finish();
 }
 
+namespace short_pieces {   // (beside the kernel of that name for longer pieces)
+
 template <int D, bool G16, bool TB, bool DENSE, bool PARTS>
-__global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
+__global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_cluster_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
                                                                        const __grid_constant__ TmaMaps maps) {
   short_body<D, G16, TB, DENSE, PARTS, false>(cv, a, maps);
 }
 template <int D, bool G16>
-__global__ void __maxnreg__(208) wnw_attn_short_uniform_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
+__global__ void __maxnreg__(208) wnw_attn_cluster_uniform_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
                                                                const __grid_constant__ TmaMaps maps) {
   short_body<D, G16, false, false, false, true>(cv, a, maps);
 }
+
+}  // namespace short_pieces
 
 // ---- host: one list of the forms there are ----
 namespace {
@@ -557,8 +563,8 @@ template <int D, bool G16, bool TB, bool DENSE, bool PARTS, bool UNI = false>
 struct ShortForm {
   typedef ShortShape<D, G16, DENSE> X;
   static auto kernel() {
-    if constexpr (UNI) return wnw_attn_short_uniform_kernel<D, G16>;
-    else return wnw_attn_short_kernel<D, G16, TB, DENSE, PARTS>;
+    if constexpr (UNI) return short_pieces::wnw_attn_cluster_uniform_kernel<D, G16>;
+    else return short_pieces::wnw_attn_cluster_kernel<D, G16, TB, DENSE, PARTS>;
   }
   static size_t smem(int g) { return (size_t)X::STAGES_B + X::P_B + (size_t)((g + 1) / 2 * (D / 2) + 16) * 16 + 8 * 16 * 16 + 1024; }
   static void config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int g, int n_ctas, int cluster, bool pdl, cudaStream_t st) {
@@ -629,10 +635,21 @@ cudaError_t launch_attn_short(const CacheView &cv, const AttnArgs &a, cudaStream
   if (cv.geo.kv8 || (cv.geo.d != 64 && cv.geo.d != 128)) return cudaErrorInvalidValue;
   return with_form(cv.geo.g, cv.geo.d, cv.geo.token_base != 0, a.short_pieces == SHORT_DENSE, a.parts != nullptr, [&](auto x) { return x.launch(cv, a, st); });
 }
-cudaError_t configure_short_kernels() {
+// Opt-in shared memory and cluster sizes, once per device: of the forms a cache of that shape uses (a kernel's first attribute call
+// loads it: some 0.3 ms each), of the uniform ones.
+cudaError_t configure_short_kernels(int device, int g, int d, bool token_base) {
+  static std::mutex mu;
+  static std::set<std::tuple<int, bool, int, bool>> done;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto key = std::make_tuple(device, g > 8, d, token_base);
+  if (done.count(key)) return cudaSuccess;
   cudaError_t e = cudaSuccess;
-  for (int k = 0; k < 32 && e == cudaSuccess; ++k)
-    e = with_form(k & 1 ? 16 : 8, k & 2 ? 64 : 128, k & 4, k & 8, k & 16, [](auto x) { return x.configure(); });
+  for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = with_form(g, d, token_base, k & 1, k & 2, [](auto x) { return x.configure(); });
+  if (e == cudaSuccess) done.insert(key);
+  return e;
+}
+cudaError_t configure_short_uniform_kernels() {
+  cudaError_t e = cudaSuccess;
   for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = with_uniform_form(k & 1 ? 16 : 8, k & 2 ? 64 : 128, [](auto x) { return x.configure(); });
   return e;
 }

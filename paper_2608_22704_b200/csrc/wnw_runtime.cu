@@ -373,6 +373,9 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
 #define CKE(expr) do { cudaError_t _e = (expr); if (_e != cudaSuccess) { return fail(_e == cudaErrorMemoryAllocation ? WNW_ERR_OOM_DEVICE : WNW_ERR_CUDA); } } while (0)
   cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
   CKE(configure_attn_kernels());
+  if (cfg->head_dim == 128 || cfg->head_dim == 64)
+    CKE(configure_short_kernels(cfg->device, cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim,
+                                cfg->mode == WNW_MODE_TIERED && cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE));
   CKE(configure_select_kernel());
   for (int k = 0; k < 2 * N_ATTN_FORMS; ++k)
     c->recall_fits_beside[k / N_ATTN_FORMS][k % N_ATTN_FORMS] = attn_leaves_recall_room(cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim,
@@ -827,7 +830,7 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
   lw.packed = true;   // the pipeline runs across a CTA's items (its merge scratch sits behind the stages)
 }
 
-// Short pieces: heads in pieces of at most 16 granules, wnw_attn_short_kernel, as wide CTAs (one to an SM, all fragments ahead
+// Short pieces: heads in pieces of at most 16 granules (wnw_attn_short.cu), as wide CTAs (one to an SM, all fragments ahead
 // of the query) where the clusters of two layers fit the GPU side by side, so that a layer's bytes land while its predecessor runs;
 // else dense ones, two to an SM.  Chained, us a replayed step of 30 layers, 32 query heads on 8 KV heads of 128, wide / dense / the
 // cut below: 3000 tokens (3 clusters of 16) 140 / 146 / 154; 2 x 3000 (6) 206 / 157 / 225; 4 x 1000 196 / 163 / 211; the paper's form
@@ -858,7 +861,7 @@ static bool build_cluster_items(const wnw_cache *c, int layer, int mode, const s
     longest_fits = longest_fits && n_work[hd] <= 16 * nw * CLUSTER_LONGEST_PER_WARP;
     longest = std::max(longest, n_gran[hd]);
   }
-  // per = 1: pieces of at most SHORT_GRANULES granules whatever they hold, which wnw_attn_short_kernel takes (bf16 tiers)
+  // per = 1: pieces of at most SHORT_GRANULES granules whatever they hold (bf16 tiers)
   const bool short_pieces = !G.kv8 && (longest <= 16 * SHORT_GRANULES || longest > 16 * nw * SHORT_PARTS_FROM);
   for (int per = short_pieces ? 1 : 2; per <= CLUSTER_MAX_PER_WARP; ++per) {
     if (per > 1 && !longest_fits) return false;

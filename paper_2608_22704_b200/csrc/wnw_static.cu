@@ -48,7 +48,7 @@ wnw_status_t scratch_for_current_device(int device, unsigned char **out) {
   if (!g_scratch_addr[device]) {
     void *p = nullptr;
     if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) { cudaGetLastError(); return WNW_ERR_CUDA; }
-    if (configure_attn_kernels() != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }  // shared-memory opt-in, no allocation
+    if (configure_attn_kernels() != cudaSuccess || configure_short_uniform_kernels() != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }  // shared-memory opt-in, no allocation
     if (cudaDeviceGetAttribute(&g_n_sm[device], cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
     g_scratch_addr[device] = (unsigned char *)p;
   }
