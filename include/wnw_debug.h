@@ -28,6 +28,11 @@ wnw_status_t wnw_debug_fill_mirror_padding(wnw_cache_t *cache, int32_t seq, int3
 wnw_status_t wnw_debug_get_slot_padding(wnw_cache_t *cache, int32_t seq, int32_t layer, int32_t kv_head, int32_t slot,
                                         int32_t which, void *rows);
 
+/* How wnw_attend_static cuts the heads of such a call: *cluster = CTAs of the thread-block cluster in which a head's pieces
+ * meet, 0 if they meet in global memory.  The answer is the call's own, whatever the process did before. */
+wnw_status_t wnw_debug_attend_static_cluster(int32_t device, int32_t n_tokens, int32_t n_q_heads, int32_t n_kv_heads,
+                                             int32_t head_dim, int32_t *cluster);
+
 /* Optional per-kernel timing: when enabled the library brackets its attention-kernel launches with CUDA events
  * on the launching stream; wnw_get_kernel_time returns the accumulated milliseconds and launch count since the
  * last call (drains the stream).  Off by default. */

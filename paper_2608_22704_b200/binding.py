@@ -87,6 +87,7 @@ _SIGNATURES = {
     "wnw_get_kernel_time": [_vp, C.POINTER(C.c_float), C.POINTER(_i32)],
     "wnw_sync": [_vp],
     "wnw_measure_host_link": [_i32, C.c_int64, _i32, C.POINTER(C.c_double), C.POINTER(C.c_double)],
+    "wnw_debug_attend_static_cluster": [_i32, _i32, _i32, _i32, _i32, C.POINTER(_i32)],
     "wnw_attend_static": [_vp, _i32, _i32, _vp, _vp, _i32, _i32, _i32, C.c_float, _i32, _vp],
     "wnw_attend_static_status": [_i32, _vp, C.POINTER(_i32)],
 }
@@ -409,3 +410,10 @@ def wnw_attend_static_status(device: int = 0, stream=None) -> bool:
     v = _i32(0)
     _ck(lib().wnw_attend_static_status(device, _stream(stream), C.byref(v)), "wnw_attend_static_status")
     return bool(v.value)
+
+
+def wnw_debug_attend_static_cluster(n_tokens: int, n_q_heads: int, n_kv_heads: int, head_dim: int, device: int = 0) -> int:
+    """CTAs of the cluster in which a head's pieces meet; 0 if they meet in global memory."""
+    v = _i32()
+    _ck(lib().wnw_debug_attend_static_cluster(device, n_tokens, n_q_heads, n_kv_heads, head_dim, C.byref(v)), "wnw_debug_attend_static_cluster")
+    return v.value

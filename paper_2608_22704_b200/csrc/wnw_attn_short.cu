@@ -590,13 +590,16 @@ struct ShortForm {
     const cudaError_t e = cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(G16 ? 16 : 8));
     return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel(), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // up to 16 CTAs
   }
-  static int cluster_room(int g, int cluster) {
+  // Clusters of that size that the GPU holds at once; 0: it takes none of them
+  static cudaError_t cluster_room(int g, int cluster, int *n) {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[2];
     config(cfg, attr, g, cluster, cluster, false, nullptr);
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, kernel(), &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
-    return n;
+    *n = 0;
+    const cudaError_t e = cudaOccupancyMaxActiveClusters(n, kernel(), &cfg);
+    if (e != cudaErrorInvalidClusterSize) return e;
+    cudaGetLastError();
+    return cudaSuccess;
   }
   static bool leaves_recall_room(int g, int rt) { return recall_room((const void *)kernel(), NW_LAT * 32, smem(g), rt); }
 };
@@ -636,7 +639,7 @@ cudaError_t launch_attn_short(const CacheView &cv, const AttnArgs &a, cudaStream
   return with_form(cv.geo.g, cv.geo.d, cv.geo.token_base != 0, a.short_pieces == SHORT_DENSE, a.parts != nullptr, [&](auto x) { return x.launch(cv, a, st); });
 }
 // Opt-in shared memory and cluster sizes, once per device: of the forms a cache of that shape uses (a kernel's first attribute call
-// loads it: some 0.3 ms each), of the uniform ones.
+// loads it: some 0.3 ms each).
 cudaError_t configure_short_kernels(int device, int g, int d, bool token_base) {
   static std::mutex mu;
   static std::set<std::tuple<int, bool, int, bool>> done;
@@ -648,13 +651,18 @@ cudaError_t configure_short_kernels(int device, int g, int d, bool token_base) {
   if (e == cudaSuccess) done.insert(key);
   return e;
 }
-cudaError_t configure_short_uniform_kernels() {
-  cudaError_t e = cudaSuccess;
-  for (int k = 0; k < 4 && e == cudaSuccess; ++k) e = with_uniform_form(k & 1 ? 16 : 8, k & 2 ? 64 : 128, [](auto x) { return x.configure(); });
-  return e;
+// The uniform form that groups of g share is configured by the question for its room, which no launch of it goes without.  One answer
+// for all of the form's groups: 208 registers a thread hold an SM to one CTA.
+cudaError_t short_uniform_room(int g, int d, int cluster, int *n) {
+  return with_uniform_form(g, d, [&](auto x) {
+    const cudaError_t e = x.configure();
+    return e != cudaSuccess ? e : x.cluster_room(g > 8 ? 16 : 8, cluster, n);
+  });
 }
 int short_cluster_room(int g, int d, bool dense, int cluster) {
-  return with_form(g, d, false, dense, false, [&](auto x) { return x.cluster_room(g, cluster); });
+  int n = 0;
+  if (with_form(g, d, false, dense, false, [&](auto x) { return x.cluster_room(g, cluster, &n); }) != cudaSuccess) { cudaGetLastError(); return 0; }
+  return n;
 }
 bool short_leaves_recall_room(int g, int d, bool token_base, bool dense, int recall_threads) {
   return with_form(g, d, token_base, dense, false, [&](auto x) { return x.leaves_recall_room(g, recall_threads); }) &&

@@ -306,7 +306,7 @@ enum { SHORT_WIDE = 1, SHORT_DENSE = 2 };   // one CTA to an SM; two
 cudaError_t launch_attn_short(const CacheView &cv, const AttnArgs &a, cudaStream_t st);
 cudaError_t launch_attn_short_uniform(const CacheView &cv, AttnArgs a, int n_heads, cudaStream_t st);
 cudaError_t configure_short_kernels(int device, int g, int d, bool token_base);
-cudaError_t configure_short_uniform_kernels();
+cudaError_t short_uniform_room(int g, int d, int cluster, int *n);   // clusters of that size, of the allocation-free call, that fit the current device at once
 int short_cluster_room(int g, int d, bool dense, int cluster);
 bool short_leaves_recall_room(int g, int d, bool token_base, bool dense, int recall_threads);
 bool recall_room(const void *kernel, int threads, size_t dynamic_smem, int recall_threads);   // room for a recall CTA on an SM full of that kernel's CTAs

@@ -9,10 +9,13 @@
 // this entry point: it calls no cudaMalloc, no cudaFree and no allocating library routine, and its host side keeps
 // no list at all.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 
 #include "../../include/wnw.h"
+#include "../../include/wnw_debug.h"
 #include "wnw_internal.cuh"
 
 using namespace wnw;
@@ -39,34 +42,90 @@ static_assert(OFF_PART_O % 256 == 0, "scratch sections are 256-byte aligned");
 // Every GPU that loads the library holds this array until the process exits.
 static __device__ __align__(256) unsigned char g_static_scratch[SCRATCH_BYTES];
 
-// In host code the array's name is only a stand-in; the device address comes from cudaGetSymbolAddress, once per device.
-unsigned char *g_scratch_addr[ST_MAX_DEVICES] = {nullptr};
-int g_n_sm[ST_MAX_DEVICES];
+// What the calls need to know of a device, found once: a call among others takes no lock and asks the driver nothing.
+struct StaticDevice {
+  std::atomic<unsigned char *> scratch;   // device address of the array (in host code its name is only a stand-in); set last
+  int n_sm;
+  std::atomic<int> room[2][2][3];         // [group of more than 8][head_dim 128][k]: 1 + the clusters of 4 << k CTAs that fit at once, 0: not asked yet
+};
+StaticDevice g_devices[ST_MAX_DEVICES];
 
-wnw_status_t scratch_for_current_device(int device, unsigned char **out) {
+wnw_status_t current_device(int device, StaticDevice **out) {
   if (device < 0 || device >= ST_MAX_DEVICES) return WNW_ERR_INVALID_ARG;
-  if (!g_scratch_addr[device]) {
+  StaticDevice &dv = g_devices[device];
+  if (!dv.scratch.load(std::memory_order_acquire)) {
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
     void *p = nullptr;
     if (cudaGetSymbolAddress(&p, g_static_scratch) != cudaSuccess || !p) { cudaGetLastError(); return WNW_ERR_CUDA; }
-    if (configure_attn_kernels() != cudaSuccess || configure_short_uniform_kernels() != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }  // shared-memory opt-in, no allocation
-    if (cudaDeviceGetAttribute(&g_n_sm[device], cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
-    g_scratch_addr[device] = (unsigned char *)p;
+    if (configure_attn_kernels() != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }  // shared-memory opt-in, no allocation
+    int n_sm = 0;
+    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
+    if (!dv.scratch.load(std::memory_order_relaxed)) {
+      dv.n_sm = n_sm;
+      dv.scratch.store((unsigned char *)p, std::memory_order_release);
+    }
   }
-  *out = g_scratch_addr[device];
+  *out = &dv;
   return WNW_OK;
 }
+
+// How the heads of a call are cut.  cluster: CTAs of a cluster that a head's pieces share; 0: the pieces meet in global memory.
+struct StaticCut { int pieces, cluster; };
+
+wnw_status_t check_shape(int n_tokens, int n_q_heads, int n_kv_heads, int head_dim) {
+  if (n_q_heads < 1 || n_kv_heads < 1 || n_q_heads % n_kv_heads || n_tokens < 1) return WNW_ERR_INVALID_ARG;
+  if (head_dim != 64 && head_dim != 128) return WNW_ERR_UNSUPPORTED;
+  // beyond the fixed scratch: refuse rather than overrun
+  if (n_kv_heads > ST_MAX_KV_HEADS || n_q_heads > ST_MAX_Q_HEADS || n_q_heads / n_kv_heads > MAX_G || n_tokens > ST_MAX_TOKENS) return WNW_ERR_CAPACITY;
+  return WNW_OK;
+}
+
+wnw_status_t cut_heads(StaticDevice &dv, int n_tokens, int n_q_heads, int n_kv_heads, int head_dim, StaticCut *cut) {
+  const int n_gran = (n_tokens + GR - 1) / GR, nw = attn_warps(false), g = n_q_heads / n_kv_heads;
+  // Where a head would be split and its pieces of 16 granules fit a cluster, all heads' clusters on the GPU at once: they meet inside
+  // the cluster instead of in global memory.  us a call among others, through global memory / in clusters: 4 KV heads of 64 (8 query
+  // heads), 129 tokens 5.6 / 4.2, 777 5.6 / 4.3, 4096 8.9 / 4.4; 2 of 128 (16 query heads) 777 6.8 / 5.1, 4096 10.3 / 5.0.  Not one
+  // piece a head (16 tokens 3.4 / 4.1), nor a second wave of clusters (8 KV heads of 128, 4096 tokens 8.6 / 9.7; 64 of 64 7.7 / 8.5).
+  const int n_short = (n_gran + SHORT_GRANULES - 1) / SHORT_GRANULES, k = n_short <= 4 ? 0 : n_short <= 8 ? 1 : 2;
+  if (n_gran > nw && n_short <= 16) {
+    std::atomic<int> &room = dv.room[g > 8][head_dim == 128][k];
+    int n = room.load(std::memory_order_acquire) - 1;
+    if (n < 0) {   // (some 0.5 ms; threads that ask at the same time get the same answer)
+      if (short_uniform_room(g, head_dim, 4 << k, &n) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
+      room.store(n + 1, std::memory_order_release);
+    }
+    if (n_kv_heads <= n) { *cut = StaticCut{n_short, 4 << k}; return WNW_OK; }
+  }
+  // Every head in the same number of pieces: at least a granule for every warp of a CTA, one wave of CTAs (one fits an SM),
+  // and no more partial rows than the scratch holds (binds only for one KV head with more than eight query heads).  All heads
+  // are alike, so a CTA computes its piece from its index and no list is built or passed.  Before, at most 96 CTAs ran, what
+  // a list in the kernel parameters held, behind a kernel that cleared counters: 50001 tokens x 8 heads 47.5 -> 40.9 us,
+  // 777 tokens x 4 heads of 64: 13.1 -> 8.5 us.
+  *cut = StaticCut{std::max(1, std::min({(n_gran + nw - 1) / nw, dv.n_sm / n_kv_heads, ST_MAX_ROWS / n_q_heads})), 0};
+  return WNW_OK;
+}
+
+struct OnDevice {   // the device is current while this lives
+  int prev = -1, dev;
+  bool ok;
+  explicit OnDevice(int device) : dev(device) {
+    ok = cudaGetDevice(&prev) == cudaSuccess && (prev == device || cudaSetDevice(device) == cudaSuccess);
+    if (!ok) cudaGetLastError();
+  }
+  ~OnDevice() { if (ok && prev != dev) cudaSetDevice(prev); }
+};
 
 }  // namespace
 
 extern "C" wnw_status_t wnw_attend_static_status(int32_t device, void *cuda_stream, int32_t *timed_out) {
   if (!timed_out) return WNW_ERR_INVALID_ARG;
-  int prev = -1;
-  if (cudaGetDevice(&prev) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
-  if (prev != device && cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
-  struct Restore { int prev, dev; ~Restore() { if (prev != dev) cudaSetDevice(prev); } } restore{prev, device};
-  unsigned char *scr = nullptr;
-  wnw_status_t rc = scratch_for_current_device(device, &scr);
+  OnDevice on(device);
+  if (!on.ok) return WNW_ERR_CUDA;
+  StaticDevice *dv = nullptr;
+  const wnw_status_t rc = current_device(device, &dv);
   if (rc != WNW_OK) return rc;
+  unsigned char *scr = dv->scratch.load(std::memory_order_relaxed);
   cudaStream_t st = (cudaStream_t)cuda_stream;
   int32_t word = 0;
   if (cudaMemcpyAsync(&word, scr + OFF_STATUS, sizeof(word), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
@@ -82,30 +141,18 @@ extern "C" wnw_status_t wnw_attend_static(const void *kv_dev, int32_t n_tokens, 
                                           void *out_dev, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim,
                                           float softmax_scale, int32_t device, void *cuda_stream) {
   if (!kv_dev || !q_dev || !out_dev) return WNW_ERR_INVALID_ARG;
-  if (n_q_heads < 1 || n_kv_heads < 1 || n_q_heads % n_kv_heads || n_tokens < 1) return WNW_ERR_INVALID_ARG;
-  if (padded_tokens < n_tokens || padded_tokens % GR) return WNW_ERR_INVALID_ARG;
+  if (n_tokens < 1 || padded_tokens < n_tokens || padded_tokens % GR) return WNW_ERR_INVALID_ARG;
   if (!(softmax_scale >= 0.f) || std::isinf(softmax_scale)) return WNW_ERR_INVALID_ARG;
-  if (head_dim != 64 && head_dim != 128) return WNW_ERR_UNSUPPORTED;
-  // beyond the fixed scratch: refuse rather than overrun
-  if (n_kv_heads > ST_MAX_KV_HEADS || n_q_heads > ST_MAX_Q_HEADS || n_q_heads / n_kv_heads > MAX_G ||
-      (long long)padded_tokens > ST_MAX_TOKENS)
-    return WNW_ERR_CAPACITY;
-  int prev = -1;
-  if (cudaGetDevice(&prev) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
-  if (prev != device && cudaSetDevice(device) != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
-  struct Restore { int prev, dev; ~Restore() { if (prev != dev) cudaSetDevice(prev); } } restore{prev, device};
-  unsigned char *scr = nullptr;
-  wnw_status_t rc = scratch_for_current_device(device, &scr);
+  wnw_status_t rc = check_shape(padded_tokens, n_q_heads, n_kv_heads, head_dim);
   if (rc != WNW_OK) return rc;
+  OnDevice on(device);
+  if (!on.ok) return WNW_ERR_CUDA;
+  StaticDevice *dv = nullptr;
+  StaticCut cut;
+  if ((rc = current_device(device, &dv)) != WNW_OK || (rc = cut_heads(*dv, n_tokens, n_q_heads, n_kv_heads, head_dim, &cut)) != WNW_OK) return rc;
+  unsigned char *scr = dv->scratch.load(std::memory_order_relaxed);
   cudaStream_t st = (cudaStream_t)cuda_stream;
-
-  // Every head in the same number of pieces: at least a granule for every warp of a CTA, one wave of CTAs (one fits an SM),
-  // and no more partial rows than the scratch holds (binds only for one KV head with more than eight query heads).  All heads
-  // are alike, so a CTA computes its piece from its index and no list is built or passed.  Before, at most 96 CTAs ran, what
-  // a list in the kernel parameters held, behind a kernel that cleared counters: 50001 tokens x 8 heads 47.5 -> 40.9 us,
-  // 777 tokens x 4 heads of 64: 13.1 -> 8.5 us.
-  const int n_gran = (n_tokens + GR - 1) / GR, nw = attn_warps(false);
-  const int n_cta = std::max(1, std::min({(n_gran + nw - 1) / nw, g_n_sm[device] / n_kv_heads, ST_MAX_ROWS / n_q_heads}));
+  const int n_gran = (n_tokens + GR - 1) / GR;
 
   CacheView cv;
   memset(&cv, 0, sizeof(cv));
@@ -126,7 +173,7 @@ extern "C" wnw_status_t wnw_attend_static(const void *kv_dev, int32_t n_tokens, 
   AttnArgs a{};
   a.maps = &maps;
   a.mode = ATTN_FULL; a.layer = 0; a.n_active = 1; a.has_new = 0; a.score_on = 0;
-  a.uni = WorkItem{0, 0, 0, n_gran, 0, ROLE_ANCHOR, 0, n_tokens, n_gran, 0, 0, 0, n_cta};
+  a.uni = WorkItem{0, 0, 0, n_gran, 0, ROLE_ANCHOR, 0, n_tokens, n_gran, 0, 0, 0, cut.pieces};
   a.pdl = 1;   // the launch overlaps the tail of the preceding kernel; nothing is read before that has completed
   a.q = (const bf16 *)q_dev;
   a.anchor_base = (const bf16 *)kv_dev; a.anchor_seq_stride = 0; a.anchor_head0 = 0;
@@ -136,18 +183,22 @@ extern "C" wnw_status_t wnw_attend_static(const void *kv_dev, int32_t n_tokens, 
   a.head_done = reinterpret_cast<int32_t *>(scr + OFF_COUNTERS);
   a.head_mz = reinterpret_cast<float2 *>(scr + OFF_HEAD_MZ);
   a.out = (bf16 *)out_dev;
-  // Where a head would be split and its pieces of 16 granules fit a cluster, all heads' clusters on the GPU at once: they meet inside
-  // the cluster instead of in global memory.  us a call among others, through global memory / in clusters: 4 KV heads of 64 (8 query
-  // heads), 129 tokens 5.6 / 4.2, 777 5.6 / 4.3, 4096 8.9 / 4.4; 2 of 128 (16 query heads) 777 6.8 / 5.1, 4096 10.3 / 5.0.  Not one
-  // piece a head (16 tokens 3.4 / 4.1), nor a second wave of clusters (8 KV heads of 128, 4096 tokens 8.6 / 9.7; 64 of 64 7.7 / 8.5).
-  const int n_short = (n_gran + SHORT_GRANULES - 1) / SHORT_GRANULES, size = n_short <= 4 ? 4 : n_short <= 8 ? 8 : 16;
-  cudaError_t e;
-  if (n_gran > nw && n_short <= 16 && n_kv_heads <= attn_cluster_room(device, G.g, head_dim, size, SHORT_WIDE)) {
-    a.uni.hd_count = n_short; a.cluster = size;
-    e = launch_attn_short_uniform(cv, a, n_kv_heads, st);
-  } else {
-    e = launch_attn_uniform(cv, a, n_kv_heads, 1, st);
-  }
+  a.cluster = cut.cluster;
+  const cudaError_t e = cut.cluster ? launch_attn_short_uniform(cv, a, n_kv_heads, st) : launch_attn_uniform(cv, a, n_kv_heads, 1, st);
   if (e != cudaSuccess) { cudaGetLastError(); return WNW_ERR_CUDA; }
+  return WNW_OK;
+}
+
+extern "C" wnw_status_t wnw_debug_attend_static_cluster(int32_t device, int32_t n_tokens, int32_t n_q_heads, int32_t n_kv_heads,
+                                                        int32_t head_dim, int32_t *cluster) {
+  if (!cluster) return WNW_ERR_INVALID_ARG;
+  wnw_status_t rc = check_shape(n_tokens, n_q_heads, n_kv_heads, head_dim);
+  if (rc != WNW_OK) return rc;
+  OnDevice on(device);
+  if (!on.ok) return WNW_ERR_CUDA;
+  StaticDevice *dv = nullptr;
+  StaticCut cut;
+  if ((rc = current_device(device, &dv)) != WNW_OK || (rc = cut_heads(*dv, n_tokens, n_q_heads, n_kv_heads, head_dim, &cut)) != WNW_OK) return rc;
+  *cluster = cut.cluster;
   return WNW_OK;
 }
