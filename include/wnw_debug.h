@@ -33,6 +33,20 @@ wnw_status_t wnw_debug_get_slot_padding(wnw_cache_t *cache, int32_t seq, int32_t
 wnw_status_t wnw_debug_attend_static_cluster(int32_t device, int32_t n_tokens, int32_t n_q_heads, int32_t n_kv_heads,
                                              int32_t head_dim, int32_t *cluster);
 
+/* How the step issued last cuts a layer: cut[0] the attention kernel, cut[1] CTAs of a thread-block cluster (0: no clusters),
+ * cut[2] 1 if a head takes several clusters.  Valid from wnw_step_begin or wnw_graph_begin on until a sequence is placed or
+ * grows. */
+typedef enum {
+  WNW_DEBUG_CUT_PERSISTENT = 0,  /* CTAs that work through several items */
+  WNW_DEBUG_CUT_CLUSTER = 1,     /* the pieces of a head in a cluster */
+  WNW_DEBUG_CUT_SHORT = 2,       /* ... short pieces, one CTA to an SM */
+  WNW_DEBUG_CUT_SHORT_DENSE = 3, /* ... two CTAs to an SM */
+  WNW_DEBUG_CUT_ONE_SHOT = 4,    /* CTAs of one item, eight warps */
+  WNW_DEBUG_CUT_NARROW = 5,      /* ... four warps */
+  WNW_DEBUG_CUT_PACKED = 6       /* eight warps, several heads to a CTA */
+} wnw_debug_cut_t;
+wnw_status_t wnw_debug_get_layer_cut(wnw_cache_t *cache, int32_t layer, int32_t cut[3]);
+
 /* Optional per-kernel timing: when enabled the library brackets its attention-kernel launches with CUDA events
  * on the launching stream; wnw_get_kernel_time returns the accumulated milliseconds and launch count since the
  * last call (drains the stream).  Off by default. */

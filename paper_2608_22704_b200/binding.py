@@ -87,6 +87,7 @@ _SIGNATURES = {
     "wnw_get_kernel_time": [_vp, C.POINTER(C.c_float), C.POINTER(_i32)],
     "wnw_sync": [_vp],
     "wnw_measure_host_link": [_i32, C.c_int64, _i32, C.POINTER(C.c_double), C.POINTER(C.c_double)],
+    "wnw_debug_get_layer_cut": [_vp, _i32, C.POINTER(_i32)],
     "wnw_debug_attend_static_cluster": [_i32, _i32, _i32, _i32, _i32, C.POINTER(_i32)],
     "wnw_attend_static": [_vp, _i32, _i32, _vp, _vp, _i32, _i32, _i32, C.c_float, _i32, _vp],
     "wnw_attend_static_status": [_i32, _vp, C.POINTER(_i32)],
@@ -366,6 +367,17 @@ def wnw_debug_get_slot_padding(cache, seq, layer, kv_head, slot, which, chunk_to
     out = np.zeros((-chunk_tokens % 16, head_dim * elem_bytes), np.uint8)
     _ck(lib().wnw_debug_get_slot_padding(cache, seq, layer, kv_head, slot, which, out.ctypes.data_as(_vp)), "wnw_debug_get_slot_padding")
     return out
+
+
+WNW_DEBUG_CUT_PERSISTENT, WNW_DEBUG_CUT_CLUSTER, WNW_DEBUG_CUT_SHORT, WNW_DEBUG_CUT_SHORT_DENSE, WNW_DEBUG_CUT_ONE_SHOT, WNW_DEBUG_CUT_NARROW, \
+    WNW_DEBUG_CUT_PACKED = range(7)
+
+
+def wnw_debug_get_layer_cut(cache, layer: int):
+    """(WNW_DEBUG_CUT_*, CTAs of a cluster or 0, whether a head takes several clusters) of the step issued last."""
+    cut = (_i32 * 3)()
+    _ck(lib().wnw_debug_get_layer_cut(cache, layer, cut), "wnw_debug_get_layer_cut")
+    return cut[0], cut[1], bool(cut[2])
 
 
 def wnw_get_launch_counts(cache):

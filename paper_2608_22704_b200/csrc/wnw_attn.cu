@@ -1250,15 +1250,27 @@ static cudaError_t launch_cluster(const CacheView &cv, const AttnArgs &a, cudaSt
   if (cv.geo.kv8) return cudaErrorInvalidValue;
   return cv.geo.token_base ? launch_cluster_t<D, G16, 1>(cv, a, st) : launch_cluster_t<D, G16, 0>(cv, a, st);
 }
-// Clusters of the given size that the GPU holds at once (0 if it takes none)
-template <int D, bool G16>
-static int cluster_room_t(int g, int cluster) {
+// Clusters of the launch's size that the GPU holds at once; 0: it takes none of them.  The kernel has to be configured.
+cudaError_t max_active_clusters(const void *kernel, const cudaLaunchConfig_t &cfg, int *n) {
+  *n = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(n, kernel, &cfg);
+  if (e != cudaErrorInvalidClusterSize) return e;
+  cudaGetLastError();
+  return cudaSuccess;
+}
+template <int D, bool G16, int VAR>
+static cudaError_t cluster_room_t(int g, int cluster, int *n) {
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute attr[2];
   cluster_attrs(cfg, attr, g, D, cluster, cluster, false, nullptr);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, wnw_attn_cluster_kernel<D, G16, 0>, &cfg) != cudaSuccess) { cudaGetLastError(); return 0; }
-  return n;
+  cudaError_t e = configure_attn_kernels();
+  return e != cudaSuccess ? e : max_active_clusters((const void *)wnw_attn_cluster_kernel<D, G16, VAR>, cfg, n);
+}
+template <int D, bool G16>
+static cudaError_t cluster_room(int g, bool kv8, bool token_base, int cluster, int *n) {
+  if constexpr (D == 128)
+    if (kv8) return cluster_room_t<D, G16, 2>(g, cluster, n);
+  return token_base ? cluster_room_t<D, G16, 1>(g, cluster, n) : cluster_room_t<D, G16, 0>(g, cluster, n);
 }
 // An SM has 64 K registers, 228 KB of shared memory (1 KB of it kept for every CTA) and 2 048 threads.
 bool recall_room(const void *kernel, int threads, size_t dynamic_smem, int recall_threads) {
@@ -1301,18 +1313,19 @@ bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, AttnForm f
   if (it == known.end()) it = known.emplace(key, find_recall_room(g, d, kv8, token_base, form, crowded ? RECALL_THREADS_CROWDED : RECALL_THREADS)).first;
   return it->second;
 }
-int attn_cluster_room(int device, int g, int d, int cluster, int short_pieces) {   // (an occupancy query takes some 0.2 ms: asked once per shape)
+cudaError_t attn_cluster_room(int device, int g, int d, bool kv8, bool token_base, int cluster, int short_pieces, int *n) {   // (an occupancy query takes some 0.2 ms: asked once per shape)
   static std::mutex mu;
-  static std::map<std::tuple<int, int, int, int, int>, int> known;
+  static std::map<std::tuple<int, int, int, bool, bool, int, int>, int> known;
   std::lock_guard<std::mutex> lock(mu);
-  auto it = known.find({device, g, d, cluster, short_pieces});
-  if (it != known.end()) return it->second;
-  int n;
-  if (short_pieces) n = short_cluster_room(g, d, short_pieces == SHORT_DENSE, cluster);
-  else if (d == 128) n = g > 8 ? cluster_room_t<128, true>(g, cluster) : cluster_room_t<128, false>(g, cluster);
-  else n = g > 8 ? cluster_room_t<64, true>(g, cluster) : cluster_room_t<64, false>(g, cluster);
-  if (n > 0) known[{device, g, d, cluster, short_pieces}] = n;
-  return n;
+  const auto key = std::make_tuple(device, g, d, kv8, token_base, cluster, short_pieces);
+  const auto it = known.find(key);
+  if (it != known.end()) { *n = it->second; return cudaSuccess; }
+  cudaError_t e;
+  if (short_pieces) e = short_cluster_room(g, d, token_base, short_pieces == SHORT_DENSE, cluster, n);
+  else if (d == 128) e = g > 8 ? cluster_room<128, true>(g, kv8, token_base, cluster, n) : cluster_room<128, false>(g, kv8, token_base, cluster, n);
+  else e = g > 8 ? cluster_room<64, true>(g, kv8, token_base, cluster, n) : cluster_room<64, false>(g, kv8, token_base, cluster, n);
+  if (e == cudaSuccess) known[key] = *n;
+  return e;
 }
 
 template <int D, bool G16, int NW>

@@ -590,16 +590,13 @@ struct ShortForm {
     const cudaError_t e = cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem(G16 ? 16 : 8));
     return e != cudaSuccess ? e : cudaFuncSetAttribute(kernel(), cudaFuncAttributeNonPortableClusterSizeAllowed, 1);   // up to 16 CTAs
   }
-  // Clusters of that size that the GPU holds at once; 0: it takes none of them
+  // The answer depends on what the kernel is allowed, so it is configured here and not left to whoever launches it.
   static cudaError_t cluster_room(int g, int cluster, int *n) {
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute attr[2];
     config(cfg, attr, g, cluster, cluster, false, nullptr);
-    *n = 0;
-    const cudaError_t e = cudaOccupancyMaxActiveClusters(n, kernel(), &cfg);
-    if (e != cudaErrorInvalidClusterSize) return e;
-    cudaGetLastError();
-    return cudaSuccess;
+    const cudaError_t e = configure();
+    return e != cudaSuccess ? e : max_active_clusters((const void *)kernel(), cfg, n);
   }
   static bool leaves_recall_room(int g, int rt) { return recall_room((const void *)kernel(), NW_LAT * 32, smem(g), rt); }
 };
@@ -651,18 +648,12 @@ cudaError_t configure_short_kernels(int device, int g, int d, bool token_base) {
   if (e == cudaSuccess) done.insert(key);
   return e;
 }
-// The uniform form that groups of g share is configured by the question for its room, which no launch of it goes without.  One answer
-// for all of the form's groups: 208 registers a thread hold an SM to one CTA.
+// One answer for all groups that share a uniform form: 208 registers a thread hold an SM to one CTA.
 cudaError_t short_uniform_room(int g, int d, int cluster, int *n) {
-  return with_uniform_form(g, d, [&](auto x) {
-    const cudaError_t e = x.configure();
-    return e != cudaSuccess ? e : x.cluster_room(g > 8 ? 16 : 8, cluster, n);
-  });
+  return with_uniform_form(g, d, [&](auto x) { return x.cluster_room(g > 8 ? 16 : 8, cluster, n); });
 }
-int short_cluster_room(int g, int d, bool dense, int cluster) {
-  int n = 0;
-  if (with_form(g, d, false, dense, false, [&](auto x) { return x.cluster_room(g, cluster, &n); }) != cudaSuccess) { cudaGetLastError(); return 0; }
-  return n;
+cudaError_t short_cluster_room(int g, int d, bool token_base, bool dense, int cluster, int *n) {
+  return with_form(g, d, token_base, dense, false, [&](auto x) { return x.cluster_room(g, cluster, n); });
 }
 bool short_leaves_recall_room(int g, int d, bool token_base, bool dense, int recall_threads) {
   return with_form(g, d, token_base, dense, false, [&](auto x) { return x.leaves_recall_room(g, recall_threads); }) &&

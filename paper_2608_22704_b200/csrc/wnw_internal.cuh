@@ -307,7 +307,8 @@ cudaError_t launch_attn_short(const CacheView &cv, const AttnArgs &a, cudaStream
 cudaError_t launch_attn_short_uniform(const CacheView &cv, AttnArgs a, int n_heads, cudaStream_t st);
 cudaError_t configure_short_kernels(int device, int g, int d, bool token_base);
 cudaError_t short_uniform_room(int g, int d, int cluster, int *n);   // clusters of that size, of the allocation-free call, that fit the current device at once
-int short_cluster_room(int g, int d, bool dense, int cluster);
+cudaError_t short_cluster_room(int g, int d, bool token_base, bool dense, int cluster, int *n);
+cudaError_t max_active_clusters(const void *kernel, const cudaLaunchConfig_t &cfg, int *n);
 bool short_leaves_recall_room(int g, int d, bool token_base, bool dense, int recall_threads);
 bool recall_room(const void *kernel, int threads, size_t dynamic_smem, int recall_threads);   // room for a recall CTA on an SM full of that kernel's CTAs
 // the CTAs of several layers' launches (one-shot variant) in one launch
@@ -332,7 +333,8 @@ enum AttnForm { FORM_PERSISTENT, FORM_CLUSTER, FORM_SHORT, FORM_SHORT_DENSE, FOR
 // whether an SM that holds as many CTAs of that form as it can has room left for a recall CTA
 bool attn_leaves_recall_room(int g, int d, bool kv8, bool token_base, AttnForm form, bool crowded);
 constexpr int RECALL_THREADS = 64, RECALL_THREADS_CROWDED = 256, RECALL_REGS_PER_THREAD = 40;   // of a recall CTA (crowded: see launch_recall)
-int attn_cluster_room(int device, int g, int d, int cluster, int short_pieces);   // clusters of that size that fit the GPU at once
+// Clusters of that size, of the kernel that a cache of that kind launches, that fit the current device at once
+cudaError_t attn_cluster_room(int device, int g, int d, bool kv8, bool token_base, int cluster, int short_pieces, int *n);
 int attn_warps(bool throughput);  // warps per attention CTA in the latency / throughput variant
 int attn_persistent_ctas_per_sm(int g, int d);  // persistent (throughput-variant) CTAs that fit one SM
 

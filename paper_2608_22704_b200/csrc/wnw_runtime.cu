@@ -372,17 +372,17 @@ extern "C" wnw_status_t wnw_create(const wnw_config_t *cfg, wnw_cache_t **out) {
 #define CKC(call) do { wnw_status_t _s = (call); if (_s != WNW_OK) return fail(_s); } while (0)
 #define CKE(expr) do { cudaError_t _e = (expr); if (_e != cudaSuccess) { return fail(_e == cudaErrorMemoryAllocation ? WNW_ERR_OOM_DEVICE : WNW_ERR_CUDA); } } while (0)
   cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, cfg->device);
+  const int group = cfg->n_q_heads / cfg->n_kv_heads;
+  const bool kv8 = cfg->mode == WNW_MODE_TIERED && cfg->tidal_kv_format == WNW_TIDAL_KV_FP8_E4M3;
+  const bool token_base = cfg->mode == WNW_MODE_TIERED && cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE;
   CKE(configure_attn_kernels());
-  if (cfg->head_dim == 128 || cfg->head_dim == 64)
-    CKE(configure_short_kernels(cfg->device, cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim,
-                                cfg->mode == WNW_MODE_TIERED && cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE));
+  if (cfg->head_dim == 128 || cfg->head_dim == 64) CKE(configure_short_kernels(cfg->device, group, cfg->head_dim, token_base));
   CKE(configure_select_kernel());
   for (int k = 0; k < 2 * N_ATTN_FORMS; ++k)
-    c->recall_fits_beside[k / N_ATTN_FORMS][k % N_ATTN_FORMS] = attn_leaves_recall_room(cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim,
-                                                       cfg->mode == WNW_MODE_TIERED && cfg->tidal_kv_format == WNW_TIDAL_KV_FP8_E4M3,
-                                                       cfg->residency == WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE, (AttnForm)(k % N_ATTN_FORMS), k >= N_ATTN_FORMS);
+    c->recall_fits_beside[k / N_ATTN_FORMS][k % N_ATTN_FORMS] =
+        attn_leaves_recall_room(group, cfg->head_dim, kv8, token_base, (AttnForm)(k % N_ATTN_FORMS), k >= N_ATTN_FORMS);
   for (int s = 0; s < 3; ++s)
-    for (int k = 0; k < 3; ++k) c->cluster_room[s][k] = attn_cluster_room(cfg->device, cfg->n_q_heads / cfg->n_kv_heads, cfg->head_dim, 4 << k, s);
+    for (int k = 0; k < 3; ++k) CKE(attn_cluster_room(cfg->device, group, cfg->head_dim, kv8, token_base, 4 << k, s, &c->cluster_room[s][k]));
   const int L = cfg->n_layers, Hkv = cfg->n_kv_heads, d = cfg->head_dim, nc = cfg->chunk_tokens;
   const bool full = cfg->mode == WNW_MODE_FULL;
   c->roles.assign(cfg->roles, cfg->roles + (size_t)L * Hkv);
@@ -2158,6 +2158,17 @@ extern "C" wnw_status_t wnw_sync(wnw_cache_t *c) {
   CK(cudaMemcpy(&st, c->cv.status, sizeof(st), cudaMemcpyDeviceToHost));
   if (st & STATUS_TIMEOUT) return WNW_ERR_TIMEOUT;   // a bounded device-side wait ran out (sticky)
   return st ? WNW_ERR_DEVICE_CHECK : WNW_OK;
+}
+
+static_assert(WNW_DEBUG_CUT_PERSISTENT == FORM_PERSISTENT && WNW_DEBUG_CUT_CLUSTER == FORM_CLUSTER && WNW_DEBUG_CUT_SHORT == FORM_SHORT &&
+              WNW_DEBUG_CUT_SHORT_DENSE == FORM_SHORT_DENSE && WNW_DEBUG_CUT_ONE_SHOT == FORM_ONE_SHOT && WNW_DEBUG_CUT_NARROW == FORM_NARROW &&
+              WNW_DEBUG_CUT_PACKED == FORM_PACKED, "");
+extern "C" wnw_status_t wnw_debug_get_layer_cut(wnw_cache_t *c, int32_t layer, int32_t *cut) {
+  if (!c || !cut || layer < 0 || layer >= c->geo.L) return WNW_ERR_INVALID_ARG;
+  if (c->wl_layers.empty()) return WNW_ERR_STATE;
+  const LayerWork &w = c->wl_layers[layer];
+  cut[0] = form_of(w); cut[1] = w.cluster; cut[2] = w.parts;
+  return WNW_OK;
 }
 
 extern "C" wnw_status_t wnw_debug_advance_step_epoch(wnw_cache_t *c, int32_t delta) {

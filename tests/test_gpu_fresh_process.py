@@ -47,3 +47,26 @@ def test_allocation_free_attention_in_clusters_before_any_cache():
         wnw.wnw_destroy(wnw.wnw_create(1, n_q, n_kv, d, 1, 1024, 16, 16, 0.25, np.array([0, 1, 1, 2], np.uint8)))
         assert torch.equal(first, attend())                                   # the same kernel before and after a cache was made
     """)
+
+
+# an anchor of one sequence: one CTA to an SM; of five (five clusters of 16 pieces): two to an SM
+@pytest.mark.parametrize("audio,d,cut", [((2000,), 128, "SHORT"), ((3000,) * 5, 128, "SHORT_DENSE"), ((1500,), 64, "SHORT")])
+def test_short_pieces_of_a_token_base_before_any_other_cache(audio, d, cut):
+    _in_fresh_process(f"""
+        import numpy as np
+        import paper_2608_22704_b200 as wnw
+        from parity_harness import Lockstep
+        from workloads import ROLE_ANCHOR as A, ROLE_FIXED as F, ROLE_TIDAL as T, tiny_custom
+        w = tiny_custom(n_layers=3, n_q_heads=8, n_kv_heads=2, head_dim={d}, n_text=7, audio_lens={audio}, chunk=25, budget=0.2, n_steps=5,
+                        roles=[[A, T], [A, F], [T, A]], region=25, jump_every=2)
+        ls = Lockstep(w, seed=61, oracle_seqs=[0], residency=wnw.WNW_RESIDENCY_SEGMENT_LAG_TOKEN_BASE, evict_lag=1, token_seg=25,
+                      token_retention=np.full((3, 2), 0.2, np.float32))
+        wnw.wnw_set_layer_dependency(ls.h, wnw.WNW_LAYERS_CHAINED)
+        ls.prefill()
+        for t in range(5):
+            ls.decode_step(t, graph=t >= 2)
+        cuts = [wnw.wnw_debug_get_layer_cut(ls.h, l) for l in range(3)]
+        assert [c[0] for c in cuts] == [wnw.WNW_DEBUG_CUT_{cut}] * 3, cuts
+        assert ls.max_out_err <= 2e-2
+        ls.close()
+    """)
