@@ -1596,16 +1596,24 @@ static void plan_step(wnw_cache *c, bool capturing, bool tiered) {
   const bool crowded = recall_crowded(c);
   bool small = true;   // no launch can fill the machine with CTAs that wait
   bool beside = true;
-  int there = 0;
+  int there = 0, most = 0;
+  long long all = 0;
   for (const LayerWork &w : c->wl_layers) {
     const int n = w.n_ctas > 0 ? w.n_ctas : w.n_items;
     const int wait = together ? n - (w.packed ? w.n_ctas_free : 0) : layers_overlap(c) ? std::min(n, w.n_tidal_items + 1) : n;
-    // (Half the SMs; of short pieces two to an SM 5/8: chained, inside and half behind the step / all behind it, 80 CTAs a layer 203 / 195 us a
-    // step of 36 layers and 213 / 209 of 30, 96 CTAs 162 / 164, 144 CTAs 223 / 237.)
+    // (Half the SMs; of short pieces two to an SM 5/8.  n counts the idle places of clusters too: the lines below were measured so.)
     small = small && !w.throughput && n <= (w.short_pieces == SHORT_DENSE ? c->n_sm * 5 / 8 : c->n_sm / 2);
+    most = std::max(most, n);
+    all += n;
     beside = beside && c->recall_fits_beside[crowded][together ? FORM_TOGETHER : form_of(w)];
     there = c->layer_dependency == WNW_LAYERS_SERIAL ? std::max(there, wait) : there + wait;
   }
+  // Between half and 5/8 what counts in a replayed step is whether the layers are so large on average or a few of them between
+  // small ones.  Half of the recall inside / all of it behind, us a step: 30 alike layers of 80 CTAs (2 x 3000 tokens) 149 / 163, with
+  // a jumping focus 229 / 270, 4 x 1000 160 / 192, 8 x 1500 of 2 KV heads 153 / 158, 12 layers 80 / 85, 4 layers 50 / 51, 3 layers
+  // 46.4 / 45.5; 36 layers of at most 80 and 48 on average 202 / 197 (15000 tokens), 247 / 237 (16 query heads a KV head), 216 / 206 (4 x
+  // 4000; with a fast focus 219 / 260).  A step issued call by call has no halves: inside / behind 444 / 205.
+  small = small && (!capturing || most <= c->n_sm / 2 || all <= (long long)G.L * c->n_sm / 2);
   small = small && (beside || there < c->n_sm);
   const bool ours = tiered && c->cfg.recall_mode != WNW_RECALL_INLINE && !c->cfg.defer_selection && (!capturing || c->graph_capturing);
   const int n_select = c->select_single_ok ? c->sel_map_single[1] : c->sel_map_update[1];

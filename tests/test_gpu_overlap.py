@@ -265,6 +265,17 @@ def test_chained_one_shot_launches_that_fill_the_machine_split_their_recall():
     assert (eager[2], replayed[2]) == (4, 5 * 3)
 
 
+@pytest.mark.parametrize("alike", [True, False])
+def test_replayed_layers_of_more_ctas_than_half_the_sms_split_their_recall_if_all_are(alike):
+    """Two sequences of short pieces, 80 CTAs a layer where it has an anchor head, 64 where not.  Replayed, half of the four layers
+    recalls inside the step where all have one; where only the first has, and in an eager step, recall follows the step."""
+    anchored, other = [ROLE_ANCHOR] + [ROLE_TIDAL] * 5 + [ROLE_FIXED] * 2, [ROLE_TIDAL] * 6 + [ROLE_FIXED] * 2
+    w = tiny_custom(n_layers=4, n_q_heads=32, n_kv_heads=8, head_dim=128, n_text=14, audio_lens=(3000, 2950), chunk=64, budget=0.2, n_steps=6,
+                    roles=[anchored] + [anchored if alike else other] * 3, region=64, jump_every=2)
+    eager, replayed = _replays(w, wnw.WNW_LAYERS_CHAINED, 5, 14)
+    assert (eager[2], replayed[2]) == (1, 5 * (3 if alike else 1))
+
+
 def test_selection_waits_for_the_recall_only_beside_free_sms():
     """All layers together, eight query heads a KV head (packed CTAs take all of an SM's shared memory): with as many selection
     and tidal CTAs as SMs the selection follows the attention instead of waiting beside it: two attention launches a step (three
