@@ -10,6 +10,12 @@ from workloads import ROLE_ANCHOR as A, ROLE_FIXED as F, ROLE_TIDAL as T, Synth,
 from workloads.synth import bf16_bits
 
 pytestmark = pytest.mark.gpu
+CLUSTER, WIDE, DENSE = wnw.WNW_DEBUG_CUT_CLUSTER, wnw.WNW_DEBUG_CUT_SHORT, wnw.WNW_DEBUG_CUT_SHORT_DENSE
+
+
+def _cuts(ls):
+    """Per layer: the attention kernel, CTAs of a cluster, whether a head takes several clusters."""
+    return [wnw.wnw_debug_get_layer_cut(ls.h, l) for l in range(ls.w.n_layers)]
 
 
 # audio tokens: one granule; a head of one piece and one of two (256 keys a piece); 16 pieces; more than 16 pieces' worth
@@ -32,13 +38,16 @@ def test_chained_layers_clustered_pieces(n_q, n_kv, d, audio, mode):
         ls.close()
 
 
-# Short pieces of one and of two CTAs to an SM (the fourth cluster of 16 decides): one piece and 16 of 16 granules exactly, one granule
-# more, groups with padding heads, the new token's row in either half of a granule and across two; chunks that fill granules partly
-@pytest.mark.parametrize("n_q,n_kv,d,chunk,audio,n_text", [
-    (8, 2, 128, 16, (224,), 6), (8, 2, 128, 16, (4064,), 14), (8, 2, 128, 16, (4065,), 14),                  # wide; 16 pieces; beyond
-    (12, 4, 128, 16, (4000, 3900, 17), 6), (8, 4, 64, 16, (4064, 4064, 900, 60), 15), (64, 4, 128, 16, (2000,) * 4, 7),   # dense
-    (64, 4, 64, 25, (1500, 2500, 1700, 26), 13), (10, 2, 128, 25, (1990,) * 8, 7), (5, 5, 64, 16, (300,), 0)])
-def test_chained_layers_of_short_pieces(n_q, n_kv, d, chunk, audio, n_text):
+# Short pieces of one and of two CTAs to an SM: one piece and 16 of 16 granules exactly, one granule more (the cut of longer pieces),
+# groups with padding heads, the new token's row in either half of a granule and across two; chunks that fill granules partly
+@pytest.mark.parametrize("n_q,n_kv,d,chunk,audio,n_text,form", [
+    (8, 2, 128, 16, (224,), 6, WIDE), (8, 2, 128, 16, (4064,), 14, WIDE), (8, 2, 128, 16, (4065,), 14, CLUSTER), (5, 5, 64, 16, (300,), 0, WIDE),
+    (12, 4, 128, 16, (4000, 3900, 3000, 17), 6, DENSE), (8, 4, 64, 16, (4064, 4064, 4064, 60), 15, DENSE),
+    (64, 4, 64, 25, (2500, 2500, 2500, 26), 13, DENSE), (10, 2, 128, 25, (1990,) * 8, 7, DENSE),
+    (12, 4, 128, 16, (4000, 3900, 17), 6, None), (8, 4, 64, 16, (4064, 4064, 900, 60), 15, None),   # near the line between the two
+    (64, 4, 64, 25, (1500, 2500, 1700, 26), 13, None),
+    (64, 4, 128, 16, (2000,) * 4, 7, None)])   # 16 query heads a KV head of 128: one kernel for both
+def test_chained_layers_of_short_pieces(n_q, n_kv, d, chunk, audio, n_text, form):
     from parity_harness import Lockstep
     roles = [[(A, T, F, T, A)[(h + l) % 5] for h in range(n_kv)] for l in range(3)]
     w = tiny_custom(n_layers=3, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=d, n_text=n_text, audio_lens=audio, chunk=chunk, budget=0.25, n_steps=6,
@@ -49,16 +58,21 @@ def test_chained_layers_of_short_pieces(n_q, n_kv, d, chunk, audio, n_text):
         ls.prefill()
         for t in range(6):
             ls.decode_step(t, graph=t >= 2)
+        cuts = _cuts(ls)
+        assert cuts[0][0] == form or form is None and cuts[0][0] in (WIDE, DENSE), cuts   # the first layer has an anchor of every sequence
+        assert all(c[0] in (WIDE, DENSE) for c in cuts[1:]) and not any(c[2] for c in cuts), cuts
         assert ls.max_out_err <= 2e-2
     finally:
         ls.close()
 
 
-# Heads of more than 384 granules take several clusters: one granule less and more, five clusters, a part of a batch; token bases
-@pytest.mark.parametrize("n_q,n_kv,d,chunk,audio,n_text,residency", [
-    (8, 2, 128, 16, (6112,), 6, 0), (8, 2, 128, 16, (6144, 40), 6, 0), (10, 2, 128, 64, (17000,), 14, 0), (32, 2, 128, 16, (6200,), 7, 0),
-    (32, 2, 64, 16, (9000, 300, 6300), 3, 0), (8, 2, 64, 25, (5000,), 15, 2), (8, 2, 128, 25, (5300, 700), 7, 2)])
-def test_chained_heads_of_several_clusters(n_q, n_kv, d, chunk, audio, n_text, residency):
+# Heads of more than 384 granules take several clusters: one granule less (the cut of longer pieces) and more, five clusters, ten, a
+# part of a batch; token bases
+@pytest.mark.parametrize("n_q,n_kv,d,chunk,audio,n_text,residency,several", [
+    (8, 2, 128, 16, (6112,), 6, 0, False), (8, 2, 128, 16, (6144, 40), 6, 0, True), (10, 2, 128, 64, (17000,), 14, 0, True),
+    (32, 2, 128, 16, (6200,), 7, 0, True), (32, 2, 64, 16, (9000, 300, 6300), 3, 0, True), (8, 2, 64, 25, (5000,), 15, 2, True),
+    (8, 2, 128, 25, (5300, 700), 7, 2, True), (8, 2, 64, 16, (40000,), 27, 0, True), (8, 2, 128, 16, (40000,), 27, 0, True)])
+def test_chained_heads_of_several_clusters(n_q, n_kv, d, chunk, audio, n_text, residency, several):
     from parity_harness import Lockstep
     w = tiny_custom(n_layers=3, n_q_heads=n_q, n_kv_heads=n_kv, head_dim=d, n_text=n_text, audio_lens=audio, chunk=chunk, budget=0.2, n_steps=5,
                     roles=[[A, T], [T, F], [F, A]], region=chunk, jump_every=2)
@@ -69,24 +83,35 @@ def test_chained_heads_of_several_clusters(n_q, n_kv, d, chunk, audio, n_text, r
         ls.prefill(check_slots=False)
         for t in range(5):
             ls.decode_step(t, graph=t >= 2)
+        cuts = _cuts(ls)
+        for l in (0, 2):   # the layers with an anchor
+            assert (cuts[l][0] in (WIDE, DENSE) and cuts[l][2]) if several else cuts[l] == (CLUSTER, 16, False), cuts
         assert ls.max_out_err <= 2e-2
     finally:
         ls.close()
 
 
-# 1408 granules, 3 of them text, are the longest head whose pieces share a cluster; layers without a long head stay clustered
-@pytest.mark.parametrize("audio,d", [((22480,), 64), ((22481,), 64), ((22600, 500), 128), ((40000,), 128)])
-def test_chained_layers_around_the_longest_clustered_head(audio, d):
+# Longer pieces: 1408 granules, 3 of them text, are the longest head whose pieces share a cluster, in an e4m3 tier and where the
+# short pieces of the long heads do not fit; alone they take several clusters.  Layers without a long head stay clustered
+@pytest.mark.parametrize("audio,d,fp8,cut", [
+    ((22480,), 128, True, "cluster"), ((22481,), 128, True, "none"), ((22600, 500), 128, True, "none"), ((40000,), 128, True, "none"),
+    ((22480,) * 3, 64, False, "cluster"), ((22481, 22000, 22000), 64, False, "none"), ((22481,) * 3, 128, False, "none"),
+    ((22480,), 64, False, "several"), ((22481,), 64, False, "several"), ((22600, 500), 128, False, "several"), ((40000,), 128, False, "several")])
+def test_chained_layers_around_the_longest_clustered_head(audio, d, fp8, cut):
     from parity_harness import Lockstep
     w = tiny_custom(n_layers=4, n_q_heads=8, n_kv_heads=2, head_dim=d, n_text=27, audio_lens=audio, chunk=16, budget=0.1, n_steps=6,
                     roles=[[A, T], [T, F], [T, A], [T, T]], region=16, jump_every=2)
-    ls = Lockstep(w, seed=47, gen_device="cuda:0")
+    ls = Lockstep(w, seed=47, gen_device="cuda:0", oracle_seqs=None if len(audio) < 3 else [0], kv_fp8=fp8)
     try:
         wnw.wnw_set_layer_dependency(ls.h, wnw.WNW_LAYERS_CHAINED)
         ls.prefill(check_slots=False)
         for t in range(6):
             ls.decode_step(t, graph=t >= 2, check_slots=(t == 5))
         ls.check_stats()
+        cuts = _cuts(ls)
+        for l in (0, 2):   # the layers with an anchor
+            assert cuts[l] == (CLUSTER, 16, False) if cut == "cluster" else cuts[l][1] == 0 if cut == "none" else cuts[l][2], cuts
+        assert all(cuts[l][1] > 0 for l in (1, 3)), cuts
         assert ls.max_out_err <= 2e-2
     finally:
         ls.close()
@@ -122,6 +147,8 @@ def test_static_attention_in_clusters(n_q, n_kv, d):
         K, V, Q = (bf16_bits_to_f64(bf16_bits(x.contiguous())) for x in (kv[:, 0, :n], kv[:, 1, :n], q))
         want = np.stack([dense_attention(Q[h], K[h * n_kv // n_q], V[h * n_kv // n_q], 1.0 / np.sqrt(d))[0] for h in range(n_q)])
         assert np.abs(out.float().cpu().numpy() - want).max() <= 2e-2, n   # bf16 weights and outputs of O(1)
+        pieces = -(-n // 256)
+        assert wnw.wnw_debug_attend_static_cluster(n, n_q, n_kv, d) == (4 if pieces <= 4 else 8 if pieces <= 8 else 16 if pieces <= 16 else 0)
     assert not wnw.wnw_attend_static_status()
 
 
