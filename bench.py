@@ -631,12 +631,18 @@ def chained_batch_sweep(wnw, dev, batches, audio_tokens, steps=8, warm=3):
             "smallest_batch_with_wnw_below_full_cache": min(below) if below else None}
 
 
-def attention_kernel(w, dep, eager):
-    """The kernel that carries a decode step's attention: all layers in three launches; one wave of clusters (layers that wait for
-    one another, a single sequence of up to 22 000 tokens); one-shot or persistent CTAs."""
+def attention_kernel(w, dep, eager, kv_fp8=False):
+    """The kernel that carries a decode step's attention: all layers in three launches; layers that wait for one another, a single
+    sequence, in clusters of short pieces or, of 257 to 384 granules a head and with an e4m3 tier, of longer ones (up to 1408
+    granules); one-shot or persistent CTAs."""
     if dep == 3 and not eager:
         return "wnw_attn_multi_kernel"
-    return "wnw_attn_cluster_kernel" if dep in (1, 2) and w.batch == 1 and max(w.audio_lens) <= 22000 else "wnw_attn_kernel"
+    if dep not in (1, 2) or w.batch > 1:
+        return "wnw_attn_kernel"
+    granules = -(-w.text_capacity // 16) + -(-max(w.audio_lens) // w.chunk) * -(-w.chunk // 16)
+    if not kv_fp8 and not 256 < granules <= 384:
+        return "wnw_attn_short_kernel"
+    return "wnw_attn_cluster_kernel" if granules <= 1408 else "wnw_attn_kernel"
 
 
 def run_ours(args, rank, world, local_rank):
@@ -931,7 +937,7 @@ def run_ours(args, rank, world, local_rank):
         # layer, each waiting for its predecessor, so the share of one is step time / layers).  The other issue forms are
         # reported under their names: `upper_bound_all_layers_together` needs every layer's q before the step starts (no
         # decoder whose layers feed one another can run it), `per_layer_overlapped` likewise; `serial` is plain stream order.
-        "roofline": {"bound": "hbm", "kernel": attention_kernel(w, DEP, args.eager),
+        "roofline": {"bound": "hbm", "kernel": attention_kernel(w, DEP, args.eager, Job.kv_fp8),
                      "achieved": region_achieved, "peak": peak_gbs, "unit": "GB/s",
                      "frac": region_achieved / peak_gbs, "peak_kind": f"of {peak_kind}", "traffic": traffic,
                      "bytes_per_launch": region_bytes_per_launch, "us_per_launch": region_us_per_launch,

@@ -541,20 +541,16 @@ __device__ __forceinline__ void short_body(const CacheView &cv, const AttnArgs &
   finish();
 }
 
-namespace short_pieces {   // (beside the kernel of that name for longer pieces)
-
 template <int D, bool G16, bool TB, bool DENSE, bool PARTS>
-__global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_cluster_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
-                                                                       const __grid_constant__ TmaMaps maps) {
+__global__ void __maxnreg__(DENSE ? 120 : 208) wnw_attn_short_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
+                                                                     const __grid_constant__ TmaMaps maps) {
   short_body<D, G16, TB, DENSE, PARTS, false>(cv, a, maps);
 }
 template <int D, bool G16>
-__global__ void __maxnreg__(208) wnw_attn_cluster_uniform_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
+__global__ void __maxnreg__(208) wnw_attn_short_uniform_kernel(const __grid_constant__ CacheView cv, const __grid_constant__ AttnArgs a,
                                                                const __grid_constant__ TmaMaps maps) {
   short_body<D, G16, false, false, false, true>(cv, a, maps);
 }
-
-}  // namespace short_pieces
 
 // ---- host: one list of the forms there are ----
 namespace {
@@ -563,8 +559,8 @@ template <int D, bool G16, bool TB, bool DENSE, bool PARTS, bool UNI = false>
 struct ShortForm {
   typedef ShortShape<D, G16, DENSE> X;
   static auto kernel() {
-    if constexpr (UNI) return short_pieces::wnw_attn_cluster_uniform_kernel<D, G16>;
-    else return short_pieces::wnw_attn_cluster_kernel<D, G16, TB, DENSE, PARTS>;
+    if constexpr (UNI) return wnw_attn_short_uniform_kernel<D, G16>;
+    else return wnw_attn_short_kernel<D, G16, TB, DENSE, PARTS>;
   }
   static size_t smem(int g) { return (size_t)X::STAGES_B + X::P_B + (size_t)((g + 1) / 2 * (D / 2) + 16) * 16 + 8 * 16 * 16 + 1024; }
   static void config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int g, int n_ctas, int cluster, bool pdl, cudaStream_t st) {

@@ -42,7 +42,8 @@ def test_roofline_names_the_kernel_that_the_step_launches():
     import bench
     one, many = bench.make_workload("cfg1", 4, 0), bench.make_workload("hbm", 4, 0)
     assert [bench.attention_kernel(one, dep, False) for dep in (0, 1, 2, 3)] == [
-        "wnw_attn_kernel", "wnw_attn_cluster_kernel", "wnw_attn_cluster_kernel", "wnw_attn_multi_kernel"]
+        "wnw_attn_kernel", "wnw_attn_short_kernel", "wnw_attn_short_kernel", "wnw_attn_multi_kernel"]
+    assert bench.attention_kernel(one, 1, False, kv_fp8=True) == "wnw_attn_cluster_kernel"
     assert bench.attention_kernel(many, 1, False) == "wnw_attn_kernel" == bench.attention_kernel(one, 3, True)
     traffic = json.load(open(os.path.join(ROOT, "profiles", "attn_traffic.json")))
     assert bench.attention_kernel(one, 1, False) in traffic["source"] and traffic[one.name] > 0
