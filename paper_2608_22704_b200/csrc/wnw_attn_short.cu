@@ -14,8 +14,9 @@
 //   - (maximum, denominator) of the piece leave ahead of P V, so that the weights of the pieces are ready when the accumulators
 //     arrive; the softmax-mass partials of anchor heads are added up while these travel.
 // From the inputs to the output a piece takes 4 200 cycles: query 600 to 1 050 (near and far half of L2), K q^T 330 (mma.sync at its
-// rate: 16 a warp, two warps a scheduler), softmax 650, P V 760, exchange 820, last sums 400.  Config 1, 30 chained layers with the
-// program's copies: 154 -> 140 us a step; 16 query heads a KV head 235 -> 174; the paper's form 204 -> 154.
+// rate: 16 a warp, two warps a scheduler), softmax 650, P V 760, exchange 820, last sums 400.  30 chained layers of 3000
+// tokens with the program's copies: 149 -> 136 us a step; the paper's form 207 -> 156; 16 query heads a KV head 235 -> 174.  Registers: wide
+// forms 148 to 197, dense ones 107 to 120 (bounds 208 and 120; of those only the ones of 16 query heads a KV head of 64 spill, 12 bytes).
 // tcgen05 does not pay here: with 8 to 16 query heads its M = 128, N = 16, K = 16 steps take 50 to 59 cycles each (485 to 567 for
 // 128 tokens), where mma.sync needs 256 for 256 tokens with its operands in registers.
 #include <mutex>

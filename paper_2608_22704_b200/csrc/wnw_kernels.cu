@@ -332,7 +332,9 @@ cudaError_t launch_select(const CacheView &cv, const SelectArgs &a, size_t smem_
 // 40 registers a thread.  48 warps, two to a CTA (one fits beside an 8-warp attention CTA of up to 240 registers, two of up to 120),
 // where layers wait for one another: the copies have the whole next step's time, and the step's own small copies and launches share
 // the link (30 chained layers with the program's copies, 1 / 2 / 4 x 3000 tokens, us a step: 64 warps 139.6 / 165.6 / 221, 48 warps
-// 136.9 / 166.8 / 213, 32 warps 135.2 / 172 / 210, 24 warps 138 / 188 / 220).  192 warps, eight to a CTA (on 96 SMs
+// 136.9 / 166.8 / 213, 32 warps 135.2 / 172 / 210, 24 warps 138 / 188 / 220), and the same where the
+// layers wait for all of it (recall in line with them: 64 and 48 warps 579 and 582 us a step, one small layer call by call 26 and 26;
+// four sequences call by call, recall beside the layers of the same step, 572 and 556).  192 warps, eight to a CTA (on 96 SMs
 // instead of 24 they disturb attention: 16 ragged sequences 49.7 -> 50.4 ms a request), where attention keeps the memory system busy
 // (overlapping layers, persistent CTAs): a host read takes several times as long then and the step waits for it (4 x 3000 tokens,
 // overlapping: 225 us a step with 64, 197 with 128, 193 with 192, 194 with 256, 198 with 384; 206 with 1 024).

@@ -693,10 +693,11 @@ static void head_granules(const wnw_cache *c, int layer, int mode, const SeqHost
 constexpr int CLUSTER_MAX_PER_WARP = 8;   // granules: with more, persistent CTAs are the better cut (8 x 3000 tokens, 12 layers: 206 us at 8, 234 at 4)
 // Granules a warp of the longest head: a cluster holds 16 pieces, so a long head's warps walk ever more granules one after
 // another, where the cuts that merge through global memory (one-shot: 32 pieces a head; persistent) take half as many and pay
-// some 2.5 us for the merge.  Chained, one sequence, us a layer, cluster / other cut: 2 KV heads of 128 elements (anchor and
-// tidal) at 8 000 tokens 9.0 / 11.9, 20 000 (10 granules) 15.3 / 16.0, 24 000 (12) 18.0 / 17.7, 32 000 (16) 22.1 / 19.9, 60 000
-// 37.3 / 28.7; 8 KV heads at 20 000 15.3 / 15.8, 24 000 17.4 / 16.2, 32 000 21.4 / 18.6; 4 KV heads of 64 at 20 000 11.5 / 11.8,
-// 24 000 13.1 / 12.6.  The lines cross between 9 (e4m3) and 14 (full cache, 2 KV heads).
+// some 2.5 us for the merge.  What takes this cut at such lengths: e4m3 tiers, and bf16 heads whose short pieces do not fit.  Chained, 12
+// layers, us a layer, cluster / other cut, at 16 000 (8 granules) / 20 000 (10) / 24 000 (12) / 32 000 tokens (16): e4m3, 8 KV heads
+// 15.5 / 16.2, 17.9 / 17.1, 20.2 / 18.7, 25.0 / 20.9; e4m3, 2 KV heads 9.8 / 13.0, 11.3 / 13.8, 12.0 / 14.5, 14.6 / 16.5; bf16, 8 KV heads
+// 18.1 / 17.7 (20 000), 19.4 / 18.3, 23.8 / 20.8; four sequences of 2 KV heads 12.1 / 13.0, 15.5 / 17.6, 16.4 / 19.9, 19.2 / 22.4.  The
+// lines cross between 9 granules and, with few heads, beyond 16.
 constexpr int CLUSTER_LONGEST_PER_WARP = 11;
 struct CutMemo {   // piece sizes found for one work list, by the launch's head sizes
   struct Entry { std::vector<int> sizes; double T; };
@@ -833,13 +834,13 @@ static void build_throughput_items(const wnw_cache *c, int layer, int mode, cons
 // Short pieces: heads in pieces of at most 16 granules (wnw_attn_short.cu), as wide CTAs (one to an SM, all fragments ahead
 // of the query) where the clusters of two layers fit the GPU side by side, so that a layer's bytes land while its predecessor runs;
 // else dense ones, two to an SM.  Chained, us a replayed step of 30 layers, 32 query heads on 8 KV heads of 128, wide / dense / the
-// cut below: 3000 tokens (3 clusters of 16) 140 / 146 / 154; 2 x 3000 (6) 206 / 157 / 225; 4 x 1000 196 / 163 / 211; the paper's form
-// (4) 182 / 154 / 204; 1000 tokens, full cache (8 clusters of 8) 117 / 127 / 132.
+// cut below: 3000 tokens (3 clusters of 16) 136 / 140 / 149; 2 x 3000 (5) 197 / 150 / 218; 4 x 1000 186 / 162 / 207; the paper's form
+// (4) 182 / 156 / 207; 1000 tokens, full cache (8 clusters of 8) 118 / 128 / 134.
 //
 // A head of more than 16 pieces takes several clusters, which meet in global memory (some 1 us: a fence, a counter, the last piece
-// reads).  That pays from the fourth granule on that a warp of the cut below would walk: 5000 tokens (3 a warp) 202 / 200 us a step,
-// 6000 243 / 209, 8000 245 / 210, 15000 355 / 279, 2 x 8000 355 / 268; 2 KV heads x 15000, 36 layers, 246 / 193; 4 KV heads of 64 x
-// 15000 353 / 240 (the cut below / several clusters).
+// reads).  That pays from the fourth granule on that a warp of the cut below would walk: 5000 tokens (3 a warp) 200 / 202 us a step,
+// 6000 238 / 206, 8000 236 / 205, 15000 340 / 262, 2 x 8000 340 / 260; 2 KV heads x 15000, 36 layers, 250 / 198; 4 KV heads of 64 x
+// 15000 295 / 197 (the cut below / several clusters).
 //
 // Chained or serial layers whose work fits one wave: the pieces of a head form (part of) a cluster and merge inside it, which
 // costs little however many there are, so heads are cut as fine as fits: two granules a warp (all bytes of a piece in flight
