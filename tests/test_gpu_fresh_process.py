@@ -70,3 +70,24 @@ def test_short_pieces_of_a_token_base_before_any_other_cache(audio, d, cut):
         assert ls.max_out_err <= 2e-2
         ls.close()
     """)
+
+
+def test_first_allocation_free_call_inside_a_capture():
+    _in_fresh_process("""
+        import torch
+        import paper_2608_22704_b200 as wnw
+        gen = torch.Generator().manual_seed(7)
+        kv = torch.randn(4, 2, 784, 64, generator=gen).to(torch.bfloat16).cuda()
+        q = torch.randn(8, 64, generator=gen).to(torch.bfloat16).cuda()
+        outs = [torch.zeros_like(q) for _ in range(2)]
+        graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=stream):
+            wnw.wnw_attend_static(kv, 777, q, outs[0], stream=stream)
+        graph.replay()
+        torch.cuda.synchronize()
+        wnw.wnw_attend_static(kv, 777, q, outs[1])
+        assert wnw.wnw_debug_attend_static_cluster(777, 8, 4, 64) == 4
+        assert not wnw.wnw_attend_static_status()
+        assert torch.equal(*outs) and outs[0].abs().max() > 0
+    """)
